@@ -196,6 +196,17 @@ static int choose_pipe_variant(const ConvParams& p, int sms) {
     return -1;
 }
 
+// Smaller layers with a deep reduction (a classifier-side 3x3 layer at batch 1-16 has 4-100 output tiles of 72-144
+// reduction words): the pipeline kernel with its narrowest channel tile, which gives the most thread blocks and walks the
+// words with all roles overlapped.  512 -> 512 3x3 at 7x7, batch 1: 66.8 -> 17.5 us; 1024 -> 256 1x1 at 14x14, batch 16:
+// 25.4 -> 10.3 us.  Below 18 words the warp-level kernels are as fast or faster (256 -> 1024 1x1 at 14x14: 5.5 against
+// 6.7 us), and layers of one wave of warp-level strip tiles (128 -> 128 3x3 at 28x28: 7.8 against 9.0 us) stay there.
+static int choose_deep_pipe_variant(const ConvParams& p) {
+    const int kwords = (p.KK + p.fold - 1) / p.fold;
+    if (p.Co < 64 || p.w_levels || kwords < 18) return -1;
+    return conv_umma_pipe_applies(p, 0) ? 0 : -1;
+}
+
 static int choose_umma_variant(const ConvParams& p, const ebs_conv_desc* d) {
     const int kwords = (p.KK + p.fold - 1) / p.fold;
     const long long outputs = (long long)p.P * p.Co;
@@ -297,7 +308,9 @@ static int conv_plan(const void* packed_x, int n, int h, int w, const void* pack
     if (variant == -2) {
         variant = choose_variant(d->w_bits, d->a_bits, p.P, p.Co, packed_next != nullptr, sm_count());
     } else if (variant < 0) {
-        const int pipe = mma_ok ? choose_pipe_variant(p, sm_count()) : -1;
+        int pipe = mma_ok ? choose_pipe_variant(p, sm_count()) : -1;
+        const bool one_wave_strip = p.Co > 64 && p.Co <= 128 && d->kh * d->kw > 1 && p.P < (1 << 10) && conv_mma_strip_applies(p, 1);
+        if (mma_ok && pipe < 0 && !one_wave_strip && !(p.Co <= 64 && conv_mma_strip_applies(p, 1))) pipe = choose_deep_pipe_variant(p);
         const int strip = (mma_ok && pipe < 0) ? choose_strip_variant(p) : -1;
         const int umma = (mma_ok && strip < 0 && pipe < 0) ? choose_umma_variant(p, d) : -1;
         // deep reductions whose weight tiles fit in shared memory: the persistent form of the same tile
@@ -314,6 +327,7 @@ static int conv_plan(const void* packed_x, int n, int h, int w, const void* pack
         else if (mma_ok && p.Co > 16 && p.Co <= 32 && d->kh * d->kw > 1 && conv_mma_strip_applies(p, 1)) variant = MS_BASE + 1;
         else if (mma_ok && p.Co > 32 && p.Co <= 64 && d->kh * d->kw > 1 && p.P < (1 << 13) && conv_mma_strip_applies(p, 1))
             variant = MS_BASE + 1;
+        else if (mma_ok && one_wave_strip) variant = MS_BASE + 1;
         else if (mma_ok && p.Co > 32 && p.Co <= 64 && d->kh * d->kw > 1 && conv_mma_strip_applies(p, 2))
             variant = MS_BASE + 2;
         else variant = mma_ok ? NUM_CONV_VARIANTS + choose_mma_variant(d->w_bits, d->a_bits, p.P, p.Co, sm_count())

@@ -482,6 +482,22 @@ int ebs_conv2d_mixed_host_noalloc(const void *x_host, int dtype, int layout, int
                                   void *stream);
 
 /*
+ * Replaying a fixed sequence of calls of this library as one launch (a CUDA graph); the paper has no counterpart.
+ *   ebs_graph_begin    creates a capture stream and starts recording on it; pass that stream to the calls to record.
+ *                      Every kernel must have run once before (first calls load code and look up device addresses).
+ *   ebs_graph_end      stops recording, instantiates the sequence and destroys the capture stream.  A null graph_exec
+ *                      discards the recording (after a call that failed).
+ *   ebs_graph_launch   enqueues the recorded sequence on `stream`, with the addresses and sizes it was recorded with;
+ *                      EBS_ERR_UNSUPPORTED while `stream` itself is being captured (issue the calls one by one then).
+ *   ebs_graph_destroy  frees it; launches in flight finish.
+ * The handle belongs to the caller and to the device that was current at ebs_graph_begin.
+ */
+int ebs_graph_begin(void **capture_stream);
+int ebs_graph_end(void *capture_stream, void **graph_exec);
+int ebs_graph_launch(void *graph_exec, void *stream);
+int ebs_graph_destroy(void *graph_exec);
+
+/*
  * Register-resident throughput probe of the execution pipes the convolution can use; the
  * measured rate is the denominator of the kernel's arithmetic roofline.  Runs `iters` loop
  * iterations on every SM, synchronizes the device, and writes the measured rate.

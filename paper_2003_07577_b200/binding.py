@@ -1,7 +1,9 @@
 """Thin ctypes binding of libebs.so: argument marshalling only.
 
 Every function has the name and argument order of its C entry point in ``include/ebs.h`` and
-does no arithmetic of its own.  Tensors are ``torch.Tensor`` objects used purely as device (or
+does no arithmetic of its own.  The calls made once per layer or batch go through the CPython
+extension ``_fastcall`` (csrc/fastcall.c: same functions, a fifth of the marshalling time), the
+others through ctypes.  Tensors are ``torch.Tensor`` objects used purely as device (or
 pinned host) memory: the binding passes ``tensor.data_ptr()`` and the current CUDA stream.
 There is no CPU fallback: if the shared library is missing, loading raises.
 """
@@ -31,6 +33,7 @@ EXPORTS = [
     "ebs_conv_variant_family", "ebs_conv_variant_applies", "ebs_check_device_status", "ebs_test_set_device_wait",
     "ebs_conv2d_i8", "ebs_maxpool_packed", "ebs_combined_scale", "ebs_reciprocal_step",
     "ebs_checked_build", "ebs_checked_status", "ebs_test_checked_shrink", "ebs_pack_acts_s2d",
+    "ebs_graph_begin", "ebs_graph_end", "ebs_graph_launch", "ebs_graph_destroy",
 ]
 
 
@@ -116,8 +119,31 @@ def lib() -> ctypes.CDLL:
         L.ebs_conv_variant_applies.argtypes = [D, i, i, i, E, i, i, i, i]
         L.ebs_check_device_status.restype = i
         L.ebs_test_set_device_wait.argtypes = [ctypes.c_uint, i]
+        L.ebs_graph_begin.argtypes = [ctypes.POINTER(p)]
+        L.ebs_graph_end.argtypes = [p, ctypes.POINTER(p)]
+        L.ebs_graph_launch.argtypes = [p, p]
+        L.ebs_graph_destroy.argtypes = [p]
         _lib = L
     return _lib
+
+
+_fast = None
+
+
+def _native():
+    """The CPython extension, bound to the loaded library's functions on first use; raises if it is not built."""
+    global _fast
+    if _fast is None:
+        from . import _fastcall
+        L = lib()
+        names = ("ebs_pack_acts", "ebs_pack_acts_s2d", "ebs_conv2d_mixed", "ebs_conv2d_mixed_variant", "ebs_dequant",
+                 "ebs_global_avgpool", "ebs_maxpool_packed", "ebs_resnet_cifar_forward", "ebs_search_weight_forward",
+                 "ebs_search_act_forward", "ebs_graph_launch")
+        torch.cuda.init()                                  # the stream lookups below need torch's CUDA state
+        _fastcall.bind({k: ctypes.cast(getattr(L, k), ctypes.c_void_p).value for k in names},
+                       torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+        _fast = _fastcall
+    return _fast
 
 
 def _ptr(t: Optional[torch.Tensor]):
@@ -186,21 +212,17 @@ def ebs_pack_weights(w_dev: torch.Tensor, dtype: int, layout: int, desc: ebs_con
 
 def ebs_pack_acts(x_dev: torch.Tensor, dtype: int, layout: int, n: int, c: int, h: int, w: int, a_bits: int,
                   a_scale: float, packed_x_dev: torch.Tensor, stream=None) -> None:
-    _check(lib().ebs_pack_acts(_ptr(x_dev), dtype, layout, n, c, h, w, a_bits, a_scale, _ptr(packed_x_dev),
-                               _stream(stream)), "ebs_pack_acts")
+    rc = (_fast or _native()).pack_acts(x_dev, dtype, layout, n, c, h, w, a_bits, a_scale, packed_x_dev, stream)
+    if rc:
+        _check(rc, "ebs_pack_acts")
 
 
 def ebs_conv2d_mixed(packed_x_dev, n, h, w, packed_w_dev, desc, epi=None, acc_out_dev=None, y_out_dev=None,
                      packed_next_dev=None, stream=None, variant: int = -1) -> None:
-    e = None if epi is None else ctypes.byref(epi)
-    if variant == -1:
-        rc = lib().ebs_conv2d_mixed(_ptr(packed_x_dev), n, h, w, _ptr(packed_w_dev), ctypes.byref(desc), e,
-                                    _ptr(acc_out_dev), _ptr(y_out_dev), _ptr(packed_next_dev), _stream(stream))
-    else:
-        rc = lib().ebs_conv2d_mixed_variant(_ptr(packed_x_dev), n, h, w, _ptr(packed_w_dev), ctypes.byref(desc), e,
-                                            _ptr(acc_out_dev), _ptr(y_out_dev), _ptr(packed_next_dev),
-                                            _stream(stream), variant)
-    _check(rc, "ebs_conv2d_mixed")
+    rc = (_fast or _native()).conv2d_mixed(packed_x_dev, n, h, w, packed_w_dev, desc, epi, acc_out_dev, y_out_dev,
+                                           packed_next_dev, stream, variant)
+    if rc:
+        _check(rc, "ebs_conv2d_mixed")
 
 
 def ebs_num_conv_variants() -> int:
@@ -209,8 +231,9 @@ def ebs_num_conv_variants() -> int:
 
 def ebs_dequant(acc_dev, n_pixels: int, c_out: int, scale: float, ch_scale_dev=None, ch_bias_dev=None,
                 relu=False, y_dev=None, stream=None) -> None:
-    _check(lib().ebs_dequant(_ptr(acc_dev), n_pixels, c_out, scale, _ptr(ch_scale_dev), _ptr(ch_bias_dev),
-                             int(bool(relu)), _ptr(y_dev), _stream(stream)), "ebs_dequant")
+    rc = (_fast or _native()).dequant(acc_dev, n_pixels, c_out, scale, ch_scale_dev, ch_bias_dev, relu, y_dev, stream)
+    if rc:
+        _check(rc, "ebs_dequant")
 
 
 def ebs_host_workspace_bytes(desc, n, h, w, dtype, next_a_bits=0) -> int:
@@ -233,7 +256,9 @@ def ebs_probe_pipe(kind: int, iters: int = 2000) -> float:
 
 
 def ebs_global_avgpool(y_dev, n: int, hw: int, c: int, out_dev, stream=None) -> None:
-    _check(lib().ebs_global_avgpool(_ptr(y_dev), n, hw, c, _ptr(out_dev), _stream(stream)), "ebs_global_avgpool")
+    rc = (_fast or _native()).global_avgpool(y_dev, n, hw, c, out_dev, stream)
+    if rc:
+        _check(rc, "ebs_global_avgpool")
 
 
 class ebs_fused_layer(ctypes.Structure):
@@ -259,9 +284,10 @@ def ebs_fused_plan_upload(layers, layers_dev: torch.Tensor, stream=None) -> None
 
 def ebs_resnet_cifar_forward(images_dev, n, img_h, img_w, layers_dev, n_layers, head: ebs_fused_head, logits_dev,
                              trace_dev=None, trace_stride: int = 0, stream=None) -> None:
-    _check(lib().ebs_resnet_cifar_forward(_ptr(images_dev), n, img_h, img_w, _ptr(layers_dev), n_layers,
-                                          ctypes.byref(head), _ptr(logits_dev), _ptr(trace_dev), trace_stride,
-                                          _stream(stream)), "ebs_resnet_cifar_forward")
+    rc = (_fast or _native()).resnet_cifar_forward(images_dev, n, img_h, img_w, layers_dev, n_layers, head, logits_dev,
+                                                   trace_dev, trace_stride, stream)
+    if rc:
+        _check(rc, "ebs_resnet_cifar_forward")
 
 
 def _cand(bits, coeff):
@@ -270,15 +296,15 @@ def _cand(bits, coeff):
 
 
 def ebs_search_weight_forward(w_dev, bits, coeff, w_hat_dev, scratch_dev, stream=None) -> None:
-    b, c, n = _cand(bits, coeff)
-    _check(lib().ebs_search_weight_forward(_ptr(w_dev), w_dev.numel(), b, c, n, _ptr(w_hat_dev), _ptr(scratch_dev),
-                                           _stream(stream)), "ebs_search_weight_forward")
+    rc = (_fast or _native()).search_weight_forward(w_dev, w_dev.numel(), bits, coeff, w_hat_dev, scratch_dev, stream)
+    if rc:
+        _check(rc, "ebs_search_weight_forward")
 
 
 def ebs_search_act_forward(x_dev, alpha: float, bits, coeff, x_hat_dev, stream=None) -> None:
-    b, c, n = _cand(bits, coeff)
-    _check(lib().ebs_search_act_forward(_ptr(x_dev), x_dev.numel(), alpha, b, c, n, _ptr(x_hat_dev), _stream(stream)),
-           "ebs_search_act_forward")
+    rc = (_fast or _native()).search_act_forward(x_dev, x_dev.numel(), alpha, bits, coeff, x_hat_dev, stream)
+    if rc:
+        _check(rc, "ebs_search_act_forward")
 
 
 def ebs_expected_flops(macs: float, bits_w, coeff_w, bits_x, coeff_x) -> float:
@@ -335,8 +361,9 @@ def ebs_checked_status(clear: bool = True):
 
 
 def ebs_pack_acts_s2d(x_dev, n, c, h, w, offset, a_bits, packed_x_dev, stream=None) -> None:
-    _check(lib().ebs_pack_acts_s2d(_ptr(x_dev), int(n), int(c), int(h), int(w), int(offset), int(a_bits),
-                                   _ptr(packed_x_dev), _stream(stream)), "ebs_pack_acts_s2d")
+    rc = (_fast or _native()).pack_acts_s2d(x_dev, n, c, h, w, offset, a_bits, packed_x_dev, stream)
+    if rc:
+        _check(rc, "ebs_pack_acts_s2d")
 
 
 def ebs_test_checked_shrink(elements: int) -> None:
@@ -356,8 +383,9 @@ def ebs_conv2d_i8(x_codes_dev, n, h, w, packed_w_dev, desc, epi=None, acc_out_de
 
 
 def ebs_maxpool_packed(packed_x_dev, n, h, w, c, a_bits, k, stride, pad, packed_out_dev, stream=None) -> None:
-    _check(lib().ebs_maxpool_packed(_ptr(packed_x_dev), n, h, w, c, a_bits, k, stride, pad, _ptr(packed_out_dev),
-                                    _stream(stream)), "ebs_maxpool_packed")
+    rc = (_fast or _native()).maxpool_packed(packed_x_dev, n, h, w, c, a_bits, k, stride, pad, packed_out_dev, stream)
+    if rc:
+        _check(rc, "ebs_maxpool_packed")
 
 
 def ebs_combined_scale(w_scale: float, a_scale: float) -> float:
@@ -366,3 +394,44 @@ def ebs_combined_scale(w_scale: float, a_scale: float) -> float:
 
 def ebs_reciprocal_step(step: float) -> float:
     return float(lib().ebs_reciprocal_step(step))
+
+
+class CaptureStream:
+    """The stream calls are recorded on between ebs_graph_begin and ebs_graph_end (passed as their ``stream``)."""
+
+    def __init__(self, raw: int):
+        self.cuda_stream = raw
+
+
+def ebs_graph_begin() -> CaptureStream:
+    raw = ctypes.c_void_p(0)
+    _check(lib().ebs_graph_begin(ctypes.byref(raw)), "ebs_graph_begin")
+    return CaptureStream(raw.value)
+
+
+def ebs_graph_end(capture: CaptureStream, keep: bool = True):
+    """The recorded sequence as a handle (int) for ebs_graph_launch; keep=False discards the recording."""
+    exec_ = ctypes.c_void_p(0)
+    rc = lib().ebs_graph_end(capture.cuda_stream, ctypes.byref(exec_) if keep else None)
+    if keep:
+        _check(rc, "ebs_graph_end")
+    return exec_.value
+
+
+def ebs_graph_launch(graph_exec: int, stream=None) -> bool:
+    """Enqueues the sequence; False if the stream is being captured (nothing enqueued)."""
+    rc = (_fast or _native()).graph_launch(graph_exec, stream)
+    if rc == EBS_ERR_UNSUPPORTED:
+        return False
+    if rc:
+        _check(rc, "ebs_graph_launch")
+    return True
+
+
+def ebs_graph_destroy(graph_exec: int) -> None:
+    _check(lib().ebs_graph_destroy(graph_exec), "ebs_graph_destroy")
+
+
+def same_bytes(structs, data: bytes) -> bool:
+    """Whether the concatenated contents of ctypes structures are exactly ``data``."""
+    return (_fast or _native()).same_bytes(structs, data)

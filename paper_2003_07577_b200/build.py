@@ -3,7 +3,8 @@
 Every translation unit under csrc/ is compiled to an object file in parallel and the objects
 are linked into ``paper_2003_07577_b200/libebs.so``.  Nothing is cached outside the tree.
 ``build(checked=True)`` builds the range-checked variant of the same sources (``-DEBS_CHECKED``,
-objects under ``build_checked/``) into ``libebs_checked.so``.
+objects under ``build_checked/``) into ``libebs_checked.so``.  ``csrc/fastcall.c`` becomes the CPython
+extension ``_fastcall.so`` (gcc), which serves either library.
 """
 from __future__ import annotations
 
@@ -13,6 +14,7 @@ import os
 import re
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -41,6 +43,7 @@ def _deps(path: str, seen: set) -> set:
     return seen
 
 
+FASTCALL = os.path.join(PKG, "_fastcall.so")
 LIB_CHECKED = os.path.join(PKG, "libebs_checked.so")
 
 
@@ -60,6 +63,18 @@ def _compile(src: str, verbose: bool, checked: bool = False) -> str:
     return obj
 
 
+def _build_fastcall(force: bool) -> None:
+    src = os.path.join(CSRC, "fastcall.c")
+    newest = max(os.path.getmtime(p) for p in _deps(src, set()))
+    if not force and os.path.exists(FASTCALL) and os.path.getmtime(FASTCALL) >= newest:
+        return
+    cmd = ["gcc", "-O2", "-Wall", "-fPIC", "-shared", "-I", os.path.join(ROOT, "include"),
+           "-I", sysconfig.get_paths()["include"], src, "-o", FASTCALL]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError(f"gcc failed for {src}:\n{res.stdout}\n{res.stderr}")
+
+
 def build(force: bool = False, verbose: bool = False, jobs: int | None = None, checked: bool = False) -> str:
     obj_dir, lib = OBJ + ("_checked" if checked else ""), (LIB_CHECKED if checked else LIB)
     os.makedirs(obj_dir, exist_ok=True)
@@ -75,6 +90,7 @@ def build(force: bool = False, verbose: bool = False, jobs: int | None = None, c
         res = subprocess.run(cmd, capture_output=True, text=True)
         if res.returncode != 0:
             raise RuntimeError(f"link failed:\n{res.stdout}\n{res.stderr}")
+    _build_fastcall(force)
     return lib
 
 

@@ -43,6 +43,12 @@ class ConvPlan:
     src_h: int = 0
     src_w: int = 0
 
+    _version = 0                  # grows with every assignment to a field: what a recorded run was made from
+
+    def __setattr__(self, name, value):
+        object.__setattr__(self, name, value)
+        object.__setattr__(self, "_version", self._version + 1)
+
 
 def space_to_depth_weights(weight_codes: torch.Tensor) -> torch.Tensor:
     """[c_out, c, k, k] -> [c_out, 4 c, ceil(k/2), ceil(k/2)]: w2[co][(2 dy + dx) c + ch][bi][bj] = w[co][ch][2 bi + dy][2 bj + dx],
@@ -80,6 +86,54 @@ def space_to_depth_stem(plan: ConvPlan, weight_codes: torch.Tensor) -> ConvPlan:
                     s2d_offset=off, src_c=c, src_h=plan.h_in, src_w=plan.w_in)
 
 
+class _Replay:
+    """One batch size of a BasicBlockNet: its calls, and from their second run on their recording."""
+
+    def __init__(self, net: "BasicBlockNet", n: int, versions: List[int]):
+        self.n, self.versions = n, versions
+        self.calls, self.px, self.logits = net._program(n)
+        self._descs = [p.desc for p in net.plans]
+        self._desc_bytes = b"".join(bytes(d) for d in self._descs)
+        self._runs, self._graph = 0, None
+
+    def descs_unchanged(self) -> bool:
+        return ebs.same_bytes(self._descs, self._desc_bytes)
+
+    def _issue(self, stream):
+        for f, args in self.calls:
+            f(*args, stream=stream)
+
+    def _record(self):
+        capture = ebs.ebs_graph_begin()
+        try:
+            self._issue(capture)
+        except BaseException:
+            ebs.ebs_graph_end(capture, keep=False)
+            raise
+        self._graph = ebs.ebs_graph_end(capture)
+
+    @staticmethod
+    def _capturing(stream) -> bool:
+        if stream is None:
+            return torch.cuda.is_current_stream_capturing()
+        with torch.cuda.stream(stream):
+            return torch.cuda.is_current_stream_capturing()
+
+    def run(self, stream):
+        if self._graph is None and self._runs > 0 and not self._capturing(stream):
+            self._record()
+        self._runs += 1
+        if self._graph is None or not ebs.ebs_graph_launch(self._graph, stream):
+            self._issue(stream)
+
+    def __del__(self):
+        if self._graph is not None:
+            try:
+                ebs.ebs_graph_destroy(self._graph)
+            except Exception:                # the interpreter or the CUDA context is already going down
+                pass
+
+
 class BasicBlockNet:
     """conv1, basic blocks named ``<block>c1`` / ``<block>c2`` (/ ``<block>ds``), average pool, classifier."""
 
@@ -98,6 +152,7 @@ class BasicBlockNet:
                 tag = p.name[:-2]
                 self.blocks.append((p, by_name[tag + "c2"], by_name.get(tag + "ds")))
         self._buf: Dict[tuple, torch.Tensor] = {}
+        self._replay: Optional[_Replay] = None
 
     # ------------------------------------------------------------------ buffers (allocated once per batch size)
     def _get(self, key, numel, dtype):
@@ -110,56 +165,72 @@ class BasicBlockNet:
     def _planes(self, key, n, h, w, c, bits):
         return self._get(key, ebs.ebs_packed_act_bytes(n, h, w, c, bits) // 4, torch.int32)
 
-    def _conv(self, p: ConvPlan, src, n, *, residual=None, res_packed=None, res_bits=0, res_step=0.0, relu=True,
-              want_y=False, stream=None):
+    def _conv(self, calls, p: ConvPlan, src, n, *, residual=None, res_packed=None, res_bits=0, res_step=0.0, relu=True,
+              want_y=False):
         d = p.desc
         ho, wo = ebs.ebs_conv_out_shape(d, p.h_in, p.w_in)
         y = self._get((p.name, "y"), n * ho * wo * d.c_out, torch.float32) if want_y else None
         out = self._planes((p.name, "q"), n, ho, wo, d.c_out, p.out_bits) if p.out_bits else None
         epi = ebs.epilogue(p.ch_scale, p.ch_bias, residual, relu, p.out_bits, p.out_step, ebs.EBS_NHWC,
                            res_packed=res_packed, res_bits=res_bits, res_scale=res_step)
-        ebs.ebs_conv2d_mixed(src, n, p.h_in, p.w_in, p.packed_w, d, epi, None, y, out, stream=stream)
+        calls.append((ebs.ebs_conv2d_mixed, (src, n, p.h_in, p.w_in, p.packed_w, d, epi, None, y, out)))
         return y, out, ho, wo
 
-    # ------------------------------------------------------------------ one batch
-    def forward(self, images_u8_nhwc: torch.Tensor, stream=None) -> torch.Tensor:
-        """images: uint8 [N, H, W, 3] on the device.  Returns fp32 logits [N, classes]."""
-        n = images_u8_nhwc.shape[0]
-        f = self.first
+    def _program(self, n):
+        """The calls of one batch behind its entry packing, with their buffers and epilogues; (calls, input planes, logits)."""
+        f, calls = self.first, []
         px = self._planes(("input", "q"), n, f.h_in, f.w_in, f.desc.c_in, 8)
-        if f.s2d_offset >= 0:                                    # stride-2 first layer in space-to-depth form
-            ebs.ebs_pack_acts_s2d(images_u8_nhwc, n, f.src_c, f.src_h, f.src_w, f.s2d_offset, 8, px, stream=stream)
-        else:
-            ebs.ebs_pack_acts(images_u8_nhwc, ebs.EBS_U8_CODES, ebs.EBS_NHWC, n, f.desc.c_in, f.h_in, f.w_in, 8, 1.0, px,
-                              stream=stream)
-        _, x, ho1, wo1 = self._conv(f, px, n, stream=stream)
+        _, x, ho1, wo1 = self._conv(calls, f, px, n)
         x_bits, x_step = f.out_bits, f.out_step
         if self.pool is not None:                                # on the packed codes; bits and step are unchanged
             k, s, pd = self.pool
             hp, wp = (ho1 + 2 * pd - k) // s + 1, (wo1 + 2 * pd - k) // s + 1
             xp = self._planes(("maxpool", "q"), n, hp, wp, f.desc.c_out, x_bits)
-            ebs.ebs_maxpool_packed(x, n, ho1, wo1, f.desc.c_out, x_bits, k, s, pd, xp, stream=stream)
+            calls.append((ebs.ebs_maxpool_packed, (x, n, ho1, wo1, f.desc.c_out, x_bits, k, s, pd, xp)))
             x = xp
         y_last, ho, wo = None, 0, 0
         for bi, (c1, c2, ds) in enumerate(self.blocks):
             last = bi == len(self.blocks) - 1
-            _, t, _, _ = self._conv(c1, x, n, stream=stream)
+            _, t, _, _ = self._conv(calls, c1, x, n)
             if ds is not None:
-                y_ds, _, _, _ = self._conv(ds, x, n, relu=False, want_y=True, stream=stream)
-                y_last, x_new, ho, wo = self._conv(c2, t, n, residual=y_ds, want_y=last, stream=stream)
+                y_ds, _, _, _ = self._conv(calls, ds, x, n, relu=False, want_y=True)
+                y_last, x_new, ho, wo = self._conv(calls, c2, t, n, residual=y_ds, want_y=last)
             else:
-                y_last, x_new, ho, wo = self._conv(c2, t, n, res_packed=x, res_bits=x_bits, res_step=x_step,
-                                                   want_y=last, stream=stream)
+                y_last, x_new, ho, wo = self._conv(calls, c2, t, n, res_packed=x, res_bits=x_bits, res_step=x_step,
+                                                   want_y=last)
             x, x_bits, x_step = x_new, c2.out_bits, c2.out_step
         c_last = self.blocks[-1][1].desc.c_out
         pooled = self._get(("pool", "y"), n * c_last, torch.float32)
-        ebs.ebs_global_avgpool(y_last, n, ho * wo, c_last, pooled, stream=stream)
+        calls.append((ebs.ebs_global_avgpool, (y_last, n, ho * wo, c_last, pooled)))
         fc = self.fc
         pq = self._planes(("pool", "q"), n, 1, 1, c_last, fc.desc.a_bits)
-        ebs.ebs_pack_acts(pooled, ebs.EBS_F32, ebs.EBS_NHWC, n, c_last, 1, 1, fc.desc.a_bits, fc.desc.a_scale, pq,
-                          stream=stream)
-        logits, _, _, _ = self._conv(fc, pq, n, relu=False, want_y=True, stream=stream)
-        return logits.view(n, fc.desc.c_out)
+        calls.append((ebs.ebs_pack_acts, (pooled, ebs.EBS_F32, ebs.EBS_NHWC, n, c_last, 1, 1, fc.desc.a_bits,
+                                          fc.desc.a_scale, pq)))
+        logits, _, _, _ = self._conv(calls, fc, pq, n, relu=False, want_y=True)
+        return calls, px, logits
+
+    # ------------------------------------------------------------------ one batch
+    def forward(self, images_u8_nhwc: torch.Tensor, stream=None) -> torch.Tensor:
+        """images: uint8 [N, H, W, 3] on the device.  Returns fp32 logits [N, classes].
+
+        The entry packing reads the caller's images; everything behind it works on this object's own buffers, so from
+        the second batch of a size on it is replayed as one graph launch (25 calls from Python cost 100 us and more, the
+        replay 10).  The calls are issued one by one on the first batch of a size, while the caller's stream is being
+        captured, and again after a plan has been changed.
+        """
+        n = images_u8_nhwc.shape[0]
+        r = self._replay
+        versions = [p._version for p in self.plans]
+        if r is None or r.n != n or r.versions != versions or not r.descs_unchanged():
+            r = self._replay = _Replay(self, n, versions)
+        f = self.first
+        if f.s2d_offset >= 0:                                    # stride-2 first layer in space-to-depth form
+            ebs.ebs_pack_acts_s2d(images_u8_nhwc, n, f.src_c, f.src_h, f.src_w, f.s2d_offset, 8, r.px, stream=stream)
+        else:
+            ebs.ebs_pack_acts(images_u8_nhwc, ebs.EBS_U8_CODES, ebs.EBS_NHWC, n, f.desc.c_in, f.h_in, f.w_in, 8, 1.0, r.px,
+                              stream=stream)
+        r.run(stream)
+        return r.logits.view(n, self.fc.desc.c_out)
 
     @property
     def launches_per_forward(self) -> int:

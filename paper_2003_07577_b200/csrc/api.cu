@@ -43,23 +43,8 @@ const ConvVariant* conv_mma_variant(int w_bits, int a_bits, int variant) {
     }
 }
 
-const ConvVariant* conv_umma_variant(int w_bits, int a_bits, int variant) {
-    switch (w_bits) {
-        case 1: return conv_umma_variant_w1(a_bits, variant);
-        case 2: return conv_umma_variant_w2(a_bits, variant);
-        case 3: return conv_umma_variant_w3(a_bits, variant);
-        case 4: return conv_umma_variant_w4(a_bits, variant);
-        case 5: return conv_umma_variant_w5(a_bits, variant);
-        case 6: return conv_umma_variant_w6(a_bits, variant);
-        case 7: return conv_umma_variant_w7(a_bits, variant);
-        case 8: return conv_umma_variant_w8(a_bits, variant);
-        default: return nullptr;
-    }
-}
-
 unsigned long long conv_umma_timeouts() {
-    return conv_umma_timeouts_w1() + conv_umma_timeouts_w2() + conv_umma_timeouts_w3() + conv_umma_timeouts_w4() +
-           conv_umma_timeouts_w5() + conv_umma_timeouts_w6() + conv_umma_timeouts_w7() + conv_umma_timeouts_w8() +
+    return conv_umma_tile_timeouts() +
            conv_umma_strip_timeouts() + conv_umma_resident_timeouts() + conv_umma_pipe_timeouts() + fused_net_timeouts();
 }
 
@@ -160,25 +145,6 @@ static int choose_mma_variant(int w_bits, int a_bits, int P, int Co, int sms) {
     return 6 + tc_idx;
 }
 
-// Stride-1 layers with at least 64 output channels and enough outputs to fill the GPU run on the strip
-// kernel (every input pixel expanded once per CTA, weights fetched as bytes).  The channel tile is the
-// largest of 256/128/64 that divides c_out, so that every tile is whole and takes the straight-line
-// epilogue; failing that the largest not above c_out.  (Rule fitted to per-variant timings of the
-// ResNet-18/20/50 layer shapes.)  Returns the strip variant or -1.
-static int choose_strip_variant(const ConvParams& p) {
-    if (p.Co < 64 || (long long)p.P * p.Co < (1LL << 20)) return -1;
-    int pick = -1;
-    for (int v = 4; v >= 2; --v)
-        if (p.Co % (16 << v) == 0) { pick = v; break; }
-    if (pick < 0) pick = p.Co >= 256 ? 4 : (p.Co >= 128 ? 3 : 2);
-    for (; pick >= 2; --pick)
-        if (conv_umma_strip_applies(p, pick)) return pick;
-    return -1;
-}
-
-// The per-tap tcgen05 kernels (any stride) pay off when a CTA's 128 x tile_n accumulator sees a deep
-// reduction, the channel tile is wide enough to amortise the activation expansion, and the layer has
-// enough output tiles; smaller layers run faster on the warp-level kernels.  Returns the variant or -1.
 // The persistent pipeline kernel covers stride-1 and strided k x k layers and 1x1 layers at any stride.  It pays off
 // when the layer has at least 64 output channels and enough outputs to fill the GPU.  Channel tile: the widest of
 // 256/128/64 that divides c_out (every tile whole: straight-line epilogue; the fewer channel tiles, the less often an
@@ -196,24 +162,24 @@ static int choose_pipe_variant(const ConvParams& p, int sms) {
     return -1;
 }
 
-// Smaller layers with a deep reduction (a classifier-side 3x3 layer at batch 1-16 has 4-100 output tiles of 72-144
-// reduction words): the pipeline kernel with its narrowest channel tile, which gives the most thread blocks and walks the
-// words with all roles overlapped.  512 -> 512 3x3 at 7x7, batch 1: 66.8 -> 17.5 us; 1024 -> 256 1x1 at 14x14, batch 16:
-// 25.4 -> 10.3 us.  Below 18 words the warp-level kernels are as fast or faster (256 -> 1024 1x1 at 14x14: 5.5 against
-// 6.7 us), and layers of one wave of warp-level strip tiles (128 -> 128 3x3 at 28x28: 7.8 against 9.0 us) stay there.
-static int choose_deep_pipe_variant(const ConvParams& p) {
-    const int kwords = (p.KK + p.fold - 1) / p.fold;
-    if (p.Co < 64 || p.w_levels || kwords < 18) return -1;
-    return conv_umma_pipe_applies(p, 0) ? 0 : -1;
+// Layers that do not fill the GPU several times over run on the tile kernel, with the channel tile of the smallest
+// estimate (32, 64 or 128; wider never was the fastest).  Measured against the other families on ResNet-18/50 shapes it is
+// ahead up to about three rounds of 128-channel tiles on all SMs -- 128 -> 128 3x3 at 28x28, batch 32: 9.6 against
+// 14.1 us; 512 -> 512 3x3 at 7x7, batch 1: 7.8 against 17.7 us -- and behind the persistent pipeline kernel beyond (64 -> 64
+// 1x1 at 56x56, batch 256: 93 against 66 us).  Returns the variant or -1.
+static int choose_tile_variant(const ConvParams& p) {
+    int pick = -1;
+    float best = 0.0f;
+    for (int v = 1; v <= 3; ++v) {
+        if (v > 1 && (16 << (v - 1)) >= p.Co) break;          // a narrower tile already covers every channel
+        const float c = conv_umma_cost(p, v);
+        if (c >= 0.0f && (pick < 0 || c < best)) { pick = v; best = c; }
+    }
+    return pick;
 }
-
-static int choose_umma_variant(const ConvParams& p, const ebs_conv_desc* d) {
-    const int kwords = (p.KK + p.fold - 1) / p.fold;
-    const long long outputs = (long long)p.P * p.Co;
-    (void)d;
-    if (p.Co < 64 || kwords < 8) return -1;
-    if (outputs < (1LL << 20) && kwords < 72) return -1;
-    return p.Co >= 128 ? 3 : 2;             // tile_n 128 or 64
+static bool tile_kernel_pays(const ConvParams& p, int sms) {
+    const long long tiles = (long long)((p.P + 127) / 128) * ((p.Co + 127) / 128);
+    return tiles <= 3LL * sms;
 }
 
 // A validated, fully decided launch: nothing has been enqueued when conv_plan returns.
@@ -291,10 +257,12 @@ static int conv_plan(const void* packed_x, int n, int h, int w, const void* pack
         p.y_nchw = epi->y_layout == EBS_NCHW;
         if (packed_next) { p.next_bits = epi->next_a_bits; p.inv_next = 1.0f / epi->next_a_scale; }
     }
-    const bool mma_ok = mma_path_supported(p, d);
+    // the tcgen05 kernels walk any reduction length; word offsets are int
+    const bool umma_ok = (long long)n * h * w * p.CW * (byte_acts ? 8 : d->a_bits) < (1LL << 31);
+    const bool mma_ok = umma_ok && mma_path_supported(p, d);
     if (byte_acts) {
         // the context path exists in the persistent pipeline kernels only: whole 32-channel words of byte codes
-        if ((d->c_in & 31) != 0 || d->w_levels || !mma_ok) return EBS_ERR_UNSUPPORTED;
+        if ((d->c_in & 31) != 0 || d->w_levels || !umma_ok) return EBS_ERR_UNSUPPORTED;
         int pick = -1;
         for (int v = 2; v >= 0 && pick < 0; --v)
             if ((p.Co % (64 << v) == 0 || v == 0) && conv_umma_pipe_applies(p, v)) pick = v;
@@ -308,50 +276,42 @@ static int conv_plan(const void* packed_x, int n, int h, int w, const void* pack
     if (variant == -2) {
         variant = choose_variant(d->w_bits, d->a_bits, p.P, p.Co, packed_next != nullptr, sm_count());
     } else if (variant < 0) {
-        int pipe = mma_ok ? choose_pipe_variant(p, sm_count()) : -1;
-        const bool one_wave_strip = p.Co > 64 && p.Co <= 128 && d->kh * d->kw > 1 && p.P < (1 << 10) && conv_mma_strip_applies(p, 1);
-        if (mma_ok && pipe < 0 && !one_wave_strip && !(p.Co <= 64 && conv_mma_strip_applies(p, 1))) pipe = choose_deep_pipe_variant(p);
-        const int strip = (mma_ok && pipe < 0) ? choose_strip_variant(p) : -1;
-        const int umma = (mma_ok && strip < 0 && pipe < 0) ? choose_umma_variant(p, d) : -1;
-        // deep reductions whose weight tiles fit in shared memory: the persistent form of the same tile
+        const bool small = tile_kernel_pays(p, sm_count());
+        const int tile = umma_ok && (p.Co > 16 || p.KK >= 18) ? choose_tile_variant(p) : -1;
+        const int pipe = umma_ok && !(small && tile >= 0) ? choose_pipe_variant(p, sm_count()) : -1;
+        // few channels on many pixels: the warp-level strip kernel (16 -> 16 3x3 at 32x32, batch 128: 7.1 us, the tile kernel,
+        // whose accumulator is then mostly empty, 22; 32 -> 32 at 16x16: 7.2 against 8.3)
+        const bool few = p.Co <= 32 && p.CW <= 2 && d->kh * d->kw > 1 && (long long)p.P > 128LL * sm_count();
         if (pipe >= 0) variant = PIPE_BASE + pipe;
-        else if (strip >= 0 && p.CW * d->kh * d->kw >= 8 && conv_umma_resident_applies(p, strip)) variant = RES_BASE + strip;
-        else if (strip >= 0) variant = STRIP_BASE + strip;
-        else if (umma >= 0) variant = NUM_CONV_VARIANTS + NUM_CONV_MMA_VARIANTS + umma;
-        // small stride-1 k x k layers with up to 64 output channels: the warp-level strip kernel (it expands every input
-        // pixel once instead of once per tap, and its time does not grow with the plane count) at any batch size --
-        // measured against every other variant on 16-, 32- and 64-channel layers from 1 to 64 images it is 15-45%
-        // faster; 1x1 layers have nothing to save there and stay on the per-tap kernel.  33-64 channels: the
-        // 32-channel tile (two CTAs per pixel tile) below 2^13 output pixels, the 64-channel tile from there.
+        else if (mma_ok && few && p.Co <= 16 && conv_mma_strip_applies(p, 0)) variant = MS_BASE;
+        else if (mma_ok && few && conv_mma_strip_applies(p, 1)) variant = MS_BASE + 1;
+        else if (tile >= 0) variant = NUM_CONV_VARIANTS + NUM_CONV_MMA_VARIANTS + tile;
         else if (mma_ok && p.Co <= 16 && d->kh * d->kw > 1 && conv_mma_strip_applies(p, 0)) variant = MS_BASE;
-        else if (mma_ok && p.Co > 16 && p.Co <= 32 && d->kh * d->kw > 1 && conv_mma_strip_applies(p, 1)) variant = MS_BASE + 1;
-        else if (mma_ok && p.Co > 32 && p.Co <= 64 && d->kh * d->kw > 1 && p.P < (1 << 13) && conv_mma_strip_applies(p, 1))
-            variant = MS_BASE + 1;
-        else if (mma_ok && one_wave_strip) variant = MS_BASE + 1;
-        else if (mma_ok && p.Co > 32 && p.Co <= 64 && d->kh * d->kw > 1 && conv_mma_strip_applies(p, 2))
-            variant = MS_BASE + 2;
         else variant = mma_ok ? NUM_CONV_VARIANTS + choose_mma_variant(d->w_bits, d->a_bits, p.P, p.Co, sm_count())
                               : choose_variant(d->w_bits, d->a_bits, p.P, p.Co, packed_next != nullptr, sm_count());
     }
-    if (variant >= NUM_CONV_VARIANTS && !mma_ok) return EBS_ERR_UNSUPPORTED;
+    constexpr int MMA_BASE = NUM_CONV_VARIANTS, UMMA_BASE = MMA_BASE + NUM_CONV_MMA_VARIANTS;
+    const bool warp_level = (variant >= MMA_BASE && variant < UMMA_BASE) || (variant >= MS_BASE && variant < PIPE_BASE);
+    if (variant >= NUM_CONV_VARIANTS && !(warp_level ? mma_ok : umma_ok)) return EBS_ERR_UNSUPPORTED;
     if (variant >= PIPE_BASE) {
         if (!conv_umma_pipe_applies(p, variant - PIPE_BASE)) return EBS_ERR_UNSUPPORTED;
     } else if (variant >= MS_BASE) {
         if (!conv_mma_strip_applies(p, variant - MS_BASE)) return EBS_ERR_UNSUPPORTED;
     } else if (variant >= RES_BASE) {
         if (!conv_umma_resident_applies(p, variant - RES_BASE)) return EBS_ERR_UNSUPPORTED;
-    } else if (variant >= STRIP_BASE && !conv_umma_strip_applies(p, variant - STRIP_BASE)) {
-        return EBS_ERR_UNSUPPORTED;
+    } else if (variant >= STRIP_BASE) {
+        if (!conv_umma_strip_applies(p, variant - STRIP_BASE)) return EBS_ERR_UNSUPPORTED;
+    } else if (variant >= UMMA_BASE) {
+        if (!conv_umma_applies(p, variant - UMMA_BASE)) return EBS_ERR_UNSUPPORTED;
     }
     const ConvVariant* v =
         variant >= PIPE_BASE ? conv_umma_pipe_variant(d->a_bits, variant - PIPE_BASE) :
         variant >= MS_BASE ? conv_mma_strip_variant(d->a_bits, variant - MS_BASE) :
         variant >= RES_BASE ? conv_umma_resident_variant(d->a_bits, variant - RES_BASE) :
         variant >= STRIP_BASE ? conv_umma_strip_variant(d->a_bits, variant - STRIP_BASE) :
-        variant >= NUM_CONV_VARIANTS + NUM_CONV_MMA_VARIANTS
-            ? conv_umma_variant(d->w_bits, d->a_bits, variant - NUM_CONV_VARIANTS - NUM_CONV_MMA_VARIANTS)
-            : (variant >= NUM_CONV_VARIANTS ? conv_mma_variant(d->w_bits, d->a_bits, variant - NUM_CONV_VARIANTS)
-                                            : conv_popc_variant(d->w_bits, d->a_bits, variant));
+        variant >= UMMA_BASE ? conv_umma_variant(d->a_bits, variant - UMMA_BASE) :
+        variant >= MMA_BASE ? conv_mma_variant(d->w_bits, d->a_bits, variant - MMA_BASE)
+                            : conv_popc_variant(d->w_bits, d->a_bits, variant);
     if (!v) return EBS_ERR_UNSUPPORTED;
     if (packed_next && (v->tile_c % 32) != 0 && v->tile_c < p.Co) return EBS_ERR_UNSUPPORTED;
     const long long gx = (P + v->tile_p - 1) / v->tile_p, gy = (p.Co + v->tile_c - 1) / v->tile_c;

@@ -1,0 +1,319 @@
+// What the strip-addressed tcgen05 kernels (conv_umma_pipe.cuh, conv_umma_tile.cuh) share: the frame of outputs with its
+// phase images and tap shifts, the transposes between plane words and channel bytes, and small PTX wrappers.
+#pragma once
+
+#include "conv_umma_strip.cuh"
+
+namespace ebs {
+
+constexpr int FRAME_MAX_TAPS = 64, FRAME_MAX_PHASES = 4;
+
+// Exact unsigned division by a run-time constant: q = (t + ((n - t) >> s1)) >> s2, t = mulhi(m, n).
+struct FastDiv {
+    uint32_t m, s1, s2;
+};
+inline FastDiv make_fastdiv(uint32_t d) {
+    FastDiv f{};
+    uint32_t l = 0;
+    while ((1ull << l) < d) ++l;
+    f.m = (uint32_t)(((1ull << 32) * ((1ull << l) - d)) / d + 1);
+    f.s1 = l < 1 ? l : 1;
+    f.s2 = l > 1 ? l - 1 : 0;
+    return f;
+}
+__device__ __forceinline__ uint32_t fastdiv(uint32_t n, const FastDiv& f) {
+    const uint32_t t = __umulhi(f.m, n);
+    return (t + ((n - t) >> f.s1)) >> f.s2;
+}
+
+// Frame of a layer's outputs (see conv_umma_pipe.cuh: one addressing scheme for all strides), computed on the host.
+struct FrameGeom {
+    int Wq, Hq, frame;                 // frame of one image and pixels of all images
+    FastDiv div_img, div_row;          // by Hq * Wq and by Wq
+    int q0r, q0s;                      // smallest tap quotients (<= 0)
+    int taps, n_ph, max_shift, max_ph_taps;
+    int ph_a[FRAME_MAX_PHASES], ph_b[FRAME_MAX_PHASES];
+    int ph_tap0[FRAME_MAX_PHASES + 1]; // tap slots of phase i: [ph_tap0[i], ph_tap0[i + 1])
+    short tap_shift[FRAME_MAX_TAPS];   // per tap slot: shift inside the strip, in pixels
+    short tap_id[FRAME_MAX_TAPS];      // per tap slot: r * kw + s (tile index in the weight byte image)
+};
+
+inline int floordiv_int(int a, int b) { return (a >= 0) ? a / b : -((-a + b - 1) / b); }
+
+// False when the layer is outside the scheme (stride above 2, more than 64 taps, ...).
+inline bool frame_geometry(const ConvParams& p, FrameGeom& g) {
+    const int taps = p.kh * p.kw;
+    if (p.sh > 2 || p.sw > 2 || taps > FRAME_MAX_TAPS || p.kh > 16 || p.kw > 16) return false;
+    if ((long long)p.CW * 8 > PIPE_ZERO_WORDS) return false;  // the zero page covers a pixel's words at 8 planes (byte codes: 8 words a word)
+    g.q0r = floordiv_int(-p.ph, p.sh);
+    g.q0s = floordiv_int(-p.pw, p.sw);
+    const int qr_max = floordiv_int(p.kh - 1 - p.ph, p.sh), qs_max = floordiv_int(p.kw - 1 - p.pw, p.sw);
+    g.Hq = p.Ho + qr_max - g.q0r;
+    g.Wq = p.Wo + qs_max - g.q0s;
+    const long long frame = (long long)p.N * g.Hq * g.Wq;
+    if (frame >= (1LL << 31) - 4096) return false;
+    g.frame = (int)frame;
+    g.div_img = make_fastdiv((uint32_t)(g.Hq * g.Wq));
+    g.div_row = make_fastdiv((uint32_t)g.Wq);
+    g.max_shift = (qr_max - g.q0r) * g.Wq + (qs_max - g.q0s);
+    if (g.max_shift > 30000) return false;
+    g.taps = taps;
+    g.n_ph = 0;
+    g.max_ph_taps = 0;
+    int slot = 0;
+    for (int a = 0; a < p.sh; ++a)
+        for (int b = 0; b < p.sw; ++b) {
+            const int first = slot;
+            for (int r = 0; r < p.kh; ++r) {
+                const int qr = floordiv_int(r - p.ph, p.sh);
+                if ((r - p.ph) - p.sh * qr != a) continue;
+                for (int s = 0; s < p.kw; ++s) {
+                    const int qs = floordiv_int(s - p.pw, p.sw);
+                    if ((s - p.pw) - p.sw * qs != b) continue;
+                    g.tap_shift[slot] = (short)((qr - g.q0r) * g.Wq + (qs - g.q0s));
+                    g.tap_id[slot] = (short)(r * p.kw + s);
+                    ++slot;
+                }
+            }
+            if (slot > first) {
+                g.ph_a[g.n_ph] = a;
+                g.ph_b[g.n_ph] = b;
+                g.ph_tap0[g.n_ph] = first;
+                ++g.n_ph;
+                if (slot - first > g.max_ph_taps) g.max_ph_taps = slot - first;
+            }
+        }
+    g.ph_tap0[g.n_ph] = slot;
+    return true;
+}
+
+// NW plane words of one (pixel, 32-channel word) item -> eight registers of four channel bytes (row byte 4b + i = channel
+// 8i + b).  With v_k = rotl(w_k, k), register b is rotr(t_b, b) where byte position (b + k) & 7 of t_b holds plane k.  The
+// eight t_b pick the planes in eight cyclic orders, and orders that agree modulo 2 (modulo 4) share their pairs (quads)
+// of planes: one bit-select per pair and parity, one per quad and residue, one per register - 24 selects for eight
+// planes where a merge per (register, plane) takes 64.
+__device__ __forceinline__ uint32_t bit_select(uint32_t a, uint32_t b, uint32_t m) { return (a & m) | (b & ~m); }
+
+template <int NW>
+__device__ __forceinline__ void planes_to_bytes(const uint32_t (&w)[NW], uint32_t (&r)[8]) {
+    uint32_t v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = k < NW ? __funnelshift_l(w[k < NW ? k : 0], w[k < NW ? k : 0], k) : 0u;
+    if constexpr (NW == 1) {
+#pragma unroll
+        for (int bb = 0; bb < 8; ++bb) {
+            const uint32_t t = v[0] & (0x01010101u << bb);
+            r[bb] = __funnelshift_r(t, t, bb);
+        }
+    } else {
+        // pairs: plane 2j on the even bit positions and plane 2j + 1 on the odd ones (parity 0), or the reverse
+        uint32_t pr[4][2];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            pr[j][0] = bit_select(v[2 * j], v[2 * j + 1], 0x55555555u);
+            pr[j][1] = bit_select(v[2 * j + 1], v[2 * j], 0x55555555u);
+        }
+        if constexpr (NW == 2) {
+#pragma unroll
+            for (int bb = 0; bb < 8; ++bb) {
+                const uint32_t t = pr[0][bb & 1] & ((0x01010101u << bb) | (0x01010101u << ((bb + 1) & 7)));
+                r[bb] = __funnelshift_r(t, t, bb);
+            }
+        } else {
+            // quads: the pair 2i on the positions = c, c + 1 (mod 4), the pair 2i + 1 on the other two
+            uint32_t qd[2][4];
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const uint32_t m2 = c == 0 ? 0x33333333u : c == 1 ? 0x66666666u : c == 2 ? 0xCCCCCCCCu : 0x99999999u;
+                    qd[i][c] = bit_select(pr[2 * i][c & 1], pr[2 * i + 1][c & 1], m2);
+                }
+#pragma unroll
+            for (int bb = 0; bb < 8; ++bb) {
+                const uint32_t m3 = 0x01010101u * (uint32_t)(((0x0Fu << bb) | (0x0Fu >> (8 - bb))) & 0xFFu);
+                const uint32_t t = bit_select(qd[0][bb & 3], qd[1][bb & 3], m3);   // planes 0-3 on positions bb .. bb + 3
+                r[bb] = __funnelshift_r(t, t, bb);
+            }
+        }
+    }
+}
+
+// Eight registers of four channel bytes (byte i of register b = channel 8i + b) -> plane words: the mirror image of
+// planes_to_bytes.  With c_b = rotl(bytes_b, b), plane j is rotr(t_j, j) where byte position (b + j) & 7 of t_j comes from
+// register b; the pair and quad selects are shared between the planes (16 + nb selects where a merge per (plane,
+// register) takes 8 * nb).
+__device__ __forceinline__ void bytes_to_planes(const uint32_t (&cr)[8], int nb, uint32_t (&planes)[8]) {
+    uint32_t pr[4][2], qd[2][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        pr[j][0] = bit_select(cr[2 * j], cr[2 * j + 1], 0x55555555u);
+        pr[j][1] = bit_select(cr[2 * j + 1], cr[2 * j], 0x55555555u);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const uint32_t m2 = c == 0 ? 0x33333333u : c == 1 ? 0x66666666u : c == 2 ? 0xCCCCCCCCu : 0x99999999u;
+            qd[i][c] = bit_select(pr[2 * i][c & 1], pr[2 * i + 1][c & 1], m2);
+        }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        if (j >= nb) break;
+        const uint32_t m3 = 0x01010101u * (uint32_t)(((0x0Fu << j) | (0x0Fu >> (8 - j))) & 0xFFu);
+        const uint32_t t = bit_select(qd[0][j & 3], qd[1][j & 3], m3);
+        planes[j] = __funnelshift_r(t, t, j);
+    }
+}
+
+// fl(t) -> the bit pattern 0x4B000000 + clamp(floor(t), 0, qmax) without the conversion pipe and with one logic-pipe
+// instruction: t + |t| is 2 * max(t, 0) exactly, the minimum with 2 * qmax + 1 bounds it (floor and clamp commute for
+// integer bounds: floor(min(max(t, 0), qmax + 1/2)) = min(max(floor(t), 0), qmax)), and the halving and the 2^23 go into
+// one multiply-add rounded toward -inf, whose low mantissa bits are the floor.
+__device__ __forceinline__ uint32_t code_pattern(float t, float hi2) {
+    const float a = __fadd_rn(t, fabsf(t));
+    return __float_as_uint(__fmaf_rd(fminf(a, hi2), 0.5f, 8388608.0f));
+}
+
+// tcgen05.mma with both descriptors given as (low word, high word): the start-address field sits in the low word, so
+// an operand is moved by a 32-bit addition.  The whole warp executes the call with the same operands and the
+// instruction is predicated on `leader` (non-zero in one lane): with the issue loop free of divergent branches its
+// address arithmetic stays warp-uniform, which measured faster than a loop run by one thread alone.
+__device__ __forceinline__ void umma_i8_split(uint32_t leader, uint32_t tmem_d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                              uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %2};\n\t"
+        "mov.b64 db, {%3, %4};\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "setp.ne.b32 q, %7, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %5, p;\n\t}\n"
+        :: "r"(tmem_d), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(leader)
+        : "memory");
+}
+// Address of the same shared-memory object in the CTA of the given rank of this cluster.
+__device__ __forceinline__ uint32_t cluster_addr(const void* ptr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(smem_u32(ptr)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_address) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(cluster_address) : "memory");
+}
+// Bounded wait on a barrier another CTA of the cluster arrives on.
+__device__ __forceinline__ bool mbar_wait_cluster_hot(uint64_t* bar, uint32_t parity, volatile int* abort_flag, unsigned limit) {
+    const uint32_t addr = smem_u32(bar);
+    for (unsigned it = 0; it < limit; ++it) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}\n"
+            : "=r"(done) : "r"(addr), "r"(parity) : "memory");
+        if (done) return true;
+        if (*abort_flag) return false;
+    }
+    *abort_flag = 1;
+    return false;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ void umma_commit_pred(uint32_t leader, uint64_t* bar) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n"
+        ::"r"(smem_u32(bar)), "r"(leader) : "memory");
+}
+
+// Two fp32 values in one 64-bit register for the packed fp32 instructions (one issue slot for two results; each lane is
+// an individually rounded IEEE operation, identical to the scalar instruction).
+__device__ __forceinline__ uint64_t f32x2_pack(float lo, float hi) {
+    return ((uint64_t)__float_as_uint(hi) << 32) | (uint64_t)__float_as_uint(lo);
+}
+__device__ __forceinline__ uint64_t f32x2_mul_rn(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t f32x2_add_rn(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t f32x2_add_rd(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// Four requantized codes (low bytes of code_pattern results) -> one register, channel order as in planes_to_bytes.
+__device__ __forceinline__ uint32_t join_codes(const uint32_t (&m)[4]) {
+    return __byte_perm(__byte_perm(m[0], m[1], 0x0040), __byte_perm(m[2], m[3], 0x0040), 0x5410);
+}
+// Byte i of a register as fp32, exactly, without the conversion pipe: 2^23 + byte, minus 2^23.
+__device__ __forceinline__ float byte_to_float(uint32_t w, int i) {
+    return __fadd_rn(__uint_as_float(__byte_perm(w, 0x4B000000u, 0x7540u + (uint32_t)i)), -8388608.0f);
+}
+
+// Per-channel terms of a 32-channel group in the order terms_codes32 reads them: entry bb = channels bb, 8 + bb, 16 + bb,
+// 24 + bb; identities (x * 1, x + (-0)) where a layer has no such term or the channel does not exist.
+__device__ __forceinline__ float term_at(const float* t, int co, int Co, float identity) {
+    return t && co < Co ? __ldg(t + co) : identity;
+}
+
+// 32 accumulators of one pixel and 32-channel group -> eight registers of requantized codes (register bb: channels bb,
+// 8 + bb, 16 + bb, 24 + bb), with per-channel scale and shift and a shortcut: RES 0 none, 1 fp32 values of the pixel's
+// 32 channels, 2 codes in byte registers of the same order.  Every fp32 step is rounded on its own, in the library's
+// order.  The terms come from shared memory as broadcast 16-byte reads (read through the cache channel by channel they
+// were two thirds of the instructions of this function); products are packed two to an instruction, additions are scalar
+// because the assembler contracts a packed product and a packed sum into a fused operation.  The ReLU is not applied: the
+// quantizer's clamp at zero gives the same codes.
+template <int RES>
+__device__ __forceinline__ void terms_codes32(const uint32_t (&v)[32], float S, const float4* cs, const float4* cb,
+                                              const float (&res)[32], const uint32_t (&rbyte)[8], float res_scale,
+                                              float inv_next, float hi2, uint32_t (&cr)[8]) {
+    const uint64_t S2 = f32x2_pack(S, S);
+#pragma unroll
+    for (int bb = 0; bb < 8; ++bb) {
+        const float4 a = cs[bb], b = cb[bb];
+        const uint64_t w0 = f32x2_mul_rn(f32x2_mul_rn(f32x2_pack((float)(int)v[bb], (float)(int)v[8 + bb]), S2), f32x2_pack(a.x, a.y));
+        const uint64_t w1 = f32x2_mul_rn(f32x2_mul_rn(f32x2_pack((float)(int)v[16 + bb], (float)(int)v[24 + bb]), S2), f32x2_pack(a.z, a.w));
+        float t[4] = {__fadd_rn(__uint_as_float((uint32_t)w0), b.x), __fadd_rn(__uint_as_float((uint32_t)(w0 >> 32)), b.y),
+                      __fadd_rn(__uint_as_float((uint32_t)w1), b.z), __fadd_rn(__uint_as_float((uint32_t)(w1 >> 32)), b.w)};
+        uint32_t m[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (RES == 1) t[i] = __fadd_rn(t[i], res[8 * i + bb]);
+            if (RES == 2) t[i] = __fadd_rn(t[i], __fmul_rn(res_scale, byte_to_float(rbyte[bb], i)));
+            m[i] = code_pattern(__fadd_rn(__fmul_rn(t[i], inv_next), 0.5f), hi2);
+        }
+        const uint32_t c4 = join_codes(m);
+        cr[bb] = __funnelshift_l(c4, c4, bb);
+    }
+}
+
+// A group's plane words in the widest stores their alignment (4 * nb bytes) allows.
+__device__ __forceinline__ void store_plane_words(const uint32_t (&planes)[8], int nb, uint32_t* dst) {
+    if (nb == 4) {
+        *reinterpret_cast<uint4*>(dst) = make_uint4(planes[0], planes[1], planes[2], planes[3]);
+    } else if (nb == 8) {
+        *reinterpret_cast<uint4*>(dst) = make_uint4(planes[0], planes[1], planes[2], planes[3]);
+        *reinterpret_cast<uint4*>(dst + 4) = make_uint4(planes[4], planes[5], planes[6], planes[7]);
+    } else if (nb == 2) {
+        *reinterpret_cast<uint2*>(dst) = make_uint2(planes[0], planes[1]);
+    } else if (nb == 6) {
+        *reinterpret_cast<uint2*>(dst) = make_uint2(planes[0], planes[1]);
+        *reinterpret_cast<uint2*>(dst + 2) = make_uint2(planes[2], planes[3]);
+        *reinterpret_cast<uint2*>(dst + 4) = make_uint2(planes[4], planes[5]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (j >= nb) break;
+            dst[j] = planes[j];
+        }
+    }
+}
+
+}  // namespace ebs

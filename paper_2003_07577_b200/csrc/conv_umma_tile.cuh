@@ -1,0 +1,617 @@
+// One thread block per (128 frame pixels, channel tile, share of the reduction): the tcgen05 kernel for layers that do not
+// fill the GPU with the pipeline kernel's super-tiles -- small batches, the deep 7x7 and 14x14 layers, odd channel
+// counts -- and for the paper's weight levels.
+//
+// Arithmetic and addressing are those of conv_umma_pipe.cuh: planes of a packed word merged back into one byte per
+// channel, one int8 MMA of 128 pixels x N channels x 32 channels of a tap, phase images and tap shifts inside a strip
+// that is expanded once.  What bounds such a layer is latency: a launch, a round trip for the packed words, the chain of
+// MMAs onto one accumulator (about 50 clocks each at N = 64) and the epilogue, with most SMs idle.  Hence
+//  * the reduction is split over the CTAs of a cluster (up to 8) by input-channel words; each accumulates its share in its
+//    own tensor memory, the partial sums meet in shared memory and every CTA of the cluster finishes its part of the
+//    pixels (exact: integer sums);
+//  * all of a CTA's operands are in flight at once where they fit (100 KB, so that two CTAs share an SM and one's epilogue
+//    runs under the other's MMAs), weight tiles by bulk copies of one warp, packed words by the expanders;
+//  * the launch may begin while its predecessor in the stream finishes (programmatic dependent launch): barriers, tables
+//    and tensor memory are set up before the wait.
+// Roles (10 warps): warps 0-7 expand and later run the epilogue, warp 8 issues the MMAs, warp 9 fetches weights.
+// Three forms: 1 = packed planes only, no per-channel terms, reduction not split, whole 32-channel words: out of tensor
+// memory with a thread per pixel; 2 = the same with per-channel terms and shortcut; 0 = everything else: the sums go
+// through shared memory and a warp finishes 32 channels of a pixel at a time (coalesced stores; the codes go back into
+// shared memory as bytes and a thread packs the 32 channels of a pixel).
+// Weight levels (w_levels): the window sum of the codes is one more accumulator column, an MMA against a tile of ones.
+// Every wait is bounded as in the other tcgen05 kernels.
+#pragma once
+
+#include "conv_frame.cuh"
+
+namespace ebs {
+
+constexpr int TILE_WORKERS = 256, TILE_ISSUER = 8, TILE_PRODUCER = 9, TILE_THREADS = 320;
+constexpr int TILE_SLOTS = 2;                       // (pixel, word) items an expander handles per stage
+constexpr int TILE_MAX_STAGES = 16, TILE_MAX_SPLIT = 8;
+constexpr int TILE_SMEM_SHARED = 104 * 1024, TILE_SMEM_MAX = 216 * 1024;   // two CTAs / one CTA per SM
+
+struct TileGeom : FrameGeom {
+    int tile_n, n_ptiles, n_ctiles, split;
+    int S, SP, kw;                     // strip pixels, rounded up to 8; words per stage
+    int words;                         // input-channel words of a CTA (the last of a cluster may have fewer)
+    int a_word_bytes, b_off, stage_bytes, n_stages;
+    int tmem_cols, smem_bytes, part_pitch;
+    float cost;                        // estimated clocks of the launch
+    bool ok;
+};
+
+inline int tile_round_up(int v, int m) { return (v + m - 1) / m * m; }
+
+// Geometry for a channel tile of tile_n and a split of the reduction (0: the split with the smallest estimate).
+inline TileGeom tile_geometry(const ConvParams& p, int tile_n, int sms, int split_req) {
+    TileGeom g{};
+    if (!frame_geometry(p, g)) return g;
+    g.tile_n = tile_n;
+    g.S = UMMA_M + g.max_shift;
+    g.SP = tile_round_up(g.S, 8);
+    if (g.S > TILE_SLOTS * TILE_WORKERS) return g;
+    g.n_ptiles = (g.frame + UMMA_M - 1) / UMMA_M;
+    g.n_ctiles = (p.Co + tile_n - 1) / tile_n;
+    if (g.n_ctiles > 65535) return g;
+    g.tmem_cols = 32;
+    while (g.tmem_cols < tile_n + (p.w_levels ? 16 : 0)) g.tmem_cols *= 2;
+    if (g.tmem_cols > 512) return g;
+    g.part_pitch = (tile_n + (p.w_levels ? 1 : 0) + 3) / 4 * 4 + 4;
+    const int b_tile = tile_n * 32;
+    TileGeom best{};
+    for (int split = 1; split <= TILE_MAX_SPLIT; split *= 2) {
+        if (split_req && split != split_req) continue;
+        // A CTA holds its tensor memory while it waits for the others of its cluster, so clusters take at most a quarter of
+        // it: no mix of resident blocks can then keep a member from starting (at most three of this kernel fit an SM).
+        if (split > p.CW || (split > 1 && g.tmem_cols > 128)) break;
+        TileGeom c = g;
+        c.words = (p.CW + split - 1) / split;
+        c.split = (p.CW + c.words - 1) / c.words;
+        if (c.split != split) continue;                        // a rank without words
+        c.kw = TILE_SLOTS * TILE_WORKERS / c.S;
+        if (c.kw > 4) c.kw = 4;
+        if (c.kw > c.words) c.kw = c.words;
+        // the strip of a word: two halves of SP x 16 bytes, skewed so that lanes on consecutive words hit different banks
+        auto stage = [&](int kw) {
+            c.a_word_bytes = c.SP * 32 + (kw == 4 ? 32 : kw == 3 ? 48 : 64);
+            c.b_off = tile_round_up(kw * c.a_word_bytes, 256);
+            return c.b_off + kw * c.max_ph_taps * b_tile;
+        };
+        const int fixed = 1024 + 512;
+        while (c.kw > 1 && 3 * stage(c.kw) + fixed > TILE_SMEM_SHARED) --c.kw;
+        c.stage_bytes = stage(c.kw);
+        const int chunks = c.n_ph * ((c.words + c.kw - 1) / c.kw);
+        const int part = UMMA_M * c.part_pitch * 4;            // the partial sums reuse the stages
+        const int need = chunks < 2 ? 1 : 2;
+        int budget = TILE_SMEM_SHARED;
+        if (need * c.stage_bytes + fixed > budget || part + fixed > budget) budget = TILE_SMEM_MAX;
+        c.n_stages = (budget - fixed) / c.stage_bytes;
+        if (c.n_stages > chunks) c.n_stages = chunks;
+        if (c.n_stages > TILE_MAX_STAGES) c.n_stages = TILE_MAX_STAGES;
+        if (c.n_stages < need) continue;
+        const int body = c.n_stages * c.stage_bytes > part ? c.n_stages * c.stage_bytes : part;
+        c.smem_bytes = body + fixed;
+        if (c.smem_bytes > TILE_SMEM_MAX) continue;
+        // Estimate of the launch, fitted to about 1000 measured (layer, channel tile, split) points: the serial chain of a
+        // CTA is the longer of its MMAs and its expansion plus an epilogue per channel, or the exchange of the sums; from
+        // about 1.2 CTAs per SM on time grows with their number.
+        const double ctas = (double)c.n_ptiles * c.n_ctiles * split;
+        if (split == TILE_MAX_SPLIT && ctas > sms / 2) continue;   // (more clusters of eight than GPCs run at once: slower)
+        const double mma = (double)c.words * c.taps * (17.0 + 0.34 * tile_n + (p.w_levels ? 20.0 : 0.0));
+        const double expand = 1.26 * c.words * c.n_ph * c.S;
+        const int cols = tile_n < tile_round_up(p.Co, 32) ? tile_n : tile_round_up(p.Co, 32);
+        const double tail = split == 1 ? 21.0 * cols : 1610.0 + 114.0 * cols / split;
+        const double load = ctas / (1.21 * sms);
+        c.cost = (float)((86.0 + (mma > expand ? mma : expand) + tail) * (load > 1.0 ? load : 1.0));
+        c.ok = true;
+        if (!best.ok || c.cost < best.cost) best = c;
+    }
+    return best;
+}
+
+template <int AB, int FORM>
+__global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const ConvParams p, const TileGeom g) {
+    extern __shared__ uint8_t dyn_smem[];
+    __shared__ __align__(8) uint64_t full[TILE_MAX_STAGES], empty[TILE_MAX_STAGES], acc_full;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag;
+    __shared__ int gp_s[UMMA_M];                         // output pixel of every row, -1: none
+    __shared__ int s_tap_shift[FRAME_MAX_TAPS], s_tap_id[FRAME_MAX_TAPS];
+    __shared__ __align__(16) float s_terms[FORM == 2 ? 512 : 4];   // FORM 2: scale and shift of the channel tile, terms_codes32 order
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)blockIdx.z, split = g.split;   // cluster of `split` CTAs along z
+    const int f0 = (int)blockIdx.x * UMMA_M, co0 = (int)blockIdx.y * g.tile_n;
+    const int N = g.tile_n, b_tile = N * 32, KW = g.kw, NST = g.n_stages, SP = g.SP, S = g.S;
+    uint8_t* ones = dyn_smem + ((1024u - (smem_u32(dyn_smem) & 1023u)) & 1023u);   // w_levels: 16 rows of ones
+    uint8_t* stages = ones + 512;                        // [NST] x { KW strips, KW * taps weight tiles }; later the partial sums
+    volatile int* abortp = &abort_flag;
+    const unsigned limit = p.wait_limit;
+    const int w0 = rank * g.words, nw = min(g.words, p.CW - w0);
+    const int nwg = (nw + KW - 1) / KW, nchunks = g.n_ph * nwg;
+
+    if (tid == 0) {
+        abort_flag = 0;
+        for (int s = 0; s < NST; ++s) {
+            mbar_init(&full[s], 8 + 1);                  // expander warps and the weight producer
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(&acc_full, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (tid < FRAME_MAX_TAPS) {
+        s_tap_shift[tid] = g.tap_shift[tid];
+        s_tap_id[tid] = g.tap_id[tid];
+    }
+    if (p.w_levels && tid < 128) reinterpret_cast<uint32_t*>(ones)[tid] = 0x01010101u;
+    if (warp == TILE_ISSUER) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_slot)),
+                     "r"((uint32_t)g.tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const uint32_t tmem = tmem_slot;
+    // The next launch may start its own set-up from here on: this CTA has its tensor memory, so nothing it still needs can
+    // be taken by a CTA that waits for it.  Global memory is touched only behind the wait for the previous launch.
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+
+    if (warp < 8) {
+        // =========================== expanders ===========================
+        int slot_q[TILE_SLOTS], slot_dst[TILE_SLOTS], slot_f[TILE_SLOTS];
+#pragma unroll
+        for (int j = 0; j < TILE_SLOTS; ++j) {
+            const int e = tid + j * TILE_WORKERS;
+            const int s = e / KW, q = e - s * KW;         // consecutive lanes: consecutive words of one pixel
+            slot_q[j] = s < S ? q : -1;
+            slot_f[j] = f0 + s;
+            slot_dst[j] = q * g.a_word_bytes + s * 16;
+        }
+        const uint32_t* src[TILE_SLOTS];
+        auto phase_pointers = [&](int ph) {
+#pragma unroll
+            for (int j = 0; j < TILE_SLOTS; ++j) {
+                src[j] = nullptr;                        // padding, past the batch, or no item: zero bytes
+                const int f = slot_f[j];
+                if (slot_q[j] < 0 || f >= g.frame) continue;
+                const uint32_t n = fastdiv((uint32_t)f, g.div_img);
+                const uint32_t rem = (uint32_t)f - n * (uint32_t)(g.Hq * g.Wq);
+                const uint32_t hq = fastdiv(rem, g.div_row), wq = rem - hq * (uint32_t)g.Wq;
+                const int h = p.sh * ((int)hq + g.q0r) + g.ph_a[ph], w = p.sw * ((int)wq + g.q0s) + g.ph_b[ph];
+                if ((unsigned)h < (unsigned)p.H && (unsigned)w < (unsigned)p.W)
+                    src[j] = p.x + (size_t)((((int)n * p.H + h) * p.W + w) * p.CW + w0 + slot_q[j]) * AB;
+            }
+        };
+        constexpr int SETS = AB <= 4 ? 4 : 3;            // packed words of SETS - 1 chunks in flight
+        uint32_t words[SETS][TILE_SLOTS][AB];
+        int ld_ph = 0, ld_wg = 0;
+        auto load_next = [&](int set) {
+            if (ld_wg == 0) phase_pointers(ld_ph);
+#pragma unroll
+            for (int j = 0; j < TILE_SLOTS; ++j) {
+                const uint32_t* a = src[j] + (size_t)ld_wg * KW * AB;
+                const bool in = src[j] != nullptr && ld_wg * KW + slot_q[j] < nw;
+                if (in && EBS_IN_RANGE(p, CHK_UT_X, (a - p.x) + AB - 1, p.lim_x)) {
+                    load_words_global<AB>(a, words[set][j]);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < AB; ++k) words[set][j][k] = 0u;
+                }
+            }
+            if (++ld_wg == nwg) { ld_wg = 0; ++ld_ph; }
+        };
+#pragma unroll
+        for (int u = 0; u < SETS - 1; ++u)
+            if (u < nchunks) load_next(u);
+        // while these are on their way: the output pixel of every row, the per-channel terms of the tile
+        if (tid < UMMA_M) {
+            const int f = f0 + tid;
+            int gp = -1;
+            if (f < g.frame) {
+                const uint32_t n = fastdiv((uint32_t)f, g.div_img);
+                const uint32_t rem = (uint32_t)f - n * (uint32_t)(g.Hq * g.Wq);
+                const uint32_t hq = fastdiv(rem, g.div_row), wq = rem - hq * (uint32_t)g.Wq;
+                if ((int)hq < p.Ho && (int)wq < p.Wo) gp = ((int)n * p.Ho + (int)hq) * p.Wo + (int)wq;
+            }
+            gp_s[tid] = gp;
+        }
+        if constexpr (FORM == 2) {
+            if (tid < N) {                               // channel tid of the tile: group tid / 32, entry tid % 8, lane (tid / 8) % 4
+                const int at = (tid >> 5) * 32 + (tid & 7) * 4 + ((tid >> 3) & 3);
+                s_terms[at] = term_at(p.ch_scale, co0 + tid, p.Co, 1.0f);
+                s_terms[256 + at] = term_at(p.ch_bias, co0 + tid, p.Co, -0.0f);
+            }
+        }
+        bool ok = true;
+        int st = 0;
+        uint32_t round = 0;
+        for (int c0 = 0; c0 < nchunks && ok; c0 += SETS) {
+#pragma unroll
+            for (int u = 0; u < SETS; ++u) {
+                if (c0 + u >= nchunks) break;
+                if (c0 + u + SETS - 1 < nchunks) load_next((u + SETS - 1) % SETS);
+                if (round > 0 && !mbar_wait_bounded(&empty[st], (round - 1) & 1u, abortp, limit)) { ok = false; break; }
+                uint8_t* A = stages + st * g.stage_bytes;
+#pragma unroll
+                for (int j = 0; j < TILE_SLOTS; ++j) {
+                    if (slot_q[j] < 0) continue;
+                    uint32_t r[8];
+                    planes_to_bytes<AB>(words[u][j], r);
+                    uint8_t* dst = A + slot_dst[j];
+                    if (!EBS_IN_RANGE(p, CHK_UT_STAGE, (dst + SP * 16 + 15) - stages, NST * g.stage_bytes)) continue;
+                    *reinterpret_cast<uint4*>(dst) = make_uint4(r[0], r[1], r[2], r[3]);
+                    *reinterpret_cast<uint4*>(dst + SP * 16) = make_uint4(r[4], r[5], r[6], r[7]);
+                }
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&full[st]);
+                if (++st == NST) { st = 0; ++round; }
+            }
+        }
+        if (ok) mbar_wait_bounded(&acc_full, 0u, abortp, limit);
+    } else if (warp == TILE_ISSUER) {
+        // =========================== issuer ===========================
+        const bool skip_mma = (p.test_flags & 1) != 0;   // test hook: issue nothing, so that waits run out
+        const uint32_t leader = lane == 0 ? 1u : 0u;
+        const uint64_t da0 = umma_desc_interleaved(smem_u32(stages), (uint32_t)(SP * 16)), db0 = umma_desc_sw32(smem_u32(stages + g.b_off));
+        const uint32_t da_hi = (uint32_t)(da0 >> 32), db_hi = (uint32_t)(db0 >> 32), ones_lo = (uint32_t)umma_desc_sw32(smem_u32(ones));
+        const uint32_t idesc = umma_idesc_i8(N), word16 = (uint32_t)g.a_word_bytes >> 4, bt16 = (uint32_t)b_tile >> 4;
+        int st = 0, ph = 0, wg = 0;
+        uint32_t round = 0;
+        for (int c = 0; c < nchunks; ++c) {
+            if (!mbar_wait_bounded_hot(&full[st], round & 1u, abortp, limit)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            if (!skip_mma) {
+                const int nq = min(KW, nw - wg * KW), t0 = g.ph_tap0[ph], t1 = g.ph_tap0[ph + 1];
+                const uint32_t stage16 = (uint32_t)(st * g.stage_bytes) >> 4;
+                uint32_t a_lo = (uint32_t)da0 + stage16, b_lo = (uint32_t)db0 + stage16;
+                uint32_t accu = c == 0 ? 0u : 1u;
+                for (int q = 0; q < nq; ++q, a_lo += word16) {
+                    uint32_t shift = (uint32_t)s_tap_shift[t0];
+                    for (int t = t0; t < t1; ++t, b_lo += bt16) {
+                        const uint32_t next = (uint32_t)s_tap_shift[min(t + 1, FRAME_MAX_TAPS - 1)];
+                        umma_i8_split(leader, tmem, a_lo + shift, da_hi, b_lo, db_hi, idesc, accu);
+                        if (p.w_levels) umma_i8_split(leader, tmem + (uint32_t)N, a_lo + shift, da_hi, ones_lo, db_hi, umma_idesc_i8(16), accu);
+                        accu = 1u;
+                        shift = next;
+                    }
+                }
+                umma_commit_pred(leader, &empty[st]);
+                if (c == nchunks - 1) umma_commit_pred(leader, &acc_full);
+            }
+            __syncwarp();
+            if (++st == NST) { st = 0; ++round; }
+            if (++wg == nwg) { wg = 0; ++ph; }
+        }
+    } else {
+        // =========================== weight tiles ===========================
+        const uint32_t bytes = (uint32_t)min(N, p.Co16 - co0) * 32u;
+        int st = 0, ph = 0, wg = 0;
+        uint32_t round = 0;
+        for (int c = 0; c < nchunks; ++c) {
+            if (round > 0) {
+                const bool got = mbar_wait_bounded_hot(&empty[st], (round - 1) & 1u, abortp, limit);
+                if (!__all_sync(0xffffffffu, got)) break;
+            }
+            const int nq = min(KW, nw - wg * KW), t0 = g.ph_tap0[ph], ntaps = g.ph_tap0[ph + 1] - t0, n = nq * ntaps;
+            if (lane == 0) mbar_arrive_expect_tx(&full[st], bytes * (uint32_t)n);
+            __syncwarp();
+            uint8_t* B = stages + st * g.stage_bytes + g.b_off;
+            for (int i = lane; i < n; i += 32) {
+                const int q = i / ntaps, ts = t0 + (i - q * ntaps);
+                const size_t at = ((size_t)(s_tap_id[ts] * p.CW + w0 + wg * KW + q) * p.Co16 + co0) * 32;
+                // (a copy skipped by the range-checked build leaves its barrier incomplete: the CTA gives up at its wait)
+                if (EBS_IN_RANGE(p, CHK_UT_W8, at + bytes - 1, p.lim_w8)) bulk_copy_g2s(B + i * b_tile, p.w8 + at, bytes, &full[st]);
+            }
+            if (++st == NST) { st = 0; ++round; }
+            if (++wg == nwg) { wg = 0; ++ph; }
+        }
+        if (*abortp)                                     // copies may still be in flight towards this CTA's shared memory
+            for (int i = 0; i < 64; ++i) __nanosleep(1000);
+    }
+
+    if constexpr (FORM != 0) {
+        // =========================== epilogue, a thread per pixel ===========================
+        if (warp < 8) {
+            asm volatile("bar.sync 1, 256;\n" ::: "memory");    // gp_s and the terms
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            if (abort_flag == 0) {
+                const int gp = gp_s[(warp & 3) * 32 + lane];
+                const bool pvalid = gp >= 0;
+                const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+                const int nb = p.next_bits, qmax = (1 << nb) - 1;
+                const float hi2 = (float)(2 * qmax + 1);
+                if (__any_sync(0xffffffffu, pvalid)) {
+#pragma unroll 1
+                    for (int c0 = (warp >> 2) * 32; c0 < N && co0 + c0 < p.Co; c0 += 64) {
+                        uint32_t v[32];
+                        uint32_t (&lo)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[0]);
+                        uint32_t (&hi)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[16]);
+                        tmem_ld16_issue(trow + (uint32_t)c0, lo);
+                        tmem_ld16_issue(trow + (uint32_t)(c0 + 16), hi);
+                        const int word = (co0 + c0) >> 5;
+                        uint32_t cr[8];
+                        if constexpr (FORM == 2) {
+                            float res[32];
+                            uint32_t rbyte[8];
+                            const float4* cs = reinterpret_cast<const float4*>(s_terms + c0);
+                            const float4* cb = reinterpret_cast<const float4*>(s_terms + 256 + c0);
+                            if (p.residual) {
+                                const float4* r4 = reinterpret_cast<const float4*>(p.residual + (size_t)(pvalid ? gp : 0) * p.Co + co0 + c0);
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) {
+                                    const float4 t = __ldg(r4 + i);
+                                    res[4 * i] = t.x; res[4 * i + 1] = t.y; res[4 * i + 2] = t.z; res[4 * i + 3] = t.w;
+                                }
+                            } else if (p.res_packed) {
+                                const uint32_t* rw = p.res_packed + ((size_t)(pvalid ? gp : 0) * p.CWo + word) * p.res_bits;
+                                uint32_t rw8[8];
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) rw8[j] = j < p.res_bits ? __ldg(rw + j) : 0u;
+                                planes_to_bytes<8>(rw8, rbyte);
+                            }
+                            tmem_ld16_wait(lo);
+                            tmem_ld16_wait(hi);
+                            if (p.residual) terms_codes32<1>(v, p.S, cs, cb, res, rbyte, 0.0f, p.inv_next, hi2, cr);
+                            else if (p.res_packed) terms_codes32<2>(v, p.S, cs, cb, res, rbyte, p.res_scale, p.inv_next, hi2, cr);
+                            else terms_codes32<0>(v, p.S, cs, cb, res, rbyte, 0.0f, p.inv_next, hi2, cr);
+                        } else {
+                            tmem_ld16_wait(lo);
+                            tmem_ld16_wait(hi);
+                            const uint64_t S2 = f32x2_pack(p.S, p.S);
+#pragma unroll
+                            for (int bb = 0; bb < 8; ++bb) {
+                                uint32_t m[4];
+#pragma unroll
+                                for (int h = 0; h < 2; ++h) {
+                                    const uint64_t w = f32x2_mul_rn(f32x2_pack((float)(int)v[16 * h + bb], (float)(int)v[16 * h + 8 + bb]), S2);
+                                    m[2 * h] = code_pattern(__fadd_rn(__fmul_rn(__uint_as_float((uint32_t)w), p.inv_next), 0.5f), hi2);
+                                    m[2 * h + 1] = code_pattern(__fadd_rn(__fmul_rn(__uint_as_float((uint32_t)(w >> 32)), p.inv_next), 0.5f), hi2);
+                                }
+                                const uint32_t c4 = join_codes(m);
+                                cr[bb] = __funnelshift_l(c4, c4, bb);
+                            }
+                        }
+                        uint32_t planes[8];
+                        bytes_to_planes(cr, nb, planes);
+                        uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + word) * nb;
+                        if (pvalid && EBS_IN_RANGE(p, CHK_UT_PN, (dst - p.packed_next) + nb - 1, p.lim_pn)) store_plane_words(planes, nb, dst);
+                    }
+                }
+            }
+        }
+    } else {
+        // =========================== epilogue through shared memory ===========================
+        // A worker's TMEM row -> its row of partial sums [128][part_pitch] (the stages are free: every MMA has finished).
+        int* part = reinterpret_cast<int*>(stages);
+        const int pitch = g.part_pitch;
+        __syncwarp();
+        if (warp < 8 && !__any_sync(0xffffffffu, abort_flag != 0)) {
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+            int* row = part + ((warp & 3) * 32 + lane) * pitch;
+            const int cols = N + (p.w_levels ? 1 : 0);
+#pragma unroll 1
+            for (int c0 = (warp >> 2) * 16; c0 < cols; c0 += 32) {
+                uint32_t v[16];
+                tmem_ld16(trow + (uint32_t)c0, v);
+                if (c0 < N) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) *reinterpret_cast<int4*>(row + c0 + 4 * i) = make_int4((int)v[4 * i], (int)v[4 * i + 1], (int)v[4 * i + 2], (int)v[4 * i + 3]);
+                } else {
+                    row[N] = (int)v[0];                  // the window sum
+                }
+            }
+        }
+        __syncwarp();
+        if (split > 1) cluster_sync_all();
+        else __syncthreads();
+        if (warp < 8 && abort_flag == 0) {
+            // This CTA finishes rows rank * 128 / split ..; a warp takes 32 channels of four pixels at a time, a lane four
+            // channels of one of them (16-byte accesses; with a channel a lane the same work took five times the instructions).
+            const int groups = (N + 31) >> 5, rows = UMMA_M / split, grp = warp & (groups - 1), rstep = 8 / groups;
+            const int sub = lane & 7, col = grp * 32 + 4 * sub, co = co0 + col, live = col < N ? min(max(p.Co - co, 0), 4) : 0;
+            const int nb = p.next_bits, qmax = (1 << nb) - 1, word = (co0 >> 5) + grp, hw = p.Ho * p.Wo;
+            const bool vec = (p.Co & 3) == 0;            // then live is 0 or 4 and every access is aligned
+            float cs[4], cb[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                cs[i] = i < live ? term_at(p.ch_scale, co + i, p.Co, 1.0f) : 1.0f;
+                cb[i] = i < live ? term_at(p.ch_bias, co + i, p.Co, -0.0f) : -0.0f;
+            }
+            const int off = min(col, N - 4);
+#pragma unroll 1
+            for (int r0 = (warp / groups) * 4; r0 < rows; r0 += rstep * 4) {
+                const int row = rank * rows + r0 + (lane >> 3), gp = gp_s[row];
+                int* sums = part + row * pitch;
+                int a[4], wsum = 0;
+                if (split == 1) {
+                    const int4 t = *reinterpret_cast<const int4*>(sums + off);
+                    a[0] = t.x; a[1] = t.y; a[2] = t.z; a[3] = t.w;
+                    if (p.w_levels) wsum = sums[N];
+                } else {                                 // exact: integer partial sums of the cluster's CTAs
+                    const uint32_t at = smem_u32(sums + off);
+                    int4 t[TILE_MAX_SPLIT];
+#pragma unroll
+                    for (int r = 0; r < TILE_MAX_SPLIT; ++r) {
+                        t[r] = make_int4(0, 0, 0, 0);
+                        if (r < split) {
+                            uint32_t peer;
+                            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(peer) : "r"(at), "r"(r));
+                            asm volatile("ld.shared::cluster.v4.s32 {%0, %1, %2, %3}, [%4];\n"
+                                         : "=r"(t[r].x), "=r"(t[r].y), "=r"(t[r].z), "=r"(t[r].w) : "r"(peer));
+                            if (p.w_levels) {
+                                int wr;
+                                asm volatile("ld.shared::cluster.s32 %0, [%1];\n" : "=r"(wr) : "r"(peer + 4u * (uint32_t)(N - off)));
+                                wsum += wr;
+                            }
+                        }
+                    }
+                    a[0] = a[1] = a[2] = a[3] = 0;
+#pragma unroll
+                    for (int r = 0; r < TILE_MAX_SPLIT; ++r) { a[0] += t[r].x; a[1] += t[r].y; a[2] += t[r].z; a[3] += t[r].w; }
+                }
+                if (p.w_levels) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) a[i] = 2 * a[i] + wsum;
+                }
+                const bool out = gp >= 0 && live > 0;
+                const size_t o = (size_t)(gp < 0 ? 0 : gp) * p.Co + co;
+                if (p.acc && out && EBS_IN_RANGE(p, CHK_UT_ACC, o + live - 1, p.lim_out)) {
+                    if (vec) *reinterpret_cast<int4*>(p.acc + o) = make_int4(a[0], a[1], a[2], a[3]);
+                    else
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (i < live) p.acc[o + i] = a[i];
+                }
+                float y[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) y[i] = __fadd_rn(__fmul_rn(__fmul_rn((float)a[i], p.S), cs[i]), cb[i]);
+                if (p.residual && out) {
+                    if (vec) {
+                        const float4 t = __ldg(reinterpret_cast<const float4*>(p.residual + o));
+                        y[0] = __fadd_rn(y[0], t.x); y[1] = __fadd_rn(y[1], t.y); y[2] = __fadd_rn(y[2], t.z); y[3] = __fadd_rn(y[3], t.w);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (i < live) y[i] = __fadd_rn(y[i], __ldg(p.residual + o + i));
+                    }
+                }
+                if (p.res_packed && out) {
+                    const uint32_t* rw = p.res_packed + ((size_t)gp * p.CWo + word) * p.res_bits;
+                    uint32_t code4 = 0u;                 // plane j of the four channels -> bit j of four bytes
+#pragma unroll 1
+                    for (int j = 0; j < p.res_bits; ++j)
+                        code4 |= ((((__ldg(rw + j) >> (4 * sub)) & 0xFu) * 0x00204081u) & 0x01010101u) << j;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) y[i] = __fadd_rn(y[i], __fmul_rn(p.res_scale, byte_to_float(code4, i)));
+                }
+                if (p.relu) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) y[i] = y[i] > 0.0f ? y[i] : 0.0f;
+                }
+                if (p.y && out && EBS_IN_RANGE(p, CHK_UT_Y, o + live - 1, p.lim_out)) {
+                    if (p.y_nchw) {
+                        const int img = gp / hw;
+                        float* dst = p.y + ((size_t)img * p.Co + co) * hw + (gp - img * hw);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (i < live) dst[(size_t)i * hw] = y[i];
+                    } else if (vec) {
+                        *reinterpret_cast<float4*>(p.y + o) = make_float4(y[0], y[1], y[2], y[3]);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (i < live) p.y[o + i] = y[i];
+                    }
+                }
+                if (p.packed_next) {                     // the four codes as bytes over the start of the group's sums
+                    uint32_t code4 = 0u;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (i < live) code4 |= (uint32_t)quantize_act_code(y[i], p.inv_next, qmax) << (8 * i);
+                    __syncwarp();                        // every lane of these rows has read its sums
+                    reinterpret_cast<uint32_t*>(sums + grp * 32)[sub] = code4;
+                }
+            }
+            if (p.packed_next) {
+                asm volatile("bar.sync 1, 256;\n" ::: "memory");
+                // a thread per (pixel, 32-channel word): 32 code bytes in channel order -> plane words
+                for (int e = tid; e < rows * groups; e += TILE_WORKERS) {
+                    const int r = e / groups, gi = e - r * groups, row = rank * rows + r, gp = gp_s[row], wd = (co0 >> 5) + gi;
+                    if (gp < 0 || wd >= p.CWo) continue;
+                    const uint4* src4 = reinterpret_cast<const uint4*>(part + row * pitch + gi * 32);
+                    const uint4 lo = src4[0], hi = src4[1];
+                    const uint32_t n[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+                    uint32_t cr[8], planes[8];
+#pragma unroll
+                    for (int bb = 0; bb < 8; ++bb) {     // register bb: channels bb, 8 + bb, 16 + bb, 24 + bb
+                        const uint32_t sel = 0x0040u + 0x11u * (uint32_t)(bb & 3);
+                        const uint32_t c4 = __byte_perm(__byte_perm(n[bb >> 2], n[2 + (bb >> 2)], sel), __byte_perm(n[4 + (bb >> 2)], n[6 + (bb >> 2)], sel), 0x5410);
+                        cr[bb] = __funnelshift_l(c4, c4, bb);
+                    }
+                    bytes_to_planes(cr, nb, planes);
+                    uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + wd) * nb;
+                    if (EBS_IN_RANGE(p, CHK_UT_PN, (dst - p.packed_next) + nb - 1, p.lim_pn)) store_plane_words(planes, nb, dst);
+                }
+            }
+        }
+        __syncwarp();
+        if (split > 1) cluster_sync_all();               // no CTA leaves while another may read its sums
+    }
+
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (abort_flag != 0 && tid == 0) atomicAdd(&g_umma_timeouts, 1ull);
+    if (warp == TILE_ISSUER)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"((uint32_t)g.tmem_cols) : "memory");
+}
+
+int tile_sm_count();
+
+// Whether the epilogue can run a thread per pixel (forms 1 and 2): packed planes only, whole 32-channel words.
+inline bool tile_thread_epilogue(const ConvParams& p, int tile_n) {
+    return p.packed_next && !p.acc && !p.y && !p.w_levels && (p.Co & 31) == 0 && (tile_n & 31) == 0 && !(p.residual && p.res_packed);
+}
+
+template <int AB, int FORM>
+int launch_conv_umma_tile_form(const ConvParams& p, const TileGeom& g, cudaStream_t st) {
+    auto kern = conv_umma_tile_kernel<AB, FORM>;
+    static bool attr_set[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !attr_set[dev]) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_SMEM_MAX);
+        attr_set[dev] = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)g.n_ptiles, (unsigned)g.n_ctiles, (unsigned)g.split);
+    cfg.blockDim = dim3(TILE_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)g.smem_bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = (unsigned)g.split;
+    cfg.attrs = attr;
+    cfg.numAttrs = g.split > 1 ? 2 : 1;
+    return check_cuda(cudaLaunchKernelEx(&cfg, kern, p, g));
+}
+
+template <int AB, int TILE_N>
+int launch_conv_umma_tile(const ConvParams& p, dim3 /*grid*/, cudaStream_t st) {
+    const TileGeom g = tile_geometry(p, TILE_N, tile_sm_count(), p.tile_split);
+    if (!g.ok) return EBS_ERR_UNSUPPORTED;                    // the geometry does not apply: nothing is launched
+    if (g.split == 1 && tile_thread_epilogue(p, TILE_N))
+        return p.ch_scale || p.ch_bias || p.residual || p.res_packed ? launch_conv_umma_tile_form<AB, 2>(p, g, st)
+                                                                     : launch_conv_umma_tile_form<AB, 1>(p, g, st);
+    return launch_conv_umma_tile_form<AB, 0>(p, g, st);
+}
+
+constexpr int NUM_TILE_VARIANTS = 5;           // TILE_N = 16, 32, 64, 128, 256
+
+// One translation unit per activation bit count (conv_umma_tile_a1.cu .. a8.cu).
+#define EBS_DEFINE_TILE_ROW(AB)                                                                            \
+    const ConvVariant* conv_umma_variant_a##AB(int variant) {                                              \
+        static const ConvVariant row[NUM_TILE_VARIANTS] = {                                                \
+            ConvVariant{&launch_conv_umma_tile<AB, 16>, UMMA_M, 16, TILE_THREADS},                         \
+            ConvVariant{&launch_conv_umma_tile<AB, 32>, UMMA_M, 32, TILE_THREADS},                         \
+            ConvVariant{&launch_conv_umma_tile<AB, 64>, UMMA_M, 64, TILE_THREADS},                         \
+            ConvVariant{&launch_conv_umma_tile<AB, 128>, UMMA_M, 128, TILE_THREADS},                       \
+            ConvVariant{&launch_conv_umma_tile<AB, 256>, UMMA_M, 256, TILE_THREADS}};                      \
+        return variant < 0 || variant >= NUM_TILE_VARIANTS ? nullptr : &row[variant];                      \
+    }                                                                                                      \
+    unsigned long long conv_umma_timeouts_a##AB() {                                                        \
+        unsigned long long v = 0;                                                                          \
+        cudaMemcpyFromSymbol(&v, g_umma_timeouts, sizeof(v));                                              \
+        return v;                                                                                          \
+    }
+
+}  // namespace ebs

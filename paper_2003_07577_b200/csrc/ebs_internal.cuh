@@ -41,6 +41,7 @@ struct ConvParams {
     int strip_pix, strip_ks;          // strip kernel only (set by its launcher): pixels of a strip, words per stage
     unsigned wait_limit;              // polls a bounded device-side wait makes before the CTA gives up
     int test_flags;                   // bit 0 (tests only): the MMA issuer issues nothing, so that waits run out
+    int tile_split;                   // tile kernel: CTAs the reduction is split over (0 = chosen by the library)
     int pipe_m_sub;                   // persistent pipeline kernel: accumulators per super-tile (0 = chosen by the library)
     int acc_small;                    // 1: every accumulator of the layer is below 2^22 in magnitude (worst case of its sizes and bit counts)
     // Extents of the buffers, for the range-checked build (EBS_CHECKED); filled in every build.
@@ -70,7 +71,7 @@ __device__ __forceinline__ bool check_in_range(unsigned long long* st, unsigned 
 #define EBS_IN_RANGE(p, site, idx, limit) true
 #endif
 // Sites (kernel family * 16 + access): 1x pipeline kernel, 2x warp-level strip kernel, 3x warp-level per-tap kernel,
-// 4x integer-pipe kernel, 5x shared epilogue helpers.
+// 4x integer-pipe kernel, 5x shared epilogue helpers, 6x tile kernel.
 enum CheckSite {
     CHK_PIPE_X = 0x10, CHK_PIPE_STAGE = 0x11, CHK_PIPE_TAB = 0x12, CHK_PIPE_ACC = 0x13, CHK_PIPE_Y = 0x14, CHK_PIPE_PN = 0x15,
     CHK_PIPE_W8 = 0x16,
@@ -78,6 +79,7 @@ enum CheckSite {
     CHK_MMA_X = 0x30, CHK_MMA_W8 = 0x31, CHK_MMA_ACC = 0x32, CHK_MMA_Y = 0x33, CHK_MMA_STAGE = 0x34,
     CHK_POPC_X = 0x40, CHK_POPC_W = 0x41, CHK_POPC_ACC = 0x42, CHK_POPC_Y = 0x43, CHK_POPC_SMEM = 0x44,
     CHK_TILE_PN = 0x50, CHK_TILE_CODES = 0x51,
+    CHK_UT_X = 0x60, CHK_UT_STAGE = 0x61, CHK_UT_W8 = 0x62, CHK_UT_ACC = 0x63, CHK_UT_Y = 0x64, CHK_UT_PN = 0x65,
 };
 
 // One instantiation of the popcount kernel: launch function + its tile geometry.
@@ -105,7 +107,7 @@ EBS_DECLARE_AB(1) EBS_DECLARE_AB(2) EBS_DECLARE_AB(3) EBS_DECLARE_AB(4)
 EBS_DECLARE_AB(5) EBS_DECLARE_AB(6) EBS_DECLARE_AB(7) EBS_DECLARE_AB(8)
 #undef EBS_DECLARE_AB
 
-// 5th-generation tensor-core kernels (conv_umma_w1.cu .. conv_umma_w8.cu); variant = log2(tile_n / 16).
+// Tile kernels on the 5th-generation tensor cores (conv_umma_tile*.cu); variant = log2(tile_n / 16).
 enum { NUM_CONV_UMMA_VARIANTS = 5, NUM_CONV_STRIP_VARIANTS = 5, NUM_CONV_RESIDENT_VARIANTS = 5, NUM_CONV_MMA_STRIP_VARIANTS = 3,
        NUM_CONV_PIPE_VARIANTS = 4 };
 // Persistent pipeline kernel for any stride (conv_umma_pipe.cu): variants 0-2 by channel tile 64 << variant, variant 3 the
@@ -125,14 +127,11 @@ unsigned long long conv_umma_resident_timeouts();
 const ConvVariant* conv_umma_strip_variant(int a_bits, int variant);
 bool conv_umma_strip_applies(const ConvParams& p, int variant);
 unsigned long long conv_umma_strip_timeouts();
-const ConvVariant* conv_umma_variant(int w_bits, int a_bits, int variant);
+const ConvVariant* conv_umma_variant(int a_bits, int variant);
+bool conv_umma_applies(const ConvParams& p, int variant);
+float conv_umma_cost(const ConvParams& p, int variant);   // estimated clocks, negative if it does not apply
+unsigned long long conv_umma_tile_timeouts();
 unsigned long long conv_umma_timeouts();
-#define EBS_DECLARE_WB(WB)                                                   \
-    const ConvVariant* conv_umma_variant_w##WB(int a_bits, int variant);     \
-    unsigned long long conv_umma_timeouts_w##WB();
-EBS_DECLARE_WB(1) EBS_DECLARE_WB(2) EBS_DECLARE_WB(3) EBS_DECLARE_WB(4)
-EBS_DECLARE_WB(5) EBS_DECLARE_WB(6) EBS_DECLARE_WB(7) EBS_DECLARE_WB(8)
-#undef EBS_DECLARE_WB
 
 // pack.cu
 int launch_pack_acts_s2d(const void* x, int n, int c, int h, int w, int off, int a_bits, uint32_t* out, cudaStream_t st);

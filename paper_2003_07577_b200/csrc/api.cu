@@ -234,6 +234,7 @@ static int conv_plan(const void* packed_x, int n, int h, int w, const void* pack
     p.acc = acc_out; p.y = y_out; p.packed_next = static_cast<uint32_t*>(packed_next);
     p.S = d->w_scale * d->a_scale;       // one rounded fp32 multiply
     p.next_bits = 1;
+    p.one = 1.0f;
     p.w_levels = d->w_levels;
     p.fold = d->c_in <= 4 ? 8 : (d->c_in <= 8 ? 4 : (d->c_in <= 16 ? 2 : 1));
     p.fold_bits = 32 / p.fold;

@@ -33,6 +33,8 @@ struct FrameGeom {
     int q0r, q0s;                      // smallest tap quotients (<= 0)
     int taps, n_ph, max_shift, max_ph_taps;
     int ph_a[FRAME_MAX_PHASES], ph_b[FRAME_MAX_PHASES];
+    int ph_rows[FRAME_MAX_PHASES], ph_cols[FRAME_MAX_PHASES], ph_shift[FRAME_MAX_PHASES];   // a phase's taps: rows x cols
+                                       // consecutive shifts (row pitch Wq) from ph_shift on
     int ph_tap0[FRAME_MAX_PHASES + 1]; // tap slots of phase i: [ph_tap0[i], ph_tap0[i + 1])
     short tap_shift[FRAME_MAX_TAPS];   // per tap slot: shift inside the strip, in pixels
     short tap_id[FRAME_MAX_TAPS];      // per tap slot: r * kw + s (tile index in the weight byte image)
@@ -79,6 +81,11 @@ inline bool frame_geometry(const ConvParams& p, FrameGeom& g) {
                 g.ph_a[g.n_ph] = a;
                 g.ph_b[g.n_ph] = b;
                 g.ph_tap0[g.n_ph] = first;
+                g.ph_shift[g.n_ph] = g.tap_shift[first];
+                g.ph_cols[g.n_ph] = 1;                       // (r = stride q + a: the quotients of a phase are consecutive)
+                while (first + g.ph_cols[g.n_ph] < slot && g.tap_shift[first + g.ph_cols[g.n_ph]] == g.tap_shift[first] + g.ph_cols[g.n_ph] &&
+                       g.tap_id[first + g.ph_cols[g.n_ph]] / p.kw == g.tap_id[first] / p.kw) ++g.ph_cols[g.n_ph];
+                g.ph_rows[g.n_ph] = (slot - first) / g.ph_cols[g.n_ph];
                 ++g.n_ph;
                 if (slot - first > g.max_ph_taps) g.max_ph_taps = slot - first;
             }
@@ -248,6 +255,100 @@ __device__ __forceinline__ uint64_t f32x2_add_rd(uint64_t a, uint64_t b) {
     return d;
 }
 
+// Two rounded additions in one instruction, as multiply-adds by one: `one2` holds 1.0f twice, passed in at run time.  A
+// packed addition behind a packed product comes out of the assembler as one fused operation, which changes codes at ties;
+// a product by a run-time value cannot be folded that way.
+__device__ __forceinline__ uint64_t f32x2_add_one(uint64_t a, uint64_t one2, uint64_t b) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(one2), "l"(b));
+    return d;
+}
+
+// Global loads of what an earlier launch in the stream wrote, for kernels that may start before that launch has ended
+// (programmatic dependent launch): neither through the read-only path (its data must not change while the kernel runs) nor
+// movable across the wait for the earlier launch.
+__device__ __forceinline__ uint32_t ld_dep(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];\n" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 ld_dep(const uint2* p) {
+    uint2 v;
+    asm volatile("ld.global.v2.u32 {%0, %1}, [%2];\n" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 ld_dep(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_dep(const float* p) { return __uint_as_float(ld_dep(reinterpret_cast<const uint32_t*>(p))); }
+__device__ __forceinline__ float4 ld_dep(const float4* p) {
+    const uint4 v = ld_dep(reinterpret_cast<const uint4*>(p));
+    return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
+}
+// NW packed words in the widest loads their alignment (4 * NW bytes) allows.
+template <int NW>
+__device__ __forceinline__ void ld_dep_words(const uint32_t* src, uint32_t (&dst)[NW]) {
+    if constexpr (NW % 4 == 0) {
+#pragma unroll
+        for (int i = 0; i < NW / 4; ++i) {
+            const uint4 t = ld_dep(reinterpret_cast<const uint4*>(src) + i);
+            dst[4 * i] = t.x; dst[4 * i + 1] = t.y; dst[4 * i + 2] = t.z; dst[4 * i + 3] = t.w;
+        }
+    } else if constexpr (NW % 2 == 0) {
+#pragma unroll
+        for (int i = 0; i < NW / 2; ++i) {
+            const uint2 t = ld_dep(reinterpret_cast<const uint2*>(src) + i);
+            dst[2 * i] = t.x; dst[2 * i + 1] = t.y;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < NW; ++i) dst[i] = ld_dep(src + i);
+    }
+}
+// The same for a run-time number of words (1 .. 8; the others become 0).
+__device__ __forceinline__ void ld_dep_planes(const uint32_t* src, int n, uint32_t (&dst)[8]) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) dst[j] = 0u;
+    if ((n & 3) == 0) {
+        const uint4 t = ld_dep(reinterpret_cast<const uint4*>(src));
+        dst[0] = t.x; dst[1] = t.y; dst[2] = t.z; dst[3] = t.w;
+        if (n == 8) {
+            const uint4 u = ld_dep(reinterpret_cast<const uint4*>(src) + 1);
+            dst[4] = u.x; dst[5] = u.y; dst[6] = u.z; dst[7] = u.w;
+        }
+    } else if ((n & 1) == 0) {
+        const uint2 t = ld_dep(reinterpret_cast<const uint2*>(src));
+        dst[0] = t.x; dst[1] = t.y;
+        if (n == 6) {
+            const uint2 u = ld_dep(reinterpret_cast<const uint2*>(src) + 1), w = ld_dep(reinterpret_cast<const uint2*>(src) + 2);
+            dst[2] = u.x; dst[3] = u.y; dst[4] = w.x; dst[5] = w.y;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 7; ++j)
+            if (j < n) dst[j] = ld_dep(src + j);
+    }
+}
+
+// Bounded wait for a whole warp: the outcome is a vote, so that the loops around it stay warp-uniform for the compiler.
+__device__ __forceinline__ bool mbar_wait_bounded_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, unsigned limit) {
+    const uint32_t addr = smem_u32(bar);
+    for (unsigned it = 0; it < limit; ++it) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}\n"
+            : "=r"(done) : "r"(addr), "r"(parity) : "memory");
+        if (__all_sync(0xffffffffu, done != 0)) return true;
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+    }
+    *abort_flag = 1;
+    return false;
+}
+
 // Four requantized codes (low bytes of code_pattern results) -> one register, channel order as in planes_to_bytes.
 __device__ __forceinline__ uint32_t join_codes(const uint32_t (&m)[4]) {
     return __byte_perm(__byte_perm(m[0], m[1], 0x0040), __byte_perm(m[2], m[3], 0x0040), 0x5410);
@@ -260,34 +361,104 @@ __device__ __forceinline__ float byte_to_float(uint32_t w, int i) {
 // Per-channel terms of a 32-channel group in the order terms_codes32 reads them: entry bb = channels bb, 8 + bb, 16 + bb,
 // 24 + bb; identities (x * 1, x + (-0)) where a layer has no such term or the channel does not exist.
 __device__ __forceinline__ float term_at(const float* t, int co, int Co, float identity) {
-    return t && co < Co ? __ldg(t + co) : identity;
+    return t && co < Co ? ld_dep(t + co) : identity;
 }
 
 // 32 accumulators of one pixel and 32-channel group -> eight registers of requantized codes (register bb: channels bb,
 // 8 + bb, 16 + bb, 24 + bb), with per-channel scale and shift and a shortcut: RES 0 none, 1 fp32 values of the pixel's
 // 32 channels, 2 codes in byte registers of the same order.  Every fp32 step is rounded on its own, in the library's
 // order.  The terms come from shared memory as broadcast 16-byte reads (read through the cache channel by channel they
-// were two thirds of the instructions of this function); products are packed two to an instruction, additions are scalar
-// because the assembler contracts a packed product and a packed sum into a fused operation.  The ReLU is not applied: the
-// quantizer's clamp at zero gives the same codes.
+// were two thirds of the instructions of this function); products and sums are packed two to an instruction
+// (f32x2_add_one).  The ReLU is not applied: the quantizer's clamp at zero gives the same codes.
 template <int RES>
-__device__ __forceinline__ void terms_codes32(const uint32_t (&v)[32], float S, const float4* cs, const float4* cb,
+__device__ __forceinline__ void terms_codes32(const uint32_t (&v)[32], float S, float one, const float4* cs, const float4* cb,
                                               const float (&res)[32], const uint32_t (&rbyte)[8], float res_scale,
                                               float inv_next, float hi2, uint32_t (&cr)[8]) {
-    const uint64_t S2 = f32x2_pack(S, S);
+    const uint64_t S2 = f32x2_pack(S, S), one2 = f32x2_pack(one, one), inv2 = f32x2_pack(inv_next, inv_next);
+    const uint64_t half2 = f32x2_pack(0.5f, 0.5f), rs2 = f32x2_pack(res_scale, res_scale);
 #pragma unroll
     for (int bb = 0; bb < 8; ++bb) {
         const float4 a = cs[bb], b = cb[bb];
-        const uint64_t w0 = f32x2_mul_rn(f32x2_mul_rn(f32x2_pack((float)(int)v[bb], (float)(int)v[8 + bb]), S2), f32x2_pack(a.x, a.y));
-        const uint64_t w1 = f32x2_mul_rn(f32x2_mul_rn(f32x2_pack((float)(int)v[16 + bb], (float)(int)v[24 + bb]), S2), f32x2_pack(a.z, a.w));
-        float t[4] = {__fadd_rn(__uint_as_float((uint32_t)w0), b.x), __fadd_rn(__uint_as_float((uint32_t)(w0 >> 32)), b.y),
-                      __fadd_rn(__uint_as_float((uint32_t)w1), b.z), __fadd_rn(__uint_as_float((uint32_t)(w1 >> 32)), b.w)};
+        uint64_t w[2] = {f32x2_mul_rn(f32x2_pack((float)(int)v[bb], (float)(int)v[8 + bb]), S2),
+                         f32x2_mul_rn(f32x2_pack((float)(int)v[16 + bb], (float)(int)v[24 + bb]), S2)};
+        w[0] = f32x2_add_one(f32x2_mul_rn(w[0], f32x2_pack(a.x, a.y)), one2, f32x2_pack(b.x, b.y));
+        w[1] = f32x2_add_one(f32x2_mul_rn(w[1], f32x2_pack(a.z, a.w)), one2, f32x2_pack(b.z, b.w));
         uint32_t m[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (RES == 1) t[i] = __fadd_rn(t[i], res[8 * i + bb]);
-            if (RES == 2) t[i] = __fadd_rn(t[i], __fmul_rn(res_scale, byte_to_float(rbyte[bb], i)));
-            m[i] = code_pattern(__fadd_rn(__fmul_rn(t[i], inv_next), 0.5f), hi2);
+        for (int h = 0; h < 2; ++h) {
+            if (RES == 1) w[h] = f32x2_add_one(w[h], one2, f32x2_pack(res[16 * h + bb], res[16 * h + 8 + bb]));
+            if (RES == 2) w[h] = f32x2_add_one(w[h], one2, f32x2_mul_rn(rs2, f32x2_pack(byte_to_float(rbyte[bb], 2 * h), byte_to_float(rbyte[bb], 2 * h + 1))));
+            w[h] = f32x2_add_one(f32x2_mul_rn(w[h], inv2), one2, half2);
+            m[2 * h] = code_pattern(__uint_as_float((uint32_t)w[h]), hi2);
+            m[2 * h + 1] = code_pattern(__uint_as_float((uint32_t)(w[h] >> 32)), hi2);
+        }
+        const uint32_t c4 = join_codes(m);
+        cr[bb] = __funnelshift_l(c4, c4, bb);
+    }
+}
+
+// The same in two steps, for layers that want the fp32 values too: pair (h, bb) = channels 16 h + bb and 16 h + 8 + bb.
+template <int RES>
+__device__ __forceinline__ void terms_values32(const uint32_t (&v)[32], float S, float one, const float4* cs, const float4* cb,
+                                               const float (&res)[32], const uint32_t (&rbyte)[8], float res_scale, uint64_t (&yy)[2][8]) {
+    const uint64_t S2 = f32x2_pack(S, S), one2 = f32x2_pack(one, one), rs2 = f32x2_pack(res_scale, res_scale);
+#pragma unroll
+    for (int bb = 0; bb < 8; ++bb) {
+        const float4 a = cs[bb], b = cb[bb];
+        uint64_t w[2] = {f32x2_mul_rn(f32x2_pack((float)(int)v[bb], (float)(int)v[8 + bb]), S2),
+                         f32x2_mul_rn(f32x2_pack((float)(int)v[16 + bb], (float)(int)v[24 + bb]), S2)};
+        w[0] = f32x2_add_one(f32x2_mul_rn(w[0], f32x2_pack(a.x, a.y)), one2, f32x2_pack(b.x, b.y));
+        w[1] = f32x2_add_one(f32x2_mul_rn(w[1], f32x2_pack(a.z, a.w)), one2, f32x2_pack(b.z, b.w));
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (RES == 1) w[h] = f32x2_add_one(w[h], one2, f32x2_pack(res[16 * h + bb], res[16 * h + 8 + bb]));
+            if (RES == 2) w[h] = f32x2_add_one(w[h], one2, f32x2_mul_rn(rs2, f32x2_pack(byte_to_float(rbyte[bb], 2 * h), byte_to_float(rbyte[bb], 2 * h + 1))));
+            yy[h][bb] = w[h];
+        }
+    }
+}
+__device__ __forceinline__ void value_codes32(const uint64_t (&yy)[2][8], float one, float inv_next, float hi2, uint32_t (&cr)[8]) {
+    const uint64_t one2 = f32x2_pack(one, one), inv2 = f32x2_pack(inv_next, inv_next), half2 = f32x2_pack(0.5f, 0.5f);
+#pragma unroll
+    for (int bb = 0; bb < 8; ++bb) {
+        uint32_t m[4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint64_t w = f32x2_add_one(f32x2_mul_rn(yy[h][bb], inv2), one2, half2);
+            m[2 * h] = code_pattern(__uint_as_float((uint32_t)w), hi2);
+            m[2 * h + 1] = code_pattern(__uint_as_float((uint32_t)(w >> 32)), hi2);
+        }
+        const uint32_t c4 = join_codes(m);
+        cr[bb] = __funnelshift_l(c4, c4, bb);
+    }
+}
+__device__ __forceinline__ void store_values32(const uint64_t (&yy)[2][8], bool relu, float* dst) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        float t[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int c = 4 * q + e;                           // channel c: pair (c / 16, c % 8), upper lane if c & 8
+            const uint64_t w = yy[c >> 4][c & 7];
+            t[e] = __uint_as_float((c & 8) ? (uint32_t)(w >> 32) : (uint32_t)w);
+            if (relu) t[e] = t[e] > 0.f ? t[e] : 0.f;
+        }
+        *reinterpret_cast<float4*>(dst + 4 * q) = make_float4(t[0], t[1], t[2], t[3]);
+    }
+}
+
+// The same without per-channel terms and shortcut.
+__device__ __forceinline__ void plain_codes32(const uint32_t (&v)[32], float S, float one, float inv_next, float hi2, uint32_t (&cr)[8]) {
+    const uint64_t S2 = f32x2_pack(S, S), one2 = f32x2_pack(one, one), inv2 = f32x2_pack(inv_next, inv_next), half2 = f32x2_pack(0.5f, 0.5f);
+#pragma unroll
+    for (int bb = 0; bb < 8; ++bb) {
+        uint32_t m[4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint64_t w = f32x2_mul_rn(f32x2_pack((float)(int)v[16 * h + bb], (float)(int)v[16 * h + 8 + bb]), S2);
+            w = f32x2_add_one(f32x2_mul_rn(w, inv2), one2, half2);
+            m[2 * h] = code_pattern(__uint_as_float((uint32_t)w), hi2);
+            m[2 * h + 1] = code_pattern(__uint_as_float((uint32_t)(w >> 32)), hi2);
         }
         const uint32_t c4 = join_codes(m);
         cr[bb] = __funnelshift_l(c4, c4, bb);

@@ -224,64 +224,15 @@ __device__ __forceinline__ void pipe_group32(const ConvParams& p, uint32_t (&v)[
 #pragma unroll
         for (int bb = 0; bb < 8; ++bb)
             yy[h][bb] = f32x2_mul_rn(f32x2_pack((float)(int)v[16 * h + bb], (float)(int)v[16 * h + 8 + bb]), S2);
-    if (p.y && pvalid && EBS_IN_RANGE(p, CHK_PIPE_Y, o + 31, p.lim_out)) {
-        const bool relu = p.relu != 0;
-#pragma unroll
-        for (int gq = 0; gq < 8; ++gq) {
-            float t[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int c = 4 * gq + e;                           // channel c: pair (c / 16, c % 8), upper lane if c & 8
-                const uint64_t w = yy[c >> 4][c & 7];
-                t[e] = __uint_as_float((c & 8) ? (uint32_t)(w >> 32) : (uint32_t)w);
-                if (relu) t[e] = t[e] > 0.f ? t[e] : 0.f;
-            }
-            *reinterpret_cast<float4*>(p.y + o + 4 * gq) = make_float4(t[0], t[1], t[2], t[3]);
-        }
-    }
+    if (p.y && pvalid && EBS_IN_RANGE(p, CHK_PIPE_Y, o + 31, p.lim_out)) store_values32(yy, p.relu != 0, p.y + o);
     if (WANT_Q) {
         // The clamp at zero of the quantizer makes an explicit ReLU redundant here: a negative y gives
         // floor(y / step + 0.5) <= 0 and is clamped to code 0, exactly what max(y, 0) would give.
-        // Floor and clamp without the conversion pipe: code_pattern above.
-        // Byte register bb holds the codes of channels {bb, 8 + bb, 16 + bb, 24 + bb}, rotated left by bb.
         uint32_t cr[8];
-        const float hi2 = (float)(2 * qmax + 1);
-#pragma unroll
-        for (int bb = 0; bb < 8; ++bb) {
-            uint32_t m[4];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                // (the multiply and the addition of 0.5 are scalar instructions with explicit rounding, which the assembler
-                // never contracts into a fused multiply-add; issued as a packed pair they came out fused)
-                const uint64_t w = yy[h][bb];
-                m[2 * h] = code_pattern(__fadd_rn(__fmul_rn(__uint_as_float((uint32_t)w), inv_next), 0.5f), hi2);
-                m[2 * h + 1] = code_pattern(__fadd_rn(__fmul_rn(__uint_as_float((uint32_t)(w >> 32)), inv_next), 0.5f), hi2);
-            }
-            const uint32_t c4 = __byte_perm(__byte_perm(m[0], m[1], 0x0040), __byte_perm(m[2], m[3], 0x0040), 0x5410);
-            cr[bb] = __funnelshift_l(c4, c4, bb);
-        }
+        value_codes32(yy, p.one, inv_next, (float)(2 * qmax + 1), cr);
         uint32_t planes[8];
         bytes_to_planes(cr, nb, planes);
-        if (pvalid && EBS_IN_RANGE(p, CHK_PIPE_PN, (dst - p.packed_next) + nb - 1, p.lim_pn)) {
-            if (nb == 4) {
-                *reinterpret_cast<uint4*>(dst) = make_uint4(planes[0], planes[1], planes[2], planes[3]);
-            } else if (nb == 8) {
-                *reinterpret_cast<uint4*>(dst) = make_uint4(planes[0], planes[1], planes[2], planes[3]);
-                *reinterpret_cast<uint4*>(dst + 4) = make_uint4(planes[4], planes[5], planes[6], planes[7]);
-            } else if (nb == 2) {
-                *reinterpret_cast<uint2*>(dst) = make_uint2(planes[0], planes[1]);
-            } else if (nb == 6) {
-                *reinterpret_cast<uint2*>(dst) = make_uint2(planes[0], planes[1]);
-                *reinterpret_cast<uint2*>(dst + 2) = make_uint2(planes[2], planes[3]);
-                *reinterpret_cast<uint2*>(dst + 4) = make_uint2(planes[4], planes[5]);
-            } else {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    if (j >= nb) break;
-                    dst[j] = planes[j];
-                }
-            }
-        }
+        if (pvalid && EBS_IN_RANGE(p, CHK_PIPE_PN, (dst - p.packed_next) + nb - 1, p.lim_pn)) store_plane_words(planes, nb, dst);
     }
 }
 
@@ -333,26 +284,7 @@ __device__ __forceinline__ void pipe_store_planes(const uint32_t (&planes)[8], i
             return;
         }
     }
-    if (pvalid && EBS_IN_RANGE(p, CHK_PIPE_PN, (dst - p.packed_next) + nb - 1, p.lim_pn)) {
-        if (nb == 4) {
-            *reinterpret_cast<uint4*>(dst) = make_uint4(planes[0], planes[1], planes[2], planes[3]);
-        } else if (nb == 8) {
-            *reinterpret_cast<uint4*>(dst) = make_uint4(planes[0], planes[1], planes[2], planes[3]);
-            *reinterpret_cast<uint4*>(dst + 4) = make_uint4(planes[4], planes[5], planes[6], planes[7]);
-        } else if (nb == 2) {
-            *reinterpret_cast<uint2*>(dst) = make_uint2(planes[0], planes[1]);
-        } else if (nb == 6) {
-            *reinterpret_cast<uint2*>(dst) = make_uint2(planes[0], planes[1]);
-            *reinterpret_cast<uint2*>(dst + 2) = make_uint2(planes[2], planes[3]);
-            *reinterpret_cast<uint2*>(dst + 4) = make_uint2(planes[4], planes[5]);
-        } else {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                if (j >= nb) break;
-                dst[j] = planes[j];
-            }
-        }
-    }
+    if (pvalid && EBS_IN_RANGE(p, CHK_PIPE_PN, (dst - p.packed_next) + nb - 1, p.lim_pn)) store_plane_words(planes, nb, dst);
 }
 
 // The same group when only packed planes are asked for (a chained network: no accumulator and no fp32 output): the
@@ -363,89 +295,112 @@ template <int G>
 __device__ __forceinline__ void pipe_group32_packed(const uint32_t (&v)[32], bool pvalid, float S, float inv_next, int nb, int qmax,
                                                     uint32_t* dst, const ConvParams& p, PlaneHold<G>& hold) {
     uint32_t cr[8];
-    const uint64_t S2 = f32x2_pack(S, S);
-    const float hi2 = (float)(2 * qmax + 1);
-#pragma unroll
-    for (int bb = 0; bb < 8; ++bb) {
-        uint32_t m[4];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint64_t w = f32x2_mul_rn(f32x2_pack((float)(int)v[16 * h + bb], (float)(int)v[16 * h + 8 + bb]), S2);
-            m[2 * h] = code_pattern(__fadd_rn(__fmul_rn(__uint_as_float((uint32_t)w), inv_next), 0.5f), hi2);
-            m[2 * h + 1] = code_pattern(__fadd_rn(__fmul_rn(__uint_as_float((uint32_t)(w >> 32)), inv_next), 0.5f), hi2);
-        }
-        const uint32_t c4 = __byte_perm(__byte_perm(m[0], m[1], 0x0040), __byte_perm(m[2], m[3], 0x0040), 0x5410);
-        cr[bb] = __funnelshift_l(c4, c4, bb);
-    }
+    plain_codes32(v, S, p.one, inv_next, (float)(2 * qmax + 1), cr);
     uint32_t planes[8];
     bytes_to_planes(cr, nb, planes);
     pipe_store_planes(planes, nb, dst, pvalid, hold, p);
 }
 
-// The packed-only group of a layer with per-channel terms and / or a shortcut (a folded batch normalisation, the
-// second convolution of a residual block): the same chain per byte register with the terms applied in the library's
-// order -- per-channel scale, per-channel shift, fp32 shortcut, shortcut from packed codes -- each an individually
-// rounded fp32 operation.  The shortcut codes come out of their planes with the rotate-merge of the expanders, which
-// leaves them in exactly the byte registers (channels bb, 8 + bb, 16 + bb, 24 + bb) this loop works on.  The ReLU is
-// not applied: the quantizer's clamp at zero gives the same codes.
-template <int G>
-__device__ __forceinline__ void pipe_group32_affine(const uint32_t (&v)[32], const ConvParams& p, size_t o, int cbase, int gp,
-                                                    bool pvalid, int nb, int qmax, uint32_t* dst, PlaneHold<G>& hold) {
-    const float S = p.S, inv_next = p.inv_next;
-    uint32_t rbyte[8];
-    const bool has_rp = p.res_packed != nullptr;
-    if (has_rp) {
-        const uint32_t* rw = p.res_packed + ((size_t)gp * p.CWo + (cbase >> 5)) * p.res_bits;
-        uint32_t rw8[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) rw8[j] = (pvalid && j < p.res_bits) ? __ldg(rw + j) : 0u;
-        planes_to_bytes<8>(rw8, rbyte);
-    }
-    uint32_t cr[8];
-    const float hi2 = (float)(2 * qmax + 1);
-#pragma unroll
-    for (int bb = 0; bb < 8; ++bb) {
-        uint32_t m[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int c = 8 * i + bb;
-            float t = __fmul_rn((float)(int)v[c], S);
-            if (p.ch_scale) t = __fmul_rn(t, __ldg(p.ch_scale + cbase + c));
-            if (p.ch_bias) t = __fadd_rn(t, __ldg(p.ch_bias + cbase + c));
-            if (p.residual && pvalid) t = __fadd_rn(t, __ldg(p.residual + o + c));
-            if (has_rp) t = __fadd_rn(t, __fmul_rn(p.res_scale, (float)((rbyte[bb] >> (8 * i)) & 0xFFu)));
-            m[i] = code_pattern(__fadd_rn(__fmul_rn(t, inv_next), 0.5f), hi2);
-        }
-        const uint32_t c4 = __byte_perm(__byte_perm(m[0], m[1], 0x0040), __byte_perm(m[2], m[3], 0x0040), 0x5410);
-        cr[bb] = __funnelshift_l(c4, c4, bb);
-    }
-    uint32_t planes[8];
-    bytes_to_planes(cr, nb, planes);
-    pipe_store_planes(planes, nb, dst, pvalid, hold, p);
-}
-
-// Packed-only epilogue with per-channel terms / shortcut of one 128-pixel accumulator (whole channel tile, NHWC).
-template <int TILE_N, int G>
-__device__ __forceinline__ void pipe_epilogue_affine_g(const ConvParams& p, uint32_t tmem_acc, int vwarp, int gp, bool pvalid,
-                                                       int co0) {
-    constexpr int COLS = TILE_N / 2;
-    const uint32_t trow = tmem_acc + ((uint32_t)((vwarp & 3) * 32) << 16);
+// Epilogue of a layer with per-channel terms and / or a shortcut (a folded batch normalisation, the second convolution of a
+// residual block): whole channel tiles, NHWC, packed planes and / or fp32 out.  The warp walks its (accumulator, 32-channel
+// group) units; the next unit's shortcut and terms are requested before the current one is packed and stored.  The terms of
+// a group pass through 64 words of shared memory of the warp's own (one load and one store a lane, then broadcast reads):
+// read channel by channel through the cache they cost more than the arithmetic (64 -> 256 1x1 at 56x56, batch 256: 225 us
+// against 119 us for the same layer without terms).  VALUES: fp32 output may be wanted too.
+template <int TILE_N, int G, bool VALUES>
+__device__ __forceinline__ void pipe_epilogue_terms(const ConvParams& p, const FrameGeom& g, uint32_t tmem_set, int m_sub, int vwarp,
+                                                    int f0, int co0, float* terms) {
+    constexpr int COLS = TILE_N / 2, NG = COLS / 32;
+    const int lane = (int)(threadIdx.x & 31), at = (lane & 7) * 4 + (lane >> 3);
+    const uint32_t trow = tmem_set + ((uint32_t)((vwarp & 3) * 32) << 16);
     const int cbeg = (vwarp >> 2) * COLS;
-    const int nb = p.next_bits, qmax = (1 << p.next_bits) - 1;
-    uint32_t v[32];
+    const int nb = p.next_bits;
+    const float hi2 = (float)(2 * ((1 << nb) - 1) + 1);
     PlaneHold<G> hold;
     hold.filled = 0;
+    float res[32], t_scale, t_bias;
+    uint32_t rw[8];
+    int gp = 0;
+    bool pvalid = false;
+    auto locate = [&](int j) {
+        const int f = f0 + j * UMMA_M;
+        pvalid = false;
+        gp = 0;
+        if (f < g.frame) {
+            const uint32_t n = fastdiv((uint32_t)f, g.div_img);
+            const uint32_t rem = (uint32_t)f - n * (uint32_t)(g.Hq * g.Wq);
+            const uint32_t hq = fastdiv(rem, g.div_row), wq = rem - hq * (uint32_t)g.Wq;
+            if ((int)hq < p.Ho && (int)wq < p.Wo) {
+                pvalid = true;
+                gp = ((int)n * p.Ho + (int)hq) * p.Wo + (int)wq;
+            }
+        }
+    };
+    auto request = [&](int c) {                              // c: first channel of the unit
+        t_scale = p.ch_scale ? __ldg(p.ch_scale + c + lane) : 1.0f;
+        t_bias = p.ch_bias ? __ldg(p.ch_bias + c + lane) : -0.0f;
+        if (p.residual) {
+            const float4* r4 = reinterpret_cast<const float4*>(p.residual + (size_t)gp * p.Co + c);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float4 t = __ldg(r4 + i);
+                res[4 * i] = t.x; res[4 * i + 1] = t.y; res[4 * i + 2] = t.z; res[4 * i + 3] = t.w;
+            }
+        } else if (p.res_packed) {
+            ld_dep_planes(p.res_packed + ((size_t)gp * p.CWo + (c >> 5)) * p.res_bits, p.res_bits, rw);
+        }
+    };
+    locate(0);
+    request(co0 + cbeg);
 #pragma unroll 1
-    for (int c0 = cbeg; c0 < cbeg + COLS; c0 += 32) {
-        uint32_t (&lo)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[0]);
-        uint32_t (&hi)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[16]);
-        tmem_ld16_issue(trow + (uint32_t)c0, lo);
-        tmem_ld16_issue(trow + (uint32_t)(c0 + 16), hi);
-        tmem_ld16_wait(lo);
-        tmem_ld16_wait(hi);
-        const size_t o = (size_t)gp * p.Co + co0 + c0;
-        uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + ((co0 + c0) >> 5)) * nb;
-        pipe_group32_affine(v, p, o, co0 + c0, gp, pvalid, nb, qmax, dst, hold);
+    for (int j = 0; j < m_sub; ++j) {
+#pragma unroll 1
+        for (int k = 0; k < NG; ++k) {
+            const int c0 = cbeg + 32 * k, c = co0 + c0;
+            const bool ok = pvalid;
+            const size_t gpz = gp;
+            __syncwarp();                                    // every lane has read the unit before
+            terms[at] = t_scale;
+            terms[32 + at] = t_bias;
+            __syncwarp();
+            const float4* cs = reinterpret_cast<const float4*>(terms);
+            const float4* cb = reinterpret_cast<const float4*>(terms + 32);
+            uint32_t cr[8];
+            const bool some = __any_sync(0xffffffffu, ok);   // else: 32 frame pixels without an output
+            if (some) {
+                uint32_t v[32], rbyte[8];
+                uint32_t (&lo)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[0]);
+                uint32_t (&hi)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[16]);
+                tmem_ld16_issue(trow + (uint32_t)(j * TILE_N + c0), lo);
+                tmem_ld16_issue(trow + (uint32_t)(j * TILE_N + c0 + 16), hi);
+                tmem_ld16_wait(lo);
+                tmem_ld16_wait(hi);
+                if (!p.residual && p.res_packed) planes_to_bytes<8>(rw, rbyte);
+                if constexpr (VALUES) {
+                    uint64_t yy[2][8];
+                    if (p.residual) terms_values32<1>(v, p.S, p.one, cs, cb, res, rbyte, 0.0f, yy);
+                    else if (p.res_packed) terms_values32<2>(v, p.S, p.one, cs, cb, res, rbyte, p.res_scale, yy);
+                    else terms_values32<0>(v, p.S, p.one, cs, cb, res, rbyte, 0.0f, yy);
+                    if (p.y && ok && EBS_IN_RANGE(p, CHK_PIPE_Y, gpz * p.Co + c + 31, p.lim_out)) store_values32(yy, p.relu != 0, p.y + gpz * p.Co + c);
+                    if (p.packed_next) value_codes32(yy, p.one, p.inv_next, hi2, cr);
+                } else {
+                    if (p.residual) terms_codes32<1>(v, p.S, p.one, cs, cb, res, rbyte, 0.0f, p.inv_next, hi2, cr);
+                    else if (p.res_packed) terms_codes32<2>(v, p.S, p.one, cs, cb, res, rbyte, p.res_scale, p.inv_next, hi2, cr);
+                    else terms_codes32<0>(v, p.S, p.one, cs, cb, res, rbyte, 0.0f, p.inv_next, hi2, cr);
+                }
+            }
+            if (k + 1 < NG) {
+                request(c + 32);
+            } else if (j + 1 < m_sub) {
+                locate(j + 1);
+                request(co0 + cbeg);
+            }
+            if (some && (!VALUES || p.packed_next)) {
+                uint32_t planes[8];
+                bytes_to_planes(cr, nb, planes);
+                pipe_store_planes(planes, nb, p.packed_next + (gpz * p.CWo + (c >> 5)) * nb, ok, hold, p);
+            }
+        }
     }
 }
 
@@ -516,13 +471,13 @@ __device__ __forceinline__ void pipe_epilogue_packed_g(const ConvParams& p, uint
 // (the usual layer of a network: its epilogue holds nothing but the lean group, or the group with per-channel terms);
 // 2 = form 1 with the held-back runs.
 inline bool pipe_packed_only(const ConvParams& p, int tile_n) {
-    return p.packed_next && !p.acc && !p.y && !p.w_levels && (p.Co % tile_n) == 0;
+    return p.packed_next && !p.acc && !p.y && !p.w_levels && (p.Co % tile_n) == 0 && !(p.residual && p.res_packed);
 }
 inline bool pipe_hold_applies(const ConvParams& p, int tile_n) {
     const int G = tile_n / 64;
     // (5 and 7 planes; with 1 or 3 the single-word stores are few and the held form measured slower)
     return G > 1 && p.packed_next && (p.next_bits == 5 || p.next_bits == 7) && (p.CWo % G) == 0 && !p.acc && !p.y && !p.y_nchw &&
-           (p.Co & 31) == 0 && !p.w_levels;
+           (p.Co & 31) == 0 && !p.w_levels && !(p.residual && p.res_packed);
 }
 
 template <int AB, int TILE_N, bool AFFINE, int FORM, bool PAIR = false>
@@ -543,6 +498,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
     __shared__ __align__(8) uint64_t bs_full[PIPE_MAX_BSLOTS], bs_empty[PIPE_MAX_BSLOTS];   // streamed weight tiles
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
+    __shared__ __align__(16) float s_terms[AFFINE ? PIPE_EPI_WARPS : 1][64];
     __shared__ uint32_t s_tap_shift[PIPE_MAX_TAPS];     // tap tables in shared memory: indexed at run time by single threads
     __shared__ int s_tap_id[PIPE_MAX_TAPS];
 
@@ -997,8 +953,8 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
         const int row = (warp & 3) * 32 + (tid & 31);
         const bool plain_ok = !AFFINE && !p.ch_scale && !p.ch_bias && !p.residual && !p.res_packed && !p.y_nchw &&
                               (p.Co & 3) == 0;
-        // layers with per-channel terms or a shortcut that only hand packed planes on (the usual layer of a network)
-        const bool affine_ok = AFFINE && p.packed_next && !p.y && !p.acc && !p.w_levels && (p.Co & 31) == 0;
+        // layers with per-channel terms or a shortcut and without integer output (the layers of a network)
+        const bool affine_ok = AFFINE && !p.acc && !p.y_nchw && (p.Co & 31) == 0 && !(p.residual && p.res_packed);
         for (int it = 0; it < my_items; ++it) {
             const int buf = g.nbuf == 2 ? (it & 1) : 0;
             const int use = g.nbuf == 2 ? (it >> 1) : it;
@@ -1007,7 +963,12 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
             int ptile, ctile;
             item_of(it, ptile, ctile);
             const int co0 = ctile * TILE_N;
-            for (int j = 0; j < g.m_sub; ++j) {
+            if (AFFINE && (FORM != 0 || (affine_ok && co0 + TILE_N <= p.Co))) {
+                if constexpr (AFFINE)
+                    pipe_epilogue_terms<TILE_N, EPI_G, FORM == 0>(p, g, tmem_base + (uint32_t)(buf * g.m_sub * TILE_N), g.m_sub, vwarp,
+                                                                  (PAIR ? 2 * ptile + crank : ptile) * g.tile_pix + row, co0,
+                                                                  s_terms[warp - PIPE_EPI_WARP0]);
+            } else for (int j = 0; j < g.m_sub; ++j) {
                 const int f = (PAIR ? 2 * ptile + crank : ptile) * g.tile_pix + j * UMMA_M + row;
                 bool pvalid = false;
                 int gp = 0;
@@ -1021,11 +982,9 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
                 if (!__any_sync(0xffffffffu, pvalid)) continue;   // 32 frame pixels without an output
                 const uint32_t tmem_acc = tmem_base + (uint32_t)((buf * g.m_sub + j) * TILE_N);
                 if constexpr (FORM != 0) {
-                    if constexpr (AFFINE) pipe_epilogue_affine_g<TILE_N, EPI_G>(p, tmem_acc, vwarp, gp, pvalid, co0);
-                    else pipe_epilogue_packed_g<TILE_N, EPI_G>(p, tmem_acc, vwarp, gp, pvalid, co0);
+                    if constexpr (!AFFINE) pipe_epilogue_packed_g<TILE_N, EPI_G>(p, tmem_acc, vwarp, gp, pvalid, co0);
                 } else {
                     if (plain_ok && co0 + TILE_N <= p.Co) pipe_epilogue_plain_g<TILE_N, 1>(p, tmem_acc, vwarp, gp, pvalid, co0);
-                    else if (affine_ok && co0 + TILE_N <= p.Co) pipe_epilogue_affine_g<TILE_N, 1>(p, tmem_acc, vwarp, gp, pvalid, co0);
                     else umma_epilogue<TILE_N, AFFINE>(p, tmem_acc, vwarp, gp, pvalid, 0, co0);
                 }
             }

@@ -7,8 +7,8 @@
 // that is expanded once.  What bounds such a layer is latency: a launch, a round trip for the packed words, the chain of
 // MMAs onto one accumulator (about 50 clocks each at N = 64) and the epilogue, with most SMs idle.  Hence
 //  * the reduction is split over the CTAs of a cluster (up to 8) by input-channel words; each accumulates its share in its
-//    own tensor memory, the partial sums meet in shared memory and every CTA of the cluster finishes its part of the
-//    pixels (exact: integer sums);
+//    own tensor memory, the copy engine brings the partial sums together in distributed shared memory and every CTA of the
+//    cluster finishes its part of the pixels (exact: integer sums);
 //  * all of a CTA's operands are in flight at once where they fit (100 KB, so that two CTAs share an SM and one's epilogue
 //    runs under the other's MMAs), weight tiles by bulk copies of one warp, packed words by the expanders;
 //  * the launch may begin while its predecessor in the stream finishes (programmatic dependent launch): barriers, tables
@@ -36,7 +36,7 @@ struct TileGeom : FrameGeom {
     int S, SP, kw;                     // strip pixels, rounded up to 8; words per stage
     int words;                         // input-channel words of a CTA (the last of a cluster may have fewer)
     int a_word_bytes, b_off, stage_bytes, n_stages;
-    int tmem_cols, smem_bytes, part_pitch;
+    int tmem_cols, smem_bytes, part_pitch, xch_off;   // xch_off: where a cluster's CTAs put their sums, from the stages on
     float cost;                        // estimated clocks of the launch
     bool ok;
 };
@@ -78,11 +78,12 @@ inline TileGeom tile_geometry(const ConvParams& p, int tile_n, int sms, int spli
             c.b_off = tile_round_up(kw * c.a_word_bytes, 256);
             return c.b_off + kw * c.max_ph_taps * b_tile;
         };
-        const int fixed = 1024 + 512;
+        const int fixed = 1024 + 512 + (split == 1 ? 0 : UMMA_M * c.part_pitch * 4);
         while (c.kw > 1 && 3 * stage(c.kw) + fixed > TILE_SMEM_SHARED) --c.kw;
         c.stage_bytes = stage(c.kw);
         const int chunks = c.n_ph * ((c.words + c.kw - 1) / c.kw);
-        const int part = UMMA_M * c.part_pitch * 4;            // the partial sums reuse the stages
+        // the sums lie over the stages; those that the CTAs of a cluster send each other lie behind them (in `fixed`)
+        const int part = UMMA_M * c.part_pitch * 4;
         const int need = chunks < 2 ? 1 : 2;
         int budget = TILE_SMEM_SHARED;
         if (need * c.stage_bytes + fixed > budget || part + fixed > budget) budget = TILE_SMEM_MAX;
@@ -91,6 +92,7 @@ inline TileGeom tile_geometry(const ConvParams& p, int tile_n, int sms, int spli
         if (c.n_stages > TILE_MAX_STAGES) c.n_stages = TILE_MAX_STAGES;
         if (c.n_stages < need) continue;
         const int body = c.n_stages * c.stage_bytes > part ? c.n_stages * c.stage_bytes : part;
+        c.xch_off = body;
         c.smem_bytes = body + fixed;
         if (c.smem_bytes > TILE_SMEM_MAX) continue;
         // Estimate of the launch, fitted to about 1000 measured (layer, channel tile, split) points: the serial chain of a
@@ -113,14 +115,16 @@ inline TileGeom tile_geometry(const ConvParams& p, int tile_n, int sms, int spli
 template <int AB, int FORM>
 __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const ConvParams p, const TileGeom g) {
     extern __shared__ uint8_t dyn_smem[];
-    __shared__ __align__(8) uint64_t full[TILE_MAX_STAGES], empty[TILE_MAX_STAGES], acc_full;
+    __shared__ __align__(8) uint64_t full[TILE_MAX_STAGES], empty[TILE_MAX_STAGES], acc_full, xch_full;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     __shared__ int gp_s[UMMA_M];                         // output pixel of every row, -1: none
-    __shared__ int s_tap_shift[FRAME_MAX_TAPS], s_tap_id[FRAME_MAX_TAPS];
+    __shared__ int s_tap_id[FRAME_MAX_TAPS];
     __shared__ __align__(16) float s_terms[FORM == 2 ? 512 : 4];   // FORM 2: scale and shift of the channel tile, terms_codes32 order
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // (read from lane 0, so that the compiler knows the role branches to be warp-uniform and keeps the issuing warp's
+    // descriptors in uniform registers)
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int rank = (int)blockIdx.z, split = g.split;   // cluster of `split` CTAs along z
     const int f0 = (int)blockIdx.x * UMMA_M, co0 = (int)blockIdx.y * g.tile_n;
     const int N = g.tile_n, b_tile = N * 32, KW = g.kw, NST = g.n_stages, SP = g.SP, S = g.S;
@@ -138,12 +142,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
             mbar_init(&empty[s], 1);
         }
         mbar_init(&acc_full, 1);
+        mbar_init(&xch_full, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    if (tid < FRAME_MAX_TAPS) {
-        s_tap_shift[tid] = g.tap_shift[tid];
-        s_tap_id[tid] = g.tap_id[tid];
-    }
+    if (tid < FRAME_MAX_TAPS) s_tap_id[tid] = g.tap_id[tid];
     if (p.w_levels && tid < 128) reinterpret_cast<uint32_t*>(ones)[tid] = 0x01010101u;
     if (warp == TILE_ISSUER) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_slot)),
@@ -158,7 +160,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
     // The next launch may start its own set-up from here on: this CTA has its tensor memory, so nothing it still needs can
     // be taken by a CTA that waits for it.  Global memory is touched only behind the wait for the previous launch.
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    if (split > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");   // this CTA runs: its memory may be written
 
     if (warp < 8) {
         // =========================== expanders ===========================
@@ -190,13 +192,13 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
         uint32_t words[SETS][TILE_SLOTS][AB];
         int ld_ph = 0, ld_wg = 0;
         auto load_next = [&](int set) {
-            if (ld_wg == 0) phase_pointers(ld_ph);
+            if (ld_wg == 0 && ld_ph > 0) phase_pointers(ld_ph);
 #pragma unroll
             for (int j = 0; j < TILE_SLOTS; ++j) {
                 const uint32_t* a = src[j] + (size_t)ld_wg * KW * AB;
                 const bool in = src[j] != nullptr && ld_wg * KW + slot_q[j] < nw;
                 if (in && EBS_IN_RANGE(p, CHK_UT_X, (a - p.x) + AB - 1, p.lim_x)) {
-                    load_words_global<AB>(a, words[set][j]);
+                    ld_dep_words<AB>(a, words[set][j]);
                 } else {
 #pragma unroll
                     for (int k = 0; k < AB; ++k) words[set][j][k] = 0u;
@@ -204,28 +206,11 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
             }
             if (++ld_wg == nwg) { ld_wg = 0; ++ld_ph; }
         };
+        phase_pointers(0);
+        asm volatile("griddepcontrol.wait;\n" ::: "memory");
 #pragma unroll
         for (int u = 0; u < SETS - 1; ++u)
             if (u < nchunks) load_next(u);
-        // while these are on their way: the output pixel of every row, the per-channel terms of the tile
-        if (tid < UMMA_M) {
-            const int f = f0 + tid;
-            int gp = -1;
-            if (f < g.frame) {
-                const uint32_t n = fastdiv((uint32_t)f, g.div_img);
-                const uint32_t rem = (uint32_t)f - n * (uint32_t)(g.Hq * g.Wq);
-                const uint32_t hq = fastdiv(rem, g.div_row), wq = rem - hq * (uint32_t)g.Wq;
-                if ((int)hq < p.Ho && (int)wq < p.Wo) gp = ((int)n * p.Ho + (int)hq) * p.Wo + (int)wq;
-            }
-            gp_s[tid] = gp;
-        }
-        if constexpr (FORM == 2) {
-            if (tid < N) {                               // channel tid of the tile: group tid / 32, entry tid % 8, lane (tid / 8) % 4
-                const int at = (tid >> 5) * 32 + (tid & 7) * 4 + ((tid >> 3) & 3);
-                s_terms[at] = term_at(p.ch_scale, co0 + tid, p.Co, 1.0f);
-                s_terms[256 + at] = term_at(p.ch_bias, co0 + tid, p.Co, -0.0f);
-            }
-        }
         bool ok = true;
         int st = 0;
         uint32_t round = 0;
@@ -252,9 +237,89 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
                 if (++st == NST) { st = 0; ++round; }
             }
         }
-        if (ok) mbar_wait_bounded(&acc_full, 0u, abortp, limit);
+        // under the last MMAs: this thread's output pixel, the per-channel terms and the first shortcut values
+        const int row = (warp & 3) * 32 + lane, f = f0 + row;
+        int gp = -1;
+        if (f < g.frame) {
+            const uint32_t n = fastdiv((uint32_t)f, g.div_img);
+            const uint32_t rem = (uint32_t)f - n * (uint32_t)(g.Hq * g.Wq);
+            const uint32_t hq = fastdiv(rem, g.div_row), wq = rem - hq * (uint32_t)g.Wq;
+            if ((int)hq < p.Ho && (int)wq < p.Wo) gp = ((int)n * p.Ho + (int)hq) * p.Wo + (int)wq;
+        }
+        if constexpr (FORM == 0) {
+            if (warp < 4) gp_s[row] = gp;
+            if (ok) mbar_wait_bounded(&acc_full, 0u, abortp, limit);
+        } else {
+            // =========================== epilogue, a thread per pixel ===========================
+            const bool pvalid = gp >= 0;
+            const size_t gpz = pvalid ? gp : 0;
+            const int half = (warp >> 2) * 32;               // this warp's first group of 32 channels; every other one is its own
+            const bool mine = half < N && co0 + half < p.Co;
+            uint32_t rw[8];
+            float res[32];
+            auto load_shortcut = [&](int c0) {
+                if constexpr (FORM == 2) {
+                    if (p.residual) {
+                        const float4* r4 = reinterpret_cast<const float4*>(p.residual + gpz * p.Co + co0 + c0);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const float4 t = ld_dep(r4 + i);
+                            res[4 * i] = t.x; res[4 * i + 1] = t.y; res[4 * i + 2] = t.z; res[4 * i + 3] = t.w;
+                        }
+                    } else if (p.res_packed) {
+                        ld_dep_planes(p.res_packed + (gpz * p.CWo + ((co0 + c0) >> 5)) * p.res_bits, p.res_bits, rw);
+                    }
+                }
+            };
+            if (mine) load_shortcut(half);
+            if constexpr (FORM == 2) {
+                if (tid < N) {                               // channel tid of the tile: group tid / 32, entry tid % 8, lane (tid / 8) % 4
+                    const int at = (tid >> 5) * 32 + (tid & 7) * 4 + ((tid >> 3) & 3);
+                    s_terms[at] = term_at(p.ch_scale, co0 + tid, p.Co, 1.0f);
+                    s_terms[256 + at] = term_at(p.ch_bias, co0 + tid, p.Co, -0.0f);
+                }
+            }
+            if (ok) mbar_wait_bounded(&acc_full, 0u, abortp, limit);
+            asm volatile("bar.sync 1, 256;\n" ::: "memory");
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            if (!__any_sync(0xffffffffu, abort_flag != 0) && __any_sync(0xffffffffu, pvalid)) {
+                const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+                const int nb = p.next_bits;
+                const float hi2 = (float)(2 * ((1 << nb) - 1) + 1);
+#pragma unroll 1
+                for (int c0 = half; c0 < N && co0 + c0 < p.Co; c0 += 64) {
+                    uint32_t v[32], cr[8], planes[8];
+                    uint32_t (&lo)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[0]);
+                    uint32_t (&hi)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[16]);
+                    tmem_ld16_issue(trow + (uint32_t)c0, lo);
+                    tmem_ld16_issue(trow + (uint32_t)(c0 + 16), hi);
+                    tmem_ld16_wait(lo);
+                    tmem_ld16_wait(hi);
+                    if constexpr (FORM == 2) {
+                        const float4* cs = reinterpret_cast<const float4*>(s_terms + c0);
+                        const float4* cb = reinterpret_cast<const float4*>(s_terms + 256 + c0);
+                        uint32_t rbyte[8];
+                        if (p.residual) {
+                            terms_codes32<1>(v, p.S, p.one, cs, cb, res, rbyte, 0.0f, p.inv_next, hi2, cr);
+                        } else if (p.res_packed) {
+                            planes_to_bytes<8>(rw, rbyte);
+                            terms_codes32<2>(v, p.S, p.one, cs, cb, res, rbyte, p.res_scale, p.inv_next, hi2, cr);
+                        } else {
+                            terms_codes32<0>(v, p.S, p.one, cs, cb, res, rbyte, 0.0f, p.inv_next, hi2, cr);
+                        }
+                    } else {
+                        plain_codes32(v, p.S, p.one, p.inv_next, hi2, cr);
+                    }
+                    if (c0 + 64 < N && co0 + c0 + 64 < p.Co) load_shortcut(c0 + 64);
+                    bytes_to_planes(cr, nb, planes);
+                    uint32_t* dst = p.packed_next + (gpz * p.CWo + ((co0 + c0) >> 5)) * nb;
+                    if (pvalid && EBS_IN_RANGE(p, CHK_UT_PN, (dst - p.packed_next) + nb - 1, p.lim_pn)) store_plane_words(planes, nb, dst);
+                }
+            }
+        }
     } else if (warp == TILE_ISSUER) {
         // =========================== issuer ===========================
+        const bool levels = p.w_levels != 0;
         const bool skip_mma = (p.test_flags & 1) != 0;   // test hook: issue nothing, so that waits run out
         const uint32_t leader = lane == 0 ? 1u : 0u;
         const uint64_t da0 = umma_desc_interleaved(smem_u32(stages), (uint32_t)(SP * 16)), db0 = umma_desc_sw32(smem_u32(stages + g.b_off));
@@ -263,21 +328,22 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
         int st = 0, ph = 0, wg = 0;
         uint32_t round = 0;
         for (int c = 0; c < nchunks; ++c) {
-            if (!mbar_wait_bounded_hot(&full[st], round & 1u, abortp, limit)) break;
+            if (!mbar_wait_bounded_warp(&full[st], round & 1u, abortp, limit)) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             if (!skip_mma) {
-                const int nq = min(KW, nw - wg * KW), t0 = g.ph_tap0[ph], t1 = g.ph_tap0[ph + 1];
+                // The taps of a phase are a rectangle of shifts, walked by additions; the weight tiles lie in the same order.
+                const int nq = min(KW, nw - wg * KW), rows = g.ph_rows[ph], cols = g.ph_cols[ph];
                 const uint32_t stage16 = (uint32_t)(st * g.stage_bytes) >> 4;
-                uint32_t a_lo = (uint32_t)da0 + stage16, b_lo = (uint32_t)db0 + stage16;
+                uint32_t a_word = (uint32_t)da0 + stage16 + (uint32_t)g.ph_shift[ph], b_lo = (uint32_t)db0 + stage16;
                 uint32_t accu = c == 0 ? 0u : 1u;
-                for (int q = 0; q < nq; ++q, a_lo += word16) {
-                    uint32_t shift = (uint32_t)s_tap_shift[t0];
-                    for (int t = t0; t < t1; ++t, b_lo += bt16) {
-                        const uint32_t next = (uint32_t)s_tap_shift[min(t + 1, FRAME_MAX_TAPS - 1)];
-                        umma_i8_split(leader, tmem, a_lo + shift, da_hi, b_lo, db_hi, idesc, accu);
-                        if (p.w_levels) umma_i8_split(leader, tmem + (uint32_t)N, a_lo + shift, da_hi, ones_lo, db_hi, umma_idesc_i8(16), accu);
-                        accu = 1u;
-                        shift = next;
+                for (int q = 0; q < nq; ++q, a_word += word16) {
+                    uint32_t a_row = a_word;
+                    for (int r = 0; r < rows; ++r, a_row += (uint32_t)g.Wq) {
+                        for (int s = 0; s < cols; ++s, b_lo += bt16) {
+                            umma_i8_split(leader, tmem, a_row + (uint32_t)s, da_hi, b_lo, db_hi, idesc, accu);
+                            if (levels) umma_i8_split(leader, tmem + (uint32_t)N, a_row + (uint32_t)s, da_hi, ones_lo, db_hi, umma_idesc_i8(16), accu);
+                            accu = 1u;
+                        }
                     }
                 }
                 umma_commit_pred(leader, &empty[st]);
@@ -289,6 +355,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
         }
     } else {
         // =========================== weight tiles ===========================
+        asm volatile("griddepcontrol.wait;\n" ::: "memory");
         const uint32_t bytes = (uint32_t)min(N, p.Co16 - co0) * 32u;
         int st = 0, ph = 0, wg = 0;
         uint32_t round = 0;
@@ -314,86 +381,34 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
             for (int i = 0; i < 64; ++i) __nanosleep(1000);
     }
 
-    if constexpr (FORM != 0) {
-        // =========================== epilogue, a thread per pixel ===========================
-        if (warp < 8) {
-            asm volatile("bar.sync 1, 256;\n" ::: "memory");    // gp_s and the terms
-            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            if (abort_flag == 0) {
-                const int gp = gp_s[(warp & 3) * 32 + lane];
-                const bool pvalid = gp >= 0;
-                const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-                const int nb = p.next_bits, qmax = (1 << nb) - 1;
-                const float hi2 = (float)(2 * qmax + 1);
-                if (__any_sync(0xffffffffu, pvalid)) {
-#pragma unroll 1
-                    for (int c0 = (warp >> 2) * 32; c0 < N && co0 + c0 < p.Co; c0 += 64) {
-                        uint32_t v[32];
-                        uint32_t (&lo)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[0]);
-                        uint32_t (&hi)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[16]);
-                        tmem_ld16_issue(trow + (uint32_t)c0, lo);
-                        tmem_ld16_issue(trow + (uint32_t)(c0 + 16), hi);
-                        const int word = (co0 + c0) >> 5;
-                        uint32_t cr[8];
-                        if constexpr (FORM == 2) {
-                            float res[32];
-                            uint32_t rbyte[8];
-                            const float4* cs = reinterpret_cast<const float4*>(s_terms + c0);
-                            const float4* cb = reinterpret_cast<const float4*>(s_terms + 256 + c0);
-                            if (p.residual) {
-                                const float4* r4 = reinterpret_cast<const float4*>(p.residual + (size_t)(pvalid ? gp : 0) * p.Co + co0 + c0);
-#pragma unroll
-                                for (int i = 0; i < 8; ++i) {
-                                    const float4 t = __ldg(r4 + i);
-                                    res[4 * i] = t.x; res[4 * i + 1] = t.y; res[4 * i + 2] = t.z; res[4 * i + 3] = t.w;
-                                }
-                            } else if (p.res_packed) {
-                                const uint32_t* rw = p.res_packed + ((size_t)(pvalid ? gp : 0) * p.CWo + word) * p.res_bits;
-                                uint32_t rw8[8];
-#pragma unroll
-                                for (int j = 0; j < 8; ++j) rw8[j] = j < p.res_bits ? __ldg(rw + j) : 0u;
-                                planes_to_bytes<8>(rw8, rbyte);
-                            }
-                            tmem_ld16_wait(lo);
-                            tmem_ld16_wait(hi);
-                            if (p.residual) terms_codes32<1>(v, p.S, cs, cb, res, rbyte, 0.0f, p.inv_next, hi2, cr);
-                            else if (p.res_packed) terms_codes32<2>(v, p.S, cs, cb, res, rbyte, p.res_scale, p.inv_next, hi2, cr);
-                            else terms_codes32<0>(v, p.S, cs, cb, res, rbyte, 0.0f, p.inv_next, hi2, cr);
-                        } else {
-                            tmem_ld16_wait(lo);
-                            tmem_ld16_wait(hi);
-                            const uint64_t S2 = f32x2_pack(p.S, p.S);
-#pragma unroll
-                            for (int bb = 0; bb < 8; ++bb) {
-                                uint32_t m[4];
-#pragma unroll
-                                for (int h = 0; h < 2; ++h) {
-                                    const uint64_t w = f32x2_mul_rn(f32x2_pack((float)(int)v[16 * h + bb], (float)(int)v[16 * h + 8 + bb]), S2);
-                                    m[2 * h] = code_pattern(__fadd_rn(__fmul_rn(__uint_as_float((uint32_t)w), p.inv_next), 0.5f), hi2);
-                                    m[2 * h + 1] = code_pattern(__fadd_rn(__fmul_rn(__uint_as_float((uint32_t)(w >> 32)), p.inv_next), 0.5f), hi2);
-                                }
-                                const uint32_t c4 = join_codes(m);
-                                cr[bb] = __funnelshift_l(c4, c4, bb);
-                            }
-                        }
-                        uint32_t planes[8];
-                        bytes_to_planes(cr, nb, planes);
-                        uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + word) * nb;
-                        if (pvalid && EBS_IN_RANGE(p, CHK_UT_PN, (dst - p.packed_next) + nb - 1, p.lim_pn)) store_plane_words(planes, nb, dst);
-                    }
-                }
-            }
-        }
-    } else {
+    if constexpr (FORM == 0) {
         // =========================== epilogue through shared memory ===========================
-        // A worker's TMEM row -> its row of partial sums [128][part_pitch] (the stages are free: every MMA has finished).
-        int* part = reinterpret_cast<int*>(stages);
-        const int pitch = g.part_pitch;
+        // A worker's TMEM row -> a row of sums [128][part_pitch] over the stages (every MMA has finished).  In a cluster each CTA
+        // finishes 128 / split rows; the copy engine carries every CTA's block of those rows to it ([split][128 / split] rows
+        // behind the stages), rows past the frame excepted: 1.7 us for eight CTAs and 64 channels, where reading the peers' sums
+        // from the finishing threads took 2.5 and pushing them with thread stores 3.8.
+        const int pitch = g.part_pitch, rows = UMMA_M / split;
+        int* dump = reinterpret_cast<int*>(stages);
+        int* part = reinterpret_cast<int*>(stages + (split == 1 ? 0 : g.xch_off));
+        auto block_bytes = [&](int r) { return (uint32_t)(min(max(g.frame - f0 - r * rows, 0), rows) * pitch * 4); };
+        // This CTA finishes rows rank * 128 / split ..; a warp takes 32 channels of four pixels at a time, a lane four
+        // channels of one of them (16-byte accesses; with a channel a lane the same work took five times the instructions).
+        const int groups = (N + 31) >> 5, grp = warp & (groups - 1), rstep = 8 / groups;
+        const int sub = lane & 7, col = grp * 32 + 4 * sub, co = co0 + col, live = col < N ? min(max(p.Co - co, 0), 4) : 0;
+        const int nb = p.next_bits, qmax = (1 << nb) - 1, word = (co0 >> 5) + grp, hw = p.Ho * p.Wo;
+        const bool vec = (p.Co & 3) == 0;            // then live is 0 or 4 and every access is aligned
+        float cs[4], cb[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            cs[i] = i < live ? term_at(p.ch_scale, co + i, p.Co, 1.0f) : 1.0f;
+            cb[i] = i < live ? term_at(p.ch_bias, co + i, p.Co, -0.0f) : -0.0f;
+        }
         __syncwarp();
+        if (split > 1) asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");   // every CTA of the cluster runs
         if (warp < 8 && !__any_sync(0xffffffffu, abort_flag != 0)) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-            int* row = part + ((warp & 3) * 32 + lane) * pitch;
+            int* row = dump + ((warp & 3) * 32 + lane) * pitch;
             const int cols = N + (p.w_levels ? 1 : 0);
 #pragma unroll 1
             for (int c0 = (warp >> 2) * 16; c0 < cols; c0 += 32) {
@@ -401,59 +416,44 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
                 tmem_ld16(trow + (uint32_t)c0, v);
                 if (c0 < N) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) *reinterpret_cast<int4*>(row + c0 + 4 * i) = make_int4((int)v[4 * i], (int)v[4 * i + 1], (int)v[4 * i + 2], (int)v[4 * i + 3]);
+                    for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4*>(row + c0 + 4 * i) = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
                 } else {
                     row[N] = (int)v[0];                  // the window sum
                 }
             }
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         }
-        __syncwarp();
-        if (split > 1) cluster_sync_all();
-        else __syncthreads();
-        if (warp < 8 && abort_flag == 0) {
-            // This CTA finishes rows rank * 128 / split ..; a warp takes 32 channels of four pixels at a time, a lane four
-            // channels of one of them (16-byte accesses; with a channel a lane the same work took five times the instructions).
-            const int groups = (N + 31) >> 5, rows = UMMA_M / split, grp = warp & (groups - 1), rstep = 8 / groups;
-            const int sub = lane & 7, col = grp * 32 + 4 * sub, co = co0 + col, live = col < N ? min(max(p.Co - co, 0), 4) : 0;
-            const int nb = p.next_bits, qmax = (1 << nb) - 1, word = (co0 >> 5) + grp, hw = p.Ho * p.Wo;
-            const bool vec = (p.Co & 3) == 0;            // then live is 0 or 4 and every access is aligned
-            float cs[4], cb[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                cs[i] = i < live ? term_at(p.ch_scale, co + i, p.Co, 1.0f) : 1.0f;
-                cb[i] = i < live ? term_at(p.ch_bias, co + i, p.Co, -0.0f) : -0.0f;
+        __syncthreads();
+        if (split > 1) {
+            if (warp == 0 && abort_flag == 0) {
+                if (lane == 0) mbar_arrive_expect_tx(&xch_full, (uint32_t)split * block_bytes(rank));
+                __syncwarp();
+                if (lane < split && block_bytes(lane) != 0u)
+                    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                                     cluster_addr(part + rank * rows * pitch, (uint32_t)lane)),
+                                 "r"(smem_u32(dump + lane * rows * pitch)), "r"(block_bytes(lane)), "r"(cluster_addr(&xch_full, (uint32_t)lane))
+                                 : "memory");
             }
+            __syncwarp();
+            if (warp < 8) mbar_wait_bounded_warp(&xch_full, 0u, abortp, limit);
+            __syncthreads();
+            // (no CTA may end while the copies out of its memory are under way: every peer reports that it has received all)
+            asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+        }
+        if (warp < 8 && abort_flag == 0) {
             const int off = min(col, N - 4);
 #pragma unroll 1
             for (int r0 = (warp / groups) * 4; r0 < rows; r0 += rstep * 4) {
-                const int row = rank * rows + r0 + (lane >> 3), gp = gp_s[row];
-                int* sums = part + row * pitch;
-                int a[4], wsum = 0;
-                if (split == 1) {
-                    const int4 t = *reinterpret_cast<const int4*>(sums + off);
-                    a[0] = t.x; a[1] = t.y; a[2] = t.z; a[3] = t.w;
-                    if (p.w_levels) wsum = sums[N];
-                } else {                                 // exact: integer partial sums of the cluster's CTAs
-                    const uint32_t at = smem_u32(sums + off);
-                    int4 t[TILE_MAX_SPLIT];
+                const int r = r0 + (lane >> 3), gp = gp_s[rank * rows + r];
+                int* sums = part + r * pitch;
+                int a[4] = {0, 0, 0, 0}, wsum = 0;
 #pragma unroll
-                    for (int r = 0; r < TILE_MAX_SPLIT; ++r) {
-                        t[r] = make_int4(0, 0, 0, 0);
-                        if (r < split) {
-                            uint32_t peer;
-                            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(peer) : "r"(at), "r"(r));
-                            asm volatile("ld.shared::cluster.v4.s32 {%0, %1, %2, %3}, [%4];\n"
-                                         : "=r"(t[r].x), "=r"(t[r].y), "=r"(t[r].z), "=r"(t[r].w) : "r"(peer));
-                            if (p.w_levels) {
-                                int wr;
-                                asm volatile("ld.shared::cluster.s32 %0, [%1];\n" : "=r"(wr) : "r"(peer + 4u * (uint32_t)(N - off)));
-                                wsum += wr;
-                            }
-                        }
+                for (int i = 0; i < TILE_MAX_SPLIT; ++i) {   // exact: integer partial sums of the cluster's CTAs
+                    if (i < split) {
+                        const int4 t = *reinterpret_cast<const int4*>(sums + i * rows * pitch + off);
+                        a[0] += t.x; a[1] += t.y; a[2] += t.z; a[3] += t.w;
+                        if (p.w_levels) wsum += sums[i * rows * pitch + N];
                     }
-                    a[0] = a[1] = a[2] = a[3] = 0;
-#pragma unroll
-                    for (int r = 0; r < TILE_MAX_SPLIT; ++r) { a[0] += t[r].x; a[1] += t[r].y; a[2] += t[r].z; a[3] += t[r].w; }
                 }
                 if (p.w_levels) {
 #pragma unroll
@@ -473,12 +473,12 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
                 for (int i = 0; i < 4; ++i) y[i] = __fadd_rn(__fmul_rn(__fmul_rn((float)a[i], p.S), cs[i]), cb[i]);
                 if (p.residual && out) {
                     if (vec) {
-                        const float4 t = __ldg(reinterpret_cast<const float4*>(p.residual + o));
+                        const float4 t = ld_dep(reinterpret_cast<const float4*>(p.residual + o));
                         y[0] = __fadd_rn(y[0], t.x); y[1] = __fadd_rn(y[1], t.y); y[2] = __fadd_rn(y[2], t.z); y[3] = __fadd_rn(y[3], t.w);
                     } else {
 #pragma unroll
                         for (int i = 0; i < 4; ++i)
-                            if (i < live) y[i] = __fadd_rn(y[i], __ldg(p.residual + o + i));
+                            if (i < live) y[i] = __fadd_rn(y[i], ld_dep(p.residual + o + i));
                     }
                 }
                 if (p.res_packed && out) {
@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
                     uint32_t code4 = 0u;                 // plane j of the four channels -> bit j of four bytes
 #pragma unroll 1
                     for (int j = 0; j < p.res_bits; ++j)
-                        code4 |= ((((__ldg(rw + j) >> (4 * sub)) & 0xFu) * 0x00204081u) & 0x01010101u) << j;
+                        code4 |= ((((ld_dep(rw + j) >> (4 * sub)) & 0xFu) * 0x00204081u) & 0x01010101u) << j;
 #pragma unroll
                     for (int i = 0; i < 4; ++i) y[i] = __fadd_rn(y[i], __fmul_rn(p.res_scale, byte_to_float(code4, i)));
                 }
@@ -522,9 +522,9 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
                 asm volatile("bar.sync 1, 256;\n" ::: "memory");
                 // a thread per (pixel, 32-channel word): 32 code bytes in channel order -> plane words
                 for (int e = tid; e < rows * groups; e += TILE_WORKERS) {
-                    const int r = e / groups, gi = e - r * groups, row = rank * rows + r, gp = gp_s[row], wd = (co0 >> 5) + gi;
+                    const int r = e / groups, gi = e - r * groups, gp = gp_s[rank * rows + r], wd = (co0 >> 5) + gi;
                     if (gp < 0 || wd >= p.CWo) continue;
-                    const uint4* src4 = reinterpret_cast<const uint4*>(part + row * pitch + gi * 32);
+                    const uint4* src4 = reinterpret_cast<const uint4*>(part + r * pitch + gi * 32);
                     const uint4 lo = src4[0], hi = src4[1];
                     const uint32_t n[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
                     uint32_t cr[8], planes[8];
@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
             }
         }
         __syncwarp();
-        if (split > 1) cluster_sync_all();               // no CTA leaves while another may read its sums
+        if (split > 1) asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");

@@ -43,6 +43,7 @@ struct ConvParams {
     int test_flags;                   // bit 0 (tests only): the MMA issuer issues nothing, so that waits run out
     int tile_split;                   // tile kernel: CTAs the reduction is split over (0 = chosen by the library)
     int pipe_m_sub;                   // persistent pipeline kernel: accumulators per super-tile (0 = chosen by the library)
+    float one;                        // 1.0f: multiplier of packed additions (see f32x2_add_one)
     int acc_small;                    // 1: every accumulator of the layer is below 2^22 in magnitude (worst case of its sizes and bit counts)
     // Extents of the buffers, for the range-checked build (EBS_CHECKED); filled in every build.
     long long lim_x, lim_w;           // 32-bit words of the packed activations (bytes / 4 on the byte-code path) and of the weight plane words

@@ -38,6 +38,8 @@
 // memory and returns.  The single-CTA forms use no clusters.
 #pragma once
 
+#include <type_traits>
+
 #include "conv_frame.cuh"
 
 namespace ebs {
@@ -307,14 +309,14 @@ __device__ __forceinline__ void pipe_group32_packed(const uint32_t (&v)[32], boo
 // a group pass through 64 words of shared memory of the warp's own (one load and one store a lane, then broadcast reads):
 // read channel by channel through the cache they cost more than the arithmetic (64 -> 256 1x1 at 56x56, batch 256: 225 us
 // against 119 us for the same layer without terms).  VALUES: fp32 output may be wanted too.
-template <int TILE_N, int G, bool VALUES>
-__device__ __forceinline__ void pipe_epilogue_terms(const ConvParams& p, const FrameGeom& g, uint32_t tmem_set, int m_sub, int vwarp,
+template <int TILE_N, int G, bool VALUES, int NB, int RES>
+__device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, const FrameGeom& g, uint32_t tmem_set, int m_sub, int vwarp,
                                                     int f0, int co0, float* terms) {
     constexpr int COLS = TILE_N / 2, NG = COLS / 32;
     const int lane = (int)(threadIdx.x & 31), at = (lane & 7) * 4 + (lane >> 3);
     const uint32_t trow = tmem_set + ((uint32_t)((vwarp & 3) * 32) << 16);
     const int cbeg = (vwarp >> 2) * COLS;
-    const int nb = p.next_bits;
+    const int nb = NB > 0 ? NB : p.next_bits;                // (a constant where only planes are written)
     const float hi2 = (float)(2 * ((1 << nb) - 1) + 1);
     PlaneHold<G> hold;
     hold.filled = 0;
@@ -339,14 +341,14 @@ __device__ __forceinline__ void pipe_epilogue_terms(const ConvParams& p, const F
     auto request = [&](int c) {                              // c: first channel of the unit
         t_scale = p.ch_scale ? __ldg(p.ch_scale + c + lane) : 1.0f;
         t_bias = p.ch_bias ? __ldg(p.ch_bias + c + lane) : -0.0f;
-        if (p.residual) {
+        if constexpr (RES == 1) {
             const float4* r4 = reinterpret_cast<const float4*>(p.residual + (size_t)gp * p.Co + c);
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const float4 t = __ldg(r4 + i);
                 res[4 * i] = t.x; res[4 * i + 1] = t.y; res[4 * i + 2] = t.z; res[4 * i + 3] = t.w;
             }
-        } else if (p.res_packed) {
+        } else if constexpr (RES == 2) {
             ld_dep_planes(p.res_packed + ((size_t)gp * p.CWo + (c >> 5)) * p.res_bits, p.res_bits, rw);
         }
     };
@@ -375,18 +377,14 @@ __device__ __forceinline__ void pipe_epilogue_terms(const ConvParams& p, const F
                 tmem_ld16_issue(trow + (uint32_t)(j * TILE_N + c0 + 16), hi);
                 tmem_ld16_wait(lo);
                 tmem_ld16_wait(hi);
-                if (!p.residual && p.res_packed) planes_to_bytes<8>(rw, rbyte);
+                if constexpr (RES == 2) planes_to_bytes<8>(rw, rbyte);
                 if constexpr (VALUES) {
                     uint64_t yy[2][8];
-                    if (p.residual) terms_values32<1>(v, p.S, p.one, cs, cb, res, rbyte, 0.0f, yy);
-                    else if (p.res_packed) terms_values32<2>(v, p.S, p.one, cs, cb, res, rbyte, p.res_scale, yy);
-                    else terms_values32<0>(v, p.S, p.one, cs, cb, res, rbyte, 0.0f, yy);
+                    terms_values32<RES>(v, p.S, p.one, cs, cb, res, rbyte, p.res_scale, yy);
                     if (p.y && ok && EBS_IN_RANGE(p, CHK_PIPE_Y, gpz * p.Co + c + 31, p.lim_out)) store_values32(yy, p.relu != 0, p.y + gpz * p.Co + c);
                     if (p.packed_next) value_codes32(yy, p.one, p.inv_next, hi2, cr);
                 } else {
-                    if (p.residual) terms_codes32<1>(v, p.S, p.one, cs, cb, res, rbyte, 0.0f, p.inv_next, hi2, cr);
-                    else if (p.res_packed) terms_codes32<2>(v, p.S, p.one, cs, cb, res, rbyte, p.res_scale, p.inv_next, hi2, cr);
-                    else terms_codes32<0>(v, p.S, p.one, cs, cb, res, rbyte, 0.0f, p.inv_next, hi2, cr);
+                    terms_codes32<RES>(v, p.S, p.one, cs, cb, res, rbyte, p.res_scale, p.inv_next, hi2, cr);
                 }
             }
             if (k + 1 < NG) {
@@ -440,13 +438,13 @@ __device__ __forceinline__ void pipe_epilogue_plain_g(const ConvParams& p, uint3
 
 // Packed-only epilogue without per-channel terms of one 128-pixel accumulator (whole channel tile): nothing but the lean
 // group, for the kernel forms that are launched only for such layers.
-template <int TILE_N, int G>
-__device__ __forceinline__ void pipe_epilogue_packed_g(const ConvParams& p, uint32_t tmem_acc, int vwarp, int gp, bool pvalid,
+template <int TILE_N, int G, int NB>
+__device__ __forceinline__ void pipe_epilogue_packed_nb(const ConvParams& p, uint32_t tmem_acc, int vwarp, int gp, bool pvalid,
                                                        int co0) {
     constexpr int COLS = TILE_N / 2;
     const uint32_t trow = tmem_acc + ((uint32_t)((vwarp & 3) * 32) << 16);
     const int cbeg = (vwarp >> 2) * COLS;
-    const int nb = p.next_bits, qmax = (1 << p.next_bits) - 1;
+    constexpr int nb = NB, qmax = (1 << NB) - 1;
     const float S = p.S, inv_next = p.inv_next;
     uint32_t v[32];
     PlaneHold<G> hold;
@@ -462,6 +460,42 @@ __device__ __forceinline__ void pipe_epilogue_packed_g(const ConvParams& p, uint
         uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + ((co0 + c0) >> 5)) * nb;
         pipe_group32_packed(v, pvalid, S, inv_next, nb, qmax, dst, p, hold);
     }
+}
+
+// The plane count as a constant of the code: with run-time counts every group ran through a dozen branches (plane loops,
+// store widths), which cost the epilogue warps more in instruction fetch than their arithmetic.
+#define EBS_PIPE_EACH_NB(CALL)                                                                                    \
+    if constexpr (G > 1) {                                                                                        \
+        if (p.next_bits == 5) { constexpr int NB = 5; CALL; }                                                     \
+        else { constexpr int NB = 7; CALL; }                                                                      \
+    } else {                                                                                                      \
+        switch (p.next_bits) {                                                                                    \
+            case 1: { constexpr int NB = 1; CALL; } break;                                                        \
+            case 2: { constexpr int NB = 2; CALL; } break;                                                        \
+            case 3: { constexpr int NB = 3; CALL; } break;                                                        \
+            case 4: { constexpr int NB = 4; CALL; } break;                                                        \
+            case 5: { constexpr int NB = 5; CALL; } break;                                                        \
+            case 6: { constexpr int NB = 6; CALL; } break;                                                        \
+            case 7: { constexpr int NB = 7; CALL; } break;                                                        \
+            default: { constexpr int NB = 8; CALL; } break;                                                       \
+        }                                                                                                         \
+    }
+template <int TILE_N, int G>
+__device__ __forceinline__ void pipe_epilogue_packed_g(const ConvParams& p, uint32_t tmem_acc, int vwarp, int gp, bool pvalid, int co0) {
+    EBS_PIPE_EACH_NB((pipe_epilogue_packed_nb<TILE_N, G, NB>(p, tmem_acc, vwarp, gp, pvalid, co0)))
+}
+
+template <int TILE_N, int G, bool VALUES>
+__device__ __forceinline__ void pipe_epilogue_terms(const ConvParams& p, const FrameGeom& g, uint32_t tmem_set, int m_sub, int vwarp,
+                                                    int f0, int co0, float* terms) {
+    auto run = [&](auto res_tag) {
+        constexpr int RES = decltype(res_tag)::value;
+        if constexpr (VALUES) pipe_epilogue_terms_nb<TILE_N, G, true, 0, RES>(p, g, tmem_set, m_sub, vwarp, f0, co0, terms);
+        else EBS_PIPE_EACH_NB((pipe_epilogue_terms_nb<TILE_N, G, false, NB, RES>(p, g, tmem_set, m_sub, vwarp, f0, co0, terms)))
+    };
+    if (p.residual) run(std::integral_constant<int, 1>{});
+    else if (p.res_packed) run(std::integral_constant<int, 2>{});
+    else run(std::integral_constant<int, 0>{});
 }
 
 // Odd plane counts of the packed output take the form that holds the groups of a run back: a kernel instantiation of

@@ -1,32 +1,40 @@
 // Whole-network kernel for basic-block CIFAR ResNets: one CTA carries one image through every layer
 // with its activations resident in shared memory.
 //
-// The per-layer kernels spend most of a ResNet-20 layer's 5-18 us on launch, prologue and moving 4-37 KB
-// of activations per image through L2.  Here the activation codes of an image live in shared memory as
-// BYTES, already in the un-swizzled K-major strip layout the tcgen05 operand descriptors read
-// ([16-byte half][frame pixel][16 bytes] per 32-channel word, frame = zero-padded image), so between
-// layers there is no bit-to-byte expansion, no global traffic and no launch.  Per layer the CTA
-//   1. has the layer's weight byte image (the second part of an ebs_pack_weights buffer) fetched into one
-//      of two shared buffers by cp.async.bulk while the previous layer runs,
-//   2. lets one thread issue all MMAs of the layer -- every 128-row tile of the frame x every tap x every
-//      32-channel word, a tap being a shifted descriptor -- into tensor-memory accumulators (tile t at
-//      columns 32 t or 64 t), then tcgen05.commit onto an mbarrier,
-//   3. runs the fp32 steps of the epilogue out of tensor memory (scale, per-channel scale/shift, shortcut,
-//      ReLU, requantize: the same individually rounded operations as the per-layer kernels) and writes the
-//      codes as bytes at frame position f + Wp + 1 of the destination strip: outputs that do not exist
-//      (frame columns >= Wo, rows >= Ho) land exactly on padding positions and are written as zero.
+// The activation codes of an image live in shared memory as BYTES, already in the un-swizzled K-major strip layout the
+// tcgen05 operand descriptors read ([16-byte half][frame pixel][16 bytes] per 32-channel word, frame = zero-padded
+// image), so between layers there is no bit-to-byte expansion, no global traffic and no launch.  Per layer
+//   1. the weight byte image (the second part of an ebs_pack_weights buffer) arrives in one of two shared buffers by
+//      cp.async.bulk while earlier layers run,
+//   2. the MMAs -- every 128-row tile of the frame x every tap x every 32-channel word, a tap being a shifted
+//      descriptor -- go into tensor-memory accumulators (tile t at columns 32 t or 64 t),
+//   3. the epilogue runs the fp32 steps out of tensor memory (scale, per-channel scale/shift, shortcut, ReLU, requantize:
+//      the same individually rounded operations as the per-layer kernels) and writes the codes as bytes at frame
+//      position f + Wp + 1 of the destination strip: outputs that do not exist (frame columns >= Wo, rows >= Ho) land
+//      exactly on padding positions and are written as zero.
+// What bounds it is the chain from layer to layer, so the layers overlap as a wavefront and nothing waits for a whole
+// layer: 16 epilogue warps take (tile, channel group) units as their accumulators complete, two warps issue MMAs, one
+// fetches weights, layer records and per-channel terms ahead.  In a run of 3x3 stride-1 layers of one geometry the MMAs of
+// tile t need the codes of tiles 0 .. t + 1 of the layer before, and no strip or accumulator is overwritten earlier than
+// that same order allows; where the geometry changes, the next layer waits for all tiles.  (With the phases of a layer one
+// after the other between block barriers a layer took 5.5 us whatever its size.)
+// A unit is the 16 channels that fill one 16-byte half of a pixel's row (channels 8 i + 4 h + e of a 32-channel word), so
+// its codes leave in one 16-byte store and its identity shortcut is one 16-byte load.
 // Stride-2 3x3 layers are computed at stride 1 and subsampled in the epilogue (4x the MMAs of two or three
 // layers, no phase logic); a 1x1 stride-2 projection runs on a subsampled copy of its input laid out in the
 // output frame, keeps its accumulators in tensor memory, and the next layer's epilogue adds them as the
 // shortcut.  The identity shortcut is read from the destination strip (the block input) just before it is
 // overwritten in place.  After the last block: average pooling (pixels added in order), 8-bit
-// quantization, and the classifier as a plain integer dot product.
-// Every wait is bounded; on a timeout the CTA sets its abort flag, skips the rest, frees tensor memory.
-#include "conv_umma_strip.cuh"
+// quantization, and the classifier as a plain integer dot product, a warp per class.
+// Every wait is bounded; on a timeout the CTA sets its abort flag, every role leaves its loop, tensor memory is freed.
+#include "conv_frame.cuh"
 
 namespace ebs {
 
-constexpr int FUSED_THREADS = 768;
+constexpr int FUSED_EPI_WARPS = 16, FUSED_ISSUER_WARP = 16, FUSED_ISSUERS = 2, FUSED_LOADER_WARP = 18;
+constexpr int FUSED_THREADS = 20 * 32;                 // (warp 19 has no role)
+constexpr int FUSED_MAX_TILES = 10;                    // 320 accumulator columns of at least 32
+constexpr int FUSED_RING = 4;                          // layer records and terms in shared memory
 constexpr int FUSED_ACT_PIX = 1360;                    // pixels an activation strip holds (34 x 34 frame + halo, 128-row tiles)
 constexpr int FUSED_ACT_BYTES = FUSED_ACT_PIX * 32;    // one 32-channel word
 constexpr int FUSED_W_BYTES = 37 * 1024;               // largest weight image (3x3 64->64)
@@ -40,54 +48,95 @@ __device__ __forceinline__ uint8_t* strip_ptr(uint8_t* acts, int buf) { return a
 // A strip holds one 32-channel word of up to 1360 frame pixels or two words of up to 680: pixels per word.
 __host__ __device__ inline int strip_cap(int channels) { return channels > 32 ? FUSED_ACT_PIX / 2 : FUSED_ACT_PIX; }
 
+// What the roles derive from a layer record.
+struct FusedGeom {
+    int cw, co16, Ho, Wo, Hf, Wf, frame, tiles, acc_stride, units;   // units: epilogue units per tile (1, 2 or 4)
+};
+__device__ __forceinline__ FusedGeom fused_geom(const FusedLayer& L) {
+    FusedGeom g;
+    g.cw = (L.c_in + 31) >> 5;
+    g.co16 = (L.c_out + 15) & ~15;
+    g.Ho = L.stride == 2 ? L.h_in / 2 : L.h_in;
+    g.Wo = L.stride == 2 ? L.w_in / 2 : L.w_in;
+    // frame in which the MMAs run: the padded input for a 3x3 layer, the padded OUTPUT frame for the projection
+    g.Hf = L.k == 3 ? L.h_in + 2 : g.Ho + 2;
+    g.Wf = L.k == 3 ? L.w_in + 2 : g.Wo + 2;
+    g.frame = g.Hf * g.Wf;
+    g.tiles = (g.frame + UMMA_M - 1) / UMMA_M;
+    g.acc_stride = g.co16 > 32 ? g.co16 : 32;
+    g.units = L.c_out <= 16 ? 1 : (L.c_out <= 32 ? 2 : 4);
+    return g;
+}
+// Layer `L` can follow `P` tile by tile: same frame, stride 1, reads what P writes, nothing to clear or copy.
+__device__ __forceinline__ bool fused_follows(const FusedLayer& P, const FusedLayer& L) {
+    return L.k == 3 && P.k == 3 && P.stride == 1 && !P.hold && !L.hold && L.stride == 1 && !L.zero_dst && L.h_in == P.h_in &&
+           L.w_in == P.w_in && L.src == P.dst && L.c_out == P.c_out;
+}
+
+struct FusedTerms {                                     // per-channel terms in the order the epilogue reads them
+    float cs[64], cb[64], pcs[64], pcb[64];             // of the layer, and of the held projection
+};
+
+__device__ __forceinline__ void tmem_ld4_issue(uint32_t taddr, uint32_t (&v)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];\n" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld4_wait(uint32_t (&a)[4], uint32_t (&b)[4], uint32_t (&c)[4], uint32_t (&d)[4]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+                 : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]),
+                   "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]) :: "memory");
+}
+__device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t n) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(n) : "memory");
+}
+
 __global__ void __launch_bounds__(FUSED_THREADS, 1)
 fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, const FusedLayer* __restrict__ layers,
-                    int n_layers, const FusedHead head, float* __restrict__ logits, uint8_t* __restrict__ trace,
+                    int n_layers, const FusedHead head, float one, float* __restrict__ logits, uint8_t* __restrict__ trace,
                     long long trace_stride) {
     extern __shared__ uint8_t dyn_smem[];
-    __shared__ __align__(8) uint64_t w_bar[2], mma_bar;
+    __shared__ __align__(8) uint64_t w_full[2], w_free[2], rec_full[FUSED_RING], rec_free[FUSED_RING];
+    __shared__ __align__(8) uint64_t acc_full[FUSED_MAX_TILES], ep_done[FUSED_MAX_TILES], hold_full, copy_ready, epi_sync;
+    __shared__ __align__(16) FusedTerms s_terms[FUSED_RING];
+    __shared__ __align__(16) FusedLayer s_rec[FUSED_RING];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     __shared__ int fc_codes[64];
-    __shared__ float s_cs[64], s_cb[64], s_pcs[64], s_pcb[64];    // per-channel terms of the layer / of the held projection
-    __shared__ float s_proj_S;
-    __shared__ int s_proj_flags;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int img = blockIdx.x;
     uint8_t* base = dyn_smem + ((1024u - (smem_u32(dyn_smem) & 1023u)) & 1023u);
     uint8_t* acts = base;                                        // three strips
     uint8_t* wbuf = base + 3 * FUSED_ACT_BYTES;                  // two weight images
     volatile int* abortp = &abort_flag;
+    const unsigned limit = UMMA_WAIT_LIMIT;
 
     if (tid == 0) {
         abort_flag = 0;
-        mbar_init(&w_bar[0], 1);
-        mbar_init(&w_bar[1], 1);
-        mbar_init(&mma_bar, 4);                                   // the four issuing threads
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&w_full[i], 1);
+            mbar_init(&w_free[i], FUSED_ISSUERS);
+        }
+        for (int i = 0; i < FUSED_RING; ++i) {
+            mbar_init(&rec_full[i], 1);
+            mbar_init(&rec_free[i], FUSED_EPI_WARPS + FUSED_ISSUERS);
+        }
+        for (int i = 0; i < FUSED_MAX_TILES; ++i) {
+            mbar_init(&acc_full[i], 1);
+            mbar_init(&ep_done[i], 16);                          // four quarters x four units (fewer units arrive with more)
+        }
+        mbar_init(&hold_full, FUSED_ISSUERS);
+        mbar_init(&copy_ready, FUSED_EPI_WARPS);
+        mbar_init(&epi_sync, FUSED_EPI_WARPS);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    if (warp == 0) {
+    if (warp == FUSED_ISSUER_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_slot)),
                      "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
     // all strips start as zeros (padding positions are never written with anything else)
     for (int i = tid; i < 3 * FUSED_ACT_BYTES / 16; i += FUSED_THREADS) reinterpret_cast<uint4*>(acts)[i] = make_uint4(0, 0, 0, 0);
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    const uint32_t tmem_base = tmem_slot;
-
-    auto fetch_weights = [&](int li) {                           // one thread: the whole byte image of layer li
-        const FusedLayer& L = layers[li];
-        const int cw = (L.c_in + 31) >> 5, co16 = (L.c_out + 15) & ~15;
-        const uint32_t bytes = (uint32_t)(L.k * L.k * cw * co16 * 32);
-        mbar_arrive_expect_tx(&w_bar[li & 1], bytes);
-        bulk_copy_g2s(wbuf + (li & 1) * FUSED_W_BYTES, L.w8, bytes, &w_bar[li & 1]);
-    };
-    if (tid == 0 && n_layers > 0) fetch_weights(0);
-
     // ---- the image: u8 NHWC, 3 channels -> bytes of strip 0 in the padded frame (channel c is byte 4c of word 0)
     {
         const int Wp = img_w + 2;
@@ -100,212 +149,356 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
         }
     }
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
-
-    bool ok = true;
-    int mma_phase = 0;
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const uint32_t tmem_base = tmem_slot;
     float* pool_scratch = reinterpret_cast<float*>(strip_ptr(acts, 0));      // [pixels][c_out] of the last layer
 
-    for (int li = 0; li < n_layers && ok; ++li) {
-        const FusedLayer L = layers[li];
-        const int cw = (L.c_in + 31) >> 5, co16 = (L.c_out + 15) & ~15;
-        const int Ho = L.stride == 2 ? L.h_in / 2 : L.h_in, Wo = L.stride == 2 ? L.w_in / 2 : L.w_in;
-        // frame in which the MMAs run: the padded input for a 3x3 layer, the padded OUTPUT frame for the projection
-        const int Hf = L.k == 3 ? L.h_in + 2 : Ho + 2, Wf = L.k == 3 ? L.w_in + 2 : Wo + 2;
-        const int frame = Hf * Wf;
-        const int tiles = (frame + UMMA_M - 1) / UMMA_M;
-        const int acc_stride = co16 > 32 ? co16 : 32;
-        const int col0 = L.hold ? FUSED_HOLD_COL : 0;
-
-        const int Wp_out = Wo + 2;                                 // frame of the destination strip
-        const int cap_in = strip_cap(L.c_in), cap_out = strip_cap(L.c_out);   // pixels per word of the strips read / written
-        uint8_t* src_strip = strip_ptr(acts, L.src);
-        uint8_t* dst_strip = L.dst >= 0 ? strip_ptr(acts, L.dst) : nullptr;
-
-        if (tid == 0 && li + 1 < n_layers) fetch_weights(li + 1);  // its buffer was last read by layer li-1, finished
-        if (tid < 64) {                                            // per-channel terms -> shared memory (read by every row)
-            const bool in = tid < L.c_out;
-            s_cs[tid] = (L.ch_scale && in) ? __ldg(L.ch_scale + tid) : 1.0f;
-            s_cb[tid] = (L.ch_bias && in) ? __ldg(L.ch_bias + tid) : 0.0f;
-            if (L.res == 2) {
-                const FusedLayer& P = layers[li - 1];              // the projection whose accumulators are held
-                s_pcs[tid] = (P.ch_scale && in) ? __ldg(P.ch_scale + tid) : 1.0f;
-                s_pcb[tid] = (P.ch_bias && in) ? __ldg(P.ch_bias + tid) : 0.0f;
-                if (tid == 0) { s_proj_S = P.S; s_proj_flags = (P.ch_scale ? 1 : 0) | (P.ch_bias ? 2 : 0); }
+    if (warp == FUSED_LOADER_WARP) {
+        // =========================== records, terms, weights ===========================
+        const float *hold_cs = nullptr, *hold_cb = nullptr;
+        for (int li = 0; li < n_layers; ++li) {
+            const int slot = li & (FUSED_RING - 1), use = li / FUSED_RING;
+            if (use > 0 && !mbar_wait_bounded_warp(&rec_free[slot], (uint32_t)((use - 1) & 1), abortp, limit)) break;
+            for (int i = lane; i < (int)(sizeof(FusedLayer) / 4); i += 32)
+                reinterpret_cast<uint32_t*>(&s_rec[slot])[i] = __ldg(reinterpret_cast<const uint32_t*>(layers + li) + i);
+            __syncwarp();
+            const FusedLayer& L = s_rec[slot];
+            FusedTerms& T = s_terms[slot];
+            for (int c = lane; c < 64; c += 32) {
+                const int at = L.c_out <= 16 ? (c < 16 ? (c & 7) * 2 + (c >> 3) : c) : (c & 32) + (c & 7) * 4 + ((c & 31) >> 3);
+                const bool in = c < L.c_out;
+                T.cs[at] = (L.ch_scale && in) ? __ldg(L.ch_scale + c) : 1.0f;    // identities: x * 1, x + (-0)
+                T.cb[at] = (L.ch_bias && in) ? __ldg(L.ch_bias + c) : -0.0f;
+                T.pcs[at] = (hold_cs && in) ? __ldg(hold_cs + c) : 1.0f;
+                T.pcb[at] = (hold_cb && in) ? __ldg(hold_cb + c) : -0.0f;
             }
-        }
-
-        if (L.k == 1) {
-            // projection: its input is the stride-2 subsample of strip src, copied into strip dst in the output frame
-            for (int i = tid; i < FUSED_ACT_BYTES / 16; i += FUSED_THREADS)
-                reinterpret_cast<uint4*>(dst_strip)[i] = make_uint4(0, 0, 0, 0);
-            __syncthreads();
-            const int Wp_in = L.w_in + 2;
-            for (int e = tid; e < Ho * Wo * cw * 2; e += FUSED_THREADS) {
-                const int half = e & 1, rest = e >> 1, wd = rest % cw, pix = rest / cw;
-                const int ho = pix / Wo, wo = pix - ho * Wo;
-                const uint8_t* s = src_strip + wd * cap_in * 32 + half * cap_in * 16 + ((2 * ho + 1) * Wp_in + 2 * wo + 1) * 16;
-                uint8_t* d = dst_strip + wd * cap_in * 32 + half * cap_in * 16 + ((ho + 1) * Wf + wo + 1) * 16;
-                *reinterpret_cast<uint4*>(d) = *reinterpret_cast<const uint4*>(s);
+            hold_cs = L.hold ? L.ch_scale : nullptr;
+            hold_cb = L.hold ? L.ch_bias : nullptr;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&rec_full[slot]);
+            if (li >= 2 && !mbar_wait_bounded_warp(&w_free[li & 1], (uint32_t)(((li >> 1) - 1) & 1), abortp, limit)) break;
+            if (lane == 0) {
+                const uint32_t bytes = (uint32_t)(L.k * L.k * ((L.c_in + 31) >> 5) * ((L.c_out + 15) & ~15) * 32);
+                mbar_arrive_expect_tx(&w_full[li & 1], bytes);
+                bulk_copy_g2s(wbuf + (li & 1) * FUSED_W_BYTES, L.w8, bytes, &w_full[li & 1]);
             }
-        } else if (L.zero_dst && dst_strip) {
-            for (int i = tid; i < FUSED_ACT_BYTES / 16; i += FUSED_THREADS)
-                reinterpret_cast<uint4*>(dst_strip)[i] = make_uint4(0, 0, 0, 0);
+            __syncwarp();
         }
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        __syncthreads();
-
-        // ---- MMAs of the whole layer
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        if (lane == 0 && warp < 4 && mbar_wait_bounded(&w_bar[li & 1], (uint32_t)((li >> 1) & 1), abortp)) {
-            // Four threads issue (lane 0 of warps 0-3, tiles dealt round-robin): the issue loop of one thread,
-            // not the tensor core, bounds a layer of many small MMAs.  Descriptors are built once and advanced
-            // by additions (start addresses are in 16-byte units).  Each thread's commit arrives once.
-            if (warp < tiles) {
-                const uint32_t idesc = umma_idesc_i8(co16);
-                const uint8_t* a_src = L.k == 1 ? dst_strip : src_strip;   // the projection reads its subsampled copy
-                const uint64_t da0 = umma_desc_interleaved(smem_u32(a_src), (uint32_t)(cap_in * 16));
-                uint64_t db = umma_desc_sw32(smem_u32(wbuf + (li & 1) * FUSED_W_BYTES));
-                const uint64_t db_step = (uint64_t)((co16 * 32) >> 4), db_word = db_step * (uint64_t)cw;
+        if (*abortp)                                     // a copy may still be in flight towards this CTA's shared memory
+            for (int i = 0; i < 64; ++i) __nanosleep(1000);
+    } else if (warp >= FUSED_ISSUER_WARP && warp < FUSED_ISSUER_WARP + FUSED_ISSUERS) {
+        // =========================== MMAs ===========================
+        const int k_iss = warp - FUSED_ISSUER_WARP;
+        const uint32_t leader = lane == 0 ? 1u : 0u;
+        uint32_t par = 0u;                               // bit t: parity of the number of layers that used tile t so far
+        int prev = -1, prev_tiles = 0, n_copies = 0;     // the last layer with an epilogue
+        bool ok = true;
+        for (int li = 0; li < n_layers && ok; ++li) {
+            const int slot = li & (FUSED_RING - 1);
+            if (!mbar_wait_bounded_warp(&rec_full[slot], (uint32_t)((li / FUSED_RING) & 1), abortp, limit)) break;
+            const FusedLayer& L = s_rec[slot];
+            const FusedGeom g = fused_geom(L);
+            // (the record before it is still in the ring: this warp has not released it while it is compared)
+            const bool wave = prev >= 0 && prev == li - 1 && fused_follows(s_rec[prev & (FUSED_RING - 1)], L);
+            if (!mbar_wait_bounded_warp(&w_full[li & 1], (uint32_t)((li >> 1) & 1), abortp, limit)) break;
+            if (L.k == 1) {                              // the subsampled copy of its input
+                if (!mbar_wait_bounded_warp(&copy_ready, (uint32_t)(n_copies & 1), abortp, limit)) break;
+                ++n_copies;
+            }
+            const int cap_in = strip_cap(L.c_in);
+            const uint64_t da0 = umma_desc_interleaved(smem_u32(strip_ptr(acts, L.k == 1 ? L.dst : L.src)), (uint32_t)(cap_in * 16));
+            const uint64_t db0 = umma_desc_sw32(smem_u32(wbuf + (li & 1) * FUSED_W_BYTES));
+            const uint32_t da_hi = (uint32_t)(da0 >> 32), db_hi = (uint32_t)(db0 >> 32);
+            const uint32_t idesc = umma_idesc_i8(g.co16), step = (uint32_t)((g.co16 * 32) >> 4);
+            const int k = L.k, cw = g.cw;
+            int waited = 0;                              // tiles of the layer before that are known to be finished
+            auto wait_tiles = [&](int upto) {
+                for (; waited < upto; ++waited)
+                    if (!mbar_wait_bounded_warp(&ep_done[waited], ((par >> waited) & 1u) ^ 1u, abortp, limit)) return false;
+                return true;
+            };
+            for (int t = k_iss; t < g.tiles; t += FUSED_ISSUERS) {
+                const int need = wave ? min(prev_tiles, (t * UMMA_M + UMMA_M + g.Wf) / UMMA_M + 1) : prev_tiles;
+                if (!wait_tiles(need)) { ok = false; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                const uint32_t tm = tmem_base + (uint32_t)((L.hold ? FUSED_HOLD_COL : 0) + t * g.acc_stride);
+                uint32_t accu = 0u;
                 for (int wd = 0; wd < cw; ++wd) {
-                    const uint64_t da_w = da0 + (uint64_t)(wd * cap_in * 2);   // one word = cap_in * 32 bytes
-                    uint64_t db_t = db + db_step * (uint64_t)wd;                // weight tiles are ordered [tap][word]
-                    for (int r = 0; r < L.k; ++r) {
-                        for (int s = 0; s < L.k; ++s, db_t += db_word) {
-                            const int shift = L.k == 3 ? r * Wf + s : Wf + 1;    // 1x1: the centre of the output frame
-                            const uint32_t acc_flag = (wd | r | s) != 0 ? 1u : 0u;
-                            uint64_t da = da_w + (uint64_t)(warp * UMMA_M + shift);
-                            uint32_t tm = tmem_base + (uint32_t)(col0 + warp * acc_stride);
-                            for (int t = warp; t < tiles; t += 4, da += 4 * UMMA_M, tm += 4 * acc_stride)
-                                umma_i8(tm, da, db_t, idesc, acc_flag);
+                    uint32_t a_row = (uint32_t)da0 + (uint32_t)(wd * cap_in * 2 + t * UMMA_M + (k == 3 ? 0 : g.Wf + 1));
+                    uint32_t b_lo = (uint32_t)db0 + step * (uint32_t)wd;      // weight tiles are ordered [tap][word]
+                    for (int r = 0; r < k; ++r, a_row += (uint32_t)g.Wf) {
+                        for (int s = 0; s < k; ++s, b_lo += step * (uint32_t)cw) {
+                            umma_i8_split(leader, tm, a_row + (uint32_t)s, da_hi, b_lo, db_hi, idesc, accu);
+                            accu = 1u;
                         }
                     }
                 }
-                umma_commit(&mma_bar);
+                if (!L.hold) umma_commit_pred(leader, &acc_full[t]);
+            }
+            if (!ok || !wait_tiles(prev_tiles)) break;   // (every phase of these barriers is waited for, so that parities stay in step)
+            if (L.hold) {
+                umma_commit_pred(leader, &hold_full);
             } else {
-                mbar_arrive(&mma_bar);
+                prev = li;
+                prev_tiles = g.tiles;
+                par ^= (1u << g.tiles) - 1u;
+            }
+            umma_commit_pred(leader, &w_free[li & 1]);
+            __syncwarp();
+            // the slot before this one is not looked at any more
+            if (li > 0 && lane == 0) mbar_arrive(&rec_free[(li - 1) & (FUSED_RING - 1)]);
+        }
+        // the last commits have arrived before the block ends
+        if (ok && n_layers > 0 && !*abortp) mbar_wait_bounded_warp(&w_free[(n_layers - 1) & 1], (uint32_t)(((n_layers - 1) >> 1) & 1), abortp, limit);
+    } else if (warp < FUSED_EPI_WARPS) {
+        // =========================== epilogue ===========================
+        const int quarter = warp & 3, quad = warp >> 2;
+        const float half = 0.5f;
+        uint32_t par = 0u;
+        int turn = 0, n_sync = 0, n_hold = 0;            // turn: units dealt so far, modulo 4
+        bool ok = true;
+        auto all_epilogue_warps = [&]() {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&epi_sync);
+            const bool good = mbar_wait_bounded_warp(&epi_sync, (uint32_t)(n_sync & 1), abortp, limit);
+            ++n_sync;
+            return good;
+        };
+        for (int li = 0; li < n_layers && ok; ++li) {
+            const int slot = li & (FUSED_RING - 1);
+            if (!mbar_wait_bounded_warp(&rec_full[slot], (uint32_t)((li / FUSED_RING) & 1), abortp, limit)) break;
+            const FusedLayer& L = s_rec[slot];
+            const FusedTerms& T = s_terms[slot];
+            const FusedGeom g = fused_geom(L);
+            uint8_t* dst_strip = L.dst >= 0 ? strip_ptr(acts, L.dst) : nullptr;
+            const int cap_out = strip_cap(L.c_out);
+            if (dst_strip && (L.zero_dst || L.k == 1)) {
+                // the strip's old contents have no reader left once every warp is here (its units waited for the MMAs)
+                if (!all_epilogue_warps()) break;
+                for (int i = tid; i < FUSED_ACT_BYTES / 16; i += FUSED_EPI_WARPS * 32) reinterpret_cast<uint4*>(dst_strip)[i] = make_uint4(0, 0, 0, 0);
+                if (!all_epilogue_warps()) break;
+            }
+            if (L.k == 1) {
+                // projection: its input is the stride-2 subsample of strip src, copied into strip dst in the output frame
+                const int Wp_in = L.w_in + 2, cap_in = strip_cap(L.c_in);
+                const uint8_t* src_strip = strip_ptr(acts, L.src);
+                for (int e = tid; e < g.Ho * g.Wo * g.cw * 2; e += FUSED_EPI_WARPS * 32) {
+                    const int hf = e & 1, rest = e >> 1, wd = rest % g.cw, pix = rest / g.cw;
+                    const int ho = pix / g.Wo, wo = pix - ho * g.Wo;
+                    const uint8_t* s = src_strip + wd * cap_in * 32 + hf * cap_in * 16 + ((2 * ho + 1) * Wp_in + 2 * wo + 1) * 16;
+                    uint8_t* d = dst_strip + wd * cap_in * 32 + hf * cap_in * 16 + ((ho + 1) * g.Wf + wo + 1) * 16;
+                    *reinterpret_cast<uint4*>(d) = *reinterpret_cast<const uint4*>(s);
+                }
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&copy_ready);
+                // its MMAs: before anything may overwrite the copy, and before the next layer reads their accumulators
+                if (!mbar_wait_bounded_warp(&hold_full, (uint32_t)(n_hold & 1), abortp, limit)) break;
+                ++n_hold;
+            } else {
+                const int Wp_out = g.Wo + 2, res = L.res, units = g.units;
+                const bool narrow = L.c_out <= 16, to_pool = L.dst < 0, relu = L.relu != 0;
+                const float hi2 = (float)(2 * ((1 << L.out_bits) - 1) + 1);
+                const uint64_t S2 = f32x2_pack(L.S, L.S), one2 = f32x2_pack(one, one), inv2 = f32x2_pack(L.out_inv_step, L.out_inv_step);
+                const uint64_t half2 = f32x2_pack(half, half), rs2 = f32x2_pack(L.res_step, L.res_step);
+                const float PS = res == 2 ? s_rec[(li - 1) & (FUSED_RING - 1)].S : 0.0f;
+                const uint64_t PS2 = f32x2_pack(PS, PS);
+                const int total = g.tiles * units;
+                if (L.src == (to_pool ? 0 : L.dst)) {    // writes over its own input: only after the last MMA
+                    for (int t = 0; t < g.tiles && ok; ++t) ok = mbar_wait_bounded_warp(&acc_full[t], (par >> t) & 1u, abortp, limit);
+                    if (!ok) break;
+                }
+                for (int u = 0; u < total; ++u) {
+                    const int t = u / units, un = u - t * units;
+                    if (un == 0 && !mbar_wait_bounded_warp(&acc_full[t], (par >> t) & 1u, abortp, limit)) { ok = false; break; }
+                    if (((turn + u) & 3) != quad) continue;
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    const int f = t * UMMA_M + quarter * 32 + lane;
+                    const int hp = f / g.Wf, wp = f - hp * g.Wf;
+                    // does this frame row have an output, and where does it go in the destination frame
+                    bool valid = f < g.frame;
+                    int ho = hp, wo = wp;
+                    if (L.stride == 2) { valid = valid && !(hp & 1) && !(wp & 1); ho = hp >> 1; wo = wp >> 1; }
+                    valid = valid && ho < g.Ho && wo < g.Wo;
+                    const int target = L.stride == 2 ? (ho + 1) * Wp_out + wo + 1 : f + g.Wf + 1;
+                    const bool in_frame = f < g.frame && (L.stride == 1 || valid);   // stride 1 also writes the zeros of the padding
+                    if (__any_sync(0xffffffffu, in_frame)) {
+                        const uint32_t trow = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(t * g.acc_stride);
+                        // word e of this unit: channels ch(e, 0 .. 3) as its bytes.  Wide: word 4 hf + e of the 32-channel
+                        // group; narrow (all 16 channels in one unit): words 0 .. 7, channels b and 8 + b
+                        const int grp = un >> 1, hf = un & 1;
+                        uint32_t words[8];
+                        uint32_t resw[8];
+                        uint8_t* at = dst_strip + grp * cap_out * 32 + target * 16;
+                        const uint8_t* rp = strip_ptr(acts, L.res_buf) + grp * cap_out * 32 + target * 16;
+                        auto value = [&](uint64_t w, uint64_t a, uint64_t b) { return f32x2_add_one(f32x2_mul_rn(w, a), one2, b); };
+                        auto code = [&](uint64_t w, uint32_t& m0, uint32_t& m1) {
+                            w = f32x2_add_one(f32x2_mul_rn(w, inv2), one2, half2);
+                            m0 = code_pattern(__uint_as_float((uint32_t)w), hi2);
+                            m1 = code_pattern(__uint_as_float((uint32_t)(w >> 32)), hi2);
+                        };
+                        auto pool = [&](uint64_t w, int c) {                  // two channels 8 apart
+                            float y0 = __uint_as_float((uint32_t)w), y1 = __uint_as_float((uint32_t)(w >> 32));
+                            if (relu) { y0 = y0 > 0.0f ? y0 : 0.0f; y1 = y1 > 0.0f ? y1 : 0.0f; }
+                            if (valid && c < L.c_out) pool_scratch[(ho * g.Wo + wo) * L.c_out + c] = y0;
+                            if (valid && c + 8 < L.c_out) pool_scratch[(ho * g.Wo + wo) * L.c_out + c + 8] = y1;
+                        };
+                        auto pair = [](uint32_t a, uint32_t b) { return f32x2_pack((float)(int)a, (float)(int)b); };
+                        if (narrow) {
+                            uint32_t v[16], pv[16];
+                            tmem_ld16_issue(trow, v);
+                            if (res == 2) tmem_ld16_issue(trow + FUSED_HOLD_COL, pv);
+                            if (res == 1) {
+                                const uint4 a = *reinterpret_cast<const uint4*>(rp), b = *reinterpret_cast<const uint4*>(rp + cap_out * 16);
+                                resw[0] = a.x; resw[1] = a.y; resw[2] = a.z; resw[3] = a.w;
+                                resw[4] = b.x; resw[5] = b.y; resw[6] = b.z; resw[7] = b.w;
+                            }
+                            tmem_ld16_wait(v);
+                            if (res == 2) tmem_ld16_wait(pv);
+#pragma unroll
+                            for (int b = 0; b < 8; ++b) {
+                                const float2 s2 = *reinterpret_cast<const float2*>(&T.cs[2 * b]), b2 = *reinterpret_cast<const float2*>(&T.cb[2 * b]);
+                                uint64_t w = value(f32x2_mul_rn(pair(v[b], v[8 + b]), S2), f32x2_pack(s2.x, s2.y), f32x2_pack(b2.x, b2.y));
+                                if (res == 2) {
+                                    const float2 ps = *reinterpret_cast<const float2*>(&T.pcs[2 * b]), pb = *reinterpret_cast<const float2*>(&T.pcb[2 * b]);
+                                    w = f32x2_add_one(w, one2, value(f32x2_mul_rn(pair(pv[b], pv[8 + b]), PS2), f32x2_pack(ps.x, ps.y), f32x2_pack(pb.x, pb.y)));
+                                }
+                                if (res == 1) w = f32x2_add_one(w, one2, f32x2_mul_rn(rs2, f32x2_pack(byte_to_float(resw[b], 0), byte_to_float(resw[b], 1))));
+                                if (to_pool) {
+                                    pool(w, b);
+                                } else {
+                                    uint32_t m0, m1;
+                                    code(w, m0, m1);
+                                    words[b] = (__byte_perm(m0, m1, 0x0040) & 0xFFFFu) & ((b < L.c_out ? 0xFFu : 0u) | (8 + b < L.c_out ? 0xFF00u : 0u));
+                                }
+                            }
+                        } else {
+                            uint32_t v[4][4], pv[4][4];
+                            const uint32_t tc = trow + (uint32_t)(32 * grp + 4 * hf);
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) tmem_ld4_issue(tc + 8u * i, v[i]);
+                            if (res == 2) {
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) tmem_ld4_issue(tc + FUSED_HOLD_COL + 8u * i, pv[i]);
+                            }
+                            if (res == 1) {
+                                const uint4 a = *reinterpret_cast<const uint4*>(rp + hf * cap_out * 16);
+                                resw[0] = a.x; resw[1] = a.y; resw[2] = a.z; resw[3] = a.w;
+                            }
+                            tmem_ld4_wait(v[0], v[1], v[2], v[3]);
+                            if (res == 2) tmem_ld4_wait(pv[0], pv[1], pv[2], pv[3]);
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const int ti = grp * 32 + (4 * hf + e) * 4, c = 32 * grp + 4 * hf + e;
+                                const float4 s4 = *reinterpret_cast<const float4*>(&T.cs[ti]), b4 = *reinterpret_cast<const float4*>(&T.cb[ti]);
+                                uint64_t w0 = value(f32x2_mul_rn(pair(v[0][e], v[1][e]), S2), f32x2_pack(s4.x, s4.y), f32x2_pack(b4.x, b4.y));
+                                uint64_t w1 = value(f32x2_mul_rn(pair(v[2][e], v[3][e]), S2), f32x2_pack(s4.z, s4.w), f32x2_pack(b4.z, b4.w));
+                                if (res == 2) {
+                                    const float4 ps = *reinterpret_cast<const float4*>(&T.pcs[ti]), pb = *reinterpret_cast<const float4*>(&T.pcb[ti]);
+                                    w0 = f32x2_add_one(w0, one2, value(f32x2_mul_rn(pair(pv[0][e], pv[1][e]), PS2), f32x2_pack(ps.x, ps.y), f32x2_pack(pb.x, pb.y)));
+                                    w1 = f32x2_add_one(w1, one2, value(f32x2_mul_rn(pair(pv[2][e], pv[3][e]), PS2), f32x2_pack(ps.z, ps.w), f32x2_pack(pb.z, pb.w)));
+                                }
+                                if (res == 1) {
+                                    w0 = f32x2_add_one(w0, one2, f32x2_mul_rn(rs2, f32x2_pack(byte_to_float(resw[e], 0), byte_to_float(resw[e], 1))));
+                                    w1 = f32x2_add_one(w1, one2, f32x2_mul_rn(rs2, f32x2_pack(byte_to_float(resw[e], 2), byte_to_float(resw[e], 3))));
+                                }
+                                if (to_pool) {
+                                    pool(w0, c);
+                                    pool(w1, c + 16);
+                                } else {
+                                    uint32_t m[4];
+                                    code(w0, m[0], m[1]);
+                                    code(w1, m[2], m[3]);
+                                    words[e] = join_codes(m);
+                                    if (L.c_out & 31) {                       // channels past c_out
+                                        const uint32_t keep = (c < L.c_out ? 0xFFu : 0u) | (c + 8 < L.c_out ? 0xFF00u : 0u) |
+                                                              (c + 16 < L.c_out ? 0xFF0000u : 0u) | (c + 24 < L.c_out ? 0xFF000000u : 0u);
+                                        words[e] &= keep;
+                                    }
+                                }
+                            }
+                        }
+                        if (!to_pool) {
+                            if (in_frame) {
+                                const uint32_t z = valid ? 0xFFFFFFFFu : 0u;
+                                const uint4 a = make_uint4(words[0] & z, words[1] & z, words[2] & z, words[3] & z);
+                                if (narrow) {
+                                    *reinterpret_cast<uint4*>(at) = a;
+                                    *reinterpret_cast<uint4*>(at + cap_out * 16) = make_uint4(words[4] & z, words[5] & z, words[6] & z, words[7] & z);
+                                } else {
+                                    *reinterpret_cast<uint4*>(at + hf * cap_out * 16) = a;
+                                }
+                            }
+                            if (trace && L.trace_off >= 0 && valid) {
+                                uint8_t* tp = trace + (size_t)img * trace_stride + L.trace_off + (size_t)(ho * g.Wo + wo) * L.c_out;
+                                const int nwords = narrow ? 8 : 4;
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) {
+                                    if (e >= nwords) break;
+#pragma unroll
+                                    for (int i = 0; i < 4; ++i) {
+                                        const int c = (narrow ? 8 * i + e : 32 * grp + 8 * i + 4 * hf + e);
+                                        if (c < L.c_out && (!narrow || i < 2)) tp[c] = (uint8_t)(words[e] >> (8 * i));
+                                    }
+                                }
+                            }
+                        }
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_n(&ep_done[t], (uint32_t)(4 / units));
+                }
+                turn = (turn + total) & 3;
+                par ^= (1u << g.tiles) - 1u;
+            }
+            __syncwarp();
+            // (a held projection's record is read once more by the layer after it)
+            if (ok && lane == 0) {
+                if (li > 0) mbar_arrive(&rec_free[(li - 1) & (FUSED_RING - 1)]);
             }
         }
-        // one warp polls for the MMAs' completion; the others sleep in the block barrier instead of spinning
-        if (warp == 4) mbar_wait_bounded(&mma_bar, (uint32_t)(mma_phase & 1), abortp);
-        __syncthreads();
-        if (abort_flag != 0) { ok = false; break; }
-        ++mma_phase;
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-
-        // ---- epilogue (a held projection has none: the next layer reads its accumulators)
-        if (!L.hold) {
-            const int qmax = (1 << L.out_bits) - 1;
-            const int quarter = warp & 3;
-            const bool has_cs = L.ch_scale != nullptr, has_cb = L.ch_bias != nullptr;
-            const bool p_cs = s_proj_flags & 1, p_cb = s_proj_flags & 2;
-            const float S = L.S, inv_step = L.out_inv_step, res_step = L.res_step, PS = s_proj_S;
-            // a unit of work is (tile, 16 channels); the four warps of a TMEM lane quarter take units in turn
-            const int nb16 = co16 >> 4, units = tiles * nb16;
-            for (int u = warp >> 2; u < units; u += FUSED_THREADS / 128) {
-                const int t = u / nb16, c0 = (u - t * nb16) << 4;
-                const int f = t * UMMA_M + quarter * 32 + lane;
-                const int hp = f / Wf, wp = f - hp * Wf;
-                // does this frame row have an output, and where does it go in the destination frame
-                bool valid = f < frame;
-                int ho = hp, wo = wp;
-                if (L.stride == 2) { valid = valid && !(hp & 1) && !(wp & 1); ho = hp >> 1; wo = wp >> 1; }
-                valid = valid && ho < Ho && wo < Wo;
-                const int target = L.stride == 2 ? (ho + 1) * Wp_out + wo + 1 : f + Wf + 1;
-                const bool in_frame = f < frame && (L.stride == 1 || valid);   // stride 1 also writes the zeros of the padding
-                const uint32_t trow = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(col0 + t * acc_stride);
-                const uint32_t prow = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(FUSED_HOLD_COL + t * acc_stride);
-                const int lane0 = (c0 & 16) >> 3;                        // byte lane of channels c0 .. c0+7 in words 0..7
-                uint32_t resw[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};      // the identity shortcut's word at the same pixel
-                if (L.res == 1 && valid) {
-                    const uint8_t* rp = strip_ptr(acts, L.res_buf) + (c0 >> 5) * cap_out * 32 + target * 16;
-                    const uint4 a = *reinterpret_cast<const uint4*>(rp), b = *reinterpret_cast<const uint4*>(rp + cap_out * 16);
-                    resw[0] = a.x; resw[1] = a.y; resw[2] = a.z; resw[3] = a.w;
-                    resw[4] = b.x; resw[5] = b.y; resw[6] = b.z; resw[7] = b.w;
-                }
-                uint32_t v[16], pv[16];
-                tmem_ld16(trow + (uint32_t)c0, v);                      // whole warp, also for rows without an output
-                if (L.res == 2) tmem_ld16(prow + (uint32_t)c0, pv);
-                int q[16];
-#pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    const int c = c0 + e;
-                    float y = __fmul_rn((float)(int)v[e], S);
-                    if (has_cs) y = __fmul_rn(y, s_cs[c]);
-                    if (has_cb) y = __fadd_rn(y, s_cb[c]);
-                    if (L.res == 2) {                               // projection shortcut: its own scale and per-channel terms
-                        float r = __fmul_rn((float)(int)pv[e], PS);
-                        if (p_cs) r = __fmul_rn(r, s_pcs[c]);
-                        if (p_cb) r = __fadd_rn(r, s_pcb[c]);
-                        y = __fadd_rn(y, r);
-                    }
-                    if (L.res == 1)                                 // identity shortcut: channel 8 i + k is byte i of word k
-                        y = __fadd_rn(y, __fmul_rn(res_step, (float)((resw[e & 7] >> (8 * (lane0 + (e >> 3)))) & 0xFFu)));
-                    if (L.relu && !(y > 0.0f)) y = 0.0f;
-                    int code = 0;
-                    if (valid && c < L.c_out) {
-                        if (L.dst < 0) pool_scratch[(ho * Wo + wo) * L.c_out + c] = y;
-                        else code = min(__float2int_rd(__fadd_rn(__fmul_rn(y, inv_step), 0.5f)), qmax);
-                    }
-                    q[e] = code;
-                }
-                if (L.dst >= 0 && in_frame) {
-                    // word k of the pixel holds channels k, 8+k, 16+k, 24+k as bytes: these 16 channels are two
-                    // adjacent bytes of each of the eight words (negative codes saturate to 0)
-                    uint8_t* wp_ = dst_strip + (c0 >> 5) * cap_out * 32 + target * 16 + lane0;
-#pragma unroll
-                    for (int k8 = 0; k8 < 8; ++k8) {
-                        uint32_t two;
-                        asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;\n" : "=r"(two) : "r"(q[8 + k8]), "r"(q[k8]), "r"(0));
-                        *reinterpret_cast<uint16_t*>(wp_ + (k8 >> 2) * cap_out * 16 + (k8 & 3) * 4) = (uint16_t)two;
-                    }
-                    if (trace && L.trace_off >= 0 && valid) {
-                        uint8_t* tp = trace + (size_t)img * trace_stride + L.trace_off + (size_t)(ho * Wo + wo) * L.c_out + c0;
-#pragma unroll
-                        for (int e = 0; e < 16; ++e)
-                            if (c0 + e < L.c_out) tp[e] = (uint8_t)max(q[e], 0);
-                    }
-                }
-            }
-        }
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     }
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
     // ---- pooling, 8-bit quantization, classifier
-    if (ok && !abort_flag && n_layers > 0) {
-        const FusedLayer L = layers[n_layers - 1];
-        const int Ho = L.stride == 2 ? L.h_in / 2 : L.h_in, Wo = L.stride == 2 ? L.w_in / 2 : L.w_in;
-        const int hw = Ho * Wo, C = L.c_out;
+    if (!abort_flag && n_layers > 0) {
+        const FusedLayer& L = s_rec[(n_layers - 1) & (FUSED_RING - 1)];
+        const FusedGeom g = fused_geom(L);
+        const int hw = g.Ho * g.Wo, C = L.c_out;
         if (tid < C && tid < 64) {
             float acc = 0.0f;
+#pragma unroll 8
             for (int p = 0; p < hw; ++p) acc = __fadd_rn(acc, pool_scratch[p * C + tid]);
             const float m = __fmul_rn(acc, 1.0f / (float)hw);
             fc_codes[tid] = quantize_act_code(m, head.a_inv_step, 255);
         }
         __syncthreads();
-        if (tid < head.c_out) {
-            const int co16 = (head.c_out + 15) & ~15, cwf = (head.c_in + 31) >> 5;
+        const int co16 = (head.c_out + 15) & ~15;
+        for (int o = warp; o < head.c_out; o += FUSED_THREADS / 32) {
             int acc = 0;
-            for (int c = 0; c < head.c_in; ++c) {
+            for (int c = lane; c < head.c_in; c += 32) {
                 const int wd = c >> 5, cc = c & 31, j = 4 * (cc & 7) + (cc >> 3);      // byte 4b + i of the row
-                const int jj = j ^ (((tid >> 2) & 1) << 4);                               // halves swapped for these rows
-                const int8_t wv = (int8_t)head.w8[((size_t)wd * co16 + tid) * 32 + jj];
-                acc += (int)wv * fc_codes[c];
+                const int jj = j ^ (((o >> 2) & 1) << 4);                                 // halves swapped for these rows
+                acc += (int)(int8_t)head.w8[((size_t)wd * co16 + o) * 32 + jj] * fc_codes[c];
             }
-            (void)cwf;
-            float y = __fmul_rn((float)acc, head.S);
-            if (head.ch_scale) y = __fmul_rn(y, __ldg(head.ch_scale + tid));
-            if (head.ch_bias) y = __fadd_rn(y, __ldg(head.ch_bias + tid));
-            logits[(size_t)img * head.c_out + tid] = y;
+            acc = __reduce_add_sync(0xffffffffu, acc);
+            if (lane == 0) {
+                float y = __fmul_rn((float)acc, head.S);
+                if (head.ch_scale) y = __fmul_rn(y, __ldg(head.ch_scale + o));
+                if (head.ch_bias) y = __fadd_rn(y, __ldg(head.ch_bias + o));
+                logits[(size_t)img * head.c_out + o] = y;
+            }
         }
     }
     if (abort_flag != 0 && tid == 0) atomicAdd(&g_umma_timeouts, 1ull);
 
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
-    if (warp == 0) {
+    if (warp == FUSED_ISSUER_WARP) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(512u) : "memory");
     }
 }
@@ -356,7 +549,7 @@ int launch_fused_resnet(const uint8_t* images, int n, int img_h, int img_w, cons
     FusedHead head;
     memcpy(&head, head_host, sizeof(head));
     fused_resnet_kernel<<<n, FUSED_THREADS, FUSED_SMEM, st>>>(images, img_h, img_w, static_cast<const FusedLayer*>(layers_dev),
-                                                               n_layers, head, logits, trace, trace_stride);
+                                                               n_layers, head, 1.0f, logits, trace, trace_stride);
     return check_cuda(cudaGetLastError());
 }
 

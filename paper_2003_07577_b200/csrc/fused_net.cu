@@ -73,6 +73,11 @@ __device__ __forceinline__ bool fused_follows(const FusedLayer& P, const FusedLa
            L.w_in == P.w_in && L.src == P.dst && L.c_out == P.c_out;
 }
 
+// The same value in every lane, known to the compiler to be so: what the issuing warps feed into descriptors and loop
+// bounds has to live in uniform registers, or every MMA moves four operands there first (130 clocks an MMA instead of 40).
+__device__ __forceinline__ int uni(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ uint32_t uni(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 struct FusedTerms {                                     // per-channel terms in the order the epilogue reads them
     float cs[64], cb[64], pcs[64], pcb[64];             // of the layer, and of the held projection
 };
@@ -87,6 +92,163 @@ __device__ __forceinline__ void tmem_ld4_wait(uint32_t (&a)[4], uint32_t (&b)[4]
 }
 __device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t n) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(n) : "memory");
+}
+
+// What the units of a layer share.
+struct FusedUnitEnv {
+    uint64_t S2, PS2, rs2, one2, inv2;
+    float hi2;
+    int c_out, cap_out;
+    uint8_t* dst;                                       // destination strip
+    const uint8_t* res;                                 // strip of the identity shortcut
+    const FusedTerms* T;
+};
+__device__ __forceinline__ uint64_t fused_value(uint64_t w, float s0, float s1, float b0, float b1, uint64_t one2) {
+    return f32x2_add_one(f32x2_mul_rn(w, f32x2_pack(s0, s1)), one2, f32x2_pack(b0, b1));
+}
+__device__ __forceinline__ uint64_t fused_pair(uint32_t a, uint32_t b) { return f32x2_pack((float)(int)a, (float)(int)b); }
+__device__ __forceinline__ void fused_code(uint64_t w, const FusedUnitEnv& E, uint32_t& m0, uint32_t& m1) {
+    w = f32x2_add_one(f32x2_mul_rn(w, E.inv2), E.one2, f32x2_pack(0.5f, 0.5f));
+    m0 = code_pattern(__uint_as_float((uint32_t)w), E.hi2);
+    m1 = code_pattern(__uint_as_float((uint32_t)(w >> 32)), E.hi2);
+}
+// The fp32 values of a unit's 16 channels at this thread's pixel, two to a register: wide layers w[2 e + j] = word 4 hf + e of
+// the 32-channel group, its bytes 2 j and 2 j + 1 (channels 8 i + 4 hf + e); narrow ones (all 16 channels in one unit) w[b] =
+// channels b and 8 + b.  RES: 0 none, 1 identity shortcut, 2 held projection.  Straight-line code for each form: a unit is
+// some 200 instructions, and branching through all forms cost ten times their issue time in instruction fetch.
+template <bool NARROW, int RES>
+__device__ __forceinline__ void fused_unit_values(const FusedUnitEnv& E, uint32_t trow, int un, int target, uint64_t (&w)[8]) {
+    const int grp = un >> 1, hf = un & 1;
+    const FusedTerms& T = *E.T;
+    uint32_t resw[8];
+    if constexpr (NARROW) {
+        uint32_t v[16], pv[16];
+        tmem_ld16_issue(trow, v);
+        if constexpr (RES == 2) tmem_ld16_issue(trow + FUSED_HOLD_COL, pv);
+        if constexpr (RES == 1) {
+            const uint8_t* rp = E.res + target * 16;
+            const uint4 a = *reinterpret_cast<const uint4*>(rp), b = *reinterpret_cast<const uint4*>(rp + E.cap_out * 16);
+            resw[0] = a.x; resw[1] = a.y; resw[2] = a.z; resw[3] = a.w;
+            resw[4] = b.x; resw[5] = b.y; resw[6] = b.z; resw[7] = b.w;
+        }
+        tmem_ld16_wait(v);
+        if constexpr (RES == 2) tmem_ld16_wait(pv);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 s4 = *reinterpret_cast<const float4*>(&T.cs[4 * q]), b4 = *reinterpret_cast<const float4*>(&T.cb[4 * q]);
+            w[2 * q] = fused_value(f32x2_mul_rn(fused_pair(v[2 * q], v[8 + 2 * q]), E.S2), s4.x, s4.y, b4.x, b4.y, E.one2);
+            w[2 * q + 1] = fused_value(f32x2_mul_rn(fused_pair(v[2 * q + 1], v[9 + 2 * q]), E.S2), s4.z, s4.w, b4.z, b4.w, E.one2);
+            if constexpr (RES == 2) {
+                const float4 ps = *reinterpret_cast<const float4*>(&T.pcs[4 * q]), pb = *reinterpret_cast<const float4*>(&T.pcb[4 * q]);
+                w[2 * q] = f32x2_add_one(w[2 * q], E.one2, fused_value(f32x2_mul_rn(fused_pair(pv[2 * q], pv[8 + 2 * q]), E.PS2), ps.x, ps.y, pb.x, pb.y, E.one2));
+                w[2 * q + 1] = f32x2_add_one(w[2 * q + 1], E.one2, fused_value(f32x2_mul_rn(fused_pair(pv[2 * q + 1], pv[9 + 2 * q]), E.PS2), ps.z, ps.w, pb.z, pb.w, E.one2));
+            }
+        }
+        if constexpr (RES == 1) {
+#pragma unroll
+            for (int b = 0; b < 8; ++b)
+                w[b] = f32x2_add_one(w[b], E.one2, f32x2_mul_rn(E.rs2, f32x2_pack(byte_to_float(resw[b], 0), byte_to_float(resw[b], 1))));
+        }
+    } else {
+        uint32_t v[4][4], pv[4][4];
+        const uint32_t tc = trow + (uint32_t)(32 * grp + 4 * hf);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tmem_ld4_issue(tc + 8u * i, v[i]);
+        if constexpr (RES == 2) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) tmem_ld4_issue(tc + FUSED_HOLD_COL + 8u * i, pv[i]);
+        }
+        if constexpr (RES == 1) {
+            const uint4 a = *reinterpret_cast<const uint4*>(E.res + grp * E.cap_out * 32 + hf * E.cap_out * 16 + target * 16);
+            resw[0] = a.x; resw[1] = a.y; resw[2] = a.z; resw[3] = a.w;
+        }
+        tmem_ld4_wait(v[0], v[1], v[2], v[3]);
+        if constexpr (RES == 2) tmem_ld4_wait(pv[0], pv[1], pv[2], pv[3]);
+        const int t0 = grp * 32 + 16 * hf;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float4 s4 = *reinterpret_cast<const float4*>(&T.cs[t0 + 4 * e]), b4 = *reinterpret_cast<const float4*>(&T.cb[t0 + 4 * e]);
+            w[2 * e] = fused_value(f32x2_mul_rn(fused_pair(v[0][e], v[1][e]), E.S2), s4.x, s4.y, b4.x, b4.y, E.one2);
+            w[2 * e + 1] = fused_value(f32x2_mul_rn(fused_pair(v[2][e], v[3][e]), E.S2), s4.z, s4.w, b4.z, b4.w, E.one2);
+            if constexpr (RES == 2) {
+                const float4 ps = *reinterpret_cast<const float4*>(&T.pcs[t0 + 4 * e]), pb = *reinterpret_cast<const float4*>(&T.pcb[t0 + 4 * e]);
+                w[2 * e] = f32x2_add_one(w[2 * e], E.one2, fused_value(f32x2_mul_rn(fused_pair(pv[0][e], pv[1][e]), E.PS2), ps.x, ps.y, pb.x, pb.y, E.one2));
+                w[2 * e + 1] = f32x2_add_one(w[2 * e + 1], E.one2, fused_value(f32x2_mul_rn(fused_pair(pv[2][e], pv[3][e]), E.PS2), ps.z, ps.w, pb.z, pb.w, E.one2));
+            }
+            if constexpr (RES == 1) {
+                w[2 * e] = f32x2_add_one(w[2 * e], E.one2, f32x2_mul_rn(E.rs2, f32x2_pack(byte_to_float(resw[e], 0), byte_to_float(resw[e], 1))));
+                w[2 * e + 1] = f32x2_add_one(w[2 * e + 1], E.one2, f32x2_mul_rn(E.rs2, f32x2_pack(byte_to_float(resw[e], 2), byte_to_float(resw[e], 3))));
+            }
+        }
+    }
+}
+// First and second channel of register i of a unit.
+__device__ __forceinline__ int fused_channel(bool narrow, int un, int i) {
+    return narrow ? i : 32 * (un >> 1) + 4 * (un & 1) + (i >> 1) + 16 * (i & 1);       // (the second one is 8 further)
+}
+// Codes of a unit to its half row of the destination strip (both half rows when narrow).
+template <bool NARROW, int RES>
+__device__ __forceinline__ void fused_unit_codes(const FusedUnitEnv& E, uint32_t trow, int un, int target, bool valid, bool in_frame,
+                                                 uint8_t* trace) {
+    uint64_t w[8];
+    fused_unit_values<NARROW, RES>(E, trow, un, target, w);
+    const int grp = un >> 1, hf = un & 1;
+    uint8_t* at = E.dst + grp * E.cap_out * 32 + hf * E.cap_out * 16 + target * 16;
+    const uint32_t z = valid ? 0xFFFFFFFFu : 0u;
+    uint32_t words[8];
+    if constexpr (NARROW) {
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            uint32_t m0, m1;
+            fused_code(w[b], E, m0, m1);
+            words[b] = __byte_perm(m0, m1, 0x0040) & z & 0xFFFFu;
+        }
+        if (E.c_out & 15) {                              // channels past c_out
+#pragma unroll
+            for (int b = 0; b < 8; ++b) words[b] &= (b < E.c_out ? 0xFFu : 0u) | (8 + b < E.c_out ? 0xFF00u : 0u);
+        }
+        if (in_frame) {
+            *reinterpret_cast<uint4*>(at) = make_uint4(words[0], words[1], words[2], words[3]);
+            *reinterpret_cast<uint4*>(at + E.cap_out * 16) = make_uint4(words[4], words[5], words[6], words[7]);
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            uint32_t m[4];
+            fused_code(w[2 * e], E, m[0], m[1]);
+            fused_code(w[2 * e + 1], E, m[2], m[3]);
+            words[e] = join_codes(m) & z;
+        }
+        if (E.c_out & 31) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int c = 32 * grp + 4 * hf + e;
+                words[e] &= (c < E.c_out ? 0xFFu : 0u) | (c + 8 < E.c_out ? 0xFF00u : 0u) | (c + 16 < E.c_out ? 0xFF0000u : 0u) | (c + 24 < E.c_out ? 0xFF000000u : 0u);
+            }
+        }
+        if (in_frame) *reinterpret_cast<uint4*>(at) = make_uint4(words[0], words[1], words[2], words[3]);
+    }
+    if (trace && valid) {
+#pragma unroll 1
+        for (int i = 0; i < 16; ++i) {
+            const int e = NARROW ? i & 7 : i & 3, byte = NARROW ? i >> 3 : i >> 2, c = NARROW ? 8 * byte + e : 32 * grp + 8 * byte + 4 * hf + e;
+            if (c < E.c_out) trace[c] = at[(e >> 2) * E.cap_out * 16 + (e & 3) * 4 + byte];
+        }
+    }
+}
+// fp32 results of the last layer's unit for pooling: [pixel][c_out].
+template <bool NARROW, int RES>
+__device__ __forceinline__ void fused_unit_pool(const FusedUnitEnv& E, uint32_t trow, int un, int target, bool valid, bool relu, float* row) {
+    uint64_t w[8];
+    fused_unit_values<NARROW, RES>(E, trow, un, target, w);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        float y0 = __uint_as_float((uint32_t)w[i]), y1 = __uint_as_float((uint32_t)(w[i] >> 32));
+        if (relu) { y0 = y0 > 0.0f ? y0 : 0.0f; y1 = y1 > 0.0f ? y1 : 0.0f; }
+        const int c = fused_channel(NARROW, un, i);
+        if (valid && c < E.c_out) row[c] = y0;
+        if (valid && c + 8 < E.c_out) row[c + 8] = y1;
+    }
 }
 
 __global__ void __launch_bounds__(FUSED_THREADS, 1)
@@ -134,24 +296,28 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                      "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
-    // all strips start as zeros (padding positions are never written with anything else)
-    for (int i = tid; i < 3 * FUSED_ACT_BYTES / 16; i += FUSED_THREADS) reinterpret_cast<uint4*>(acts)[i] = make_uint4(0, 0, 0, 0);
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
-    // ---- the image: u8 NHWC, 3 channels -> bytes of strip 0 in the padded frame (channel c is byte 4c of word 0)
-    {
-        const int Wp = img_w + 2;
-        const uint8_t* src = images + (size_t)img * img_h * img_w * 3;
-        for (int pix = tid; pix < img_h * img_w; pix += FUSED_THREADS) {
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    if (warp != FUSED_LOADER_WARP) {                             // (the loader goes ahead)
+        constexpr int NT = FUSED_THREADS - 32;
+        const int i0 = warp > FUSED_LOADER_WARP ? tid - 32 : tid;
+        // all strips start as zeros (padding positions are never written with anything else)
+        for (int i = i0; i < 3 * FUSED_ACT_BYTES / 16; i += NT) reinterpret_cast<uint4*>(acts)[i] = make_uint4(0, 0, 0, 0);
+        asm volatile("bar.sync 1, %0;\n" ::"n"(FUSED_THREADS - 32) : "memory");
+        // the image: u8 NHWC, 3 channels -> bytes of strip 0 in the padded frame (channel c is byte 4c of word 0)
+        const int Wp = img_w + 2, pixels = img_h * img_w;
+        const uint8_t* src = images + (size_t)img * pixels * 3;
+#pragma unroll 2
+        for (int pix = i0; pix < pixels; pix += NT) {
             const int h = pix / img_w, w = pix - h * img_w;
             const uint32_t r = src[pix * 3], g = src[pix * 3 + 1], b = src[pix * 3 + 2];
             uint32_t* dst = reinterpret_cast<uint32_t*>(strip_ptr(acts, 0) + ((h + 1) * Wp + (w + 1)) * 16);
             dst[0] = r; dst[1] = g; dst[2] = b;                   // words 0..2 of the first 16-byte half: channels 0, 1, 2
         }
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        asm volatile("bar.sync 1, %0;\n" ::"n"(FUSED_THREADS - 32) : "memory");
     }
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem_base = tmem_slot;
     float* pool_scratch = reinterpret_cast<float*>(strip_ptr(acts, 0));      // [pixels][c_out] of the last layer
 
@@ -207,43 +373,53 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                 if (!mbar_wait_bounded_warp(&copy_ready, (uint32_t)(n_copies & 1), abortp, limit)) break;
                 ++n_copies;
             }
-            const int cap_in = strip_cap(L.c_in);
+            const int cap_in = uni(strip_cap(L.c_in));
             const uint64_t da0 = umma_desc_interleaved(smem_u32(strip_ptr(acts, L.k == 1 ? L.dst : L.src)), (uint32_t)(cap_in * 16));
             const uint64_t db0 = umma_desc_sw32(smem_u32(wbuf + (li & 1) * FUSED_W_BYTES));
-            const uint32_t da_hi = (uint32_t)(da0 >> 32), db_hi = (uint32_t)(db0 >> 32);
-            const uint32_t idesc = umma_idesc_i8(g.co16), step = (uint32_t)((g.co16 * 32) >> 4);
-            const int k = L.k, cw = g.cw;
+            const uint32_t da_lo = uni((uint32_t)da0), da_hi = uni((uint32_t)(da0 >> 32)), db_lo = uni((uint32_t)db0), db_hi = uni((uint32_t)(db0 >> 32));
+            const uint32_t idesc = uni(umma_idesc_i8(g.co16)), step = uni((uint32_t)((g.co16 * 32) >> 4));
+            const int k = uni(L.k), cw = uni(g.cw), tiles = uni(g.tiles), Wf = uni(g.Wf), hold = uni(L.hold);
+            const uint32_t tm0 = uni(tmem_base + (uint32_t)(L.hold ? FUSED_HOLD_COL : 0)), tm_step = uni((uint32_t)g.acc_stride);
             int waited = 0;                              // tiles of the layer before that are known to be finished
             auto wait_tiles = [&](int upto) {
                 for (; waited < upto; ++waited)
                     if (!mbar_wait_bounded_warp(&ep_done[waited], ((par >> waited) & 1u) ^ 1u, abortp, limit)) return false;
                 return true;
             };
-            for (int t = k_iss; t < g.tiles; t += FUSED_ISSUERS) {
-                const int need = wave ? min(prev_tiles, (t * UMMA_M + UMMA_M + g.Wf) / UMMA_M + 1) : prev_tiles;
+            for (int t = k_iss; t < tiles; t += FUSED_ISSUERS) {
+                const int need = wave ? min(prev_tiles, (t * UMMA_M + UMMA_M + Wf) / UMMA_M + 1) : prev_tiles;
                 if (!wait_tiles(need)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const uint32_t tm = tmem_base + (uint32_t)((L.hold ? FUSED_HOLD_COL : 0) + t * g.acc_stride);
+                const uint32_t tm = tm0 + (uint32_t)t * tm_step;
+                const uint32_t a_tile = da_lo + (uint32_t)(t * UMMA_M);
                 uint32_t accu = 0u;
-                for (int wd = 0; wd < cw; ++wd) {
-                    uint32_t a_row = (uint32_t)da0 + (uint32_t)(wd * cap_in * 2 + t * UMMA_M + (k == 3 ? 0 : g.Wf + 1));
-                    uint32_t b_lo = (uint32_t)db0 + step * (uint32_t)wd;      // weight tiles are ordered [tap][word]
-                    for (int r = 0; r < k; ++r, a_row += (uint32_t)g.Wf) {
-                        for (int s = 0; s < k; ++s, b_lo += step * (uint32_t)cw) {
-                            umma_i8_split(leader, tm, a_row + (uint32_t)s, da_hi, b_lo, db_hi, idesc, accu);
-                            accu = 1u;
+                if (k == 3) {
+                    for (int wd = 0; wd < cw; ++wd) {
+                        uint32_t a_row = a_tile + (uint32_t)(wd * cap_in * 2);
+                        uint32_t b = db_lo + step * (uint32_t)wd;             // weight tiles are ordered [tap][word]
+                        const uint32_t bs = step * (uint32_t)cw;
+#pragma unroll
+                        for (int r = 0; r < 3; ++r, a_row += (uint32_t)Wf) {
+#pragma unroll
+                            for (int s = 0; s < 3; ++s, b += bs) {
+                                umma_i8_split(leader, tm, a_row + (uint32_t)s, da_hi, b, db_hi, idesc, accu);
+                                accu = 1u;
+                            }
                         }
                     }
+                } else {
+                    for (int wd = 0; wd < cw; ++wd, accu = 1u)
+                        umma_i8_split(leader, tm, a_tile + (uint32_t)(wd * cap_in * 2 + Wf + 1), da_hi, db_lo + step * (uint32_t)wd, db_hi, idesc, accu);
                 }
-                if (!L.hold) umma_commit_pred(leader, &acc_full[t]);
+                if (!hold) umma_commit_pred(leader, &acc_full[t]);
             }
             if (!ok || !wait_tiles(prev_tiles)) break;   // (every phase of these barriers is waited for, so that parities stay in step)
             if (L.hold) {
                 umma_commit_pred(leader, &hold_full);
             } else {
                 prev = li;
-                prev_tiles = g.tiles;
-                par ^= (1u << g.tiles) - 1u;
+                prev_tiles = tiles;
+                par ^= (1u << tiles) - 1u;
             }
             umma_commit_pred(leader, &w_free[li & 1]);
             __syncwarp();
@@ -255,7 +431,6 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
     } else if (warp < FUSED_EPI_WARPS) {
         // =========================== epilogue ===========================
         const int quarter = warp & 3, quad = warp >> 2;
-        const float half = 0.5f;
         uint32_t par = 0u;
         int turn = 0, n_sync = 0, n_hold = 0;            // turn: units dealt so far, modulo 4
         bool ok = true;
@@ -298,158 +473,65 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                 if (!mbar_wait_bounded_warp(&hold_full, (uint32_t)(n_hold & 1), abortp, limit)) break;
                 ++n_hold;
             } else {
-                const int Wp_out = g.Wo + 2, res = L.res, units = g.units;
-                const bool narrow = L.c_out <= 16, to_pool = L.dst < 0, relu = L.relu != 0;
-                const float hi2 = (float)(2 * ((1 << L.out_bits) - 1) + 1);
-                const uint64_t S2 = f32x2_pack(L.S, L.S), one2 = f32x2_pack(one, one), inv2 = f32x2_pack(L.out_inv_step, L.out_inv_step);
-                const uint64_t half2 = f32x2_pack(half, half), rs2 = f32x2_pack(L.res_step, L.res_step);
-                const float PS = res == 2 ? s_rec[(li - 1) & (FUSED_RING - 1)].S : 0.0f;
-                const uint64_t PS2 = f32x2_pack(PS, PS);
-                const int total = g.tiles * units;
+                const int units = g.units, ushift = units == 1 ? 0 : (units == 2 ? 1 : 2), Wp_out = g.Wo + 2;
+                const bool to_pool = L.dst < 0, relu = L.relu != 0, two = L.stride == 2;
+                const int Wf = g.Wf, Ho = g.Ho, Wo = g.Wo, frame = g.frame;
+                const float rcp_w = __frcp_rn((float)Wf);
+                FusedUnitEnv E;
+                E.S2 = f32x2_pack(L.S, L.S);
+                E.rs2 = f32x2_pack(L.res_step, L.res_step);
+                E.one2 = f32x2_pack(one, one);
+                E.inv2 = f32x2_pack(L.out_inv_step, L.out_inv_step);
+                E.hi2 = (float)(2 * ((1 << L.out_bits) - 1) + 1);
+                const float PS = L.res == 2 ? s_rec[(li - 1) & (FUSED_RING - 1)].S : 0.0f;
+                E.PS2 = f32x2_pack(PS, PS);
+                E.c_out = L.c_out;
+                E.cap_out = cap_out;
+                E.dst = dst_strip;
+                E.res = strip_ptr(acts, L.res_buf);
+                E.T = &T;
+                uint8_t* tr = trace && L.trace_off >= 0 ? trace + (size_t)img * trace_stride + L.trace_off : nullptr;
+                const int form = uni((L.c_out <= 16 ? 3 : 0) + L.res + (to_pool ? 6 : 0));
+                const int total = g.tiles << ushift;
                 if (L.src == (to_pool ? 0 : L.dst)) {    // writes over its own input: only after the last MMA
                     for (int t = 0; t < g.tiles && ok; ++t) ok = mbar_wait_bounded_warp(&acc_full[t], (par >> t) & 1u, abortp, limit);
                     if (!ok) break;
                 }
                 for (int u = 0; u < total; ++u) {
-                    const int t = u / units, un = u - t * units;
+                    const int t = u >> ushift, un = u & (units - 1);
                     if (un == 0 && !mbar_wait_bounded_warp(&acc_full[t], (par >> t) & 1u, abortp, limit)) { ok = false; break; }
                     if (((turn + u) & 3) != quad) continue;
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     const int f = t * UMMA_M + quarter * 32 + lane;
-                    const int hp = f / g.Wf, wp = f - hp * g.Wf;
+                    const int hp = __float2int_rd(__fmul_rn((float)f + 0.5f, rcp_w)), wp = f - hp * Wf;   // (exact: f < 2^20)
                     // does this frame row have an output, and where does it go in the destination frame
-                    bool valid = f < g.frame;
-                    int ho = hp, wo = wp;
-                    if (L.stride == 2) { valid = valid && !(hp & 1) && !(wp & 1); ho = hp >> 1; wo = wp >> 1; }
-                    valid = valid && ho < g.Ho && wo < g.Wo;
-                    const int target = L.stride == 2 ? (ho + 1) * Wp_out + wo + 1 : f + g.Wf + 1;
-                    const bool in_frame = f < g.frame && (L.stride == 1 || valid);   // stride 1 also writes the zeros of the padding
+                    const int ho = two ? hp >> 1 : hp, wo = two ? wp >> 1 : wp;
+                    const bool valid = f < frame && !(two && ((hp | wp) & 1)) && ho < Ho && wo < Wo;
+                    const int target = two ? (ho + 1) * Wp_out + wo + 1 : f + Wf + 1;
+                    const bool in_frame = f < frame && (!two || valid);              // stride 1 also writes the zeros of the padding
                     if (__any_sync(0xffffffffu, in_frame)) {
                         const uint32_t trow = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(t * g.acc_stride);
-                        // word e of this unit: channels ch(e, 0 .. 3) as its bytes.  Wide: word 4 hf + e of the 32-channel
-                        // group; narrow (all 16 channels in one unit): words 0 .. 7, channels b and 8 + b
-                        const int grp = un >> 1, hf = un & 1;
-                        uint32_t words[8];
-                        uint32_t resw[8];
-                        uint8_t* at = dst_strip + grp * cap_out * 32 + target * 16;
-                        const uint8_t* rp = strip_ptr(acts, L.res_buf) + grp * cap_out * 32 + target * 16;
-                        auto value = [&](uint64_t w, uint64_t a, uint64_t b) { return f32x2_add_one(f32x2_mul_rn(w, a), one2, b); };
-                        auto code = [&](uint64_t w, uint32_t& m0, uint32_t& m1) {
-                            w = f32x2_add_one(f32x2_mul_rn(w, inv2), one2, half2);
-                            m0 = code_pattern(__uint_as_float((uint32_t)w), hi2);
-                            m1 = code_pattern(__uint_as_float((uint32_t)(w >> 32)), hi2);
-                        };
-                        auto pool = [&](uint64_t w, int c) {                  // two channels 8 apart
-                            float y0 = __uint_as_float((uint32_t)w), y1 = __uint_as_float((uint32_t)(w >> 32));
-                            if (relu) { y0 = y0 > 0.0f ? y0 : 0.0f; y1 = y1 > 0.0f ? y1 : 0.0f; }
-                            if (valid && c < L.c_out) pool_scratch[(ho * g.Wo + wo) * L.c_out + c] = y0;
-                            if (valid && c + 8 < L.c_out) pool_scratch[(ho * g.Wo + wo) * L.c_out + c + 8] = y1;
-                        };
-                        auto pair = [](uint32_t a, uint32_t b) { return f32x2_pack((float)(int)a, (float)(int)b); };
-                        if (narrow) {
-                            uint32_t v[16], pv[16];
-                            tmem_ld16_issue(trow, v);
-                            if (res == 2) tmem_ld16_issue(trow + FUSED_HOLD_COL, pv);
-                            if (res == 1) {
-                                const uint4 a = *reinterpret_cast<const uint4*>(rp), b = *reinterpret_cast<const uint4*>(rp + cap_out * 16);
-                                resw[0] = a.x; resw[1] = a.y; resw[2] = a.z; resw[3] = a.w;
-                                resw[4] = b.x; resw[5] = b.y; resw[6] = b.z; resw[7] = b.w;
-                            }
-                            tmem_ld16_wait(v);
-                            if (res == 2) tmem_ld16_wait(pv);
-#pragma unroll
-                            for (int b = 0; b < 8; ++b) {
-                                const float2 s2 = *reinterpret_cast<const float2*>(&T.cs[2 * b]), b2 = *reinterpret_cast<const float2*>(&T.cb[2 * b]);
-                                uint64_t w = value(f32x2_mul_rn(pair(v[b], v[8 + b]), S2), f32x2_pack(s2.x, s2.y), f32x2_pack(b2.x, b2.y));
-                                if (res == 2) {
-                                    const float2 ps = *reinterpret_cast<const float2*>(&T.pcs[2 * b]), pb = *reinterpret_cast<const float2*>(&T.pcb[2 * b]);
-                                    w = f32x2_add_one(w, one2, value(f32x2_mul_rn(pair(pv[b], pv[8 + b]), PS2), f32x2_pack(ps.x, ps.y), f32x2_pack(pb.x, pb.y)));
-                                }
-                                if (res == 1) w = f32x2_add_one(w, one2, f32x2_mul_rn(rs2, f32x2_pack(byte_to_float(resw[b], 0), byte_to_float(resw[b], 1))));
-                                if (to_pool) {
-                                    pool(w, b);
-                                } else {
-                                    uint32_t m0, m1;
-                                    code(w, m0, m1);
-                                    words[b] = (__byte_perm(m0, m1, 0x0040) & 0xFFFFu) & ((b < L.c_out ? 0xFFu : 0u) | (8 + b < L.c_out ? 0xFF00u : 0u));
-                                }
-                            }
-                        } else {
-                            uint32_t v[4][4], pv[4][4];
-                            const uint32_t tc = trow + (uint32_t)(32 * grp + 4 * hf);
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) tmem_ld4_issue(tc + 8u * i, v[i]);
-                            if (res == 2) {
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) tmem_ld4_issue(tc + FUSED_HOLD_COL + 8u * i, pv[i]);
-                            }
-                            if (res == 1) {
-                                const uint4 a = *reinterpret_cast<const uint4*>(rp + hf * cap_out * 16);
-                                resw[0] = a.x; resw[1] = a.y; resw[2] = a.z; resw[3] = a.w;
-                            }
-                            tmem_ld4_wait(v[0], v[1], v[2], v[3]);
-                            if (res == 2) tmem_ld4_wait(pv[0], pv[1], pv[2], pv[3]);
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const int ti = grp * 32 + (4 * hf + e) * 4, c = 32 * grp + 4 * hf + e;
-                                const float4 s4 = *reinterpret_cast<const float4*>(&T.cs[ti]), b4 = *reinterpret_cast<const float4*>(&T.cb[ti]);
-                                uint64_t w0 = value(f32x2_mul_rn(pair(v[0][e], v[1][e]), S2), f32x2_pack(s4.x, s4.y), f32x2_pack(b4.x, b4.y));
-                                uint64_t w1 = value(f32x2_mul_rn(pair(v[2][e], v[3][e]), S2), f32x2_pack(s4.z, s4.w), f32x2_pack(b4.z, b4.w));
-                                if (res == 2) {
-                                    const float4 ps = *reinterpret_cast<const float4*>(&T.pcs[ti]), pb = *reinterpret_cast<const float4*>(&T.pcb[ti]);
-                                    w0 = f32x2_add_one(w0, one2, value(f32x2_mul_rn(pair(pv[0][e], pv[1][e]), PS2), f32x2_pack(ps.x, ps.y), f32x2_pack(pb.x, pb.y)));
-                                    w1 = f32x2_add_one(w1, one2, value(f32x2_mul_rn(pair(pv[2][e], pv[3][e]), PS2), f32x2_pack(ps.z, ps.w), f32x2_pack(pb.z, pb.w)));
-                                }
-                                if (res == 1) {
-                                    w0 = f32x2_add_one(w0, one2, f32x2_mul_rn(rs2, f32x2_pack(byte_to_float(resw[e], 0), byte_to_float(resw[e], 1))));
-                                    w1 = f32x2_add_one(w1, one2, f32x2_mul_rn(rs2, f32x2_pack(byte_to_float(resw[e], 2), byte_to_float(resw[e], 3))));
-                                }
-                                if (to_pool) {
-                                    pool(w0, c);
-                                    pool(w1, c + 16);
-                                } else {
-                                    uint32_t m[4];
-                                    code(w0, m[0], m[1]);
-                                    code(w1, m[2], m[3]);
-                                    words[e] = join_codes(m);
-                                    if (L.c_out & 31) {                       // channels past c_out
-                                        const uint32_t keep = (c < L.c_out ? 0xFFu : 0u) | (c + 8 < L.c_out ? 0xFF00u : 0u) |
-                                                              (c + 16 < L.c_out ? 0xFF0000u : 0u) | (c + 24 < L.c_out ? 0xFF000000u : 0u);
-                                        words[e] &= keep;
-                                    }
-                                }
-                            }
-                        }
-                        if (!to_pool) {
-                            if (in_frame) {
-                                const uint32_t z = valid ? 0xFFFFFFFFu : 0u;
-                                const uint4 a = make_uint4(words[0] & z, words[1] & z, words[2] & z, words[3] & z);
-                                if (narrow) {
-                                    *reinterpret_cast<uint4*>(at) = a;
-                                    *reinterpret_cast<uint4*>(at + cap_out * 16) = make_uint4(words[4] & z, words[5] & z, words[6] & z, words[7] & z);
-                                } else {
-                                    *reinterpret_cast<uint4*>(at + hf * cap_out * 16) = a;
-                                }
-                            }
-                            if (trace && L.trace_off >= 0 && valid) {
-                                uint8_t* tp = trace + (size_t)img * trace_stride + L.trace_off + (size_t)(ho * g.Wo + wo) * L.c_out;
-                                const int nwords = narrow ? 8 : 4;
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) {
-                                    if (e >= nwords) break;
-#pragma unroll
-                                    for (int i = 0; i < 4; ++i) {
-                                        const int c = (narrow ? 8 * i + e : 32 * grp + 8 * i + 4 * hf + e);
-                                        if (c < L.c_out && (!narrow || i < 2)) tp[c] = (uint8_t)(words[e] >> (8 * i));
-                                    }
-                                }
-                            }
+                        uint8_t* tp = tr ? tr + (size_t)(ho * Wo + wo) * L.c_out : nullptr;
+                        float* pr = pool_scratch + (ho * Wo + wo) * L.c_out;
+                        switch (form) {
+                            case 0: fused_unit_codes<false, 0>(E, trow, un, target, valid, in_frame, tp); break;
+                            case 1: fused_unit_codes<false, 1>(E, trow, un, target, valid, in_frame, tp); break;
+                            case 2: fused_unit_codes<false, 2>(E, trow, un, target, valid, in_frame, tp); break;
+                            case 3: fused_unit_codes<true, 0>(E, trow, un, target, valid, in_frame, tp); break;
+                            case 4: fused_unit_codes<true, 1>(E, trow, un, target, valid, in_frame, tp); break;
+                            case 5: fused_unit_codes<true, 2>(E, trow, un, target, valid, in_frame, tp); break;
+                            case 6: fused_unit_pool<false, 0>(E, trow, un, target, valid, relu, pr); break;
+                            case 7: fused_unit_pool<false, 1>(E, trow, un, target, valid, relu, pr); break;
+                            case 8: fused_unit_pool<false, 2>(E, trow, un, target, valid, relu, pr); break;
+                            case 9: fused_unit_pool<true, 0>(E, trow, un, target, valid, relu, pr); break;
+                            case 10: fused_unit_pool<true, 1>(E, trow, un, target, valid, relu, pr); break;
+                            default: fused_unit_pool<true, 2>(E, trow, un, target, valid, relu, pr); break;
                         }
                     }
                     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) mbar_arrive_n(&ep_done[t], (uint32_t)(4 / units));
+                    if (lane == 0) mbar_arrive_n(&ep_done[t], 4u >> ushift);
                 }
                 turn = (turn + total) & 3;
                 par ^= (1u << g.tiles) - 1u;

@@ -18,6 +18,10 @@
 // tile t need the codes of tiles 0 .. t + 1 of the layer before, and no strip or accumulator is overwritten earlier than
 // that same order allows; where the geometry changes, the next layer waits for all tiles.  (With the phases of a layer one
 // after the other between block barriers a layer took 5.5 us whatever its size.)
+// Layers with at most 16 input channels would leave half of every MMA's 32 reduction bytes empty: their strips hold 16 bytes
+// a pixel, and an MMA takes two taps -- the distance between the two 16-byte halves of an operand row is a descriptor
+// field, here the distance between the taps.  The loader re-lays their weights accordingly (5 MMAs a tile instead of 9; an
+// MMA costs 41-50 clocks of operand reads and issue however narrow it is).
 // A unit is the 16 channels that fill one 16-byte half of a pixel's row (channels 8 i + 4 h + e of a 32-channel word), so
 // its codes leave in one 16-byte store and its identity shortcut is one 16-byte load.
 // Stride-2 3x3 layers are computed at stride 1 and subsampled in the epilogue (4x the MMAs of two or three
@@ -39,6 +43,7 @@ constexpr int FUSED_ACT_PIX = 1360;                    // pixels an activation s
 constexpr int FUSED_ACT_BYTES = FUSED_ACT_PIX * 32;    // one 32-channel word
 constexpr int FUSED_W_BYTES = 37 * 1024;               // largest weight image (3x3 64->64)
 constexpr int FUSED_SMEM = 3 * FUSED_ACT_BYTES + 2 * FUSED_W_BYTES + 1024;
+constexpr int FUSED_PACKED_W = 20 * 1024;             // where a narrow layer's re-laid weights lie in its weight buffer (raw: <= 18.4 KB)
 constexpr int FUSED_HOLD_COL = 320;                    // accumulator columns of a held projection
 
 using FusedLayer = ebs_fused_layer;
@@ -107,6 +112,11 @@ __device__ __forceinline__ uint64_t fused_value(uint64_t w, float s0, float s1, 
     return f32x2_add_one(f32x2_mul_rn(w, f32x2_pack(s0, s1)), one2, f32x2_pack(b0, b1));
 }
 __device__ __forceinline__ uint64_t fused_pair(uint32_t a, uint32_t b) { return f32x2_pack((float)(int)a, (float)(int)b); }
+// Bytes 2 j and 2 j + 1 of a register as fp32, exactly (2^23 + byte, minus 2^23).
+__device__ __forceinline__ uint64_t fused_byte_pair(uint32_t r, int j, uint64_t one2) {
+    const float lo = __uint_as_float(__byte_perm(r, 0x4B000000u, 0x7540u + 2u * (uint32_t)j)), hi = __uint_as_float(__byte_perm(r, 0x4B000000u, 0x7541u + 2u * (uint32_t)j));
+    return f32x2_add_one(f32x2_pack(lo, hi), one2, f32x2_pack(-8388608.0f, -8388608.0f));
+}
 __device__ __forceinline__ void fused_code(uint64_t w, const FusedUnitEnv& E, uint32_t& m0, uint32_t& m1) {
     w = f32x2_add_one(f32x2_mul_rn(w, E.inv2), E.one2, f32x2_pack(0.5f, 0.5f));
     m0 = code_pattern(__uint_as_float((uint32_t)w), E.hi2);
@@ -126,10 +136,8 @@ __device__ __forceinline__ void fused_unit_values(const FusedUnitEnv& E, uint32_
         tmem_ld16_issue(trow, v);
         if constexpr (RES == 2) tmem_ld16_issue(trow + FUSED_HOLD_COL, pv);
         if constexpr (RES == 1) {
-            const uint8_t* rp = E.res + target * 16;
-            const uint4 a = *reinterpret_cast<const uint4*>(rp), b = *reinterpret_cast<const uint4*>(rp + E.cap_out * 16);
+            const uint4 a = *reinterpret_cast<const uint4*>(E.res + target * 16);
             resw[0] = a.x; resw[1] = a.y; resw[2] = a.z; resw[3] = a.w;
-            resw[4] = b.x; resw[5] = b.y; resw[6] = b.z; resw[7] = b.w;
         }
         tmem_ld16_wait(v);
         if constexpr (RES == 2) tmem_ld16_wait(pv);
@@ -146,8 +154,7 @@ __device__ __forceinline__ void fused_unit_values(const FusedUnitEnv& E, uint32_
         }
         if constexpr (RES == 1) {
 #pragma unroll
-            for (int b = 0; b < 8; ++b)
-                w[b] = f32x2_add_one(w[b], E.one2, f32x2_mul_rn(E.rs2, f32x2_pack(byte_to_float(resw[b], 0), byte_to_float(resw[b], 1))));
+            for (int b = 0; b < 8; ++b) w[b] = f32x2_add_one(w[b], E.one2, f32x2_mul_rn(E.rs2, fused_byte_pair(resw[b & 3], b >> 2, E.one2)));
         }
     } else {
         uint32_t v[4][4], pv[4][4];
@@ -176,8 +183,8 @@ __device__ __forceinline__ void fused_unit_values(const FusedUnitEnv& E, uint32_
                 w[2 * e + 1] = f32x2_add_one(w[2 * e + 1], E.one2, fused_value(f32x2_mul_rn(fused_pair(pv[2][e], pv[3][e]), E.PS2), ps.z, ps.w, pb.z, pb.w, E.one2));
             }
             if constexpr (RES == 1) {
-                w[2 * e] = f32x2_add_one(w[2 * e], E.one2, f32x2_mul_rn(E.rs2, f32x2_pack(byte_to_float(resw[e], 0), byte_to_float(resw[e], 1))));
-                w[2 * e + 1] = f32x2_add_one(w[2 * e + 1], E.one2, f32x2_mul_rn(E.rs2, f32x2_pack(byte_to_float(resw[e], 2), byte_to_float(resw[e], 3))));
+                w[2 * e] = f32x2_add_one(w[2 * e], E.one2, f32x2_mul_rn(E.rs2, fused_byte_pair(resw[e], 0, E.one2)));
+                w[2 * e + 1] = f32x2_add_one(w[2 * e + 1], E.one2, f32x2_mul_rn(E.rs2, fused_byte_pair(resw[e], 1, E.one2)));
             }
         }
     }
@@ -186,7 +193,7 @@ __device__ __forceinline__ void fused_unit_values(const FusedUnitEnv& E, uint32_
 __device__ __forceinline__ int fused_channel(bool narrow, int un, int i) {
     return narrow ? i : 32 * (un >> 1) + 4 * (un & 1) + (i >> 1) + 16 * (i & 1);       // (the second one is 8 further)
 }
-// Codes of a unit to its half row of the destination strip (both half rows when narrow).
+// Codes of a unit to its 16 bytes of a pixel in the destination strip.
 template <bool NARROW, int RES>
 __device__ __forceinline__ void fused_unit_codes(const FusedUnitEnv& E, uint32_t trow, int un, int target, bool valid, bool in_frame,
                                                  uint8_t* trace) {
@@ -195,21 +202,19 @@ __device__ __forceinline__ void fused_unit_codes(const FusedUnitEnv& E, uint32_t
     const int grp = un >> 1, hf = un & 1;
     uint8_t* at = E.dst + grp * E.cap_out * 32 + hf * E.cap_out * 16 + target * 16;
     const uint32_t z = valid ? 0xFFFFFFFFu : 0u;
-    uint32_t words[8];
-    if constexpr (NARROW) {
+    uint32_t words[4];
+    if constexpr (NARROW) {                              // 16 bytes a pixel: word j = channels j, 8 + j, 4 + j, 12 + j
 #pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            uint32_t m0, m1;
-            fused_code(w[b], E, m0, m1);
-            words[b] = __byte_perm(m0, m1, 0x0040) & z & 0xFFFFu;
+        for (int e = 0; e < 4; ++e) {
+            uint32_t m[4];
+            fused_code(w[e], E, m[0], m[1]);
+            fused_code(w[4 + e], E, m[2], m[3]);
+            words[e] = join_codes(m) & z;
         }
         if (E.c_out & 15) {                              // channels past c_out
 #pragma unroll
-            for (int b = 0; b < 8; ++b) words[b] &= (b < E.c_out ? 0xFFu : 0u) | (8 + b < E.c_out ? 0xFF00u : 0u);
-        }
-        if (in_frame) {
-            *reinterpret_cast<uint4*>(at) = make_uint4(words[0], words[1], words[2], words[3]);
-            *reinterpret_cast<uint4*>(at + E.cap_out * 16) = make_uint4(words[4], words[5], words[6], words[7]);
+            for (int e = 0; e < 4; ++e)
+                words[e] &= (e < E.c_out ? 0xFFu : 0u) | (e + 8 < E.c_out ? 0xFF00u : 0u) | (e + 4 < E.c_out ? 0xFF0000u : 0u) | (e + 12 < E.c_out ? 0xFF000000u : 0u);
         }
     } else {
 #pragma unroll
@@ -226,13 +231,13 @@ __device__ __forceinline__ void fused_unit_codes(const FusedUnitEnv& E, uint32_t
                 words[e] &= (c < E.c_out ? 0xFFu : 0u) | (c + 8 < E.c_out ? 0xFF00u : 0u) | (c + 16 < E.c_out ? 0xFF0000u : 0u) | (c + 24 < E.c_out ? 0xFF000000u : 0u);
             }
         }
-        if (in_frame) *reinterpret_cast<uint4*>(at) = make_uint4(words[0], words[1], words[2], words[3]);
     }
+    if (in_frame) *reinterpret_cast<uint4*>(at) = make_uint4(words[0], words[1], words[2], words[3]);
     if (trace && valid) {
 #pragma unroll 1
         for (int i = 0; i < 16; ++i) {
-            const int e = NARROW ? i & 7 : i & 3, byte = NARROW ? i >> 3 : i >> 2, c = NARROW ? 8 * byte + e : 32 * grp + 8 * byte + 4 * hf + e;
-            if (c < E.c_out) trace[c] = at[(e >> 2) * E.cap_out * 16 + (e & 3) * 4 + byte];
+            const int e = i & 3, byte = i >> 2, c = NARROW ? 8 * (byte & 1) + 4 * (byte >> 1) + e : 32 * grp + 8 * byte + 4 * hf + e;
+            if (c < E.c_out) trace[c] = at[e * 4 + byte];
         }
     }
 }
@@ -256,7 +261,7 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                     int n_layers, const FusedHead head, float one, float* __restrict__ logits, uint8_t* __restrict__ trace,
                     long long trace_stride) {
     extern __shared__ uint8_t dyn_smem[];
-    __shared__ __align__(8) uint64_t w_full[2], w_free[2], rec_full[FUSED_RING], rec_free[FUSED_RING];
+    __shared__ __align__(8) uint64_t w_full[2], w_raw[2], w_free[2], rec_full[FUSED_RING], rec_free[FUSED_RING];
     __shared__ __align__(8) uint64_t acc_full[FUSED_MAX_TILES], ep_done[FUSED_MAX_TILES], hold_full, copy_ready, epi_sync;
     __shared__ __align__(16) FusedTerms s_terms[FUSED_RING];
     __shared__ __align__(16) FusedLayer s_rec[FUSED_RING];
@@ -276,6 +281,7 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
         abort_flag = 0;
         for (int i = 0; i < 2; ++i) {
             mbar_init(&w_full[i], 1);
+            mbar_init(&w_raw[i], 1);
             mbar_init(&w_free[i], FUSED_ISSUERS);
         }
         for (int i = 0; i < FUSED_RING; ++i) {
@@ -324,6 +330,7 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
     if (warp == FUSED_LOADER_WARP) {
         // =========================== records, terms, weights ===========================
         const float *hold_cs = nullptr, *hold_cb = nullptr;
+        int n_raw[2] = {0, 0};
         for (int li = 0; li < n_layers; ++li) {
             const int slot = li & (FUSED_RING - 1), use = li / FUSED_RING;
             if (use > 0 && !mbar_wait_bounded_warp(&rec_free[slot], (uint32_t)((use - 1) & 1), abortp, limit)) break;
@@ -345,12 +352,35 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
             __syncwarp();
             if (lane == 0) mbar_arrive(&rec_full[slot]);
             if (li >= 2 && !mbar_wait_bounded_warp(&w_free[li & 1], (uint32_t)(((li >> 1) - 1) & 1), abortp, limit)) break;
+            const int co16 = (L.c_out + 15) & ~15, taps = L.k * L.k;
+            uint8_t* raw = wbuf + (li & 1) * FUSED_W_BYTES;
+            uint64_t* bar = L.c_in <= 16 ? &w_raw[li & 1] : &w_full[li & 1];
             if (lane == 0) {
-                const uint32_t bytes = (uint32_t)(L.k * L.k * ((L.c_in + 31) >> 5) * ((L.c_out + 15) & ~15) * 32);
-                mbar_arrive_expect_tx(&w_full[li & 1], bytes);
-                bulk_copy_g2s(wbuf + (li & 1) * FUSED_W_BYTES, L.w8, bytes, &w_full[li & 1]);
+                const uint32_t bytes = (uint32_t)(taps * ((L.c_in + 31) >> 5) * co16 * 32);
+                mbar_arrive_expect_tx(bar, bytes);
+                bulk_copy_g2s(raw, L.w8, bytes, bar);
             }
             __syncwarp();
+            if (L.c_in <= 16) {
+                // 16 bytes a tap and row -- word j = channels j, 8 + j, 4 + j, 12 + j -- two taps to a 32-byte row, rows
+                // swizzled as in the image
+                const int uses = n_raw[li & 1]++;
+                if (!mbar_wait_bounded_warp(bar, (uint32_t)(uses & 1), abortp, limit)) break;
+                for (int e = lane; e < ((taps + 1) & ~1) * co16; e += 32) {
+                    const int t = e / co16, row = e - t * co16, sw = (row >> 2) & 1;
+                    uint4 v = make_uint4(0, 0, 0, 0);                 // the partner of an odd last tap
+                    if (t < taps) {
+                        const uint4* src = reinterpret_cast<const uint4*>(raw + (t * co16 + row) * 32);
+                        const uint4 lo = src[sw], hi = src[sw ^ 1];
+                        v = make_uint4(__byte_perm(lo.x, hi.x, 0x5410), __byte_perm(lo.y, hi.y, 0x5410), __byte_perm(lo.z, hi.z, 0x5410),
+                                       __byte_perm(lo.w, hi.w, 0x5410));
+                    }
+                    reinterpret_cast<uint4*>(raw + FUSED_PACKED_W + ((t >> 1) * co16 + row) * 32)[(t & 1) ^ sw] = v;
+                }
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&w_full[li & 1]);
+            }
         }
         if (*abortp)                                     // a copy may still be in flight towards this CTA's shared memory
             for (int i = 0; i < 64; ++i) __nanosleep(1000);
@@ -374,10 +404,12 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                 ++n_copies;
             }
             const int cap_in = uni(strip_cap(L.c_in));
-            const uint64_t da0 = umma_desc_interleaved(smem_u32(strip_ptr(acts, L.k == 1 ? L.dst : L.src)), (uint32_t)(cap_in * 16));
-            const uint64_t db0 = umma_desc_sw32(smem_u32(wbuf + (li & 1) * FUSED_W_BYTES));
-            const uint32_t da_lo = uni((uint32_t)da0), da_hi = uni((uint32_t)(da0 >> 32)), db_lo = uni((uint32_t)db0), db_hi = uni((uint32_t)(db0 >> 32));
-            const uint32_t idesc = uni(umma_idesc_i8(g.co16)), step = uni((uint32_t)((g.co16 * 32) >> 4));
+            const bool narrow = uni(L.c_in) <= 16;
+            // (narrow: the field for the distance between the halves is added per MMA)
+            const uint64_t da0 = umma_desc_interleaved(smem_u32(strip_ptr(acts, L.k == 1 ? L.dst : L.src)), narrow ? 0u : (uint32_t)(cap_in * 16));
+            const uint64_t db0 = umma_desc_sw32(smem_u32(wbuf + (li & 1) * FUSED_W_BYTES + (narrow ? FUSED_PACKED_W : 0)));
+            const uint32_t idesc = umma_idesc_i8(g.co16);
+            const uint64_t step = (uint64_t)((g.co16 * 32) >> 4);
             const int k = uni(L.k), cw = uni(g.cw), tiles = uni(g.tiles), Wf = uni(g.Wf), hold = uni(L.hold);
             const uint32_t tm0 = uni(tmem_base + (uint32_t)(L.hold ? FUSED_HOLD_COL : 0)), tm_step = uni((uint32_t)g.acc_stride);
             int waited = 0;                              // tiles of the layer before that are known to be finished
@@ -390,27 +422,43 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                 const int need = wave ? min(prev_tiles, (t * UMMA_M + UMMA_M + Wf) / UMMA_M + 1) : prev_tiles;
                 if (!wait_tiles(need)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const uint32_t tm = tm0 + (uint32_t)t * tm_step;
-                const uint32_t a_tile = da_lo + (uint32_t)(t * UMMA_M);
-                uint32_t accu = 0u;
-                if (k == 3) {
-                    for (int wd = 0; wd < cw; ++wd) {
-                        uint32_t a_row = a_tile + (uint32_t)(wd * cap_in * 2);
-                        uint32_t b = db_lo + step * (uint32_t)wd;             // weight tiles are ordered [tap][word]
-                        const uint32_t bs = step * (uint32_t)cw;
-#pragma unroll
-                        for (int r = 0; r < 3; ++r, a_row += (uint32_t)Wf) {
-#pragma unroll
-                            for (int s = 0; s < 3; ++s, b += bs) {
-                                umma_i8_split(leader, tm, a_row + (uint32_t)s, da_hi, b, db_hi, idesc, accu);
-                                accu = 1u;
-                            }
+                if (leader) {
+                    const uint32_t tm = tm0 + (uint32_t)t * tm_step;
+                    const uint64_t da_t = da0 + (uint64_t)(t * UMMA_M);
+                    uint64_t db = db0;
+                    if (narrow) {
+                        // taps in pairs (the ninth alone): operand row = 16 bytes at the first tap, 16 at the second
+                        constexpr uint64_t LBO1 = 1ull << 16;
+                        if (k == 3) {
+                            const uint64_t w = (uint64_t)Wf;
+                            umma_i8(tm, da_t + LBO1, db, idesc, 0u);
+                            umma_i8(tm, da_t + 2 + ((w - 2) << 16), db + step, idesc, 1u);
+                            umma_i8(tm, da_t + w + 1 + LBO1, db + 2 * step, idesc, 1u);
+                            umma_i8(tm, da_t + 2 * w + LBO1, db + 3 * step, idesc, 1u);
+                            umma_i8(tm, da_t + 2 * w + 2 + LBO1, db + 4 * step, idesc, 1u);
+                        } else {
+                            umma_i8(tm, da_t + (uint64_t)(Wf + 1) + LBO1, db, idesc, 0u);
                         }
+                    } else if (k == 3) {
+                        const uint64_t bs = step * (uint64_t)cw;              // weight tiles are ordered [tap][word]
+                        for (int wd = 0; wd < cw; ++wd, db += step) {
+                            const uint64_t r0 = da_t + (uint64_t)(wd * cap_in * 2), r1 = r0 + (uint64_t)Wf, r2 = r1 + (uint64_t)Wf;
+                            umma_i8(tm, r0, db, idesc, wd > 0 ? 1u : 0u);
+                            umma_i8(tm, r0 + 1, db + bs, idesc, 1u);
+                            umma_i8(tm, r0 + 2, db + 2 * bs, idesc, 1u);
+                            umma_i8(tm, r1, db + 3 * bs, idesc, 1u);
+                            umma_i8(tm, r1 + 1, db + 4 * bs, idesc, 1u);
+                            umma_i8(tm, r1 + 2, db + 5 * bs, idesc, 1u);
+                            umma_i8(tm, r2, db + 6 * bs, idesc, 1u);
+                            umma_i8(tm, r2 + 1, db + 7 * bs, idesc, 1u);
+                            umma_i8(tm, r2 + 2, db + 8 * bs, idesc, 1u);
+                        }
+                    } else {
+                        for (int wd = 0; wd < cw; ++wd, db += step)
+                            umma_i8(tm, da_t + (uint64_t)(wd * cap_in * 2 + Wf + 1), db, idesc, wd > 0 ? 1u : 0u);
                     }
-                } else {
-                    for (int wd = 0; wd < cw; ++wd, accu = 1u)
-                        umma_i8_split(leader, tm, a_tile + (uint32_t)(wd * cap_in * 2 + Wf + 1), da_hi, db_lo + step * (uint32_t)wd, db_hi, idesc, accu);
                 }
+                __syncwarp();
                 if (!hold) umma_commit_pred(leader, &acc_full[t]);
             }
             if (!ok || !wait_tiles(prev_tiles)) break;   // (every phase of these barriers is waited for, so that parities stay in step)
@@ -459,8 +507,9 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                 // projection: its input is the stride-2 subsample of strip src, copied into strip dst in the output frame
                 const int Wp_in = L.w_in + 2, cap_in = strip_cap(L.c_in);
                 const uint8_t* src_strip = strip_ptr(acts, L.src);
-                for (int e = tid; e < g.Ho * g.Wo * g.cw * 2; e += FUSED_EPI_WARPS * 32) {
-                    const int hf = e & 1, rest = e >> 1, wd = rest % g.cw, pix = rest / g.cw;
+                const int hshift = L.c_in <= 16 ? 0 : 1;         // 16-byte halves of a pixel and word: one or two
+                for (int e = tid; e < (g.Ho * g.Wo * g.cw) << hshift; e += FUSED_EPI_WARPS * 32) {
+                    const int hf = e & hshift, rest = e >> hshift, wd = rest % g.cw, pix = rest / g.cw;
                     const int ho = pix / g.Wo, wo = pix - ho * g.Wo;
                     const uint8_t* s = src_strip + wd * cap_in * 32 + hf * cap_in * 16 + ((2 * ho + 1) * Wp_in + 2 * wo + 1) * 16;
                     uint8_t* d = dst_strip + wd * cap_in * 32 + hf * cap_in * 16 + ((ho + 1) * g.Wf + wo + 1) * 16;

@@ -95,10 +95,6 @@ __device__ __forceinline__ void tmem_ld4_wait(uint32_t (&a)[4], uint32_t (&b)[4]
                  : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]),
                    "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]) :: "memory");
 }
-__device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t n) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(n) : "memory");
-}
-
 // What the units of a layer share.
 struct FusedUnitEnv {
     uint64_t S2, PS2, rs2, one2, inv2;
@@ -289,8 +285,11 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
             mbar_init(&rec_free[i], FUSED_EPI_WARPS + FUSED_ISSUERS);
         }
         for (int i = 0; i < FUSED_MAX_TILES; ++i) {
-            mbar_init(&acc_full[i], 1);
-            mbar_init(&ep_done[i], 16);                          // four quarters x four units (fewer units arrive with more)
+            // Every issuing warp and every epilogue warp arrives once per tile and layer, also where another one has the
+            // work, once it has waited for what its turn waits for: so no barrier can run a phase ahead of a warp that has
+            // not looked at it yet, and parities suffice.
+            mbar_init(&acc_full[i], FUSED_ISSUERS);
+            mbar_init(&ep_done[i], FUSED_EPI_WARPS);
         }
         mbar_init(&hold_full, FUSED_ISSUERS);
         mbar_init(&copy_ready, FUSED_EPI_WARPS);
@@ -418,9 +417,13 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                     if (!mbar_wait_bounded_warp(&ep_done[waited], ((par >> waited) & 1u) ^ 1u, abortp, limit)) return false;
                 return true;
             };
-            for (int t = k_iss; t < tiles; t += FUSED_ISSUERS) {
+            for (int t = 0; t < tiles; ++t) {
                 const int need = wave ? min(prev_tiles, (t * UMMA_M + UMMA_M + Wf) / UMMA_M + 1) : prev_tiles;
                 if (!wait_tiles(need)) { ok = false; break; }
+                if ((t & (FUSED_ISSUERS - 1)) != k_iss) {
+                    if (!hold && leader) mbar_arrive(&acc_full[t]);
+                    continue;
+                }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 if (leader) {
                     const uint32_t tm = tm0 + (uint32_t)t * tm_step;
@@ -546,10 +549,17 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                     for (int t = 0; t < g.tiles && ok; ++t) ok = mbar_wait_bounded_warp(&acc_full[t], (par >> t) & 1u, abortp, limit);
                     if (!ok) break;
                 }
-                for (int u = 0; u < total; ++u) {
-                    const int t = u >> ushift, un = u & (units - 1);
-                    if (un == 0 && !mbar_wait_bounded_warp(&acc_full[t], (par >> t) & 1u, abortp, limit)) { ok = false; break; }
-                    if (((turn + u) & 3) != quad) continue;
+                for (int t = 0; t < g.tiles; ++t) {
+                    const int u = t << ushift;
+                    if (!mbar_wait_bounded_warp(&acc_full[t], (par >> t) & 1u, abortp, limit)) { ok = false; break; }
+                    // the unit of this tile that is this warp's, if any: at most one, there are as many groups of warps as units
+                    const int own = (quad - turn - u) & 3;       // (u is the tile's first unit here)
+                    if (own >= units) {
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&ep_done[t]);
+                        continue;
+                    }
+                    const int un = own;
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     const int f = t * UMMA_M + quarter * 32 + lane;
                     const int hp = __float2int_rd(__fmul_rn((float)f + 0.5f, rcp_w)), wp = f - hp * Wf;   // (exact: f < 2^20)
@@ -580,7 +590,7 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) mbar_arrive_n(&ep_done[t], 4u >> ushift);
+                    if (lane == 0) mbar_arrive(&ep_done[t]);
                 }
                 turn = (turn + total) & 3;
                 par ^= (1u << g.tiles) - 1u;

@@ -31,6 +31,8 @@
 // overwritten in place.  After the last block: average pooling (pixels added in order), 8-bit
 // quantization, and the classifier as a plain integer dot product, a warp per class.
 // Every wait is bounded; on a timeout the CTA sets its abort flag, every role leaves its loop, tensor memory is freed.
+#include <type_traits>
+
 #include "conv_frame.cuh"
 
 namespace ebs {
@@ -543,55 +545,56 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                 E.res = strip_ptr(acts, L.res_buf);
                 E.T = &T;
                 uint8_t* tr = trace && L.trace_off >= 0 ? trace + (size_t)img * trace_stride + L.trace_off : nullptr;
-                const int form = uni((L.c_out <= 16 ? 3 : 0) + L.res + (to_pool ? 6 : 0));
+                const int res = uni(L.res);
+                const bool narrow = uni(L.c_out) <= 16;
                 const int total = g.tiles << ushift;
                 if (L.src == (to_pool ? 0 : L.dst)) {    // writes over its own input: only after the last MMA
                     for (int t = 0; t < g.tiles && ok; ++t) ok = mbar_wait_bounded_warp(&acc_full[t], (par >> t) & 1u, abortp, limit);
                     if (!ok) break;
                 }
-                for (int t = 0; t < g.tiles; ++t) {
-                    const int u = t << ushift;
-                    if (!mbar_wait_bounded_warp(&acc_full[t], (par >> t) & 1u, abortp, limit)) { ok = false; break; }
-                    // the unit of this tile that is this warp's, if any: at most one, there are as many groups of warps as units
-                    const int own = (quad - turn - u) & 3;       // (u is the tile's first unit here)
-                    if (own >= units) {
+                // One loop over the tiles per form, so that a unit is straight-line code: with the choice of form (a jump through
+                // a table) and the layer's fields read per unit, what preceded the arithmetic took longer than it.
+                const int tiles = g.tiles, c_out = L.c_out;
+                const uint32_t acc_stride = (uint32_t)g.acc_stride, trow0 = tmem_base + ((uint32_t)(quarter * 32) << 16);
+                auto run = [&](auto narrow_t, auto res_t, auto pool_t) {
+                    constexpr bool NARROW = decltype(narrow_t)::value, POOL = decltype(pool_t)::value;
+                    constexpr int RES = decltype(res_t)::value;
+#pragma unroll 1
+                    for (int t = 0; t < tiles; ++t) {
+                        const int f = t * UMMA_M + quarter * 32 + lane;
+                        const int hp = __float2int_rd(__fmul_rn((float)f + 0.5f, rcp_w)), wp = f - hp * Wf;   // (exact: f < 2^20)
+                        // does this frame row have an output, and where does it go in the destination frame
+                        const int ho = two ? hp >> 1 : hp, wo = two ? wp >> 1 : wp;
+                        const bool valid = f < frame && !(two && ((hp | wp) & 1)) && ho < Ho && wo < Wo;
+                        const int target = two ? (ho + 1) * Wp_out + wo + 1 : f + Wf + 1;
+                        const bool in_frame = f < frame && (!two || valid);          // stride 1 also writes the zeros of the padding
+                        // the unit of this tile that is this warp's, if any: at most one, there are as many groups of warps as units
+                        const int un = (quad - turn - (t << ushift)) & 3;
+                        const bool work = un < units && __any_sync(0xffffffffu, in_frame);
+                        if (!mbar_wait_bounded_warp(&acc_full[t], (par >> t) & 1u, abortp, limit)) return false;
+                        if (work) {
+                            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                            const uint32_t trow = trow0 + (uint32_t)t * acc_stride;
+                            if constexpr (POOL) fused_unit_pool<NARROW, RES>(E, trow, un, target, valid, relu, pool_scratch + (ho * Wo + wo) * c_out);
+                            else fused_unit_codes<NARROW, RES>(E, trow, un, target, valid, in_frame, tr ? tr + (size_t)(ho * Wo + wo) * c_out : nullptr);
+                            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                            asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                        }
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&ep_done[t]);
-                        continue;
                     }
-                    const int un = own;
-                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    const int f = t * UMMA_M + quarter * 32 + lane;
-                    const int hp = __float2int_rd(__fmul_rn((float)f + 0.5f, rcp_w)), wp = f - hp * Wf;   // (exact: f < 2^20)
-                    // does this frame row have an output, and where does it go in the destination frame
-                    const int ho = two ? hp >> 1 : hp, wo = two ? wp >> 1 : wp;
-                    const bool valid = f < frame && !(two && ((hp | wp) & 1)) && ho < Ho && wo < Wo;
-                    const int target = two ? (ho + 1) * Wp_out + wo + 1 : f + Wf + 1;
-                    const bool in_frame = f < frame && (!two || valid);              // stride 1 also writes the zeros of the padding
-                    if (__any_sync(0xffffffffu, in_frame)) {
-                        const uint32_t trow = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(t * g.acc_stride);
-                        uint8_t* tp = tr ? tr + (size_t)(ho * Wo + wo) * L.c_out : nullptr;
-                        float* pr = pool_scratch + (ho * Wo + wo) * L.c_out;
-                        switch (form) {
-                            case 0: fused_unit_codes<false, 0>(E, trow, un, target, valid, in_frame, tp); break;
-                            case 1: fused_unit_codes<false, 1>(E, trow, un, target, valid, in_frame, tp); break;
-                            case 2: fused_unit_codes<false, 2>(E, trow, un, target, valid, in_frame, tp); break;
-                            case 3: fused_unit_codes<true, 0>(E, trow, un, target, valid, in_frame, tp); break;
-                            case 4: fused_unit_codes<true, 1>(E, trow, un, target, valid, in_frame, tp); break;
-                            case 5: fused_unit_codes<true, 2>(E, trow, un, target, valid, in_frame, tp); break;
-                            case 6: fused_unit_pool<false, 0>(E, trow, un, target, valid, relu, pr); break;
-                            case 7: fused_unit_pool<false, 1>(E, trow, un, target, valid, relu, pr); break;
-                            case 8: fused_unit_pool<false, 2>(E, trow, un, target, valid, relu, pr); break;
-                            case 9: fused_unit_pool<true, 0>(E, trow, un, target, valid, relu, pr); break;
-                            case 10: fused_unit_pool<true, 1>(E, trow, un, target, valid, relu, pr); break;
-                            default: fused_unit_pool<true, 2>(E, trow, un, target, valid, relu, pr); break;
-                        }
-                    }
-                    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&ep_done[t]);
-                }
+                    return true;
+                };
+                auto by_res = [&](auto narrow_t, auto pool_t) {
+                    if (res == 0) return run(narrow_t, std::integral_constant<int, 0>{}, pool_t);
+                    if (res == 1) return run(narrow_t, std::integral_constant<int, 1>{}, pool_t);
+                    return run(narrow_t, std::integral_constant<int, 2>{}, pool_t);
+                };
+                using True = std::true_type;
+                using False = std::false_type;
+                if (to_pool) ok = narrow ? by_res(True{}, True{}) : by_res(False{}, True{});
+                else ok = narrow ? by_res(True{}, False{}) : by_res(False{}, False{});
+                if (!ok) break;
                 turn = (turn + total) & 3;
                 par ^= (1u << g.tiles) - 1u;
             }

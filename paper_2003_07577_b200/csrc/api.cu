@@ -155,11 +155,16 @@ static int choose_pipe_variant(const ConvParams& p, int sms) {
     // (layers with few input channels too: the kernel spends a whole 32-channel word per tap on them, and is still
     // six times faster on an ImageNet stem, 3 -> 64 channels 7x7 stride 2, than the tap-folding per-tap kernels)
     if (p.Co < 64 || (long long)p.P * p.Co < (1LL << 20) || p.w_levels) return -1;
-    for (int v = 2; v >= 0; --v) {
-        if (p.Co % (64 << v) != 0 && v != 0) continue;
-        if (conv_umma_pipe_applies(p, v)) return v;
-    }
-    return -1;
+    // Ragged channel groups leave the lean epilogues only as packed planes; with 32-bit results the tile kernel's epilogue is
+    // up to twice as fast (48 -> 77 3x3 at 28x28, batch 128: 44 us against 83).
+    if ((p.Co & 31) != 0 && (p.acc || p.y)) return -1;
+    // The widest channel tile that does not add much to the padding of the narrowest: a wide tile expands the activations
+    // fewer times (512 -> 224 1x1 at 28x28, batch 256: 119, 66 and 44 us with 64, 128 and 256 channels; 256 -> 300 at
+    // 14x14: 31, 20, 21; 192 -> 192 3x3 at 28x28: 123, 201, 134).
+    auto padded = [&](int v) { return (p.Co + (64 << v) - 1) / (64 << v) * (64 << v); };
+    if (padded(2) * 8 <= padded(0) * 9 && conv_umma_pipe_applies(p, 2)) return 2;
+    if (padded(1) * 4 <= padded(0) * 5 && conv_umma_pipe_applies(p, 1)) return 1;
+    return conv_umma_pipe_applies(p, 0) ? 0 : -1;
 }
 
 // Layers that do not fill the GPU several times over run on the tile kernel, with the channel tile of the smallest
@@ -229,6 +234,7 @@ static int conv_plan(const void* packed_x, int n, int h, int w, const void* pack
     p.N = n; p.H = h; p.W = w; p.CW = (d->c_in + 31) / 32;
     p.Co = d->c_out; p.Ho = Ho; p.Wo = Wo; p.CWo = (d->c_out + 31) / 32;
     p.kh = d->kh; p.kw = d->kw; p.sh = d->stride_h; p.sw = d->stride_w; p.ph = d->pad_h; p.pw = d->pad_w;
+    p.x_words = byte_acts ? 8 : d->a_bits;
     p.KK = d->kh * d->kw * p.CW;
     p.P = (int)P;
     p.acc = acc_out; p.y = y_out; p.packed_next = static_cast<uint32_t*>(packed_next);
@@ -238,10 +244,6 @@ static int conv_plan(const void* packed_x, int n, int h, int w, const void* pack
     p.w_levels = d->w_levels;
     p.fold = d->c_in <= 4 ? 8 : (d->c_in <= 8 ? 4 : (d->c_in <= 16 ? 2 : 1));
     p.fold_bits = 32 / p.fold;
-    {
-        const long long wmax = d->w_levels ? (1LL << d->w_bits) - 1 : (1LL << (d->w_bits - 1));
-        p.acc_small = (long long)d->c_in * d->kh * d->kw * wmax * ((1LL << d->a_bits) - 1) < (1LL << 22) ? 1 : 0;
-    }
     p.wait_limit = g_wait_limit;
     p.test_flags = g_test_flags;
     p.lim_x = byte_acts ? in_pixels * p.CW * 8 : in_pixels * p.CW * d->a_bits;

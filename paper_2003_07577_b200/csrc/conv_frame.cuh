@@ -208,7 +208,7 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_address) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(cluster_address) : "memory");
 }
 // Bounded wait on a barrier another CTA of the cluster arrives on.
-__device__ __forceinline__ bool mbar_wait_cluster_hot(uint64_t* bar, uint32_t parity, volatile int* abort_flag, unsigned limit) {
+__device__ __forceinline__ bool mbar_wait_cluster_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, unsigned limit) {
     const uint32_t addr = smem_u32(bar);
     for (unsigned it = 0; it < limit; ++it) {
         uint32_t done;
@@ -217,14 +217,24 @@ __device__ __forceinline__ bool mbar_wait_cluster_hot(uint64_t* bar, uint32_t pa
             "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}\n"
             : "=r"(done) : "r"(addr), "r"(parity) : "memory");
-        if (done) return true;
-        if (*abort_flag) return false;
+        if (__all_sync(0xffffffffu, done != 0)) return true;
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
     }
     *abort_flag = 1;
     return false;
 }
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+// The same value in every lane, known to the compiler to be so: what the issuing warps feed into descriptors and loop
+// bounds has to live in uniform registers, or every MMA moves four operands there first (130 clocks an MMA instead of 40).
+__device__ __forceinline__ int uni(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ uint32_t uni(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+// True in one lane of a converged warp, always the same one.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
+    return r != 0;
 }
 __device__ __forceinline__ void umma_commit_pred(uint32_t leader, uint64_t* bar) {
     asm volatile(
@@ -463,6 +473,12 @@ __device__ __forceinline__ void plain_codes32(const uint32_t (&v)[32], float S, 
         const uint32_t c4 = join_codes(m);
         cr[bb] = __funnelshift_l(c4, c4, bb);
     }
+}
+
+// Zero bits behind the last `left` channels of a group that is not whole.
+__device__ __forceinline__ void mask_planes(uint32_t (&planes)[8], int left) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) planes[j] &= (1u << left) - 1u;
 }
 
 // A group's plane words in the widest stores their alignment (4 * nb bytes) allows.

@@ -53,8 +53,20 @@ constexpr int PIPE_SLOTS = 2;                      // (pixel, word) items an exp
 constexpr int PIPE_MAX_ITEMS = PIPE_SLOTS * PIPE_EXPANDERS;
 constexpr int PIPE_MAX_TAPS = FRAME_MAX_TAPS, PIPE_MAX_STAGES = 4;
 constexpr int PIPE_MAX_BSLOTS = 32;                // weight tiles in flight when the weights stream
-constexpr int PIPE_MAX_MMAS = 512;                 // MMAs of one chunk (table of their operand offsets in shared memory)
 constexpr int PIPE_SMEM_MAX = 220 * 1024;
+
+// What one slot of the weight ring holds of a phase with rows x cols taps: whole words, or whole rows of taps of one word,
+// or a part of a row, so that the MMAs of a slot are straight runs along the taps.  cap: tiles a slot has room for.
+struct PipeSlot {
+    int words, rows, cols;
+};
+inline PipeSlot pipe_slot(int rows, int cols, int cap) {
+    PipeSlot s;
+    s.cols = cols < cap ? cols : cap;
+    s.rows = cols > cap ? 1 : rows * cols <= cap ? rows : cap / cols;
+    s.words = rows * cols <= cap ? cap / (rows * cols) : 1;
+    return s;
+}
 
 // Launch geometry, computed on the host and passed to the kernel by value.
 struct PipeGeom : FrameGeom {
@@ -66,6 +78,7 @@ struct PipeGeom : FrameGeom {
     int nchunks;                       // chunks per tile = n_ph * nwg (phase-major)
     int n_stages, a_word_bytes, a_stage_bytes, stage_bytes;
     int b_resident, b_total_bytes;
+    PipeSlot slot[FRAME_MAX_PHASES];   // of each phase
     int b_slots, b_group;              // streamed weights: ring of slots of b_group (tap, word) tiles of TILE_N x 32 bytes
     int nbuf, tmem_cols, smem_bytes;
     int pair;                          // 1: two CTAs of a cluster share every MMA (256 pixels x 256 channels, half a weight tile each)
@@ -98,6 +111,10 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
         if (nb == 1 && deep < 64 && !m_sub_req) continue;        // shallow reductions want the epilogue overlapped
         if (m * UMMA_M + max_shift > PIPE_MAX_ITEMS) continue;
         const long long pt = (frame + (long long)m * UMMA_M * pw - 1) / ((long long)m * UMMA_M * pw);
+        // Expander lanes run over the words of a pass first: with one word a pass every lane of a load reads a line of its
+        // own, which for pixels of about a line or more, expanded for one tap only, costs more than the larger strip saves (256 -> 64 1x1 at 56x56, batch 256:
+        // 4 bits 81.8 -> 73.7 us with half the pixels and two words, 5 bits 132 -> 92).
+        if (!m_sub_req && m > 1 && taps == 1 && m * UMMA_M > PIPE_MAX_ITEMS / 2 && p.CW > 2 && p.CW * p.x_words >= 24) continue;
         if (!m_sub_req && m > 1 && pt * g.n_ctiles < (deep >= 64 ? 1LL : 2LL) * sms) continue;
         m_sub = m;
         break;
@@ -114,14 +131,12 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
     g.a_word_bytes = g.SP * 32 + 64;                           // sized with the largest skew; fixed once ks is known
     if (g.SP * 16 >= (1 << 18)) return g;
     // weights resident when they leave room for at least two activation stages
-    const int budget = PIPE_SMEM_MAX - 2048 - PIPE_MAX_MMAS * 8;   // the MMA table sits behind the rings
+    const int budget = PIPE_SMEM_MAX - 2048;
     g.b_resident = g.b_total_bytes + 2 * ((g.a_word_bytes + 255) & ~255) <= budget && g.b_total_bytes <= 160 * 1024;
     int ks = PIPE_MAX_ITEMS / g.S;
     if (ks > 4) ks = 4;
     if (ks > p.CW) ks = p.CW;
     if (ks < 1) return g;
-    while (ks > 1 && ks * taps * m_sub >= PIPE_MAX_MMAS - 2) --ks;     // (the issue loops read up to two entries ahead)
-    if (ks * taps * m_sub >= PIPE_MAX_MMAS - 2) return g;
     // Streamed weights go through a ring of their own (slots of a few consecutive (tap, word) tiles), so that copies are
     // in flight all the time (a stage-sized unit would leave the copy engine idle while a stage's MMAs run).
     auto stage_bytes = [&](int k) { return (k * g.a_word_bytes + 255) & ~255; };
@@ -131,11 +146,12 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
     if (2 * stage_bytes(ks) > avail) return g;
     // fewer words per pass when that buys a deeper ring (latency hiding matters more than stage size)
     while (ks > 1 && avail / stage_bytes(ks) < 3) --ks;
-    // A stage is filled in nsub expander passes of ks words: the thread that issues the MMAs retires an instruction
-    // only every ten clocks or so, so its per-stage bookkeeping has to be spread over about a dozen MMAs.
+    // A stage is filled in nsub expander passes of ks words: the waits, addresses and commits of a stage cost an issuing
+    // warp a thousand clocks, to be spread over some forty MMAs (64 -> 64 3x3 at 56x56, batch 256: 55.6 us with a word a
+    // stage, 18 MMAs, 50.3 with two; 256 -> 256 3x3 stride 2 at 28x28: 65.1 and 49.9).
     int nsub = 1;
-    while (nsub < 4 && ks * nsub * taps * m_sub < 12 && ks * nsub < p.CW &&
-           ks * 2 * nsub * taps * m_sub < PIPE_MAX_MMAS - 2 && 3 * stage_bytes(ks * 2 * nsub) <= avail)
+    while (nsub < 4 && ks * nsub * taps * m_sub < 40 && ks * nsub < p.CW &&
+           3 * stage_bytes(ks * 2 * nsub) <= avail)
         nsub *= 2;
     // Skew between the word tiles of a pass: the 8 lanes of a quarter warp store 16 bytes each for ks words of 8 / ks
     // pixels; a skew of 128 / ks bytes (48 for three words) puts them on eight different 16-byte bank groups.
@@ -151,16 +167,18 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
     const int st_cap = g.b_resident ? PIPE_MAX_STAGES : (pair ? PIPE_MAX_STAGES : 3);
     if (g.n_stages > st_cap) g.n_stages = st_cap;
     if (!g.b_resident) {
-        // a slot holds up to 32 KB of consecutive tiles of a chunk (one wait and one commit per slot, not per MMA)
-        g.b_group = 32768 / b_tile;
-        if (g.b_group > g.kss * max_ph_taps) g.b_group = g.kss * max_ph_taps;
-        if (g.b_group < 1) g.b_group = 1;
+        // a slot holds up to 32 KB of consecutive tiles (one wait and one commit per slot, not per MMA)
+        const int most = 32768 / b_tile > g.kss * max_ph_taps ? g.kss * max_ph_taps : 32768 / b_tile;
+        g.b_group = 1;
+        for (int i = 0; i < g.n_ph; ++i) {
+            const PipeSlot sl = g.slot[i] = pipe_slot(g.ph_rows[i], g.ph_cols[i], most);
+            if (sl.words * sl.rows * sl.cols > g.b_group) g.b_group = sl.words * sl.rows * sl.cols;
+        }
         g.b_slots = (budget - g.n_stages * g.stage_bytes) / (g.b_group * b_tile);
         if (g.b_slots > PIPE_MAX_BSLOTS) g.b_slots = PIPE_MAX_BSLOTS;
         if (g.b_slots < 3) return g;
     }
-    g.smem_bytes = (g.b_resident ? g.b_total_bytes : g.b_slots * g.b_group * b_tile) + g.n_stages * g.stage_bytes + 1024 +
-                   PIPE_MAX_MMAS * 8;
+    g.smem_bytes = (g.b_resident ? g.b_total_bytes : g.b_slots * g.b_group * b_tile) + g.n_stages * g.stage_bytes + 1024;
     if (g.b_resident) {                                        // a CTA keeps one channel tile
         g.grid_y = g.n_ctiles;
         long long gx = sms / g.n_ctiles;
@@ -293,18 +311,20 @@ __device__ __forceinline__ void pipe_store_planes(const uint32_t (&planes)[8], i
 // four channels of a byte register go from accumulator to code in one short chain, so that nothing but the 32
 // accumulators and the finished code registers is alive at a time -- the general form above keeps the 32 fp32 images
 // as well, which at 96 registers costs spills and the parallelism of the instruction stream.
+// left: channels of the layer from this group on (a last group of fewer than 32 writes zero bits behind them).
 template <int G>
 __device__ __forceinline__ void pipe_group32_packed(const uint32_t (&v)[32], bool pvalid, float S, float inv_next, int nb, int qmax,
-                                                    uint32_t* dst, const ConvParams& p, PlaneHold<G>& hold) {
+                                                    uint32_t* dst, const ConvParams& p, PlaneHold<G>& hold, int left) {
     uint32_t cr[8];
     plain_codes32(v, S, p.one, inv_next, (float)(2 * qmax + 1), cr);
     uint32_t planes[8];
     bytes_to_planes(cr, nb, planes);
+    if (left < 32) mask_planes(planes, left);
     pipe_store_planes(planes, nb, dst, pvalid, hold, p);
 }
 
 // Epilogue of a layer with per-channel terms and / or a shortcut (a folded batch normalisation, the second convolution of a
-// residual block): whole channel tiles, NHWC, packed planes and / or fp32 out.  The warp walks its (accumulator, 32-channel
+// residual block): NHWC, packed planes and / or fp32 out.  The warp walks its (accumulator, 32-channel
 // group) units; the next unit's shortcut and terms are requested before the current one is packed and stored.  The terms of
 // a group pass through 64 words of shared memory of the warp's own (one load and one store a lane, then broadcast reads):
 // read channel by channel through the cache they cost more than the arithmetic (64 -> 256 1x1 at 56x56, batch 256: 225 us
@@ -312,10 +332,11 @@ __device__ __forceinline__ void pipe_group32_packed(const uint32_t (&v)[32], boo
 template <int TILE_N, int G, bool VALUES, int NB, int RES>
 __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, const FrameGeom& g, uint32_t tmem_set, int m_sub, int vwarp,
                                                     int f0, int co0, float* terms) {
-    constexpr int COLS = TILE_N / 2, NG = COLS / 32;
     const int lane = (int)(threadIdx.x & 31), at = (lane & 7) * 4 + (lane >> 3);
     const uint32_t trow = tmem_set + ((uint32_t)((vwarp & 3) * 32) << 16);
-    const int cbeg = (vwarp >> 2) * COLS;
+    constexpr int COLS = TILE_N / 2;
+    const int cbeg = (vwarp >> 2) * COLS, cend = COLS == 32 ? cbeg + 32 : min(cbeg + COLS, p.Co - co0);   // (cend: groups start below)
+    if (co0 + cbeg >= p.Co) return;
     const int nb = NB > 0 ? NB : p.next_bits;                // (a constant where only planes are written)
     const float hi2 = (float)(2 * ((1 << nb) - 1) + 1);
     PlaneHold<G> hold;
@@ -339,8 +360,9 @@ __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, cons
         }
     };
     auto request = [&](int c) {                              // c: first channel of the unit
-        t_scale = p.ch_scale ? __ldg(p.ch_scale + c + lane) : 1.0f;
-        t_bias = p.ch_bias ? __ldg(p.ch_bias + c + lane) : -0.0f;
+        const bool in = c + lane < p.Co;
+        t_scale = p.ch_scale && in ? __ldg(p.ch_scale + c + lane) : 1.0f;
+        t_bias = p.ch_bias && in ? __ldg(p.ch_bias + c + lane) : -0.0f;
         if constexpr (RES == 1) {
             const float4* r4 = reinterpret_cast<const float4*>(p.residual + (size_t)gp * p.Co + c);
 #pragma unroll
@@ -357,8 +379,8 @@ __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, cons
 #pragma unroll 1
     for (int j = 0; j < m_sub; ++j) {
 #pragma unroll 1
-        for (int k = 0; k < NG; ++k) {
-            const int c0 = cbeg + 32 * k, c = co0 + c0;
+        for (int c0 = cbeg; c0 < cend; c0 += 32) {
+            const int c = co0 + c0;
             const bool ok = pvalid;
             const size_t gpz = gp;
             __syncwarp();                                    // every lane has read the unit before
@@ -387,7 +409,7 @@ __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, cons
                     terms_codes32<RES>(v, p.S, p.one, cs, cb, res, rbyte, p.res_scale, p.inv_next, hi2, cr);
                 }
             }
-            if (k + 1 < NG) {
+            if (c0 + 32 < cend) {
                 request(c + 32);
             } else if (j + 1 < m_sub) {
                 locate(j + 1);
@@ -396,19 +418,20 @@ __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, cons
             if (some && (!VALUES || p.packed_next)) {
                 uint32_t planes[8];
                 bytes_to_planes(cr, nb, planes);
+                if (p.Co - c < 32) mask_planes(planes, p.Co - c);
                 pipe_store_planes(planes, nb, p.packed_next + (gpz * p.CWo + (c >> 5)) * nb, ok, hold, p);
             }
         }
     }
 }
 
-// Plain epilogue (no per-channel terms, no shortcut, NHWC, whole channel tile, c_out % 4 == 0) of one
+// Plain epilogue (no per-channel terms, no shortcut, NHWC, c_out a multiple of 32) of one
 // 128-pixel accumulator.  vwarp 0..7: TMEM lane quarter vwarp % 4, channel half vwarp / 4.
 template <int TILE_N, int G>
 __device__ __forceinline__ void pipe_epilogue_plain_g(const ConvParams& p, uint32_t tmem_acc, int vwarp, int gp, bool pvalid,
                                                       int co0) {
-    constexpr int COLS = TILE_N / 2;
     const uint32_t trow = tmem_acc + ((uint32_t)((vwarp & 3) * 32) << 16);
+    constexpr int COLS = TILE_N / 2;
     const int cbeg = (vwarp >> 2) * COLS;
     const bool want_q = p.packed_next != nullptr;
     const int nb = want_q ? p.next_bits : 0, qmax = (1 << p.next_bits) - 1;
@@ -418,6 +441,7 @@ __device__ __forceinline__ void pipe_epilogue_plain_g(const ConvParams& p, uint3
     hold.filled = 0;
 #pragma unroll 1
     for (int c0 = cbeg; c0 < cbeg + COLS; c0 += 32) {
+        if (co0 + c0 >= p.Co) break;
         uint32_t (&lo)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[0]);
         uint32_t (&hi)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[16]);
         tmem_ld16_issue(trow + (uint32_t)c0, lo);
@@ -427,7 +451,7 @@ __device__ __forceinline__ void pipe_epilogue_plain_g(const ConvParams& p, uint3
         const size_t o = (size_t)gp * p.Co + co0 + c0;
         uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + ((co0 + c0) >> 5)) * nb;
         if (want_q && !p.acc && !p.y) {
-            pipe_group32_packed(v, pvalid, S, inv_next, nb, qmax, dst, p, hold);
+            pipe_group32_packed(v, pvalid, S, inv_next, nb, qmax, dst, p, hold, 32);
         } else if (want_q) {
             pipe_group32<true>(p, v, o, pvalid, S, inv_next, nb, qmax, dst);
         } else {
@@ -436,13 +460,13 @@ __device__ __forceinline__ void pipe_epilogue_plain_g(const ConvParams& p, uint3
     }
 }
 
-// Packed-only epilogue without per-channel terms of one 128-pixel accumulator (whole channel tile): nothing but the lean
+// Packed-only epilogue without per-channel terms of one 128-pixel accumulator: nothing but the lean
 // group, for the kernel forms that are launched only for such layers.
 template <int TILE_N, int G, int NB>
 __device__ __forceinline__ void pipe_epilogue_packed_nb(const ConvParams& p, uint32_t tmem_acc, int vwarp, int gp, bool pvalid,
                                                        int co0) {
-    constexpr int COLS = TILE_N / 2;
     const uint32_t trow = tmem_acc + ((uint32_t)((vwarp & 3) * 32) << 16);
+    constexpr int COLS = TILE_N / 2;
     const int cbeg = (vwarp >> 2) * COLS;
     constexpr int nb = NB, qmax = (1 << NB) - 1;
     const float S = p.S, inv_next = p.inv_next;
@@ -451,6 +475,7 @@ __device__ __forceinline__ void pipe_epilogue_packed_nb(const ConvParams& p, uin
     hold.filled = 0;
 #pragma unroll 1
     for (int c0 = cbeg; c0 < cbeg + COLS; c0 += 32) {
+        if (co0 + c0 >= p.Co) break;
         uint32_t (&lo)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[0]);
         uint32_t (&hi)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[16]);
         tmem_ld16_issue(trow + (uint32_t)c0, lo);
@@ -458,7 +483,7 @@ __device__ __forceinline__ void pipe_epilogue_packed_nb(const ConvParams& p, uin
         tmem_ld16_wait(lo);
         tmem_ld16_wait(hi);
         uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + ((co0 + c0) >> 5)) * nb;
-        pipe_group32_packed(v, pvalid, S, inv_next, nb, qmax, dst, p, hold);
+        pipe_group32_packed(v, pvalid, S, inv_next, nb, qmax, dst, p, hold, p.Co - co0 - c0);
     }
 }
 
@@ -501,17 +526,17 @@ __device__ __forceinline__ void pipe_epilogue_terms(const ConvParams& p, const F
 // Odd plane counts of the packed output take the form that holds the groups of a run back: a kernel instantiation of
 // its own (HOLD), chosen by the launcher, because the shift register costs the other layers registers and time even
 // as an untaken branch of the same kernel (even counts 15-25% slower when both forms were compiled into one kernel).
-// Kernel form for a layer: 0 = every output mode and ragged channel tiles; 1 = packed planes only, whole channel tiles
+// Kernel form for a layer: 0 = every output mode; 1 = packed planes only
 // (the usual layer of a network: its epilogue holds nothing but the lean group, or the group with per-channel terms);
 // 2 = form 1 with the held-back runs.
-inline bool pipe_packed_only(const ConvParams& p, int tile_n) {
-    return p.packed_next && !p.acc && !p.y && !p.w_levels && (p.Co % tile_n) == 0 && !(p.residual && p.res_packed);
+inline bool pipe_packed_only(const ConvParams& p) {
+    return p.packed_next && !p.acc && !p.y && !p.y_nchw && !p.w_levels && !(p.residual && (p.res_packed || (p.Co & 31) != 0));
 }
 inline bool pipe_hold_applies(const ConvParams& p, int tile_n) {
     const int G = tile_n / 64;
     // (5 and 7 planes; with 1 or 3 the single-word stores are few and the held form measured slower)
     return G > 1 && p.packed_next && (p.next_bits == 5 || p.next_bits == 7) && (p.CWo % G) == 0 && !p.acc && !p.y && !p.y_nchw &&
-           (p.Co & 31) == 0 && !p.w_levels && !(p.residual && p.res_packed);
+           (p.Co % tile_n) == 0 && !p.w_levels && !(p.residual && p.res_packed);
 }
 
 template <int AB, int TILE_N, bool AFFINE, int FORM, bool PAIR = false>
@@ -540,30 +565,6 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
     if (tid < PIPE_MAX_TAPS) {
         s_tap_shift[tid] = (uint32_t)g.tap_shift[tid];
         s_tap_id[tid] = (int)g.tap_id[tid];
-    }
-    // Table of the MMAs of a chunk, per phase, in issue order (word, tap, accumulator): x = offset of the activation
-    // operand from the stage start (16-byte units: word, tap shift, 128 pixels per accumulator) | accumulator column
-    // offset << 22, y = offset of the weight tile (16-byte units) from the chunk's first tile (resident weights) or from
-    // the start of its ring slot (streamed).  An issuing warp then spends a load, three additions and the MMA per step;
-    // with operand addresses computed in its loop it was the slowest stage of the pipeline.
-    uint2* mma_tab = reinterpret_cast<uint2*>(dyn_smem + ((1024u - (smem_u32(dyn_smem) & 1023u)) & 1023u) +
-                                              (g.smem_bytes - 1024 - PIPE_MAX_MMAS * 8));
-    {
-        const int per_tap = g.kss * g.m_sub, total_e = per_tap * g.taps;
-        const uint32_t bt16 = (uint32_t)B_TILE_BYTES >> 4;
-        for (int e = tid; e < total_e; e += PIPE_THREADS) {
-            int ph = 0;
-            while (ph + 1 < g.n_ph && e >= per_tap * g.ph_tap0[ph + 1]) ++ph;
-            const int t0 = g.ph_tap0[ph], ntp = g.ph_tap0[ph + 1] - t0;
-            const int local = e - per_tap * t0;
-            const int q = local / (ntp * g.m_sub), r = local - q * (ntp * g.m_sub);
-            const int tl = r / g.m_sub, j = r - tl * g.m_sub;
-            const uint32_t a_off = (uint32_t)(q * (g.a_word_bytes >> 4) + g.tap_shift[t0 + tl] + j * UMMA_M);
-            const uint32_t b_off = g.b_resident ? (uint32_t)(q * g.taps + tl) * bt16
-                                                : (uint32_t)((q * ntp + tl) % g.b_group) * bt16;
-            if (EBS_IN_RANGE(p, CHK_PIPE_TAB, e, PIPE_MAX_MMAS))
-                mma_tab[e] = make_uint2(a_off | ((uint32_t)(j * TILE_N) << 22), b_off);
-        }
     }
     const int NST = g.n_stages, KS = g.ks, KSS = g.kss, NSUB = g.nsub, SP = g.SP, S = g.S;
     const int nchunks = g.nchunks, nwg = g.nwg;
@@ -641,7 +642,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
     // lost its parallelism (wide 1x1 layers 15-20% slower, and no better with twelve epilogue warps).  The other roles
     // need fewer than 96.  The increase waits in hardware until the CTA's pool has the registers, so the counts must fit
     // into what the launch allots: checked at compile time.  (80 / 56 / 128 measured best of three splits.)
-    constexpr int REG_LAUNCH = 96, REG_EXP = 80, REG_MID = 56, REG_EPI = 128;
+    constexpr int REG_LAUNCH = 96, REG_EXP = 80, REG_MID = 64, REG_EPI = 128;
     static_assert(8 * REG_EXP + 4 * REG_MID + 8 * REG_EPI <= 20 * REG_LAUNCH, "setmaxnreg: the roles' registers exceed the CTA's pool");
     static_assert(PIPE_EPI_WARP0 == 12 && PIPE_EPI_WARPS == 8 && PIPE_THREADS == 640, "role layout changed: revisit the register split");
     if (warp < 8) {
@@ -798,7 +799,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
             const uint32_t r_acc = cluster_addr(&acc_peer[0], 0), r_b = cluster_addr(&b_peer, 0);
             bool ok = true;
             if (my_items > 0 && resident) {
-                ok = mbar_wait_bounded_hot(&b_full, 0u, abortp, wait_limit);
+                ok = mbar_wait_bounded_warp(&b_full, 0u, abortp, wait_limit);
                 if (ok && lane0) mbar_arrive_cluster(r_b);
             }
             int st = 0, bs = 0;
@@ -807,19 +808,21 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
                 const int buf = g.nbuf == 2 ? (it & 1) : 0;
                 const int use = g.nbuf == 2 ? (it >> 1) : it;
                 if (use > 0) {
-                    if (!mbar_wait_bounded_hot(&acc_empty[buf], (uint32_t)((use - 1) & 1), abortp, wait_limit)) break;
+                    if (!mbar_wait_bounded_warp(&acc_empty[buf], (uint32_t)((use - 1) & 1), abortp, wait_limit)) break;
                     if (lane0) mbar_arrive_cluster(r_acc + 8u * (uint32_t)buf);
                 }
                 int ph = 0, wg = 0;
                 for (int c = 0; c < nchunks && ok; ++c) {
-                    if (!mbar_wait_bounded_hot(&st_full[st], st_round & 1u, abortp, wait_limit)) { ok = false; break; }
+                    if (!mbar_wait_bounded_warp(&st_full[st], st_round & 1u, abortp, wait_limit)) { ok = false; break; }
                     if (lane0) mbar_arrive_cluster(r_st + 8u * (uint32_t)st);
                     if (!resident) {
                         const int wgr = wg + wg_rot >= nwg ? wg + wg_rot - nwg : wg + wg_rot;
                         const int words = min(KSS, p.CW - wgr * KSS);
-                        const int ntiles = words * (g.ph_tap0[ph + 1] - g.ph_tap0[ph]);
-                        for (int i0 = 0; i0 < ntiles; i0 += GB) {
-                            if (!mbar_wait_bounded_hot(&bs_full[bs], bs_round & 1u, abortp, wait_limit)) { ok = false; break; }
+                        const int rows = g.ph_rows[ph], cols = g.ph_cols[ph];
+                        const PipeSlot sl = g.slot[ph];
+                        for (int q = 0, r = 0, s = 0; q < words;) {
+                            if ((s += sl.cols) >= cols) { s = 0; if ((r += sl.rows) >= rows) { r = 0; q += sl.words; } }
+                            if (!mbar_wait_bounded_warp(&bs_full[bs], bs_round & 1u, abortp, wait_limit)) { ok = false; break; }
                             if (lane0) mbar_arrive_cluster(r_bs + 8u * (uint32_t)bs);
                             if (++bs == NBS) { bs = 0; ++bs_round; }
                         }
@@ -832,24 +835,57 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
         }
       } else if (warp >= PIPE_ISSUER_WARP && warp < PIPE_ISSUER_WARP + n_iss) {
         // =========================== issuers ===========================
-        const int k_iss = warp - PIPE_ISSUER_WARP;                // this warp takes the MMAs k_iss, k_iss + n_iss, ... of a chunk
+        const int k_iss = warp - PIPE_ISSUER_WARP;                // this warp owns the accumulators k_iss, k_iss + n_iss, ...
         // The issuing thread is a pipeline stage of its own: every address is advanced by additions (descriptor start
         // addresses are in 16-byte units), a handful of instructions per MMA.
         constexpr uint32_t IDESC = PAIR ? (umma_idesc_i8(TILE_N) & ~(0x1Fu << 24)) | ((256u >> 4) << 24) : umma_idesc_i8(TILE_N);
         constexpr uint32_t BT16 = B_TILE_BYTES >> 4;
         const bool skip_mma = (p.test_flags & 1) != 0;            // test hook: issue nothing, so that waits run out
-        bool ok = my_items == 0 || !resident || mbar_wait_bounded_hot(&b_full, 0u, abortp, wait_limit);
-        if (PAIR && ok && my_items > 0 && resident) ok = mbar_wait_cluster_hot(&b_peer, 0u, abortp, wait_limit);
+        bool ok = my_items == 0 || !resident || mbar_wait_bounded_warp(&b_full, 0u, abortp, wait_limit);
+        if (PAIR && ok && my_items > 0 && resident) ok = mbar_wait_cluster_warp(&b_peer, 0u, abortp, wait_limit);
         const uint64_t da_ring = umma_desc_interleaved(smem_u32(stages), (uint32_t)(SP * 16));
         const uint64_t db_res = umma_desc_sw32(smem_u32(b_res));   // resident tiles, or slot 0 of the ring
         const uint32_t da_lo = (uint32_t)da_ring, da_hi = (uint32_t)(da_ring >> 32);
         const uint32_t db_lo = (uint32_t)db_res, db_hi = (uint32_t)(db_res >> 32);
-        const uint32_t stage16 = (uint32_t)(g.stage_bytes >> 4);
-        const int m_sub = g.m_sub;
-        const uint32_t leader = (tid & 31) == 0 ? 1u : 0u;
-        auto mma_issue = [](uint32_t ld, uint32_t d, uint32_t al, uint32_t ah, uint32_t bl, uint32_t bh, uint32_t idesc, uint32_t accu) {
-            if constexpr (PAIR) umma_i8_split_pair(ld, d, al, ah, bl, bh, idesc, accu);
-            else umma_i8_split(ld, d, al, ah, bl, bh, idesc, accu);
+        const uint32_t stage16 = (uint32_t)(g.stage_bytes >> 4), word16 = (uint32_t)(g.a_word_bytes >> 4);
+        const int m_sub = g.m_sub, my_acc = m_sub / n_iss;        // accumulators k_iss, k_iss + n_iss, ... of a tile
+        const uint32_t a_first = (uint32_t)(uni(k_iss) * UMMA_M), a_step = (uint32_t)(n_iss * UMMA_M);
+        const uint32_t d_first = (uint32_t)(uni(k_iss) * TILE_N), d_step = (uint32_t)(n_iss * TILE_N), b_first = uni(db_lo);
+        const uint32_t leader = elect_one() ? 1u : 0u;
+        // `steps` rows of `cols` taps (or `steps` words of a 1 x 1 layer), into every accumulator of this warp: straight-line
+        // code for the tap rows and accumulator counts that occur, run by one elected lane.  (Behind a test of the lane number
+        // instead of elect.sync every MMA moves its operands to uniform registers on its own: 64 -> 64 3x3 at 56x56, batch 256
+        // takes 75 us instead of 62.)
+        auto issue_n = [&](auto cols_tag, auto acc_tag, int steps, uint32_t d0, uint32_t a, uint32_t a_inc, uint32_t b, uint32_t b_inc,
+                           uint32_t accu) {
+            constexpr int COLS = decltype(cols_tag)::value, ACC = decltype(acc_tag)::value;
+            if (elect_one()) {
+#pragma unroll 1
+                for (int i = 0; i < steps; ++i, a += a_inc, b += b_inc) {
+#pragma unroll
+                    for (int s = 0; s < COLS; ++s) {
+#pragma unroll
+                        for (int j = 0; j < ACC; ++j) {
+                            const uint32_t d = d0 + (uint32_t)j * d_step, al = a + (uint32_t)s + (uint32_t)j * a_step, bl = b + (uint32_t)s * BT16;
+                            if constexpr (PAIR) umma_i8_split_pair(1u, d, al, da_hi, bl, db_hi, IDESC, s > 0 ? 1u : accu);
+                            else umma_i8_split(1u, d, al, da_hi, bl, db_hi, IDESC, s > 0 ? 1u : accu);
+                        }
+                    }
+                    accu = 1u;
+                }
+            }
+            __syncwarp();
+        };
+        auto issue = [&](int steps, int cols, uint32_t d0, uint32_t a, uint32_t a_inc, uint32_t b, uint32_t b_inc, uint32_t accu) {
+            auto with = [&](auto acc_tag) {
+                if (cols == 1) issue_n(std::integral_constant<int, 1>{}, acc_tag, steps, d0, a, a_inc, b, b_inc, accu);
+                else if (cols == 2) issue_n(std::integral_constant<int, 2>{}, acc_tag, steps, d0, a, a_inc, b, b_inc, accu);
+                else if (cols == 3) issue_n(std::integral_constant<int, 3>{}, acc_tag, steps, d0, a, a_inc, b, b_inc, accu);
+                else for (int i = 0; i < steps; ++i, accu = 1u)
+                    issue_n(std::integral_constant<int, 1>{}, acc_tag, cols, d0, a + (uint32_t)i * a_inc, 1u, b + (uint32_t)i * b_inc, BT16, accu);
+            };
+            if (my_acc == 1) with(std::integral_constant<int, 1>{});
+            else with(std::integral_constant<int, 2>{});
         };
         // (a pair: the odd CTA's shared window lies at a fixed distance from this one's in the cluster window)
         const uint32_t peer_delta = PAIR ? cluster_addr(&abort_flag, 1) - smem_u32(&abort_flag) : 0u;
@@ -863,52 +899,53 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
             const int buf = g.nbuf == 2 ? (it & 1) : 0;
             const int use = g.nbuf == 2 ? (it >> 1) : it;          // how often this accumulator set was used before
             if (use > 0) {                                          // its epilogue must have drained it
-                if (!mbar_wait_bounded_hot(&acc_empty[buf], (uint32_t)((use - 1) & 1), abortp, wait_limit)) break;
-                if (PAIR && !mbar_wait_cluster_hot(&acc_peer[buf], (uint32_t)((use - 1) & 1), abortp, wait_limit)) break;
+                if (!mbar_wait_bounded_warp(&acc_empty[buf], (uint32_t)((use - 1) & 1), abortp, wait_limit)) break;
+                if (PAIR && !mbar_wait_cluster_warp(&acc_peer[buf], (uint32_t)((use - 1) & 1), abortp, wait_limit)) break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const uint32_t tmem_d = tmem_base + (uint32_t)(buf * m_sub * TILE_N);
             int ph = 0, wg = 0;
             for (int c = 0; c < nchunks; ++c) {
-                if (!mbar_wait_bounded_hot(&st_full[st], st_round & 1u, abortp, wait_limit)) { ok = false; break; }
-                if (PAIR && !mbar_wait_cluster_hot(&st_peer[st], st_round & 1u, abortp, wait_limit)) { ok = false; break; }
+                if (!mbar_wait_bounded_warp(&st_full[st], st_round & 1u, abortp, wait_limit)) { ok = false; break; }
+                if (PAIR && !mbar_wait_cluster_warp(&st_peer[st], st_round & 1u, abortp, wait_limit)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 if (!skip_mma) {
-                    const int wgr = wg + wg_rot >= nwg ? wg + wg_rot - nwg : wg + wg_rot;
-                    const int words = min(KSS, p.CW - wgr * KSS);
-                    const int t0 = g.ph_tap0[ph], ntp = g.ph_tap0[ph + 1] - t0;
-                    const uint2* tab = mma_tab + KSS * m_sub * t0;
-                    const int zero_n = c == 0 ? m_sub : 0;         // the first MMA into each accumulator of a tile overwrites it
-                    const uint32_t a_lo = da_lo + (uint32_t)st * stage16;
+                    const int wgr = uni(wg + wg_rot >= nwg ? wg + wg_rot - nwg : wg + wg_rot);
+                    const int words = min(KSS, p.CW - wgr * KSS), rows = uni(g.ph_rows[ph]), cols = uni(g.ph_cols[ph]);
+                    const uint32_t a0 = uni(da_lo + (uint32_t)st * stage16 + (uint32_t)g.ph_shift[ph]) + a_first;
+                    const uint32_t d0 = uni(tmem_d) + d_first;
+                    uint32_t accu = c == 0 ? 0u : 1u;              // the first MMA into each accumulator of a tile overwrites it
                     if (resident) {
-                        const uint32_t b_lo = db_lo + (uint32_t)((wgr * KSS) * g.taps + t0) * BT16;
-                        const int n = words * ntp * m_sub;
-                        uint2 e = tab[k_iss];
-                        for (int i = k_iss; i < n; i += n_iss) {
-                            const uint2 nxt = tab[i + n_iss];             // (past the end: inside the table's allocation)
-                            mma_issue(leader, tmem_d + (e.x >> 22), a_lo + (e.x & 0x3FFFFFu), da_hi, b_lo + e.y, db_hi, IDESC,
-                                          i >= zero_n ? 1u : 0u);
-                            e = nxt;
+                        const uint32_t b0 = b_first + (uint32_t)((wgr * KSS) * g.taps + uni(g.ph_tap0[ph])) * BT16;
+                        if (rows * cols == 1) {
+                            issue(words, 1, d0, a0, word16, b0, (uint32_t)g.taps * BT16, accu);
+                        } else {
+                            for (int q = 0; q < words; ++q, accu = 1u)
+                                issue(rows, cols, d0, a0 + (uint32_t)q * word16, (uint32_t)g.Wq, b0 + (uint32_t)(q * g.taps) * BT16,
+                                      (uint32_t)cols * BT16, accu);
                         }
                     } else {
-                        // streamed weights: the chunk's (word, tap) tiles in order, GB consecutive tiles per ring slot
-                        const int ntiles = words * ntp;
-                        int i = k_iss;
-                        for (int i0 = 0; i0 < ntiles; i0 += GB) {
-                            if (!mbar_wait_bounded_hot(&bs_full[bs], bs_round & 1u, abortp, wait_limit)) { ok = false; break; }
-                            if (PAIR && !mbar_wait_cluster_hot(&bs_peer[bs], bs_round & 1u, abortp, wait_limit)) { ok = false; break; }
-                            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                            const uint32_t b_lo = db_lo + (uint32_t)(bs * GB) * BT16;
-                            const int n = (i0 + min(GB, ntiles - i0)) * m_sub;
-                            uint2 e = tab[i];
-                            for (; i < n; i += n_iss) {
-                                const uint2 nxt = tab[i + n_iss];
-                                mma_issue(leader, tmem_d + (e.x >> 22), a_lo + (e.x & 0x3FFFFFu), da_hi, b_lo + e.y, db_hi, IDESC,
-                                              i >= zero_n ? 1u : 0u);
-                                e = nxt;
+                        // streamed weights, slot by slot
+                        const PipeSlot sl = g.slot[ph];
+                        for (int q = 0; q < words && ok; q += sl.words) {
+                            for (int r = 0; r < rows && ok; r += sl.rows) {
+                                for (int s = 0; s < cols; s += sl.cols) {
+                                    if (!mbar_wait_bounded_warp(&bs_full[bs], bs_round & 1u, abortp, wait_limit)) { ok = false; break; }
+                                    if (PAIR && !mbar_wait_cluster_warp(&bs_peer[bs], bs_round & 1u, abortp, wait_limit)) { ok = false; break; }
+                                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                                    const int nq = min(sl.words, words - q), nr = min(sl.rows, rows - r), ns = min(sl.cols, cols - s);
+                                    uint32_t b_lo = uni(db_lo + (uint32_t)(bs * GB) * BT16), a_lo = a0 + (uint32_t)q * word16 + (uint32_t)(r * g.Wq + s);
+                                    if (rows * cols == 1) {
+                                        issue(nq, 1, d0, a_lo, word16, b_lo, BT16, accu);
+                                    } else {
+                                        for (int i = 0; i < nq; ++i, a_lo += word16, b_lo += (uint32_t)(nr * ns) * BT16, accu = 1u)
+                                            issue(nr, ns, d0, a_lo, (uint32_t)g.Wq, b_lo, (uint32_t)ns * BT16, accu);
+                                    }
+                                    accu = 1u;
+                                    mma_commit(leader, &bs_empty[bs]);
+                                    if (++bs == NBS) { bs = 0; ++bs_round; }
+                                }
                             }
-                            mma_commit(leader, &bs_empty[bs]);
-                            if (++bs == NBS) { bs = 0; ++bs_round; }
                         }
                         if (!ok) break;
                     }
@@ -954,18 +991,20 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
                         if (++wg == nwg) { wg = 0; ++ph; }
                         const int wgr = wg + wg_rot >= nwg ? wg + wg_rot - nwg : wg + wg_rot;
                         const int words = min(KSS, p.CW - wgr * KSS);
-                        const int t0 = g.ph_tap0[ph], ntaps = g.ph_tap0[ph + 1] - t0, ntiles = words * ntaps;
-                        for (int i0 = 0; i0 < ntiles; i0 += GB) {
+                        const int rows = g.ph_rows[ph], cols = g.ph_cols[ph], t0 = g.ph_tap0[ph];
+                        const PipeSlot sl = g.slot[ph];
+                        int q0 = 0, r0 = 0, s0 = 0;
+                        while (q0 < words) {
                             if (bs_round > 0) {                     // the MMAs that read this slot one round ago must be done
                                 const bool free = mbar_wait_bounded_hot(&bs_empty[bs], (bs_round - 1) & 1u, abortp, wait_limit);
                                 if (!__all_sync(0xffffffffu, free)) { ok = false; break; }
                             }
-                            const int n = min(GB, ntiles - i0);
+                            const int nr = min(sl.rows, rows - r0), ns = min(sl.cols, cols - s0), n = min(sl.words, words - q0) * nr * ns;
                             if (lane == 0) mbar_arrive_expect_tx(&bs_full[bs], bytes * (uint32_t)n);
                             __syncwarp();
-                            if (lane < n) {
-                                const int t = i0 + lane;                          // tile of the chunk: word-major, taps inside
-                                const int q = t / ntaps, ts = t0 + (t - q * ntaps);
+                            if (lane < n) {                          // tile of the slot: word-major, rows, taps of a row
+                                const int per = nr * ns, w = per == 1 ? lane : lane / per, t = lane - w * per, rr = nr == 1 ? 0 : t / ns;
+                                const int q = q0 + w, ts = t0 + (r0 + rr) * cols + s0 + (t - rr * ns);
                                 const size_t src = ((size_t)(s_tap_id[ts] * p.CW + wgr * KSS + q) * p.Co16 + co0) * 32;
                                 // (a copy skipped by the range-checked build leaves its barrier incomplete: the CTA then gives
                                 // up at its bounded wait, which is reported as well)
@@ -973,6 +1012,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
                                     bulk_copy_g2s(b_res + (bs * GB + lane) * B_TILE_BYTES, p.w8 + src, bytes, &bs_full[bs]);
                             }
                             if (++bs == NBS) { bs = 0; ++bs_round; }
+                            if ((s0 += sl.cols) >= cols) { s0 = 0; if ((r0 += sl.rows) >= rows) { r0 = 0; q0 += sl.words; } }
                         }
                     }
                 }
@@ -986,7 +1026,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
         const int vwarp = (warp & 3) + 4 * half;                 // TMEM lane quarter = warp % 4 (hardware rule)
         const int row = (warp & 3) * 32 + (tid & 31);
         const bool plain_ok = !AFFINE && !p.ch_scale && !p.ch_bias && !p.residual && !p.res_packed && !p.y_nchw &&
-                              (p.Co & 3) == 0;
+                              (p.Co & 31) == 0;
         // layers with per-channel terms or a shortcut and without integer output (the layers of a network)
         const bool affine_ok = AFFINE && !p.acc && !p.y_nchw && (p.Co & 31) == 0 && !(p.residual && p.res_packed);
         for (int it = 0; it < my_items; ++it) {
@@ -997,7 +1037,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
             int ptile, ctile;
             item_of(it, ptile, ctile);
             const int co0 = ctile * TILE_N;
-            if (AFFINE && (FORM != 0 || (affine_ok && co0 + TILE_N <= p.Co))) {
+            if (AFFINE && (FORM != 0 || affine_ok)) {
                 if constexpr (AFFINE)
                     pipe_epilogue_terms<TILE_N, EPI_G, FORM == 0>(p, g, tmem_base + (uint32_t)(buf * g.m_sub * TILE_N), g.m_sub, vwarp,
                                                                   (PAIR ? 2 * ptile + crank : ptile) * g.tile_pix + row, co0,
@@ -1018,7 +1058,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
                 if constexpr (FORM != 0) {
                     if constexpr (!AFFINE) pipe_epilogue_packed_g<TILE_N, EPI_G>(p, tmem_acc, vwarp, gp, pvalid, co0);
                 } else {
-                    if (plain_ok && co0 + TILE_N <= p.Co) pipe_epilogue_plain_g<TILE_N, 1>(p, tmem_acc, vwarp, gp, pvalid, co0);
+                    if (plain_ok) pipe_epilogue_plain_g<TILE_N, 1>(p, tmem_acc, vwarp, gp, pvalid, co0);
                     else umma_epilogue<TILE_N, AFFINE>(p, tmem_acc, vwarp, gp, pvalid, 0, co0);
                 }
             }
@@ -1104,7 +1144,7 @@ int launch_conv_umma_pipe_pair(const ConvParams& p, dim3 /*grid*/, cudaStream_t 
     const PipeGeom g = pipe_geometry(p, 256, pipe_sm_count(), p.pipe_m_sub, true);
     if (!g.ok) return EBS_ERR_UNSUPPORTED;
     if (!p.zero_words) return EBS_ERR_CUDA;                   // the device's zero page could not be found
-    if (pipe_packed_only(p, 256)) return launch_conv_umma_pipe_pair_form<AB, 1>(p, g, st);
+    if (pipe_packed_only(p)) return launch_conv_umma_pipe_pair_form<AB, 1>(p, g, st);
     return launch_conv_umma_pipe_pair_form<AB, 0>(p, g, st);
 }
 
@@ -1113,7 +1153,7 @@ int launch_conv_umma_pipe(const ConvParams& p, dim3 /*grid*/, cudaStream_t st) {
     const PipeGeom g = pipe_geometry(p, TILE_N, pipe_sm_count(), p.pipe_m_sub);
     if (!g.ok) return EBS_ERR_UNSUPPORTED;                    // the geometry does not apply: nothing is launched
     if (!p.zero_words) return EBS_ERR_CUDA;                   // the device's zero page could not be found
-    if (pipe_packed_only(p, TILE_N)) {
+    if (pipe_packed_only(p)) {
         if constexpr (TILE_N >= 128) {
             if (pipe_hold_applies(p, TILE_N)) return launch_conv_umma_pipe_form<AB, TILE_N, 2>(p, g, st);
         }

@@ -312,6 +312,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
                     }
                     if (c0 + 64 < N && co0 + c0 + 64 < p.Co) load_shortcut(c0 + 64);
                     bytes_to_planes(cr, nb, planes);
+                    if (p.Co - co0 - c0 < 32) mask_planes(planes, p.Co - co0 - c0);
                     uint32_t* dst = p.packed_next + (gpz * p.CWo + ((co0 + c0) >> 5)) * nb;
                     if (pvalid && EBS_IN_RANGE(p, CHK_UT_PN, (dst - p.packed_next) + nb - 1, p.lim_pn)) store_plane_words(planes, nb, dst);
                 }
@@ -321,7 +322,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
         // =========================== issuer ===========================
         const bool levels = p.w_levels != 0;
         const bool skip_mma = (p.test_flags & 1) != 0;   // test hook: issue nothing, so that waits run out
-        const uint32_t leader = lane == 0 ? 1u : 0u;
+        const uint32_t leader = elect_one() ? 1u : 0u;
         const uint64_t da0 = umma_desc_interleaved(smem_u32(stages), (uint32_t)(SP * 16)), db0 = umma_desc_sw32(smem_u32(stages + g.b_off));
         const uint32_t da_hi = (uint32_t)(da0 >> 32), db_hi = (uint32_t)(db0 >> 32), ones_lo = (uint32_t)umma_desc_sw32(smem_u32(ones));
         const uint32_t idesc = umma_idesc_i8(N), word16 = (uint32_t)g.a_word_bytes >> 4, bt16 = (uint32_t)b_tile >> 4;
@@ -336,16 +337,27 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
                 const uint32_t stage16 = (uint32_t)(st * g.stage_bytes) >> 4;
                 uint32_t a_word = (uint32_t)da0 + stage16 + (uint32_t)g.ph_shift[ph], b_lo = (uint32_t)db0 + stage16;
                 uint32_t accu = c == 0 ? 0u : 1u;
-                for (int q = 0; q < nq; ++q, a_word += word16) {
-                    uint32_t a_row = a_word;
-                    for (int r = 0; r < rows; ++r, a_row += (uint32_t)g.Wq) {
-                        for (int s = 0; s < cols; ++s, b_lo += bt16) {
-                            umma_i8_split(leader, tmem, a_row + (uint32_t)s, da_hi, b_lo, db_hi, idesc, accu);
-                            if (levels) umma_i8_split(leader, tmem + (uint32_t)N, a_row + (uint32_t)s, da_hi, ones_lo, db_hi, umma_idesc_i8(16), accu);
-                            accu = 1u;
+                if (elect_one()) {
+                    for (int q = 0; q < nq; ++q, a_word += word16) {
+                        uint32_t a_row = a_word;
+                        for (int r = 0; r < rows; ++r, a_row += (uint32_t)g.Wq) {
+                            if (cols == 3 && !levels) {
+                                umma_i8_split(1u, tmem, a_row, da_hi, b_lo, db_hi, idesc, accu);
+                                umma_i8_split(1u, tmem, a_row + 1u, da_hi, b_lo + bt16, db_hi, idesc, 1u);
+                                umma_i8_split(1u, tmem, a_row + 2u, da_hi, b_lo + 2u * bt16, db_hi, idesc, 1u);
+                                b_lo += 3u * bt16;
+                                accu = 1u;
+                                continue;
+                            }
+                            for (int s = 0; s < cols; ++s, b_lo += bt16) {
+                                umma_i8_split(1u, tmem, a_row + (uint32_t)s, da_hi, b_lo, db_hi, idesc, accu);
+                                if (levels) umma_i8_split(1u, tmem + (uint32_t)N, a_row + (uint32_t)s, da_hi, ones_lo, db_hi, umma_idesc_i8(16), accu);
+                                accu = 1u;
+                            }
                         }
                     }
                 }
+                __syncwarp();
                 umma_commit_pred(leader, &empty[st]);
                 if (c == nchunks - 1) umma_commit_pred(leader, &acc_full);
             }
@@ -553,9 +565,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
 
 int tile_sm_count();
 
-// Whether the epilogue can run a thread per pixel (forms 1 and 2): packed planes only, whole 32-channel words.
+// Whether the epilogue can run a thread per pixel (forms 1 and 2): packed planes only; an fp32 shortcut is read in whole
+// 32-channel groups.
 inline bool tile_thread_epilogue(const ConvParams& p, int tile_n) {
-    return p.packed_next && !p.acc && !p.y && !p.w_levels && (p.Co & 31) == 0 && (tile_n & 31) == 0 && !(p.residual && p.res_packed);
+    return p.packed_next && !p.acc && !p.y && !p.w_levels && (tile_n & 31) == 0 && !(p.residual && (p.res_packed || (p.Co & 31) != 0));
 }
 
 template <int AB, int FORM>

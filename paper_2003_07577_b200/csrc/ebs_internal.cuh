@@ -19,6 +19,7 @@ struct ConvParams {
     int N, H, W, CW;
     int Co, Ho, Wo, CWo;              // CWo = ceil(Co/32)
     int kh, kw, sh, sw, ph, pw;
+    int x_words;                      // 32-bit words of one pixel and 32-channel word of x: the plane count, 8 for byte codes
     int KK;                           // kh*kw*CW reduction words per plane pair
     int P;                            // N*Ho*Wo output pixels
     int32_t* __restrict__ acc;        // nullable, [P][Co]
@@ -44,7 +45,6 @@ struct ConvParams {
     int tile_split;                   // tile kernel: CTAs the reduction is split over (0 = chosen by the library)
     int pipe_m_sub;                   // persistent pipeline kernel: accumulators per super-tile (0 = chosen by the library)
     float one;                        // 1.0f: multiplier of packed additions (see f32x2_add_one)
-    int acc_small;                    // 1: every accumulator of the layer is below 2^22 in magnitude (worst case of its sizes and bit counts)
     // Extents of the buffers, for the range-checked build (EBS_CHECKED); filled in every build.
     long long lim_x, lim_w;           // 32-bit words of the packed activations (bytes / 4 on the byte-code path) and of the weight plane words
     long long lim_w8;                 // bytes of the weight byte image

@@ -80,11 +80,6 @@ __device__ __forceinline__ bool fused_follows(const FusedLayer& P, const FusedLa
            L.w_in == P.w_in && L.src == P.dst && L.c_out == P.c_out;
 }
 
-// The same value in every lane, known to the compiler to be so: what the issuing warps feed into descriptors and loop
-// bounds has to live in uniform registers, or every MMA moves four operands there first (130 clocks an MMA instead of 40).
-__device__ __forceinline__ int uni(int v) { return __shfl_sync(0xffffffffu, v, 0); }
-__device__ __forceinline__ uint32_t uni(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
-
 struct FusedTerms {                                     // per-channel terms in the order the epilogue reads them
     float cs[64], cb[64], pcs[64], pcb[64];             // of the layer, and of the held projection
 };
@@ -388,7 +383,7 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
     } else if (warp >= FUSED_ISSUER_WARP && warp < FUSED_ISSUER_WARP + FUSED_ISSUERS) {
         // =========================== MMAs ===========================
         const int k_iss = warp - FUSED_ISSUER_WARP;
-        const uint32_t leader = lane == 0 ? 1u : 0u;
+        const uint32_t leader = elect_one() ? 1u : 0u;
         uint32_t par = 0u;                               // bit t: parity of the number of layers that used tile t so far
         int prev = -1, prev_tiles = 0, n_copies = 0;     // the last layer with an epilogue
         bool ok = true;
@@ -427,7 +422,7 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                     continue;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                if (leader) {
+                if (elect_one()) {
                     const uint32_t tm = tm0 + (uint32_t)t * tm_step;
                     const uint64_t da_t = da0 + (uint64_t)(t * UMMA_M);
                     uint64_t db = db0;

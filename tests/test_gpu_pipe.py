@@ -90,6 +90,21 @@ def test_pipe_geometries(ebs, U, oracle, case, affine):
     _check(ebs, U, oracle, n, c, co, k, s, pad, h, w, 3, 4, 4, affine=affine)
 
 
+@pytest.mark.parametrize("affine", [False, True])
+@pytest.mark.parametrize("case", [
+    # n, c, co, k, stride, pad, h, w, nb
+    (3, 64, 96, 3, 1, 1, 13, 12, 5),      # whole groups, the last tile of 64 or 128 channels partly empty
+    (2, 96, 33, 1, 1, 0, 17, 9, 3),       # one channel in the last group
+    (2, 64, 159, 3, 2, 1, 15, 14, 8),     # one channel short of a whole group
+    (1, 160, 300, 5, 1, 2, 12, 11, 4),    # streamed weights: slots of parts of a tap row (256-channel tile)
+    (1, 96, 256, 7, 1, 3, 12, 11, 7),     # seven taps a row
+    (2, 320, 256, 3, 2, 1, 12, 11, 6),    # streamed weights: the four phases' slots differ
+])
+def test_pipe_ragged_tiles_and_ring_slots(ebs, U, oracle, case, affine):
+    n, c, co, k, s, pad, h, w, nb = case
+    _check(ebs, U, oracle, n, c, co, k, s, pad, h, w, 3, 5, nb, affine=affine)
+
+
 @pytest.mark.parametrize("case", [
     # n, c, co, k, stride, pad, h, w, ab
     (3, 64, 256, 1, 1, 0, 20, 19, 6),     # resident weights, one pair-tile and a ragged second one

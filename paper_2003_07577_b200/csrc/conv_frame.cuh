@@ -363,6 +363,35 @@ __device__ __forceinline__ bool mbar_wait_bounded_warp(uint64_t* bar, uint32_t p
 __device__ __forceinline__ uint32_t join_codes(const uint32_t (&m)[4]) {
     return __byte_perm(__byte_perm(m[0], m[1], 0x0040), __byte_perm(m[2], m[3], 0x0040), 0x5410);
 }
+// Codes of a pair of values w = fl(y / step).  NB = 0: planes counted at run time, or eight of them.  NB = 1..7: without a
+// logic-pipe instruction -- fl(w + 1/2) / 2^NB, clamped to [0, 1] by the addition itself (the scaling is exact), times 2^NB
+// rounded down.  What is clamped above comes out as 2^NB: codes_to_planes spreads that bit over the planes.
+template <int NB>
+__device__ __forceinline__ void code_pair(uint64_t w, uint64_t one2, uint64_t half2, float hi2, uint32_t& lo, uint32_t& hi) {
+    if constexpr (NB == 0 || NB == 8) {
+        w = f32x2_add_one(w, one2, half2);
+        lo = code_pattern(__uint_as_float((uint32_t)w), hi2);
+        hi = code_pattern(__uint_as_float((uint32_t)(w >> 32)), hi2);
+    } else {
+        constexpr float UP = (float)(1 << NB), DOWN = 1.0f / UP;
+        float a, b;
+        asm("fma.rn.sat.f32 %0, %1, %2, %3;\n" : "=f"(a) : "f"(__uint_as_float((uint32_t)w)), "f"(DOWN), "f"(0.5f * DOWN));
+        asm("fma.rn.sat.f32 %0, %1, %2, %3;\n" : "=f"(b) : "f"(__uint_as_float((uint32_t)(w >> 32))), "f"(DOWN), "f"(0.5f * DOWN));
+        lo = __float_as_uint(__fmaf_rd(a, UP, 8388608.0f));
+        hi = __float_as_uint(__fmaf_rd(b, UP, 8388608.0f));
+    }
+}
+// Code registers of code_pair<NB> -> plane words.
+template <int NB>
+__device__ __forceinline__ void codes_to_planes(const uint32_t (&cr)[8], int nb, uint32_t (&planes)[8]) {
+    if constexpr (NB == 0 || NB == 8) {
+        bytes_to_planes(cr, nb, planes);
+    } else {
+        bytes_to_planes(cr, NB + 1, planes);
+#pragma unroll
+        for (int j = 0; j < NB; ++j) planes[j] |= planes[NB];
+    }
+}
 // Byte i of a register as fp32, exactly, without the conversion pipe: 2^23 + byte, minus 2^23.
 __device__ __forceinline__ float byte_to_float(uint32_t w, int i) {
     return __fadd_rn(__uint_as_float(__byte_perm(w, 0x4B000000u, 0x7540u + (uint32_t)i)), -8388608.0f);
@@ -380,7 +409,7 @@ __device__ __forceinline__ float term_at(const float* t, int co, int Co, float i
 // order.  The terms come from shared memory as broadcast 16-byte reads (read through the cache channel by channel they
 // were two thirds of the instructions of this function); products and sums are packed two to an instruction
 // (f32x2_add_one).  The ReLU is not applied: the quantizer's clamp at zero gives the same codes.
-template <int RES>
+template <int RES, int NB = 0>
 __device__ __forceinline__ void terms_codes32(const uint32_t (&v)[32], float S, float one, const float4* cs, const float4* cb,
                                               const float (&res)[32], const uint32_t (&rbyte)[8], float res_scale,
                                               float inv_next, float hi2, uint32_t (&cr)[8]) {
@@ -398,9 +427,7 @@ __device__ __forceinline__ void terms_codes32(const uint32_t (&v)[32], float S, 
         for (int h = 0; h < 2; ++h) {
             if (RES == 1) w[h] = f32x2_add_one(w[h], one2, f32x2_pack(res[16 * h + bb], res[16 * h + 8 + bb]));
             if (RES == 2) w[h] = f32x2_add_one(w[h], one2, f32x2_mul_rn(rs2, f32x2_pack(byte_to_float(rbyte[bb], 2 * h), byte_to_float(rbyte[bb], 2 * h + 1))));
-            w[h] = f32x2_add_one(f32x2_mul_rn(w[h], inv2), one2, half2);
-            m[2 * h] = code_pattern(__uint_as_float((uint32_t)w[h]), hi2);
-            m[2 * h + 1] = code_pattern(__uint_as_float((uint32_t)(w[h] >> 32)), hi2);
+            code_pair<NB>(f32x2_mul_rn(w[h], inv2), one2, half2, hi2, m[2 * h], m[2 * h + 1]);
         }
         const uint32_t c4 = join_codes(m);
         cr[bb] = __funnelshift_l(c4, c4, bb);
@@ -458,6 +485,7 @@ __device__ __forceinline__ void store_values32(const uint64_t (&yy)[2][8], bool 
 }
 
 // The same without per-channel terms and shortcut.
+template <int NB = 0>
 __device__ __forceinline__ void plain_codes32(const uint32_t (&v)[32], float S, float one, float inv_next, float hi2, uint32_t (&cr)[8]) {
     const uint64_t S2 = f32x2_pack(S, S), one2 = f32x2_pack(one, one), inv2 = f32x2_pack(inv_next, inv_next), half2 = f32x2_pack(0.5f, 0.5f);
 #pragma unroll
@@ -465,10 +493,8 @@ __device__ __forceinline__ void plain_codes32(const uint32_t (&v)[32], float S, 
         uint32_t m[4];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            uint64_t w = f32x2_mul_rn(f32x2_pack((float)(int)v[16 * h + bb], (float)(int)v[16 * h + 8 + bb]), S2);
-            w = f32x2_add_one(f32x2_mul_rn(w, inv2), one2, half2);
-            m[2 * h] = code_pattern(__uint_as_float((uint32_t)w), hi2);
-            m[2 * h + 1] = code_pattern(__uint_as_float((uint32_t)(w >> 32)), hi2);
+            const uint64_t w = f32x2_mul_rn(f32x2_pack((float)(int)v[16 * h + bb], (float)(int)v[16 * h + 8 + bb]), S2);
+            code_pair<NB>(f32x2_mul_rn(w, inv2), one2, half2, hi2, m[2 * h], m[2 * h + 1]);
         }
         const uint32_t c4 = join_codes(m);
         cr[bb] = __funnelshift_l(c4, c4, bb);

@@ -312,13 +312,13 @@ __device__ __forceinline__ void pipe_store_planes(const uint32_t (&planes)[8], i
 // accumulators and the finished code registers is alive at a time -- the general form above keeps the 32 fp32 images
 // as well, which at 96 registers costs spills and the parallelism of the instruction stream.
 // left: channels of the layer from this group on (a last group of fewer than 32 writes zero bits behind them).
-template <int G>
+template <int G, int NB = 0>
 __device__ __forceinline__ void pipe_group32_packed(const uint32_t (&v)[32], bool pvalid, float S, float inv_next, int nb, int qmax,
                                                     uint32_t* dst, const ConvParams& p, PlaneHold<G>& hold, int left) {
     uint32_t cr[8];
-    plain_codes32(v, S, p.one, inv_next, (float)(2 * qmax + 1), cr);
+    plain_codes32<NB>(v, S, p.one, inv_next, (float)(2 * qmax + 1), cr);
     uint32_t planes[8];
-    bytes_to_planes(cr, nb, planes);
+    codes_to_planes<NB>(cr, nb, planes);
     if (left < 32) mask_planes(planes, left);
     pipe_store_planes(planes, nb, dst, pvalid, hold, p);
 }
@@ -406,7 +406,7 @@ __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, cons
                     if (p.y && ok && EBS_IN_RANGE(p, CHK_PIPE_Y, gpz * p.Co + c + 31, p.lim_out)) store_values32(yy, p.relu != 0, p.y + gpz * p.Co + c);
                     if (p.packed_next) value_codes32(yy, p.one, p.inv_next, hi2, cr);
                 } else {
-                    terms_codes32<RES>(v, p.S, p.one, cs, cb, res, rbyte, p.res_scale, p.inv_next, hi2, cr);
+                    terms_codes32<RES, NB>(v, p.S, p.one, cs, cb, res, rbyte, p.res_scale, p.inv_next, hi2, cr);
                 }
             }
             if (c0 + 32 < cend) {
@@ -417,7 +417,7 @@ __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, cons
             }
             if (some && (!VALUES || p.packed_next)) {
                 uint32_t planes[8];
-                bytes_to_planes(cr, nb, planes);
+                codes_to_planes<NB>(cr, nb, planes);
                 if (p.Co - c < 32) mask_planes(planes, p.Co - c);
                 pipe_store_planes(planes, nb, p.packed_next + (gpz * p.CWo + (c >> 5)) * nb, ok, hold, p);
             }
@@ -451,7 +451,7 @@ __device__ __forceinline__ void pipe_epilogue_plain_g(const ConvParams& p, uint3
         const size_t o = (size_t)gp * p.Co + co0 + c0;
         uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + ((co0 + c0) >> 5)) * nb;
         if (want_q && !p.acc && !p.y) {
-            pipe_group32_packed(v, pvalid, S, inv_next, nb, qmax, dst, p, hold, 32);
+            pipe_group32_packed<G>(v, pvalid, S, inv_next, nb, qmax, dst, p, hold, 32);
         } else if (want_q) {
             pipe_group32<true>(p, v, o, pvalid, S, inv_next, nb, qmax, dst);
         } else {
@@ -483,7 +483,7 @@ __device__ __forceinline__ void pipe_epilogue_packed_nb(const ConvParams& p, uin
         tmem_ld16_wait(lo);
         tmem_ld16_wait(hi);
         uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + ((co0 + c0) >> 5)) * nb;
-        pipe_group32_packed(v, pvalid, S, inv_next, nb, qmax, dst, p, hold, p.Co - co0 - c0);
+        pipe_group32_packed<G, NB>(v, pvalid, S, inv_next, nb, qmax, dst, p, hold, p.Co - co0 - c0);
     }
 }
 

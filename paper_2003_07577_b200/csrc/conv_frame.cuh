@@ -360,9 +360,11 @@ __device__ __forceinline__ bool mbar_wait_bounded_warp(uint64_t* bar, uint32_t p
 }
 
 // Four requantized codes (low bytes of code_pattern results) -> one register, channel order as in planes_to_bytes.
-__device__ __forceinline__ uint32_t join_codes(const uint32_t (&m)[4]) {
-    return __byte_perm(__byte_perm(m[0], m[1], 0x0040), __byte_perm(m[2], m[3], 0x0040), 0x5410);
+// k256 = 256, unknown to the compiler: the first step as multiply-adds, which the logic pipe has no part in.
+__device__ __forceinline__ uint32_t join_codes(const uint32_t (&m)[4], uint32_t k256) {
+    return __byte_perm(m[1] * k256 + m[0], m[3] * k256 + m[2], 0x5410);
 }
+__device__ __forceinline__ uint32_t k256_of(float one) { return (__float_as_uint(one) & 0x00800000u) >> 15; }
 // Codes of a pair of values w = fl(y / step).  NB = 0: planes counted at run time, or eight of them.  NB = 1..7: without a
 // logic-pipe instruction -- fl(w + 1/2) / 2^NB, clamped to [0, 1] by the addition itself (the scaling is exact), times 2^NB
 // rounded down.  What is clamped above comes out as 2^NB: codes_to_planes spreads that bit over the planes.
@@ -413,6 +415,7 @@ template <int RES, int NB = 0>
 __device__ __forceinline__ void terms_codes32(const uint32_t (&v)[32], float S, float one, const float4* cs, const float4* cb,
                                               const float (&res)[32], const uint32_t (&rbyte)[8], float res_scale,
                                               float inv_next, float hi2, uint32_t (&cr)[8]) {
+    const uint32_t k256 = k256_of(one);
     const uint64_t S2 = f32x2_pack(S, S), one2 = f32x2_pack(one, one), inv2 = f32x2_pack(inv_next, inv_next);
     const uint64_t half2 = f32x2_pack(0.5f, 0.5f), rs2 = f32x2_pack(res_scale, res_scale);
 #pragma unroll
@@ -429,7 +432,7 @@ __device__ __forceinline__ void terms_codes32(const uint32_t (&v)[32], float S, 
             if (RES == 2) w[h] = f32x2_add_one(w[h], one2, f32x2_mul_rn(rs2, f32x2_pack(byte_to_float(rbyte[bb], 2 * h), byte_to_float(rbyte[bb], 2 * h + 1))));
             code_pair<NB>(f32x2_mul_rn(w[h], inv2), one2, half2, hi2, m[2 * h], m[2 * h + 1]);
         }
-        const uint32_t c4 = join_codes(m);
+        const uint32_t c4 = join_codes(m, k256);
         cr[bb] = __funnelshift_l(c4, c4, bb);
     }
 }
@@ -455,6 +458,7 @@ __device__ __forceinline__ void terms_values32(const uint32_t (&v)[32], float S,
     }
 }
 __device__ __forceinline__ void value_codes32(const uint64_t (&yy)[2][8], float one, float inv_next, float hi2, uint32_t (&cr)[8]) {
+    const uint32_t k256 = k256_of(one);
     const uint64_t one2 = f32x2_pack(one, one), inv2 = f32x2_pack(inv_next, inv_next), half2 = f32x2_pack(0.5f, 0.5f);
 #pragma unroll
     for (int bb = 0; bb < 8; ++bb) {
@@ -465,7 +469,7 @@ __device__ __forceinline__ void value_codes32(const uint64_t (&yy)[2][8], float 
             m[2 * h] = code_pattern(__uint_as_float((uint32_t)w), hi2);
             m[2 * h + 1] = code_pattern(__uint_as_float((uint32_t)(w >> 32)), hi2);
         }
-        const uint32_t c4 = join_codes(m);
+        const uint32_t c4 = join_codes(m, k256);
         cr[bb] = __funnelshift_l(c4, c4, bb);
     }
 }
@@ -487,6 +491,7 @@ __device__ __forceinline__ void store_values32(const uint64_t (&yy)[2][8], bool 
 // The same without per-channel terms and shortcut.
 template <int NB = 0>
 __device__ __forceinline__ void plain_codes32(const uint32_t (&v)[32], float S, float one, float inv_next, float hi2, uint32_t (&cr)[8]) {
+    const uint32_t k256 = k256_of(one);
     const uint64_t S2 = f32x2_pack(S, S), one2 = f32x2_pack(one, one), inv2 = f32x2_pack(inv_next, inv_next), half2 = f32x2_pack(0.5f, 0.5f);
 #pragma unroll
     for (int bb = 0; bb < 8; ++bb) {
@@ -496,7 +501,7 @@ __device__ __forceinline__ void plain_codes32(const uint32_t (&v)[32], float S, 
             const uint64_t w = f32x2_mul_rn(f32x2_pack((float)(int)v[16 * h + bb], (float)(int)v[16 * h + 8 + bb]), S2);
             code_pair<NB>(f32x2_mul_rn(w, inv2), one2, half2, hi2, m[2 * h], m[2 * h + 1]);
         }
-        const uint32_t c4 = join_codes(m);
+        const uint32_t c4 = join_codes(m, k256);
         cr[bb] = __funnelshift_l(c4, c4, bb);
     }
 }

@@ -202,7 +202,7 @@ __device__ __forceinline__ void fused_unit_codes(const FusedUnitEnv& E, uint32_t
             uint32_t m[4];
             fused_code(w[e], E, m[0], m[1]);
             fused_code(w[4 + e], E, m[2], m[3]);
-            words[e] = join_codes(m) & z;
+            words[e] = join_codes(m, k256_of(__uint_as_float((uint32_t)E.one2))) & z;
         }
         if (E.c_out & 15) {                              // channels past c_out
 #pragma unroll
@@ -215,7 +215,7 @@ __device__ __forceinline__ void fused_unit_codes(const FusedUnitEnv& E, uint32_t
             uint32_t m[4];
             fused_code(w[2 * e], E, m[0], m[1]);
             fused_code(w[2 * e + 1], E, m[2], m[3]);
-            words[e] = join_codes(m) & z;
+            words[e] = join_codes(m, k256_of(__uint_as_float((uint32_t)E.one2))) & z;
         }
         if (E.c_out & 31) {
 #pragma unroll

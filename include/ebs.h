@@ -204,8 +204,9 @@ int ebs_conv2d_mixed(const void *packed_x_dev, int n, int h, int w, const void *
  *           (AND + POPC + shift-add per plane pair);
  *   10..18  warp-level tensor-pipe kernels (int8 mma.sync; the planes of a channel merged into
  *           its byte in registers, one MMA per 32 channels of a tap);
- *   19..23  tcgen05 kernels, any stride (same product, 128 pixels x 16/32/64/128/256 channels
- *           per CTA, accumulator in tensor memory);
+ *   19..23  tcgen05 tile kernels, strides up to 2 (same product, a thread block per 128 pixels x
+ *           16/32/64/128/256 channels, accumulator in tensor memory; a deep reduction on few tiles is
+ *           split over a cluster of up to eight blocks);
  *   24..28  tcgen05 strip kernels for stride-1 layers and strided 1x1 layers (every input
  *           pixel expanded once per CTA; weights read from the byte image);
  *   29..33  the same as persistent CTAs that keep the weight bytes of their channel tile in

@@ -437,6 +437,67 @@ __device__ __forceinline__ void terms_codes32(const uint32_t (&v)[32], float S, 
     }
 }
 
+// Tensor memory -> registers in fragments: 16 rows x 32 columns, lane l holds columns 8 o + 2 (l % 4) + {0, 1}, o = 0..3, of rows
+// l / 4 (v[4 o], v[4 o + 1]) and l / 4 + 8 (v[4 o + 2], v[4 o + 3]).
+__device__ __forceinline__ void tmem_ld_frag_issue(uint32_t taddr, uint32_t (&v)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(taddr));
+}
+// 4 x 4 transposition among the lanes of a quad: t[r][.] of lane q <-> t[q][.] of lane r.
+__device__ __forceinline__ void quad_transpose(uint32_t (&t)[4][2]) {
+    const uint32_t q = threadIdx.x & 3u;
+#pragma unroll
+    for (int d = 1; d <= 2; d *= 2) {
+        const bool up = (q & (uint32_t)d) != 0;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            if (r & d) continue;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? t[r][e] : t[r | d][e], d);
+                if (up) t[r][e] = got;
+                else t[r | d][e] = got;
+            }
+        }
+    }
+}
+// terms_codes32 on fragments: lo / hi hold rows 0-15 / 16-31 of the group, so a lane needs the terms of eight channels only
+// (s, b: channel 8 o + 2 q + e at 2 o + e) for four pixels, rows l / 4 + 8 r.  The codes pass through the quad afterwards:
+// cr = those of row l / 4 + 8 q.  rb[r][e]: byte o = shortcut code of row r, that channel; res likewise.
+template <int RES, int NB>
+__device__ __forceinline__ void terms_codes_frag(const uint32_t (&lo)[16], const uint32_t (&hi)[16], float S, float one, const float (&s)[8],
+                                                 const float (&b)[8], const float (&res)[32], const uint32_t (&rb)[4][2], float res_scale,
+                                                 float inv_next, float hi2, uint32_t (&cr)[8]) {
+    const uint32_t k256 = k256_of(one);
+    const uint64_t S2 = f32x2_pack(S, S), one2 = f32x2_pack(one, one), inv2 = f32x2_pack(inv_next, inv_next);
+    const uint64_t half2 = f32x2_pack(0.5f, 0.5f), rs2 = f32x2_pack(res_scale, res_scale);
+    const int q = (int)(threadIdx.x & 3u);
+    uint32_t t[4][2];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        uint32_t m0[4], m1[4];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            const uint32_t a0 = r < 2 ? lo[4 * o + 2 * (r & 1)] : hi[4 * o + 2 * (r & 1)];
+            const uint32_t a1 = r < 2 ? lo[4 * o + 2 * (r & 1) + 1] : hi[4 * o + 2 * (r & 1) + 1];
+            uint64_t w = f32x2_mul_rn(f32x2_pack((float)(int)a0, (float)(int)a1), S2);
+            w = f32x2_add_one(f32x2_mul_rn(w, f32x2_pack(s[2 * o], s[2 * o + 1])), one2, f32x2_pack(b[2 * o], b[2 * o + 1]));
+            if (RES == 1) w = f32x2_add_one(w, one2, f32x2_pack(res[8 * r + 2 * o], res[8 * r + 2 * o + 1]));
+            if (RES == 2) w = f32x2_add_one(w, one2, f32x2_mul_rn(rs2, f32x2_pack(byte_to_float(rb[r][0], o), byte_to_float(rb[r][1], o))));
+            code_pair<NB>(f32x2_mul_rn(w, inv2), one2, half2, hi2, m0[o], m1[o]);
+        }
+        const uint32_t c0 = join_codes(m0, k256), c1 = join_codes(m1, k256);
+        t[r][0] = __funnelshift_l(c0, c0, 2 * q);
+        t[r][1] = __funnelshift_l(c1, c1, 2 * q + 1);
+    }
+    quad_transpose(t);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) { cr[2 * j] = t[j][0]; cr[2 * j + 1] = t[j][1]; }
+}
+
 // The same in two steps, for layers that want the fp32 values too: pair (h, bb) = channels 16 h + bb and 16 h + 8 + bb.
 template <int RES>
 __device__ __forceinline__ void terms_values32(const uint32_t (&v)[32], float S, float one, const float4* cs, const float4* cb,

@@ -1,7 +1,7 @@
 // Persistent, warp-specialised bit-plane convolution on the tcgen05 tensor cores for every layer
 // geometry the ResNet stacks contain: stride-1 k x k, strided k x k, and 1 x 1 at any stride.
 //
-// Arithmetic as in conv_umma_kernel (Eq. 13-14 regrouped channel by channel): the planes of a packed
+// Arithmetic (Eq. 13-14 regrouped channel by channel): the planes of a packed
 // word are merged back into one byte per channel and one int8 MMA per (tap, reduction word) retires
 // all Wb*Ab plane pairs of its 32 channels.  What this kernel adds:
 //
@@ -21,7 +21,7 @@
 //    stream through the stage ring by cp.async.bulk, a stage ahead of the MMAs.
 //  * Roles (20 warps): warps 0-7 expand (packed words -> byte strips, global loads two chunks ahead), warps 8-9
 //    issue the MMAs (two warps when a tile has an even number of accumulators: each owns the accumulators of one
-//    parity; a single warp needs 140-180 clocks per MMA and was the bound of the k x k layers), warp 10 fetches weight
+//    parity, so that one's waits and addresses run while the other issues), warp 10 fetches weight
 //    tiles (every lane one tile of a ring slot), warps 12-19 run the epilogue out of tensor memory while the next
 //    tile's MMAs fill the other accumulator set.
 //  * Bit <-> byte transposes by rotate and bit-select: with v_k = rotl(w_k, k) the byte register of
@@ -327,12 +327,19 @@ __device__ __forceinline__ void pipe_group32_packed(const uint32_t (&v)[32], boo
 // residual block): NHWC, packed planes and / or fp32 out.  The warp walks its (accumulator, 32-channel
 // group) units; the next unit's shortcut and terms are requested before the current one is packed and stored.  The terms of
 // a group pass through 64 words of shared memory of the warp's own (one load and one store a lane, then broadcast reads):
-// read channel by channel through the cache they cost more than the arithmetic (64 -> 256 1x1 at 56x56, batch 256: 225 us
-// against 119 us for the same layer without terms).  VALUES: fp32 output may be wanted too.
+// read channel by channel through the cache they cost more than the arithmetic (64 -> 256 1x1 at 56x56, batch 256: 225 us,
+// and 97 us for the same layer without terms).  With packed planes only, the accumulators are loaded as fragments, so that a
+// lane reads the terms of eight channels instead of 32 (that layer 194 -> 182 us, 8 bits 230 -> 206; 128 -> 128 3x3 at
+// 28x28 50.5 -> 44.6).  VALUES: fp32 output may be wanted too.
 template <int TILE_N, int G, bool VALUES, int NB, int RES>
 __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, const FrameGeom& g, uint32_t tmem_set, int m_sub, int vwarp,
                                                     int f0, int co0, float* terms) {
-    const int lane = (int)(threadIdx.x & 31), at = (lane & 7) * 4 + (lane >> 3);
+    // Packed planes only: the accumulators come as fragments (terms_codes_frag), a lane's own pixel is row l / 4 + 8 (l % 4) of
+    // the warp's 32 and its terms are those of eight channels; else the lane's pixel is row l and it reads all terms.
+    constexpr bool FRAG = !VALUES;
+    const int lane = (int)(threadIdx.x & 31), quad = lane & 3;
+    const int at = FRAG ? ((lane & 7) >> 1) * 8 + (lane >> 3) * 2 + (lane & 1) : (lane & 7) * 4 + (lane >> 3);
+    if constexpr (FRAG) f0 += (lane >> 2) + 8 * quad - lane;
     const uint32_t trow = tmem_set + ((uint32_t)((vwarp & 3) * 32) << 16);
     constexpr int COLS = TILE_N / 2;
     const int cbeg = (vwarp >> 2) * COLS, cend = COLS == 32 ? cbeg + 32 : min(cbeg + COLS, p.Co - co0);   // (cend: groups start below)
@@ -363,7 +370,18 @@ __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, cons
         const bool in = c + lane < p.Co;
         t_scale = p.ch_scale && in ? __ldg(p.ch_scale + c + lane) : 1.0f;
         t_bias = p.ch_bias && in ? __ldg(p.ch_bias + c + lane) : -0.0f;
-        if constexpr (RES == 1) {
+        if constexpr (RES == 1 && FRAG) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int gr = __shfl_sync(0xffffffffu, gp, (lane & ~3) | r);      // the pixel of row r
+                const float2* r2 = reinterpret_cast<const float2*>(p.residual + (size_t)gr * p.Co + c + 2 * quad);
+#pragma unroll
+                for (int o = 0; o < 4; ++o) {
+                    const float2 t = __ldg(r2 + 4 * o);
+                    res[8 * r + 2 * o] = t.x; res[8 * r + 2 * o + 1] = t.y;
+                }
+            }
+        } else if constexpr (RES == 1) {
             const float4* r4 = reinterpret_cast<const float4*>(p.residual + (size_t)gp * p.Co + c);
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
@@ -395,18 +413,31 @@ __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, cons
                 uint32_t v[32], rbyte[8];
                 uint32_t (&lo)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[0]);
                 uint32_t (&hi)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[16]);
-                tmem_ld16_issue(trow + (uint32_t)(j * TILE_N + c0), lo);
-                tmem_ld16_issue(trow + (uint32_t)(j * TILE_N + c0 + 16), hi);
+                if constexpr (FRAG) {
+                    tmem_ld_frag_issue(trow + (uint32_t)(j * TILE_N + c0), lo);
+                    tmem_ld_frag_issue(trow + (16u << 16) + (uint32_t)(j * TILE_N + c0), hi);
+                } else {
+                    tmem_ld16_issue(trow + (uint32_t)(j * TILE_N + c0), lo);
+                    tmem_ld16_issue(trow + (uint32_t)(j * TILE_N + c0 + 16), hi);
+                }
+                if constexpr (RES == 2) planes_to_bytes<8>(rw, rbyte);
                 tmem_ld16_wait(lo);
                 tmem_ld16_wait(hi);
-                if constexpr (RES == 2) planes_to_bytes<8>(rw, rbyte);
                 if constexpr (VALUES) {
                     uint64_t yy[2][8];
                     terms_values32<RES>(v, p.S, p.one, cs, cb, res, rbyte, p.res_scale, yy);
                     if (p.y && ok && EBS_IN_RANGE(p, CHK_PIPE_Y, gpz * p.Co + c + 31, p.lim_out)) store_values32(yy, p.relu != 0, p.y + gpz * p.Co + c);
                     if (p.packed_next) value_codes32(yy, p.one, p.inv_next, hi2, cr);
                 } else {
-                    terms_codes32<RES, NB>(v, p.S, p.one, cs, cb, res, rbyte, p.res_scale, p.inv_next, hi2, cr);
+                    uint32_t rb[4][2];
+                    if constexpr (RES == 2) {
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) { rb[r][0] = rbyte[2 * r]; rb[r][1] = rbyte[2 * r + 1]; }
+                        quad_transpose(rb);
+                    }
+                    const float4 s0 = cs[2 * quad], s1 = cs[2 * quad + 1], b0 = cb[2 * quad], b1 = cb[2 * quad + 1];
+                    const float s[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w}, b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+                    terms_codes_frag<RES, NB>(lo, hi, p.S, p.one, s, b, res, rb, p.res_scale, p.inv_next, hi2, cr);
                 }
             }
             if (c0 + 32 < cend) {
@@ -589,9 +620,9 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
         else { ptile = idx / g.n_ctiles; ctile = idx - ptile * g.n_ctiles; }
     };
 
-    // Issuing warps: a single warp issuing every MMA of a CTA needs 140-180 clocks per MMA (measured: its busy time, not
-    // the tensor pipe, bounded the k x k layers and the GEMM), so with two or four accumulators per tile two warps share the
-    // work, each owning the accumulators of one parity -- MMAs of different warps never touch the same accumulator, so
+    // Issuing warps: the tensor pipe needs 49, 65 and 129 clocks for an MMA of 64, 128 and 256 channels (operands from shared
+    // memory) and one warp can issue that fast, but its waits and addresses between the runs of MMAs cannot hide, so with two
+    // or four accumulators per tile two warps share the work, each owning the accumulators of one parity -- MMAs of different warps never touch the same accumulator, so
     // no order between the warps is needed.  One accumulator: one issuing warp.
     const int n_iss = (g.m_sub & 1) == 0 ? PIPE_ISSUERS : 1;
     if (tid == 0) {

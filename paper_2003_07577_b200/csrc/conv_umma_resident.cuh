@@ -17,7 +17,7 @@
 //                   pack, arrive on the accumulator's "empty" barrier;
 //     so the expansion of tile i+1, the MMAs of tile i and the epilogue of tile i-1 overlap.
 // Applies when the strip kernel does, the weight tiles fit (<= 150 KB) and the layer has no window-sum
-// term (w_levels = 0).  Bounded waits and the abort path as in conv_umma_kernel.
+// term (w_levels = 0).  Bounded waits and the abort path as in the other tcgen05 kernels.
 #pragma once
 
 #include "conv_umma_strip.cuh"

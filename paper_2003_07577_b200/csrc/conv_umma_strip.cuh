@@ -1,7 +1,7 @@
 // Stride-1 (and strided 1x1) bit-plane convolution on the tcgen05 tensor cores with every input pixel
 // expanded ONCE per thread block, however many filter taps read it.
 //
-// Arithmetic as in conv_umma_kernel: the planes of a packed word are merged back into one byte per
+// Arithmetic: the planes of a packed word are merged back into one byte per
 // channel and one int8 MMA per (tap, reduction word) retires all Wb*Ab plane pairs of its 32 channels.
 // What differs is the addressing.  Output pixels are numbered in the zero-padded input frame,
 //     f = (n * Hp + hp) * Wp + wp,   Hp = H + 2 pad_h,  Wp = W + 2 pad_w,
@@ -20,7 +20,7 @@
 // reads, so one thread fetches it with cp.async.bulk straight into shared memory, completing on the
 // stage's "full" mbarrier; no thread touches weight bits.
 //
-// Roles, barriers, bounded waits and the epilogue are those of conv_umma_kernel (warps 0-7 expand,
+// Roles, barriers, bounded waits and the epilogue as in the other tcgen05 kernels (warps 0-7 expand,
 // warp 8 issues; two stages).
 #pragma once
 

@@ -672,7 +672,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
     // registers want about 126 registers; with the 96 a CTA of 20 warps starts with it spilled and its instruction stream
     // lost its parallelism (wide 1x1 layers 15-20% slower, and no better with twelve epilogue warps).  The other roles
     // need fewer than 96.  The increase waits in hardware until the CTA's pool has the registers, so the counts must fit
-    // into what the launch allots: checked at compile time.  (80 / 56 / 128 measured best of three splits.)
+    // into what the launch allots: checked at compile time.  (The middle role spilled at 56, which cost the GEMM a fifth.)
     constexpr int REG_LAUNCH = 96, REG_EXP = 80, REG_MID = 64, REG_EPI = 128;
     static_assert(8 * REG_EXP + 4 * REG_MID + 8 * REG_EPI <= 20 * REG_LAUNCH, "setmaxnreg: the roles' registers exceed the CTA's pool");
     static_assert(PIPE_EPI_WARP0 == 12 && PIPE_EPI_WARPS == 8 && PIPE_THREADS == 640, "role layout changed: revisit the register split");

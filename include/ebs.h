@@ -204,9 +204,10 @@ int ebs_conv2d_mixed(const void *packed_x_dev, int n, int h, int w, const void *
  *           (AND + POPC + shift-add per plane pair);
  *   10..18  warp-level tensor-pipe kernels (int8 mma.sync; the planes of a channel merged into
  *           its byte in registers, one MMA per 32 channels of a tap);
- *   19..23  tcgen05 tile kernels, strides up to 2 (same product, a thread block per 128 pixels x
+ *   19..23  tcgen05 tile kernels (same product, a thread block per 128 pixels x
  *           16/32/64/128/256 channels, accumulator in tensor memory; a deep reduction on few tiles is
- *           split over a cluster of up to eight blocks);
+ *           split over a cluster of up to eight blocks; strides above 2, more than 64 taps and images
+ *           too wide for a strip of input pixels: every tap's pixels expanded anew);
  *   24..28  tcgen05 strip kernels for stride-1 layers and strided 1x1 layers (every input
  *           pixel expanded once per CTA; weights read from the byte image);
  *   29..33  the same as persistent CTAs that keep the weight bytes of their channel tile in

@@ -187,6 +187,31 @@ static bool tile_kernel_pays(const ConvParams& p, int sms) {
     return tiles <= 3LL * sms;
 }
 
+// What a layer that the tile kernel fits only in its per-tap form runs on instead of it; -1: nothing is better.  The per-tap
+// form expands 128 pixels for every (tap, word), whatever the channels and bits, and its epilogue for 32-bit results and
+// weight levels takes long beside a short reduction; the warp-level kernels' time grows with the plane pairs.
+static int choose_beside_tap_form(const ConvParams& p, const ebs_conv_desc* d, int sms) {
+    constexpr int MS_BASE = NUM_CONV_VARIANTS + NUM_CONV_MMA_VARIANTS + NUM_CONV_UMMA_VARIANTS + NUM_CONV_STRIP_VARIANTS +
+                            NUM_CONV_RESIDENT_VARIANTS;
+    const int mma = NUM_CONV_VARIANTS + choose_mma_variant(d->w_bits, d->a_bits, p.P, p.Co, sms);
+    const bool words32 = p.acc || p.y;
+    auto strip = [&](int v) { return p.kh * p.kw > 1 && conv_mma_strip_applies(p, v); };
+    // at most 32 channels leave most of an accumulator empty (64 -> 16 3x3 at 200x224, two images: 10-13 us by strip, 25)
+    if (p.Co <= 32) return strip(p.Co <= 16 ? 0 : 1) ? MS_BASE + (p.Co <= 16 ? 0 : 1) : mma;
+    if (p.KK <= 18 && p.Co * p.CW <= 256) {
+        // few pixels (64 -> 64 3x3 at 16x224: 6.9 against 8.5 us), or 32-bit results of not too many channels (64 -> 64 at 200x224,
+        // two images: 29 against 34; 16 -> 48: 12 against 28; 64 -> 96: 43 either way; 8 -> 128 behind the per-tap warp-level
+        // kernel); the 16-channel tile cannot pack, and is the faster one for the results
+        const bool results = words32 && p.Co <= 96 && p.Co * p.CW <= 128;
+        if ((p.P < (1 << 13) || (results && p.packed_next)) && strip(2)) return MS_BASE + 2;
+        if (results && !p.packed_next && strip(0)) return MS_BASE;
+    }
+    // no strip at all: the per-tap warp-level kernel while there are few plane pairs (3 -> 64 3x3 at 200x224, 32-bit results: 16-20
+    // against 28 us up to four bits, 38 against 29 at six; 64 -> 64 3x3 stride 3, two bits: 18 against 22, four bits: 23 and 22)
+    if ((words32 || p.w_levels) && p.KK * (d->w_bits + d->a_bits) <= 72) return mma;
+    return -1;
+}
+
 // A validated, fully decided launch: nothing has been enqueued when conv_plan returns.
 struct ConvPlan {
     ConvParams p;
@@ -285,9 +310,11 @@ static int conv_plan(const void* packed_x, int n, int h, int w, const void* pack
         // few channels on many pixels: the warp-level strip kernel (16 -> 16 3x3 at 32x32, batch 128: 7.1 us, the tile kernel,
         // whose accumulator is then mostly empty, 22; 32 -> 32 at 16x16: 7.2 against 8.3)
         const bool few = p.Co <= 32 && p.CW <= 2 && d->kh * d->kw > 1 && (long long)p.P > 128LL * sm_count();
+        const int beside = mma_ok && tile >= 0 && conv_umma_tap_form(p) ? choose_beside_tap_form(p, d, sm_count()) : -1;
         if (pipe >= 0) variant = PIPE_BASE + pipe;
         else if (mma_ok && few && p.Co <= 16 && conv_mma_strip_applies(p, 0)) variant = MS_BASE;
         else if (mma_ok && few && conv_mma_strip_applies(p, 1)) variant = MS_BASE + 1;
+        else if (beside >= 0) variant = beside;
         else if (tile >= 0) variant = NUM_CONV_VARIANTS + NUM_CONV_MMA_VARIANTS + tile;
         else if (mma_ok && p.Co <= 16 && d->kh * d->kw > 1 && conv_mma_strip_applies(p, 0)) variant = MS_BASE;
         else variant = mma_ok ? NUM_CONV_VARIANTS + choose_mma_variant(d->w_bits, d->a_bits, p.P, p.Co, sm_count())

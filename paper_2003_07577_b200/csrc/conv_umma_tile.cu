@@ -37,6 +37,11 @@ float conv_umma_cost(const ConvParams& p, int variant) {
     return g.ok ? g.cost : -1.0f;
 }
 
+bool conv_umma_tap_form(const ConvParams& p) {
+    FrameGeom g{};
+    return tile_tap_form(p, g);
+}
+
 unsigned long long conv_umma_tile_timeouts() {
     unsigned long long v = 0;
 #define EBS_TILE_SUM(AB) v += conv_umma_timeouts_a##AB();

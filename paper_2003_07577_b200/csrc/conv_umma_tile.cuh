@@ -18,6 +18,8 @@
 // memory with a thread per pixel; 2 = the same with per-channel terms and shortcut; 0 = everything else: the sums go
 // through shared memory and a warp finishes 32 channels of a pixel at a time (coalesced stores; the codes go back into
 // shared memory as bytes and a thread packs the 32 channels of a pixel).
+// TAP: the per-tap form (tap_geometry), a kernel of its own because its addresses cost the strip layers 0.4 us a launch where
+// both were compiled into one.
 // Weight levels (w_levels): the window sum of the codes is one more accumulator column, an MMA against a tile of ones.
 // Every wait is bounded as in the other tcgen05 kernels.
 #pragma once
@@ -32,9 +34,12 @@ constexpr int TILE_MAX_STAGES = 16, TILE_MAX_SPLIT = 8;
 constexpr int TILE_SMEM_SHARED = 104 * 1024, TILE_SMEM_MAX = 216 * 1024;   // two CTAs / one CTA per SM
 
 struct TileGeom : FrameGeom {
+    int per_tap;                       // 1: per-tap form (tap_geometry)
+    FastDiv div_cw, div_kw;            // per-tap form: reduction word -> tap and channel word, tap -> row and column
     int tile_n, n_ptiles, n_ctiles, split;
     int S, SP, kw;                     // strip pixels, rounded up to 8; words per stage
-    int words;                         // input-channel words of a CTA (the last of a cluster may have fewer)
+    int n_words, words;                // reduction words: input-channel words (per-tap form: times taps), and those of a CTA (the
+                                       // last of a cluster may have fewer)
     int a_word_bytes, b_off, stage_bytes, n_stages;
     int tmem_cols, smem_bytes, part_pitch, xch_off;   // xch_off: where a cluster's CTAs put their sums, from the stages on
     float cost;                        // estimated clocks of the launch
@@ -43,14 +48,40 @@ struct TileGeom : FrameGeom {
 
 inline int tile_round_up(int v, int m) { return (v + m - 1) / m * m; }
 
+// Whether a layer has no strip: one that the expanders cannot hold (3x3 taps on more than 189 pixels of width, 5x5 on more than
+// 91) or no phases in the frame scheme (strides above 2, more than 64 taps).
+inline bool tile_tap_form(const ConvParams& p, FrameGeom& g) {
+    return !frame_geometry(p, g) || UMMA_M + g.max_shift > TILE_SLOTS * TILE_WORKERS;
+}
+// The per-tap form for such layers.  The frame is the outputs
+// themselves and every (tap, word) pair is a word of the reduction with a strip of its own, the 128 input pixels that the
+// tap reads, expanded anew for every tap; the weight byte image has the pairs in that order.
+inline bool tap_geometry(const ConvParams& p, FrameGeom& g) {
+    g = FrameGeom{};
+    const long long frame = (long long)p.N * p.Ho * p.Wo;
+    if (frame >= (1LL << 31) - 4096 || (long long)p.CW * 8 > PIPE_ZERO_WORDS) return false;
+    g.Wq = p.Wo;
+    g.Hq = p.Ho;
+    g.frame = (int)frame;
+    g.div_img = make_fastdiv((uint32_t)(g.Hq * g.Wq));
+    g.div_row = make_fastdiv((uint32_t)g.Wq);
+    g.taps = g.n_ph = g.max_ph_taps = g.ph_rows[0] = g.ph_cols[0] = g.ph_tap0[1] = 1;
+    return true;
+}
+
 // Geometry for a channel tile of tile_n and a split of the reduction (0: the split with the smallest estimate).
 inline TileGeom tile_geometry(const ConvParams& p, int tile_n, int sms, int split_req) {
     TileGeom g{};
-    if (!frame_geometry(p, g)) return g;
+    if (tile_tap_form(p, g)) {
+        if (!tap_geometry(p, g)) return g;
+        g.per_tap = 1;
+        g.div_cw = make_fastdiv((uint32_t)p.CW);
+        g.div_kw = make_fastdiv((uint32_t)p.kw);
+    }
+    g.n_words = p.CW * (g.per_tap ? p.kh * p.kw : 1);
     g.tile_n = tile_n;
     g.S = UMMA_M + g.max_shift;
     g.SP = tile_round_up(g.S, 8);
-    if (g.S > TILE_SLOTS * TILE_WORKERS) return g;
     g.n_ptiles = (g.frame + UMMA_M - 1) / UMMA_M;
     g.n_ctiles = (p.Co + tile_n - 1) / tile_n;
     if (g.n_ctiles > 65535) return g;
@@ -64,10 +95,10 @@ inline TileGeom tile_geometry(const ConvParams& p, int tile_n, int sms, int spli
         if (split_req && split != split_req) continue;
         // A CTA holds its tensor memory while it waits for the others of its cluster, so clusters take at most a quarter of
         // it: no mix of resident blocks can then keep a member from starting (at most three of this kernel fit an SM).
-        if (split > p.CW || (split > 1 && g.tmem_cols > 128)) break;
+        if (split > g.n_words || (split > 1 && g.tmem_cols > 128)) break;
         TileGeom c = g;
-        c.words = (p.CW + split - 1) / split;
-        c.split = (p.CW + c.words - 1) / c.words;
+        c.words = (g.n_words + split - 1) / split;
+        c.split = (g.n_words + c.words - 1) / c.words;
         if (c.split != split) continue;                        // a rank without words
         c.kw = TILE_SLOTS * TILE_WORKERS / c.S;
         if (c.kw > 4) c.kw = 4;
@@ -101,10 +132,13 @@ inline TileGeom tile_geometry(const ConvParams& p, int tile_n, int sms, int spli
         const double ctas = (double)c.n_ptiles * c.n_ctiles * split;
         if (split == TILE_MAX_SPLIT && ctas > sms / 2) continue;   // (more clusters of eight than GPCs run at once: slower)
         const double mma = (double)c.words * c.taps * (17.0 + 0.34 * tile_n + (p.w_levels ? 20.0 : 0.0));
-        const double expand = 1.26 * c.words * c.n_ph * c.S;
         const int cols = tile_n < tile_round_up(p.Co, 32) ? tile_n : tile_round_up(p.Co, 32);
         const double tail = split == 1 ? 21.0 * cols : 1610.0 + 114.0 * cols / split;
-        const double load = ctas / (1.21 * sms);
+        double expand = 1.26 * c.words * c.n_ph * c.S, load = ctas / (1.21 * sms);
+        if (c.per_tap) {                                       // a stage has one MMA per word: its waits dominate, and two CTAs on an
+            expand = chunks * (1150.0 + 200.0 * c.kw);         // SM hide them (fitted to 50 layers x 4 channel tiles)
+            load = ctas / ((split == 1 && c.smem_bytes <= TILE_SMEM_SHARED ? 1.6 : 1.0) * sms);
+        }
         c.cost = (float)((86.0 + (mma > expand ? mma : expand) + tail) * (load > 1.0 ? load : 1.0));
         c.ok = true;
         if (!best.ok || c.cost < best.cost) best = c;
@@ -112,7 +146,7 @@ inline TileGeom tile_geometry(const ConvParams& p, int tile_n, int sms, int spli
     return best;
 }
 
-template <int AB, int FORM>
+template <int AB, int FORM, bool TAP>
 __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const ConvParams p, const TileGeom g) {
     extern __shared__ uint8_t dyn_smem[];
     __shared__ __align__(8) uint64_t full[TILE_MAX_STAGES], empty[TILE_MAX_STAGES], acc_full, xch_full;
@@ -132,7 +166,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
     uint8_t* stages = ones + 512;                        // [NST] x { KW strips, KW * taps weight tiles }; later the partial sums
     volatile int* abortp = &abort_flag;
     const unsigned limit = p.wait_limit;
-    const int w0 = rank * g.words, nw = min(g.words, p.CW - w0);
+    const int w0 = rank * g.words, nw = min(g.words, g.n_words - w0);
     const int nwg = (nw + KW - 1) / KW, nchunks = g.n_ph * nwg;
 
     if (tid == 0) {
@@ -188,15 +222,42 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
                     src[j] = p.x + (size_t)((((int)n * p.H + h) * p.W + w) * p.CW + w0 + slot_q[j]) * AB;
             }
         };
+        // TAP: first input pixel of a slot's window; its image, -1: none
+        int slot_h[TILE_SLOTS], slot_w[TILE_SLOTS], slot_img[TILE_SLOTS];
+        auto window_starts = [&]() {
+#pragma unroll
+            for (int j = 0; j < TILE_SLOTS; ++j) {
+                const uint32_t f = (uint32_t)slot_f[j], n = fastdiv(f, g.div_img), rem = f - n * (uint32_t)(g.Hq * g.Wq);
+                const uint32_t ho = fastdiv(rem, g.div_row), wo = rem - ho * (uint32_t)g.Wq;
+                slot_h[j] = p.sh * (int)ho - p.ph;
+                slot_w[j] = p.sw * (int)wo - p.pw;
+                slot_img[j] = slot_q[j] >= 0 && slot_f[j] < g.frame ? (int)n : -1;
+            }
+        };
+        // TAP: packed words of reduction word q of this CTA for slot j, null: zero bytes
+        auto tap_item = [&](int j, int q) -> const uint32_t* {
+            if (slot_img[j] < 0 || q >= nw) return nullptr;
+            const uint32_t kk = (uint32_t)(w0 + q), tap = fastdiv(kk, g.div_cw), r = fastdiv(tap, g.div_kw);
+            const int h = slot_h[j] + (int)r, w = slot_w[j] + (int)(tap - r * (uint32_t)p.kw);
+            if ((unsigned)h >= (unsigned)p.H || (unsigned)w >= (unsigned)p.W) return nullptr;
+            return p.x + (size_t)(((slot_img[j] * p.H + h) * p.W + w) * p.CW + (int)(kk - tap * (uint32_t)p.CW)) * AB;
+        };
         constexpr int SETS = AB <= 4 ? 4 : 3;            // packed words of SETS - 1 chunks in flight
         uint32_t words[SETS][TILE_SLOTS][AB];
         int ld_ph = 0, ld_wg = 0;
         auto load_next = [&](int set) {
-            if (ld_wg == 0 && ld_ph > 0) phase_pointers(ld_ph);
+            if (!TAP && ld_wg == 0 && ld_ph > 0) phase_pointers(ld_ph);
 #pragma unroll
             for (int j = 0; j < TILE_SLOTS; ++j) {
-                const uint32_t* a = src[j] + (size_t)ld_wg * KW * AB;
-                const bool in = src[j] != nullptr && ld_wg * KW + slot_q[j] < nw;
+                const uint32_t* a;
+                bool in;
+                if constexpr (TAP) {
+                    a = tap_item(j, ld_wg * KW + slot_q[j]);
+                    in = a != nullptr;
+                } else {
+                    a = src[j] + (size_t)ld_wg * KW * AB;
+                    in = src[j] != nullptr && ld_wg * KW + slot_q[j] < nw;
+                }
                 if (in && EBS_IN_RANGE(p, CHK_UT_X, (a - p.x) + AB - 1, p.lim_x)) {
                     ld_dep_words<AB>(a, words[set][j]);
                 } else {
@@ -206,7 +267,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
             }
             if (++ld_wg == nwg) { ld_wg = 0; ++ld_ph; }
         };
-        phase_pointers(0);
+        if constexpr (TAP) window_starts();
+        else phase_pointers(0);
         asm volatile("griddepcontrol.wait;\n" ::: "memory");
 #pragma unroll
         for (int u = 0; u < SETS - 1; ++u)
@@ -571,9 +633,9 @@ inline bool tile_thread_epilogue(const ConvParams& p, int tile_n) {
     return p.packed_next && !p.acc && !p.y && !p.w_levels && (tile_n & 31) == 0 && !(p.residual && (p.res_packed || (p.Co & 31) != 0));
 }
 
-template <int AB, int FORM>
+template <int AB, int FORM, bool TAP>
 int launch_conv_umma_tile_form(const ConvParams& p, const TileGeom& g, cudaStream_t st) {
-    auto kern = conv_umma_tile_kernel<AB, FORM>;
+    auto kern = conv_umma_tile_kernel<AB, FORM, TAP>;
     static bool attr_set[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
@@ -602,10 +664,13 @@ template <int AB, int TILE_N>
 int launch_conv_umma_tile(const ConvParams& p, dim3 /*grid*/, cudaStream_t st) {
     const TileGeom g = tile_geometry(p, TILE_N, tile_sm_count(), p.tile_split);
     if (!g.ok) return EBS_ERR_UNSUPPORTED;                    // the geometry does not apply: nothing is launched
-    if (g.split == 1 && tile_thread_epilogue(p, TILE_N))
-        return p.ch_scale || p.ch_bias || p.residual || p.res_packed ? launch_conv_umma_tile_form<AB, 2>(p, g, st)
-                                                                     : launch_conv_umma_tile_form<AB, 1>(p, g, st);
-    return launch_conv_umma_tile_form<AB, 0>(p, g, st);
+    const bool terms = p.ch_scale || p.ch_bias || p.residual || p.res_packed;
+    const int form = g.split > 1 || !tile_thread_epilogue(p, TILE_N) ? 0 : terms ? 2 : 1;
+    if (g.per_tap)
+        return form == 0 ? launch_conv_umma_tile_form<AB, 0, true>(p, g, st) :
+               form == 1 ? launch_conv_umma_tile_form<AB, 1, true>(p, g, st) : launch_conv_umma_tile_form<AB, 2, true>(p, g, st);
+    return form == 0 ? launch_conv_umma_tile_form<AB, 0, false>(p, g, st) :
+           form == 1 ? launch_conv_umma_tile_form<AB, 1, false>(p, g, st) : launch_conv_umma_tile_form<AB, 2, false>(p, g, st);
 }
 
 constexpr int NUM_TILE_VARIANTS = 5;           // TILE_N = 16, 32, 64, 128, 256

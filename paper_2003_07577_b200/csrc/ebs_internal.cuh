@@ -131,6 +131,7 @@ unsigned long long conv_umma_strip_timeouts();
 const ConvVariant* conv_umma_variant(int a_bits, int variant);
 bool conv_umma_applies(const ConvParams& p, int variant);
 float conv_umma_cost(const ConvParams& p, int variant);   // estimated clocks, negative if it does not apply
+bool conv_umma_tap_form(const ConvParams& p);             // no strip fits the layer: a tile kernel expands every tap anew
 unsigned long long conv_umma_tile_timeouts();
 unsigned long long conv_umma_timeouts();
 

@@ -382,6 +382,9 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
         }
     } else if (warp == TILE_ISSUER) {
         // =========================== issuer ===========================
+        // its waits start with the data's: polls counted while the previous launch still runs would make a slow predecessor
+        // look like a stage that never fills
+        asm volatile("griddepcontrol.wait;\n" ::: "memory");
         const bool levels = p.w_levels != 0;
         const bool skip_mma = (p.test_flags & 1) != 0;   // test hook: issue nothing, so that waits run out
         const uint32_t leader = elect_one() ? 1u : 0u;

@@ -370,8 +370,8 @@ def ebs_test_checked_shrink(elements: int) -> None:
     _check(lib().ebs_test_checked_shrink(int(elements)), "ebs_test_checked_shrink")
 
 
-def ebs_test_set_device_wait(limit: int, skip_mma: bool) -> None:
-    _check(lib().ebs_test_set_device_wait(int(limit), int(bool(skip_mma))), "ebs_test_set_device_wait")
+def ebs_test_set_device_wait(limit: int, skip_mma: int) -> None:
+    _check(lib().ebs_test_set_device_wait(int(limit), int(skip_mma)), "ebs_test_set_device_wait")
 
 
 def ebs_conv2d_i8(x_codes_dev, n, h, w, packed_w_dev, desc, epi=None, acc_out_dev=None, y_out_dev=None,

@@ -509,7 +509,7 @@ int ebs_conv_variant_applies(const ebs_conv_desc* desc, int n, int h, int w, con
 
 int ebs_test_set_device_wait(unsigned int limit, int skip_mma) {
     g_wait_limit = limit == 0 ? (1u << 20) : limit;
-    g_test_flags = skip_mma ? 1 : 0;
+    g_test_flags = skip_mma == 2 ? 2 : skip_mma ? 1 : 0;
     return EBS_OK;
 }
 
@@ -616,7 +616,7 @@ int ebs_resnet_cifar_forward(const unsigned char* images_dev, int n, int img_h, 
     if (!head_host->w8 || head_host->c_in < 1 || head_host->c_in > 64 || head_host->c_out < 1 || head_host->c_out > 256)
         return EBS_ERR_INVALID_ARG;
     return launch_fused_resnet(images_dev, n, img_h, img_w, layers_dev, n_layers, head_host, logits_dev, trace_dev,
-                               trace_stride, static_cast<cudaStream_t>(stream));
+                               trace_stride, g_wait_limit, g_test_flags, static_cast<cudaStream_t>(stream));
 }
 
 int ebs_global_avgpool(const float* y_dev, int n, int hw, int c, float* out_dev, void* stream) {

@@ -66,6 +66,12 @@ __device__ __forceinline__ bool mbar_wait_bounded_hot(uint64_t* bar, uint32_t pa
     return false;
 }
 
+// What a CTA that gave up does before it frees its memory: copies into its shared memory and MMAs that were started may still
+// be under way, and nothing waits for them any more (64 us; either takes a few).
+__device__ __forceinline__ void giveup_drain() {
+    for (int i = 0; i < 64; ++i) __nanosleep(1000);
+}
+
 // Shared-memory matrix descriptor: K-major operand, 32-byte swizzle, rows of 32 bytes (K = 32 int8),
 // 8-row groups 256 bytes apart.
 __device__ __forceinline__ uint64_t umma_desc_sw32(uint32_t smem_addr) {

@@ -1099,16 +1099,19 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
         }
     }
 
-    // a CTA that gave up may still have weight copies in flight towards its shared memory: give them time to land
-    // (bounded) before the block ends and the memory is handed to another block
-    if (warp == PIPE_PRODUCER_WARP && *abortp) {
-        for (int i = 0; i < 64; ++i) __nanosleep(1000);
-    }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
-    if constexpr (PAIR) cluster_sync_all();                   // neither CTA leaves while the other may still arrive on its barriers
-    if (abort_flag != 0 && tid == 0) atomicAdd(&g_umma_timeouts, 1ull);
-    if (warp == PIPE_ISSUER_WARP) {
+    if constexpr (PAIR) {
+        if (abort_flag != 0) giveup_drain();
+        __syncwarp();
+        cluster_sync_all();                                   // neither CTA leaves while the other may still arrive on its barriers
+    }
+    if (warp == PIPE_ISSUER_WARP) {                           // (the block's memory is its own until this warp leaves)
+        if (abort_flag != 0) {
+            giveup_drain();
+            if ((tid & 31) == 0) atomicAdd(&g_umma_timeouts, 1ull);
+        }
+        __syncwarp();
         if constexpr (PAIR)
             asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"((uint32_t)g.tmem_cols)
                          : "memory");

@@ -21,7 +21,8 @@
 // TAP: the per-tap form (tap_geometry), a kernel of its own because its addresses cost the strip layers 0.4 us a launch where
 // both were compiled into one.
 // Weight levels (w_levels): the window sum of the codes is one more accumulator column, an MMA against a tile of ones.
-// Every wait is bounded as in the other tcgen05 kernels.
+// Every wait on an mbarrier is bounded as in the other tcgen05 kernels.  The two cluster barriers of a split launch have no
+// limit of their own: every thread of every CTA reaches both whether it gave up or not, after bounded waits only.
 #pragma once
 
 #include "conv_frame.cuh"
@@ -382,9 +383,6 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
         }
     } else if (warp == TILE_ISSUER) {
         // =========================== issuer ===========================
-        // its waits start with the data's: polls counted while the previous launch still runs would make a slow predecessor
-        // look like a stage that never fills
-        asm volatile("griddepcontrol.wait;\n" ::: "memory");
         const bool levels = p.w_levels != 0;
         const bool skip_mma = (p.test_flags & 1) != 0;   // test hook: issue nothing, so that waits run out
         const uint32_t leader = elect_one() ? 1u : 0u;
@@ -393,6 +391,9 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
         const uint32_t idesc = umma_idesc_i8(N), word16 = (uint32_t)g.a_word_bytes >> 4, bt16 = (uint32_t)b_tile >> 4;
         int st = 0, ph = 0, wg = 0;
         uint32_t round = 0;
+        // its waits start with the data's: polls counted while the previous launch still runs would make a slow predecessor
+        // look like a stage that never fills
+        asm volatile("griddepcontrol.wait;\n" ::: "memory");
         for (int c = 0; c < nchunks; ++c) {
             if (!mbar_wait_bounded_warp(&full[st], round & 1u, abortp, limit)) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
@@ -454,8 +455,6 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
             if (++st == NST) { st = 0; ++round; }
             if (++wg == nwg) { wg = 0; ++ph; }
         }
-        if (*abortp)                                     // copies may still be in flight towards this CTA's shared memory
-            for (int i = 0; i < 64; ++i) __nanosleep(1000);
     }
 
     if constexpr (FORM == 0) {
@@ -505,16 +504,18 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
             if (warp == 0 && abort_flag == 0) {
                 if (lane == 0) mbar_arrive_expect_tx(&xch_full, (uint32_t)split * block_bytes(rank));
                 __syncwarp();
-                if (lane < split && block_bytes(lane) != 0u)
+                const bool mute = (p.test_flags & 2) != 0 && rank == 0;
+                if (lane < split && block_bytes(lane) != 0u && !mute)
                     asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
                                      cluster_addr(part + rank * rows * pitch, (uint32_t)lane)),
                                  "r"(smem_u32(dump + lane * rows * pitch)), "r"(block_bytes(lane)), "r"(cluster_addr(&xch_full, (uint32_t)lane))
                                  : "memory");
             }
             __syncwarp();
-            if (warp < 8) mbar_wait_bounded_warp(&xch_full, 0u, abortp, limit);
+            if (warp < 8 && !mbar_wait_bounded_warp(&xch_full, 0u, abortp, limit)) giveup_drain();
             __syncthreads();
-            // (no CTA may end while the copies out of its memory are under way: every peer reports that it has received all)
+            // (no CTA may end while the copies out of its memory are under way: every peer reports that it has received all, or
+            // has given up and waited for its own)
             asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
         }
         if (warp < 8 && abort_flag == 0) {
@@ -623,9 +624,14 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
 
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
-    if (abort_flag != 0 && tid == 0) atomicAdd(&g_umma_timeouts, 1ull);
-    if (warp == TILE_ISSUER)
+    if (warp == TILE_ISSUER) {                           // (the block's memory is its own until this warp leaves)
+        if (abort_flag != 0) {
+            giveup_drain();
+            if (lane == 0) atomicAdd(&g_umma_timeouts, 1ull);
+        }
+        __syncwarp();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"((uint32_t)g.tmem_cols) : "memory");
+    }
 }
 
 int tile_sm_count();

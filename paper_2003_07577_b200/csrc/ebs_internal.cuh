@@ -41,7 +41,8 @@ struct ConvParams {
     int fold_bits;                    // 32 / fold: bits each folded tap occupies (>= c_in)
     int strip_pix, strip_ks;          // strip kernel only (set by its launcher): pixels of a strip, words per stage
     unsigned wait_limit;              // polls a bounded device-side wait makes before the CTA gives up
-    int test_flags;                   // bit 0 (tests only): the MMA issuer issues nothing, so that waits run out
+    int test_flags;                   // tests only, so that waits run out: bit 0 the MMA issuer issues nothing, bit 1 the first
+                                      // CTA of a tile kernel's cluster sends no sums
     int tile_split;                   // tile kernel: CTAs the reduction is split over (0 = chosen by the library)
     int pipe_m_sub;                   // persistent pipeline kernel: accumulators per super-tile (0 = chosen by the library)
     float one;                        // 1.0f: multiplier of packed additions (see f32x2_add_one)
@@ -153,7 +154,8 @@ int launch_search_acts(const float* x, size_t n, float alpha, const int* bits, c
                        float* x_hat, cudaStream_t st);
 int fused_plan_upload(const void* layers_host, int n_layers, void* layers_dev, cudaStream_t st);
 int launch_fused_resnet(const uint8_t* images, int n, int img_h, int img_w, const void* layers_dev, int n_layers,
-                        const void* head_host, float* logits, uint8_t* trace, long long trace_stride, cudaStream_t st);
+                        const void* head_host, float* logits, uint8_t* trace, long long trace_stride, unsigned wait_limit, int test_flags,
+                        cudaStream_t st);
 unsigned long long fused_net_timeouts();
 int launch_avgpool(const float* y, int n, int hw, int c, float* out, cudaStream_t st);
 int launch_maxpool_packed(const uint32_t* x, int n, int h, int w, int c, int bits, int k, int stride, int pad, int ho,

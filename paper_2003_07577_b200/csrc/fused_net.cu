@@ -252,7 +252,7 @@ __device__ __forceinline__ void fused_unit_pool(const FusedUnitEnv& E, uint32_t 
 __global__ void __launch_bounds__(FUSED_THREADS, 1)
 fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, const FusedLayer* __restrict__ layers,
                     int n_layers, const FusedHead head, float one, float* __restrict__ logits, uint8_t* __restrict__ trace,
-                    long long trace_stride) {
+                    long long trace_stride, unsigned limit, int test_flags) {
     extern __shared__ uint8_t dyn_smem[];
     __shared__ __align__(8) uint64_t w_full[2], w_raw[2], w_free[2], rec_full[FUSED_RING], rec_free[FUSED_RING];
     __shared__ __align__(8) uint64_t acc_full[FUSED_MAX_TILES], ep_done[FUSED_MAX_TILES], hold_full, copy_ready, epi_sync;
@@ -268,7 +268,7 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
     uint8_t* acts = base;                                        // three strips
     uint8_t* wbuf = base + 3 * FUSED_ACT_BYTES;                  // two weight images
     volatile int* abortp = &abort_flag;
-    const unsigned limit = UMMA_WAIT_LIMIT;
+    const bool skip_mma = (test_flags & 1) != 0;                 // test hook: issue nothing, so that waits run out
 
     if (tid == 0) {
         abort_flag = 0;
@@ -378,8 +378,6 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                 if (lane == 0) mbar_arrive(&w_full[li & 1]);
             }
         }
-        if (*abortp)                                     // a copy may still be in flight towards this CTA's shared memory
-            for (int i = 0; i < 64; ++i) __nanosleep(1000);
     } else if (warp >= FUSED_ISSUER_WARP && warp < FUSED_ISSUER_WARP + FUSED_ISSUERS) {
         // =========================== MMAs ===========================
         const int k_iss = warp - FUSED_ISSUER_WARP;
@@ -421,6 +419,7 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                     if (!hold && leader) mbar_arrive(&acc_full[t]);
                     continue;
                 }
+                if (skip_mma) continue;
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 if (elect_one()) {
                     const uint32_t tm = tm0 + (uint32_t)t * tm_step;
@@ -463,7 +462,7 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
             }
             if (!ok || !wait_tiles(prev_tiles)) break;   // (every phase of these barriers is waited for, so that parities stay in step)
             if (L.hold) {
-                umma_commit_pred(leader, &hold_full);
+                if (!skip_mma) umma_commit_pred(leader, &hold_full);
             } else {
                 prev = li;
                 prev_tiles = tiles;
@@ -633,11 +632,15 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
             }
         }
     }
-    if (abort_flag != 0 && tid == 0) atomicAdd(&g_umma_timeouts, 1ull);
 
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
-    if (warp == FUSED_ISSUER_WARP) {
+    if (warp == FUSED_ISSUER_WARP) {                             // (the block's memory is its own until this warp leaves)
+        if (abort_flag != 0) {
+            giveup_drain();
+            if (lane == 0) atomicAdd(&g_umma_timeouts, 1ull);
+        }
+        __syncwarp();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(512u) : "memory");
     }
 }
@@ -676,7 +679,8 @@ int fused_plan_upload(const void* layers_host, int n_layers, void* layers_dev, c
 }
 
 int launch_fused_resnet(const uint8_t* images, int n, int img_h, int img_w, const void* layers_dev, int n_layers,
-                        const void* head_host, float* logits, uint8_t* trace, long long trace_stride, cudaStream_t st) {
+                        const void* head_host, float* logits, uint8_t* trace, long long trace_stride, unsigned wait_limit, int test_flags,
+                        cudaStream_t st) {
     static bool attr_set[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
@@ -688,7 +692,7 @@ int launch_fused_resnet(const uint8_t* images, int n, int img_h, int img_w, cons
     FusedHead head;
     memcpy(&head, head_host, sizeof(head));
     fused_resnet_kernel<<<n, FUSED_THREADS, FUSED_SMEM, st>>>(images, img_h, img_w, static_cast<const FusedLayer*>(layers_dev),
-                                                               n_layers, head, 1.0f, logits, trace, trace_stride);
+                                                               n_layers, head, 1.0f, logits, trace, trace_stride, wait_limit, test_flags);
     return check_cuda(cudaGetLastError());
 }
 

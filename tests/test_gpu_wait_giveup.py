@@ -83,3 +83,59 @@ def test_tile_kernel_does_not_count_the_launch_before_it(ebs, U, oracle):
         torch.cuda.synchronize()
         assert ebs.ebs_device_wait_timeouts() == before
         assert np.array_equal(out.cpu().numpy().transpose(0, 3, 1, 2), oracle.conv2d_codes(qa, qw, (1, 1), (1, 1)))
+
+
+@pytest.mark.parametrize("c,hw,limit,skip", [
+    (64, 12, 64, 1),            # one thread block per tile
+    (512, 7, 64, 1),            # a cluster per tile, every member gives up before the exchange of the sums
+    (512, 7, 4000, 2),          # ... in the exchange: one member's sums never come
+    (64, 300, 64, 1),           # per-tap form (a row of 300 pixels)
+])
+def test_tile_bounded_waits_give_up_and_recover(ebs, U, oracle, c, hw, limit, skip):
+    rng = np.random.default_rng(c + hw)
+    h, w = (3, hw) if hw > 100 else (hw, hw)
+    qa, qw = U.rand_codes(rng, (1, c, h, w), 3, False), U.rand_codes(rng, (64, c, 3, 3), 2, True)
+    d = U.desc_for(c, 64, 3, 1, 1, 2, 3)
+    variant = U.variants_of("umma")[2]
+    assert ebs.ebs_check_device_status() == ebs.EBS_OK
+    before = ebs.ebs_device_wait_timeouts()
+    ebs.ebs_test_set_device_wait(limit, skip)
+    try:
+        U.run_conv(qa, qw, d, variant=variant)              # returns: every wait is bounded
+    finally:
+        ebs.ebs_test_set_device_wait(0, 0)
+    after = ebs.ebs_device_wait_timeouts()
+    assert after > before, "no thread block reported that it gave up"
+    assert ebs.ebs_check_device_status() == ebs.EBS_ERR_TIMEOUT
+    got = U.run_conv(qa, qw, d, variant=variant)["acc"]
+    assert np.array_equal(got, oracle.conv2d_codes(qa, qw, (1, 1), (1, 1)))
+    assert ebs.ebs_device_wait_timeouts() == after
+
+
+def test_whole_network_bounded_waits_give_up_and_recover(ebs):
+    from types import SimpleNamespace
+    from paper_2003_07577_b200 import network
+    g = torch.Generator(device="cuda")
+    g.manual_seed(7)
+    shapes = [("conv1", "first", 3, 16, 3, 1, 1, 16, 8), ("s1b1c1", "conv", 16, 16, 3, 1, 1, 16, 2),
+              ("s1b1c2", "conv", 16, 16, 3, 1, 1, 16, 3), ("s2b1c1", "conv", 16, 32, 3, 2, 1, 16, 4),
+              ("s2b1c2", "conv", 32, 32, 3, 1, 1, 8, 1), ("s2b1ds", "shortcut", 16, 32, 1, 2, 0, 16, 4),
+              ("fc", "fc", 32, 10, 1, 1, 0, 1, 8)]
+    layers = [SimpleNamespace(name=n, role=r, c_in=ci, c_out=co, k=k, stride=s, pad=p, h_in=h, w_in=h, w_bits=3, a_bits=a,
+                              w_scale=0.05) for n, r, ci, co, k, s, p, h, a in shapes]
+    codes = {L.name: torch.randint(-4, 4, (L.c_out, L.c_in, L.k, L.k), generator=g, device="cuda", dtype=torch.int8) for L in layers}
+    x = torch.randint(0, 256, (3, 16, 16, 3), generator=g, device="cuda", dtype=torch.uint8)
+    plans = network.calibrated_plans(layers, codes, x)
+    want = network.BasicBlockNet(plans).forward(x).clone()
+    net = network.FusedBasicBlockNet(plans)
+    before = ebs.ebs_device_wait_timeouts()
+    ebs.ebs_test_set_device_wait(64, 1)
+    try:
+        net.forward(x)
+        torch.cuda.synchronize()
+    finally:
+        ebs.ebs_test_set_device_wait(0, 0)
+    assert ebs.ebs_device_wait_timeouts() == before + 3       # one thread block an image
+    assert ebs.ebs_check_device_status() == ebs.EBS_ERR_TIMEOUT
+    assert torch.equal(net.forward(x), want)
+    assert ebs.ebs_device_wait_timeouts() == before + 3

@@ -141,7 +141,7 @@ def _native():
                  "ebs_search_act_forward", "ebs_graph_launch")
         torch.cuda.init()                                  # the stream lookups below need torch's CUDA state
         _fastcall.bind({k: ctypes.cast(getattr(L, k), ctypes.c_void_p).value for k in names},
-                       torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+                       torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice, ebs_conv_desc, ebs_epilogue, ebs_fused_head)
         _fast = _fastcall
     return _fast
 

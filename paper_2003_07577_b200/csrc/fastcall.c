@@ -12,7 +12,7 @@
 
 #include "ebs.h"
 
-static PyObject *s_data_ptr, *s_cuda_stream, *f_raw_stream, *f_get_device;
+static PyObject *s_data_ptr, *s_cuda_stream, *f_raw_stream, *f_get_device, *t_desc, *t_epilogue, *t_head;
 
 #define EACH_ENTRY(X)                                                                                                 \
     X(ebs_pack_acts) X(ebs_pack_acts_s2d) X(ebs_conv2d_mixed) X(ebs_conv2d_mixed_variant) X(ebs_dequant)              \
@@ -47,11 +47,9 @@ static int as_stream(PyObject *o, void **out) {
     Py_DECREF(v);
     return !(*out == NULL && PyErr_Occurred());
 }
+/* An integer: int or a type that is one by __index__ (no conversion: 2.7 or "5" is an error, as it is for a ctypes c_int). */
 static int as_int(PyObject *o, int *out) {
-    PyObject *whole = PyLong_CheckExact(o) ? NULL : PyNumber_Long(o);
-    if (!whole && PyErr_Occurred()) return 0;
-    const long v = PyLong_AsLong(whole ? whole : o);
-    Py_XDECREF(whole);
+    const long v = PyLong_AsLong(o);                        /* (takes __index__, not __int__) */
     if (v == -1 && PyErr_Occurred()) return 0;
     if (v < INT_MIN || v > INT_MAX) {
         PyErr_SetString(PyExc_OverflowError, "integer argument out of range");
@@ -67,20 +65,24 @@ static int as_float(PyObject *o, float *out) {
     return 1;
 }
 static int as_size(PyObject *o, size_t *out) {
-    *out = PyLong_AsSize_t(o);
+    PyObject *whole = PyNumber_Index(o);
+    if (!whole) return 0;
+    *out = PyLong_AsSize_t(whole);
+    Py_DECREF(whole);
     return !(*out == (size_t)-1 && PyErr_Occurred());
 }
-/* A ctypes structure (descriptor, epilogue) by value; *given = 0 for None. */
-static int as_struct(PyObject *o, void *out, size_t size, int *given) {
-    *given = 0;
-    if (o == Py_None) return 1;
+/* A ctypes structure of the given type by value. */
+static int as_struct(PyObject *o, PyObject *type, void *out, size_t size) {
+    if (!PyObject_TypeCheck(o, (PyTypeObject *)type)) {
+        PyErr_Format(PyExc_TypeError, "%s expected instead of %s", ((PyTypeObject *)type)->tp_name, Py_TYPE(o)->tp_name);
+        return 0;
+    }
     Py_buffer b;
     if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE)) return 0;
     const int fits = (size_t)b.len == size;
     if (fits) memcpy(out, b.buf, size);
     PyBuffer_Release(&b);
     if (!fits) PyErr_SetString(PyExc_TypeError, "structure argument has another size than the C type");
-    *given = 1;
     return fits;
 }
 static int arg_count(Py_ssize_t got, Py_ssize_t want) {
@@ -120,19 +122,19 @@ FAST(pack_acts_s2d) {
 
 FAST(conv2d_mixed) {
     void *x, *w, *acc, *y, *pn, *st;
-    int i[3], variant, has_d, has_e;
+    int i[3], variant;
     ebs_conv_desc d;
     ebs_epilogue e;
     if (!arg_count(n, 12) || !as_ptr(a[0], &x)) return NULL;
     for (int k = 0; k < 3; ++k)
         if (!as_int(a[1 + k], &i[k])) return NULL;
-    if (!as_ptr(a[4], &w) || !as_struct(a[5], &d, sizeof(d), &has_d) || !as_struct(a[6], &e, sizeof(e), &has_e) ||
+    if (!as_ptr(a[4], &w) || !as_struct(a[5], t_desc, &d, sizeof(d)) ||
+        (a[6] != Py_None && !as_struct(a[6], t_epilogue, &e, sizeof(e))) ||
         !as_ptr(a[7], &acc) || !as_ptr(a[8], &y) || !as_ptr(a[9], &pn) || !as_stream(a[10], &st) || !as_int(a[11], &variant))
         return NULL;
-    const ebs_conv_desc *dp = has_d ? &d : NULL;
-    const ebs_epilogue *ep = has_e ? &e : NULL;
-    if (variant == -1) CALL(p_ebs_conv2d_mixed(x, i[0], i[1], i[2], w, dp, ep, acc, y, pn, st));
-    CALL(p_ebs_conv2d_mixed_variant(x, i[0], i[1], i[2], w, dp, ep, acc, y, pn, st, variant));
+    const ebs_epilogue *ep = a[6] != Py_None ? &e : NULL;
+    if (variant == -1) CALL(p_ebs_conv2d_mixed(x, i[0], i[1], i[2], w, &d, ep, acc, y, pn, st));
+    CALL(p_ebs_conv2d_mixed_variant(x, i[0], i[1], i[2], w, &d, ep, acc, y, pn, st, variant));
 }
 
 FAST(dequant) {
@@ -169,21 +171,23 @@ FAST(maxpool_packed) {
 
 FAST(resnet_cifar_forward) {
     void *img, *layers, *logits, *trace, *st;
-    int i[3], nl, has_h;
+    int i[3], nl;
     ebs_fused_head head;
     if (!arg_count(n, 11) || !as_ptr(a[0], &img)) return NULL;
     for (int k = 0; k < 3; ++k)
         if (!as_int(a[1 + k], &i[k])) return NULL;
-    if (!as_ptr(a[4], &layers) || !as_int(a[5], &nl) || !as_struct(a[6], &head, sizeof(head), &has_h) ||
+    if (!as_ptr(a[4], &layers) || !as_int(a[5], &nl) || !as_struct(a[6], t_head, &head, sizeof(head)) ||
         !as_ptr(a[7], &logits) || !as_ptr(a[8], &trace))
         return NULL;
     const long long stride = PyLong_AsLongLong(a[9]);
     if ((stride == -1 && PyErr_Occurred()) || !as_stream(a[10], &st)) return NULL;
-    CALL(p_ebs_resnet_cifar_forward(img, i[0], i[1], i[2], layers, nl, has_h ? &head : NULL, logits, trace, stride, st));
+    CALL(p_ebs_resnet_cifar_forward(img, i[0], i[1], i[2], layers, nl, &head, logits, trace, stride, st));
 }
 
-/* bits / coefficients: sequences of numbers.  More candidates than the library takes are its error to report. */
+/* bits / coefficients: sequences of whatever int() and float() take.  More candidates than the library takes are its error
+ * to report. */
 static int candidates(PyObject *bits, PyObject *coeff, int *b, float *c, int *n_cand) {
+    if (PyObject_Size(bits) < 0 || PyObject_Size(coeff) < 0) return 0;
     PyObject *fb = PySequence_Fast(bits, "bits is not a sequence");
     if (!fb) return 0;
     PyObject *fc = PySequence_Fast(coeff, "coeff is not a sequence");
@@ -194,8 +198,13 @@ static int candidates(PyObject *bits, PyObject *coeff, int *b, float *c, int *n_
         PyErr_SetString(PyExc_ValueError, "bits and coeff have different lengths");
         ok = 0;
     }
-    for (Py_ssize_t k = 0; ok && k < n && k < EBS_MAX_CANDIDATES; ++k)
-        ok = as_int(PySequence_Fast_GET_ITEM(fb, k), &b[k]) && as_float(PySequence_Fast_GET_ITEM(fc, k), &c[k]);
+    for (Py_ssize_t k = 0; ok && k < n && k < EBS_MAX_CANDIDATES; ++k) {
+        PyObject *whole = PyNumber_Long(PySequence_Fast_GET_ITEM(fb, k));
+        PyObject *real = whole ? PyNumber_Float(PySequence_Fast_GET_ITEM(fc, k)) : NULL;
+        ok = real && as_int(whole, &b[k]) && as_float(real, &c[k]);
+        Py_XDECREF(whole);
+        Py_XDECREF(real);
+    }
     Py_DECREF(fb);
     Py_XDECREF(fc);
     return ok;
@@ -254,11 +263,13 @@ FAST(same_bytes) {
     return same < 0 ? NULL : PyBool_FromLong(same && left == 0);
 }
 
-/* bind(addresses, raw_stream, get_device): library entry points by name, torch's raw current stream of a device and
- * torch's current device. */
+/* bind(addresses, raw_stream, get_device, desc, epilogue, head): library entry points by name, torch's raw current stream of
+ * a device, torch's current device and the ctypes structure types. */
 static PyObject *bind(PyObject *self, PyObject *args) {
-    PyObject *addr, *raw, *dev;
-    if (!PyArg_ParseTuple(args, "O!OO", &PyDict_Type, &addr, &raw, &dev)) return NULL;
+    PyObject *addr, *raw, *dev, *desc, *epi, *head;
+    if (!PyArg_ParseTuple(args, "O!OOO!O!O!", &PyDict_Type, &addr, &raw, &dev, &PyType_Type, &desc, &PyType_Type, &epi,
+                          &PyType_Type, &head))
+        return NULL;
 #define BIND_ENTRY(name)                                                                                              \
     {                                                                                                                 \
         PyObject *v = PyDict_GetItemString(addr, #name);                                                              \
@@ -271,6 +282,12 @@ static PyObject *bind(PyObject *self, PyObject *args) {
     Py_XSETREF(f_raw_stream, raw);
     Py_INCREF(dev);
     Py_XSETREF(f_get_device, dev);
+    Py_INCREF(desc);
+    Py_XSETREF(t_desc, desc);
+    Py_INCREF(epi);
+    Py_XSETREF(t_epilogue, epi);
+    Py_INCREF(head);
+    Py_XSETREF(t_head, head);
     Py_RETURN_NONE;
 }
 

@@ -11,6 +11,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from typing import Optional
 
 import torch
@@ -430,6 +431,16 @@ def ebs_graph_launch(graph_exec: int, stream=None) -> bool:
 
 def ebs_graph_destroy(graph_exec: int) -> None:
     _check(lib().ebs_graph_destroy(graph_exec), "ebs_graph_destroy")
+
+
+def addresses(tensors) -> bytes:
+    """The data pointers of tensors, for same_addresses."""
+    return struct.pack(f"{len(tensors)}P", *(t.data_ptr() for t in tensors))
+
+
+def same_addresses(tensors, data: bytes) -> bool:
+    """Whether the tensors' data pointers are those of ``addresses``."""
+    return (_fast or _native()).same_addresses(tensors, data)
 
 
 def same_bytes(structs, data: bytes) -> bool:

@@ -263,6 +263,24 @@ FAST(same_bytes) {
     return same < 0 ? NULL : PyBool_FromLong(same && left == 0);
 }
 
+/* same_addresses(tensors, bytes): whether the tensors' data pointers, in order, are exactly those in `bytes`. */
+FAST(same_addresses) {
+    if (!arg_count(n, 2)) return NULL;
+    PyObject *seq = PySequence_Fast(a[0], "tensors is not a sequence");
+    if (!seq) return NULL;
+    char *want;
+    Py_ssize_t left;
+    int same = PyBytes_AsStringAndSize(a[1], &want, &left) == 0 ? 1 : -1;
+    if (same > 0) same = left == PySequence_Fast_GET_SIZE(seq) * (Py_ssize_t)sizeof(void *);
+    for (Py_ssize_t k = 0; same > 0 && k < PySequence_Fast_GET_SIZE(seq); ++k, want += sizeof(void *)) {
+        void *ptr;
+        if (!as_ptr(PySequence_Fast_GET_ITEM(seq, k), &ptr)) same = -1;
+        else same = memcmp(&ptr, want, sizeof(ptr)) == 0;
+    }
+    Py_DECREF(seq);
+    return same < 0 ? NULL : PyBool_FromLong(same);
+}
+
 /* bind(addresses, raw_stream, get_device, desc, epilogue, head): library entry points by name, torch's raw current stream of
  * a device, torch's current device and the ctypes structure types. */
 static PyObject *bind(PyObject *self, PyObject *args) {
@@ -304,6 +322,7 @@ static PyMethodDef methods[] = {{"bind", bind, METH_VARARGS, NULL},
                                 FAST_METHOD(search_act_forward),
                                 FAST_METHOD(graph_launch),
                                 FAST_METHOD(same_bytes),
+                                FAST_METHOD(same_addresses),
                                 {NULL, NULL, 0, NULL}};
 
 static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_fastcall", NULL, -1, methods, NULL, NULL, NULL, NULL};

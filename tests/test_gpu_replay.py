@@ -70,3 +70,49 @@ def test_forward_inside_a_callers_capture():
     out.zero_()
     graph.replay()
     assert torch.equal(out, want)
+
+
+def test_replay_follows_pooling_and_storage_changes():
+    """What the calls read when they are issued: the pooling, the plan objects, the storage behind a weight tensor."""
+    from paper_2003_07577_b200 import network
+    net, g = _net(3)
+    x = _images(2, g)
+    want = [net.forward(x).clone() for _ in range(3)][-1]
+
+    w = net.plans[1].packed_w                            # other storage behind the same tensor object
+    kept = w.data
+    w.data = torch.zeros_like(w)
+    zeroed = net.forward(x).clone()
+    assert torch.equal(zeroed, _one_by_one(net, x)) and not torch.equal(zeroed, want)
+    w.data = kept
+    assert torch.equal(net.forward(x), want)
+
+    import copy
+    other = copy.copy(net.fc)                            # another plan object in the place of one
+    other.ch_bias = other.ch_bias + 1.0
+    mine, net.fc = net.fc, other
+    shifted = net.forward(x).clone()
+    assert torch.allclose(shifted, want + 1.0)
+    net.fc = mine
+    assert torch.equal(net.forward(x), want)
+
+
+def test_replay_follows_an_assigned_pooling():
+    """The maximum pooling after the first convolution of an ImageNet network, changed on the object: window and padding, so
+    that the sizes behind it stay."""
+    from paper_2003_07577_b200 import network
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    shapes = [("conv1", "first", 3, 16, 3, 2, 1, 32, 8), ("s1b1c1", "conv", 16, 16, 3, 1, 1, 8, 2),
+              ("s1b1c2", "conv", 16, 16, 3, 1, 1, 8, 3), ("fc", "fc", 16, 10, 1, 1, 0, 1, 8)]
+    layers = [SimpleNamespace(name=n, role=r, c_in=ci, c_out=co, k=k, stride=s, pad=p, h_in=h, w_in=h, w_bits=3, a_bits=a,
+                              w_scale=0.05) for n, r, ci, co, k, s, p, h, a in shapes]
+    codes = {L.name: torch.randint(-4, 4, (L.c_out, L.c_in, L.k, L.k), generator=g, device="cuda", dtype=torch.int8) for L in layers}
+    x = torch.randint(0, 256, (2, 32, 32, 3), generator=g, device="cuda", dtype=torch.uint8)
+    plans = network.calibrated_plans(layers, codes, x, pool=(3, 2, 1))
+    net = network.BasicBlockNet(plans, pool=(3, 2, 1))
+    before = [net.forward(x).clone() for _ in range(3)][-1]
+    net.pool = (2, 2, 0)
+    after = [net.forward(x).clone() for _ in range(3)]
+    want = network.BasicBlockNet(plans, pool=(2, 2, 0)).forward(x)
+    assert all(torch.equal(a, want) for a in after) and not torch.equal(want, before)

@@ -69,6 +69,7 @@ __device__ __forceinline__ bool mbar_wait_bounded_hot(uint64_t* bar, uint32_t pa
 // What a CTA that gave up does before it frees its memory: copies into its shared memory and MMAs that were started may still
 // be under way, and nothing waits for them any more (64 us; either takes a few).
 __device__ __forceinline__ void giveup_drain() {
+#pragma unroll 1
     for (int i = 0; i < 64; ++i) __nanosleep(1000);
 }
 

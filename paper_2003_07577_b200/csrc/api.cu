@@ -145,13 +145,10 @@ static int choose_mma_variant(int w_bits, int a_bits, int P, int Co, int sms) {
     return 6 + tc_idx;
 }
 
-// The persistent pipeline kernel covers stride-1 and strided k x k layers and 1x1 layers at any stride.  It pays off
-// when the layer has at least 64 output channels and enough outputs to fill the GPU.  Channel tile: the widest of
-// 256/128/64 that divides c_out (every tile whole: straight-line epilogue; the fewer channel tiles, the less often an
-// input pixel is expanded and the less weight traffic per multiply -- measured faster even where it leaves some SMs
-// without a tile).  Returns the pipeline variant (0..2) or -1.
-static int choose_pipe_variant(const ConvParams& p, int sms) {
-    (void)sms;
+// The persistent pipeline kernel covers layers of strides up to 2 whose strip fits.  It pays off when the layer has at least
+// 64 output channels and enough outputs to fill the GPU.  Returns the pipeline variant (0..2: channel tiles of 64, 128
+// and 256) or -1.
+static int choose_pipe_variant(const ConvParams& p) {
     // (layers with few input channels too: the kernel spends a whole 32-channel word per tap on them, and is still
     // six times faster on an ImageNet stem, 3 -> 64 channels 7x7 stride 2, than the tap-folding per-tap kernels)
     if (p.Co < 64 || (long long)p.P * p.Co < (1LL << 20) || p.w_levels) return -1;
@@ -306,7 +303,7 @@ static int conv_plan(const void* packed_x, int n, int h, int w, const void* pack
     } else if (variant < 0) {
         const bool small = tile_kernel_pays(p, sm_count());
         const int tile = umma_ok && (p.Co > 16 || p.KK >= 18) ? choose_tile_variant(p) : -1;
-        const int pipe = umma_ok && !(small && tile >= 0) ? choose_pipe_variant(p, sm_count()) : -1;
+        const int pipe = umma_ok && !(small && tile >= 0) ? choose_pipe_variant(p) : -1;
         // few channels on many pixels: the warp-level strip kernel (16 -> 16 3x3 at 32x32, batch 128: 7.1 us, the tile kernel,
         // whose accumulator is then mostly empty, 22; 32 -> 32 at 16x16: 7.2 against 8.3)
         const bool few = p.Co <= 32 && p.CW <= 2 && d->kh * d->kw > 1 && (long long)p.P > 128LL * sm_count();

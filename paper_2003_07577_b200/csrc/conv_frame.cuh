@@ -8,7 +8,8 @@ namespace ebs {
 
 constexpr int FRAME_MAX_TAPS = 64, FRAME_MAX_PHASES = 4;
 
-// Exact unsigned division by a run-time constant: q = (t + ((n - t) >> s1)) >> s2, t = mulhi(m, n).
+// Exact unsigned division by a run-time constant (Granlund and Montgomery, "Division by Invariant Integers using
+// Multiplication", 1994): q = (t + ((n - t) >> s1)) >> s2, t = mulhi(m, n).
 struct FastDiv {
     uint32_t m, s1, s2;
 };
@@ -252,16 +253,6 @@ __device__ __forceinline__ uint64_t f32x2_pack(float lo, float hi) {
 __device__ __forceinline__ uint64_t f32x2_mul_rn(uint64_t a, uint64_t b) {
     uint64_t d;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t f32x2_add_rn(uint64_t a, uint64_t b) {
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t f32x2_add_rd(uint64_t a, uint64_t b) {
-    uint64_t d;
-    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
 

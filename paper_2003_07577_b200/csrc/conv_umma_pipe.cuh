@@ -86,7 +86,7 @@ struct PipeGeom : FrameGeom {
     bool ok;
 };
 
-// m_sub_req / ks_req = 0: chosen here.  Returns ok = false when the kernel does not apply.
+// m_sub_req = 0: chosen here.  Returns ok = false when the kernel does not apply.
 inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_sub_req = 0, bool pair = false) {
     PipeGeom g{};
     if (pair && (tile_n != 256 || (p.Co % 256) != 0 || sms < 2)) return g;
@@ -194,9 +194,7 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
     return g;
 }
 
-// One 32-channel group of the plain epilogue: 32 accumulators of this thread's pixel -> stores, fp32 steps,
-// requantized codes -> plane words.
-// The same for a CTA pair: M = 256 over the two CTAs' tensor memory, issued by the even CTA; the commit arrives on the
+// umma_i8_split for a CTA pair: M = 256 over the two CTAs' tensor memory, issued by the even CTA; the commit arrives on the
 // barrier at this offset in both CTAs.
 __device__ __forceinline__ void umma_i8_split_pair(uint32_t leader, uint32_t tmem_d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
                                                    uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
@@ -222,8 +220,8 @@ __device__ __forceinline__ void umma_commit_pred_pair(uint32_t leader, uint64_t*
         ::"r"(own), "r"(own + peer_delta), "r"(leader) : "memory");
 }
 
-
-//
+// One 32-channel group of the plain epilogue with 32-bit results: 32 accumulators of this thread's pixel -> stores, fp32
+// steps, requantized codes -> plane words.
 // The float -> int conversion issues at an eighth of the fp32 rate on this machine (16 results per clock and SM against
 // 128 fp32 operations) and was what bounded the epilogue, so the floor and the clamp are done with an fp32 addition and
 // integer min / max instead (see below); the fp32 steps run as packed two-lane instructions.
@@ -456,10 +454,10 @@ __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, cons
     }
 }
 
-// Plain epilogue (no per-channel terms, no shortcut, NHWC, c_out a multiple of 32) of one
-// 128-pixel accumulator.  vwarp 0..7: TMEM lane quarter vwarp % 4, channel half vwarp / 4.
-template <int TILE_N, int G>
-__device__ __forceinline__ void pipe_epilogue_plain_g(const ConvParams& p, uint32_t tmem_acc, int vwarp, int gp, bool pvalid,
+// Plain epilogue with 32-bit results (no per-channel terms, no shortcut, NHWC, c_out a multiple of 32; without such results:
+// pipe_epilogue_packed_nb) of one 128-pixel accumulator.  vwarp 0..7: TMEM lane quarter vwarp % 4, channel half vwarp / 4.
+template <int TILE_N>
+__device__ __forceinline__ void pipe_epilogue_plain(const ConvParams& p, uint32_t tmem_acc, int vwarp, int gp, bool pvalid,
                                                       int co0) {
     const uint32_t trow = tmem_acc + ((uint32_t)((vwarp & 3) * 32) << 16);
     constexpr int COLS = TILE_N / 2;
@@ -468,8 +466,6 @@ __device__ __forceinline__ void pipe_epilogue_plain_g(const ConvParams& p, uint3
     const int nb = want_q ? p.next_bits : 0, qmax = (1 << p.next_bits) - 1;
     const float S = p.S, inv_next = p.inv_next;
     uint32_t v[32];
-    PlaneHold<G> hold;
-    hold.filled = 0;
 #pragma unroll 1
     for (int c0 = cbeg; c0 < cbeg + COLS; c0 += 32) {
         if (co0 + c0 >= p.Co) break;
@@ -481,9 +477,7 @@ __device__ __forceinline__ void pipe_epilogue_plain_g(const ConvParams& p, uint3
         tmem_ld16_wait(hi);
         const size_t o = (size_t)gp * p.Co + co0 + c0;
         uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + ((co0 + c0) >> 5)) * nb;
-        if (want_q && !p.acc && !p.y) {
-            pipe_group32_packed<G>(v, pvalid, S, inv_next, nb, qmax, dst, p, hold, 32);
-        } else if (want_q) {
+        if (want_q) {
             pipe_group32<true>(p, v, o, pvalid, S, inv_next, nb, qmax, dst);
         } else {
             pipe_group32<false>(p, v, o, pvalid, S, inv_next, nb, qmax, dst);
@@ -589,14 +583,10 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     __shared__ __align__(16) float s_terms[AFFINE ? PIPE_EPI_WARPS : 1][64];
-    __shared__ uint32_t s_tap_shift[PIPE_MAX_TAPS];     // tap tables in shared memory: indexed at run time by single threads
-    __shared__ int s_tap_id[PIPE_MAX_TAPS];
+    __shared__ int s_tap_id[PIPE_MAX_TAPS];             // (in shared memory: indexed at run time by single threads)
 
     const int tid = threadIdx.x, warp = tid >> 5;
-    if (tid < PIPE_MAX_TAPS) {
-        s_tap_shift[tid] = (uint32_t)g.tap_shift[tid];
-        s_tap_id[tid] = (int)g.tap_id[tid];
-    }
+    if (tid < PIPE_MAX_TAPS) s_tap_id[tid] = (int)g.tap_id[tid];
     const int NST = g.n_stages, KS = g.ks, KSS = g.kss, NSUB = g.nsub, SP = g.SP, S = g.S;
     const int nchunks = g.nchunks, nwg = g.nwg;
     const bool resident = g.b_resident != 0;
@@ -680,11 +670,11 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(REG_EXP));
         // =========================== expanders ===========================
         int slot_q[PIPE_SLOTS], slot_pix[PIPE_SLOTS], slot_dst[PIPE_SLOTS];
-#pragma unroll
         // An even number of words per pass: a thread takes two adjacent words of one pixel, so that for an odd plane count
         // its 2 * AB packed words still start on an 8-byte boundary and load as pairs.  Otherwise items tid and tid + 256.
         constexpr int NW = AB == 0 ? 8 : AB;                  // words of one (pixel, 32-channel word) item; AB = 0: byte codes
         const bool paired = (NW & 1) != 0 && (KS & 1) == 0 && (p.CW & 1) == 0;
+#pragma unroll
         for (int j = 0; j < PIPE_SLOTS; ++j) {
             const int e = paired ? 2 * tid + j : tid + j * PIPE_EXPANDERS;
             const int s = e / KS, q = e - s * KS;            // consecutive lanes: consecutive words of one pixel
@@ -1089,7 +1079,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
                 if constexpr (FORM != 0) {
                     if constexpr (!AFFINE) pipe_epilogue_packed_g<TILE_N, EPI_G>(p, tmem_acc, vwarp, gp, pvalid, co0);
                 } else {
-                    if (plain_ok) pipe_epilogue_plain_g<TILE_N, 1>(p, tmem_acc, vwarp, gp, pvalid, co0);
+                    if (plain_ok) pipe_epilogue_plain<TILE_N>(p, tmem_acc, vwarp, gp, pvalid, co0);
                     else umma_epilogue<TILE_N, AFFINE>(p, tmem_acc, vwarp, gp, pvalid, 0, co0);
                 }
             }

@@ -7,8 +7,9 @@ largest single-GPU workload: the ImageNet ResNet-50 bottleneck stack at batch 25
 layers chained through fused requantization.  A step is one pass of the whole path over one batch:
 ebs_pack_acts at the network entry, one ebs_conv2d_mixed per layer whose epilogue writes the next
 layer's packed planes, ebs_dequant of the last layer's accumulators at the exit; weight packing is
-done once before timing (it is off the inference path).  `per_config` holds, for each of the five
-configurations, the step time, binary and int8 TOPS, the roofline fractions in both output modes
+done once before timing (it is off the inference path).  The line carries the headline and a summary
+(under 4 KB, so that whoever captures it gets it whole); the full record goes to bench_detail.json beside
+this file (`--detail FILE` for another place): its `per_config` holds, for each of the five configurations, the step time, binary and int8 TOPS, the roofline fractions in both output modes
 (raw: int32 accumulators + packed planes; fused: packed planes only), cold and warm L2, the literal
 AND+POPC path against the POPC pipe, and the CPU oracle timed on a stated sample.
 
@@ -715,6 +716,28 @@ def resnet18_leg(ebs, dev, stream, flush, reps, batch=64):
             "finite_logits": bool(torch.isfinite(out["logits"]).all().item())}
 
 
+def short_line(full: dict) -> dict:
+    """The line printed of a full record: everything a reader of the headline needs, and the other legs' results in brief."""
+    keep = ["metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+            "dtype", "data", "config", "clocks", "gpu_launches", "device_wait_timeouts"]
+    line = {k: full[k] for k in keep}
+    roof = full["roofline"]
+    line["roofline"] = {k: roof[k] for k in ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic", "conv_ms_per_step",
+                                             "conv_launches_per_step", "hbm_peak_gbs", "sum_layer_roofs_ms")}
+    if "e2e" in full:
+        line["e2e"] = {k: full["e2e"][k] for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step")}
+    if "cpu_baseline" in full:
+        line["cpu_baseline"] = {k: (v[:160] if isinstance(v, str) else v) for k, v in full["cpu_baseline"].items()}
+    summary = {name: {"conv_ms_" + mode: round(m["conv_ms_cold"], 4) for mode, m in res.get("modes", {}).items() if "conv_ms_cold" in m}
+               for name, res in full["per_config"].items()}
+    net = full.get("network") or {}
+    for name, leg in (("resnet20", net), ("resnet20_fused", net.get("fused")), ("resnet18_imagenet", net.get("resnet18_imagenet"))):
+        if leg:
+            summary[name] = {k: round(leg[k], 4) for k in ("ms_per_batch", "imgs_per_s", "e2e_imgs_per_s") if k in leg}
+    line["summary"] = summary
+    return line
+
+
 def run_gpu(args):
     from paper_2003_07577_b200 import binding as ebs
     ebs.lib()
@@ -962,7 +985,14 @@ def run_gpu(args):
     if cpu is not None:
         line["cpu_baseline"] = cpu
         per_config[headline]["cpu_baseline"] = cpu
-    print(json.dumps(line))
+    short = short_line(line)
+    try:
+        with open(args.detail, "w") as f:
+            json.dump(line, f)
+        short["detail"] = os.path.basename(args.detail)
+    except OSError as exc:                                       # a read-only place: the line is what counts
+        short["detail"] = f"not written: {exc.strerror}"
+    print(json.dumps(short))
 
 
 def main():
@@ -973,6 +1003,8 @@ def main():
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--quick", action="store_true", help="skip the streaming-kernel and whole-network legs")
+    ap.add_argument("--detail", default=os.path.join(ROOT, "bench_detail.json"),
+                    help="where the full record goes (per layer, per mode and context legs)")
     ap.add_argument("--step-only", action="store_true",
                     help="time the steps of --workload and print a short line: no per-layer, per-mode or context legs "
                          "(the command profiler captures run)")

@@ -70,3 +70,34 @@ def test_reference_arm_under_two_ranks_prints_once():
     assert all(p.returncode == 0 for p in procs), [o[1] for o in outs]
     printed = [o[0].strip() for o in outs if o[0].strip()]
     assert len(printed) == 1 and json.loads(printed[0])["impl"] == "reference"
+
+
+def test_printed_line_is_short_and_complete():
+    """Whatever the record holds (per-layer lists of five workloads, long notes), the printed line stays under 4 KB and has
+    every key of the headline."""
+    import sys as _sys
+    _sys.path.insert(0, ROOT)
+    import bench
+    x = 123.4567890123456
+    layers = [{"name": f"l{i}", "us": x, "frac_of_roof": x, "roof": "tensor"} for i in range(64)]
+    mode = {"conv_ms_cold": x, "conv_ms_warm": x, "outputs": "o" * 80, "algorithmic_bytes": 10 ** 10}
+    res = {"modes": {"raw": mode, "fused": mode}, "per_layer": {"raw": layers, "fused": layers}}
+    leg = {"ms_per_batch": x, "imgs_per_s": x, "e2e_imgs_per_s": x, "model": "m" * 300}
+    roof = {k: x for k in ("achieved", "peak", "frac", "traffic", "conv_ms_per_step", "conv_launches_per_step", "hbm_peak_gbs",
+                           "sum_layer_roofs_ms")}
+    full = {"metric": bench.METRIC, "value": x, "unit": bench.UNIT, "n_gpus": 1, "steps": 100, "warmup": 10, "ms_per_step": x,
+            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "int32", "data": "synthetic",
+            "config": {"workload": "w" * 300, "step": "s" * 300, "l2": "l" * 100}, "clocks": {"sm_mhz": 1965, "reasons": []},
+            "gpu_launches": 10 ** 6, "device_wait_timeouts": 0,
+            "roofline": dict(roof, bound="tensor", kernel="k" * 160, unit="TOPS", accounting="a" * 500),
+            "per_config": {f"config{i}": res for i in range(1, 6)}, "network": dict(leg, fused=leg, resnet18_imagenet=leg),
+            "streaming_kernels": {"note": "n" * 2000},
+            "e2e": {"value": x, "unit": "TOPS", "h2d_bytes_per_step": 1, "d2h_bytes_per_step": 1, "ms_per_step": x, "note": "n" * 400},
+            "cpu_baseline": {"value": x, "unit": "TOPS", "cores": 16, "kind": "oracle", "sample": "s" * 500}}
+    text = json.dumps(bench.short_line(full))
+    line = json.loads(text)
+    assert len(text) < 4096 < len(json.dumps(full))
+    for key in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                "vs_baseline", "dtype", "data", "config", "clocks", "gpu_launches", "roofline", "e2e", "cpu_baseline"):
+        assert key in line, key
+    assert set(line["summary"]) == {f"config{i}" for i in range(1, 6)} | {"resnet20", "resnet20_fused", "resnet18_imagenet"}

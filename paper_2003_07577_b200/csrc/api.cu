@@ -307,10 +307,17 @@ static int conv_plan(const void* packed_x, int n, int h, int w, const void* pack
         // few channels on many pixels: the warp-level strip kernel (16 -> 16 3x3 at 32x32, batch 128: 7.1 us, the tile kernel,
         // whose accumulator is then mostly empty, 22; 32 -> 32 at 16x16: 7.2 against 8.3)
         const bool few = p.Co <= 32 && p.CW <= 2 && d->kh * d->kw > 1 && (long long)p.P > 128LL * sm_count();
+        // short reductions with 32-bit results: the tile kernel's epilogue through shared memory takes longer than the warp-level
+        // strip kernel's (accumulators and planes, 4 bits: 64 -> 64 3x3 at 32x32, batch 1: 5.4 against 6.5 us; 32 -> 32: 4.5 and
+        // 5.9; 32 -> 64 at 28x28, batch 32: 8.3 and 9.5); not on many pixels of two words (64 -> 64 at 28x28, batch 32: 12.0 and 10.0)
+        const int short32 = p.Co <= 16 ? 0 : 1;
+        const bool short_results = (p.acc || p.y) && d->kh * d->kw > 1 && p.KK <= 18 && p.Co <= 64 &&
+                                   (p.Co * p.CW <= 64 || p.P <= (1 << 14)) && mma_ok && conv_mma_strip_applies(p, short32);
         const int beside = mma_ok && tile >= 0 && conv_umma_tap_form(p) ? choose_beside_tap_form(p, d, sm_count()) : -1;
         if (pipe >= 0) variant = PIPE_BASE + pipe;
         else if (mma_ok && few && p.Co <= 16 && conv_mma_strip_applies(p, 0)) variant = MS_BASE;
         else if (mma_ok && few && conv_mma_strip_applies(p, 1)) variant = MS_BASE + 1;
+        else if (short_results) variant = MS_BASE + short32;
         else if (beside >= 0) variant = beside;
         else if (tile >= 0) variant = NUM_CONV_VARIANTS + NUM_CONV_MMA_VARIANTS + tile;
         else if (mma_ok && p.Co <= 16 && d->kh * d->kw > 1 && conv_mma_strip_applies(p, 0)) variant = MS_BASE;

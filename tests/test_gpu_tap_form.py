@@ -85,9 +85,10 @@ def test_tap_form(ebs, U, oracle, case, shortcut):
 
 
 def test_library_choice_without_packing(ebs, U, oracle):
-    """32-bit results alone, where the choice lies between the per-tap form and the warp-level kernels."""
+    """32-bit results alone, where the choice lies between the tile kernel and the warp-level kernels."""
     for n, c, co, k, s, h, w, b in [(1, 16, 48, 3, 1, 4, 200, 4), (1, 64, 64, 3, 1, 48, 200, 2), (1, 64, 96, 3, 1, 5, 200, 3),
-                                    (1, 3, 64, 3, 1, 4, 200, 2), (1, 3, 64, 3, 1, 4, 200, 6), (2, 64, 64, 3, 3, 20, 20, 2)]:
+                                    (1, 3, 64, 3, 1, 4, 200, 2), (1, 3, 64, 3, 1, 4, 200, 6), (2, 64, 64, 3, 3, 20, 20, 2),
+                                    (1, 64, 64, 3, 1, 32, 32, 2), (2, 20, 50, 3, 1, 9, 11, 5), (3, 33, 16, 3, 1, 7, 7, 8)]:
         rng = np.random.default_rng(c + co + h)
         qa, qw = U.rand_codes(rng, (n, c, h, w), b, False), U.rand_codes(rng, (co, c, k, k), b, True)
         d = U.desc_for(c, co, k, s, 1, b, b)

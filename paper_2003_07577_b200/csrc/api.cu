@@ -209,6 +209,30 @@ static int choose_beside_tap_form(const ConvParams& p, const ebs_conv_desc* d, i
     return -1;
 }
 
+// Layers with 32-bit results and a short reduction: the tile kernel's epilogue through shared memory takes longer than those of
+// the warp-level kernels.  Returns the variant of the faster one, or -1.  (us at 4 bits, accumulators and planes, this choice
+// against the tile kernel.)
+static int choose_for_results(const ConvParams& p, const ebs_conv_desc* d, int sms) {
+    constexpr int MS_BASE = NUM_CONV_VARIANTS + NUM_CONV_MMA_VARIANTS + NUM_CONV_UMMA_VARIANTS + NUM_CONV_STRIP_VARIANTS +
+                            NUM_CONV_RESIDENT_VARIANTS;
+    if (!p.acc && !p.y) return -1;
+    const int tile = p.Co <= 16 ? 0 : 1;
+    const long long outputs = (long long)p.P * p.Co;
+    if (conv_mma_strip_applies(p, tile)) {
+        // 1x1: 64 -> 64 at 32x32, batch 1: 4.0 and 5.9; 128 -> 256 stride 2 at 28x28: 4.3 and 6.2; 64 -> 64 at 56x56, batch 16: 9.2 and
+        // 15.7.  k x k: 64 -> 64 3x3 at 32x32, batch 1: 5.4 and 6.5; 32 -> 64 at 28x28, batch 32: 8.3 and 9.5; 32 -> 32 5x5 at
+        // 32x32, batch 8: 6.9 and 7.6; not on many pixels of two words (64 -> 64 3x3 at 28x28, batch 32: 12.0 and 10.0).
+        const bool shallow = p.kh * p.kw == 1 ? p.Co <= 256 && outputs <= (1LL << 22)
+                                              : (p.Co * p.CW <= 64 && p.KK <= 25) || (p.Co <= 64 && p.KK <= 18 && p.P <= (1 << 14));
+        return shallow ? MS_BASE + tile : -1;
+    }
+    // strided k x k with few plane pairs: 16 -> 32 3x3 stride 2 at 32x32, batch 128: 8.9 and 9.4, 2 bits 8.1 and 10.1 (8 bits: 13.6 and
+    // 9.6); 32 -> 64 at 28x28, batch 4: 6.9 and 7.5
+    const bool few_pairs = (p.sh > 1 || p.sw > 1) && p.kh * p.kw > 1 && !p.w_levels && p.Co <= 64 && outputs <= (1LL << 20) &&
+                           p.KK * (d->w_bits + d->a_bits) <= 72;
+    return few_pairs ? NUM_CONV_VARIANTS + choose_mma_variant(d->w_bits, d->a_bits, p.P, p.Co, sms) : -1;
+}
+
 // A validated, fully decided launch: nothing has been enqueued when conv_plan returns.
 struct ConvPlan {
     ConvParams p;
@@ -307,17 +331,12 @@ static int conv_plan(const void* packed_x, int n, int h, int w, const void* pack
         // few channels on many pixels: the warp-level strip kernel (16 -> 16 3x3 at 32x32, batch 128: 7.1 us, the tile kernel,
         // whose accumulator is then mostly empty, 22; 32 -> 32 at 16x16: 7.2 against 8.3)
         const bool few = p.Co <= 32 && p.CW <= 2 && d->kh * d->kw > 1 && (long long)p.P > 128LL * sm_count();
-        // short reductions with 32-bit results: the tile kernel's epilogue through shared memory takes longer than the warp-level
-        // strip kernel's (accumulators and planes, 4 bits: 64 -> 64 3x3 at 32x32, batch 1: 5.4 against 6.5 us; 32 -> 32: 4.5 and
-        // 5.9; 32 -> 64 at 28x28, batch 32: 8.3 and 9.5); not on many pixels of two words (64 -> 64 at 28x28, batch 32: 12.0 and 10.0)
-        const int short32 = p.Co <= 16 ? 0 : 1;
-        const bool short_results = (p.acc || p.y) && d->kh * d->kw > 1 && p.KK <= 18 && p.Co <= 64 &&
-                                   (p.Co * p.CW <= 64 || p.P <= (1 << 14)) && mma_ok && conv_mma_strip_applies(p, short32);
+        const int results = mma_ok ? choose_for_results(p, d, sm_count()) : -1;
         const int beside = mma_ok && tile >= 0 && conv_umma_tap_form(p) ? choose_beside_tap_form(p, d, sm_count()) : -1;
         if (pipe >= 0) variant = PIPE_BASE + pipe;
         else if (mma_ok && few && p.Co <= 16 && conv_mma_strip_applies(p, 0)) variant = MS_BASE;
         else if (mma_ok && few && conv_mma_strip_applies(p, 1)) variant = MS_BASE + 1;
-        else if (short_results) variant = MS_BASE + short32;
+        else if (results >= 0) variant = results;
         else if (beside >= 0) variant = beside;
         else if (tile >= 0) variant = NUM_CONV_VARIANTS + NUM_CONV_MMA_VARIANTS + tile;
         else if (mma_ok && p.Co <= 16 && d->kh * d->kw > 1 && conv_mma_strip_applies(p, 0)) variant = MS_BASE;

@@ -88,8 +88,14 @@ def test_library_choice_without_packing(ebs, U, oracle):
     """32-bit results alone, where the choice lies between the tile kernel and the warp-level kernels."""
     for n, c, co, k, s, h, w, b in [(1, 16, 48, 3, 1, 4, 200, 4), (1, 64, 64, 3, 1, 48, 200, 2), (1, 64, 96, 3, 1, 5, 200, 3),
                                     (1, 3, 64, 3, 1, 4, 200, 2), (1, 3, 64, 3, 1, 4, 200, 6), (2, 64, 64, 3, 3, 20, 20, 2),
-                                    (1, 64, 64, 3, 1, 32, 32, 2), (2, 20, 50, 3, 1, 9, 11, 5), (3, 33, 16, 3, 1, 7, 7, 8)]:
+                                    (1, 64, 64, 3, 1, 32, 32, 2), (2, 20, 50, 3, 1, 9, 11, 5), (3, 33, 16, 3, 1, 7, 7, 8),
+                                    (2, 30, 40, 5, 1, 9, 9, 3), (2, 16, 32, 3, 2, 13, 12, 4)]:
         rng = np.random.default_rng(c + co + h)
         qa, qw = U.rand_codes(rng, (n, c, h, w), b, False), U.rand_codes(rng, (co, c, k, k), b, True)
         d = U.desc_for(c, co, k, s, 1, b, b)
         assert np.array_equal(U.run_conv(qa, qw, d)["acc"], oracle.conv2d_codes(qa, qw, (s, s), (1, 1))), (c, co, s)
+    for n, c, co, s, h, w, b in [(1, 64, 64, 1, 32, 32, 4), (2, 100, 129, 2, 9, 8, 3), (3, 33, 10, 1, 5, 7, 8)]:      # 1x1
+        rng = np.random.default_rng(c + co + h)
+        qa, qw = U.rand_codes(rng, (n, c, h, w), b, False), U.rand_codes(rng, (co, c, 1, 1), b, True)
+        d = U.desc_for(c, co, 1, s, 0, b, b)
+        assert np.array_equal(U.run_conv(qa, qw, d)["acc"], oracle.conv2d_codes(qa, qw, (s, s), (0, 0))), (c, co, s)

@@ -112,8 +112,9 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
         if (m * UMMA_M + max_shift > PIPE_MAX_ITEMS) continue;
         const long long pt = (frame + (long long)m * UMMA_M * pw - 1) / ((long long)m * UMMA_M * pw);
         // Expander lanes run over the words of a pass first: with one word a pass every lane of a load reads a line of its
-        // own, which for pixels of about a line or more, expanded for one tap only, costs more than the larger strip saves (256 -> 64 1x1 at 56x56, batch 256:
-        // 4 bits 81.8 -> 73.7 us with half the pixels and two words, 5 bits 132 -> 92).
+        // own, which for pixels of about a line or more, expanded for one tap only, costs more than the larger strip saves (256 -> 64
+        // 1x1 at 56x56, batch 128: 4 bits 40.3 -> 36.6 us with half the pixels and two words, 5 bits 56.1 -> 40.7).  Over 42
+        // layers of 64 channels the gain is 1.00-1.38 from 24 words a pixel on and would be 1.00-1.11 below.
         if (!m_sub_req && m > 1 && taps == 1 && m * UMMA_M > PIPE_MAX_ITEMS / 2 && p.CW > 2 && p.CW * p.x_words >= 24) continue;
         if (!m_sub_req && m > 1 && pt * g.n_ctiles < (deep >= 64 ? 1LL : 2LL) * sms) continue;
         m_sub = m;

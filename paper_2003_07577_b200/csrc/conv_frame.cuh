@@ -350,28 +350,32 @@ __device__ __forceinline__ bool mbar_wait_bounded_warp(uint64_t* bar, uint32_t p
     return false;
 }
 
-// Four requantized codes (low bytes of code_pattern results) -> one register, channel order as in planes_to_bytes.
+// Four requantized codes -> one register, channel order as in planes_to_bytes.
 // k256 = 256, unknown to the compiler: the first step as multiply-adds, which the logic pipe has no part in.
 __device__ __forceinline__ uint32_t join_codes(const uint32_t (&m)[4], uint32_t k256) {
     return __byte_perm(m[1] * k256 + m[0], m[3] * k256 + m[2], 0x5410);
 }
 __device__ __forceinline__ uint32_t k256_of(float one) { return (__float_as_uint(one) & 0x00800000u) >> 15; }
-// Codes of a pair of values w = fl(y / step).  NB = 0: planes counted at run time, or eight of them.  NB = 1..7: without a
-// logic-pipe instruction -- fl(w + 1/2) / 2^NB, clamped to [0, 1] by the addition itself (the scaling is exact), times 2^NB
-// rounded down.  What is clamped above comes out as 2^NB: codes_to_planes spreads that bit over the planes.
+// Codes of a pair of values w = fl(y / step), nb planes.  t = fl(w + 1/2) / 2^nb is clamped to [0, 1] by the addition itself
+// (the scaling is exact; NaN becomes 0).  Its product with the denormal 2^nb * 2^-149, rounded down, is floor(t * 2^nb) units
+// of 2^-149: the register then holds that integer, and one packed instruction serves both values.  What is clamped above comes
+// out as 2^nb: with the plane count in the code (NB = 1..7) codes_to_planes spreads that bit over the planes, else (NB = 0: nb
+// counted at run time; 8) it is brought down to 2^nb - 1 here.
 template <int NB>
-__device__ __forceinline__ void code_pair(uint64_t w, uint64_t one2, uint64_t half2, float hi2, uint32_t& lo, uint32_t& hi) {
+__device__ __forceinline__ void code_pair(uint64_t w, int nb, uint32_t& lo, uint32_t& hi) {
+    const int n = NB == 0 ? nb : NB;
+    const float down = __uint_as_float((uint32_t)(127 - n) << 23), half = 0.5f * down;
+    float a, b;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;\n" : "=f"(a) : "f"(__uint_as_float((uint32_t)w)), "f"(down), "f"(half));
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;\n" : "=f"(b) : "f"(__uint_as_float((uint32_t)(w >> 32))), "f"(down), "f"(half));
+    uint64_t d;
+    const uint64_t up2 = ((uint64_t)(1u << n) << 32) | (uint64_t)(1u << n);
+    asm("mul.rm.f32x2 %0, %1, %2;\n" : "=l"(d) : "l"(f32x2_pack(a, b)), "l"(up2));
+    lo = (uint32_t)d;
+    hi = (uint32_t)(d >> 32);
     if constexpr (NB == 0 || NB == 8) {
-        w = f32x2_add_one(w, one2, half2);
-        lo = code_pattern(__uint_as_float((uint32_t)w), hi2);
-        hi = code_pattern(__uint_as_float((uint32_t)(w >> 32)), hi2);
-    } else {
-        constexpr float UP = (float)(1 << NB), DOWN = 1.0f / UP;
-        float a, b;
-        asm("fma.rn.sat.f32 %0, %1, %2, %3;\n" : "=f"(a) : "f"(__uint_as_float((uint32_t)w)), "f"(DOWN), "f"(0.5f * DOWN));
-        asm("fma.rn.sat.f32 %0, %1, %2, %3;\n" : "=f"(b) : "f"(__uint_as_float((uint32_t)(w >> 32))), "f"(DOWN), "f"(0.5f * DOWN));
-        lo = __float_as_uint(__fmaf_rd(a, UP, 8388608.0f));
-        hi = __float_as_uint(__fmaf_rd(b, UP, 8388608.0f));
+        lo = min(lo, (1u << n) - 1u);
+        hi = min(hi, (1u << n) - 1u);
     }
 }
 // Code registers of code_pair<NB> -> plane words.
@@ -390,42 +394,9 @@ __device__ __forceinline__ float byte_to_float(uint32_t w, int i) {
     return __fadd_rn(__uint_as_float(__byte_perm(w, 0x4B000000u, 0x7540u + (uint32_t)i)), -8388608.0f);
 }
 
-// Per-channel terms of a 32-channel group in the order terms_codes32 reads them: entry bb = channels bb, 8 + bb, 16 + bb,
-// 24 + bb; identities (x * 1, x + (-0)) where a layer has no such term or the channel does not exist.
+// Per-channel terms: identities (x * 1, x + (-0)) where a layer has no such term or the channel does not exist.
 __device__ __forceinline__ float term_at(const float* t, int co, int Co, float identity) {
     return t && co < Co ? ld_dep(t + co) : identity;
-}
-
-// 32 accumulators of one pixel and 32-channel group -> eight registers of requantized codes (register bb: channels bb,
-// 8 + bb, 16 + bb, 24 + bb), with per-channel scale and shift and a shortcut: RES 0 none, 1 fp32 values of the pixel's
-// 32 channels, 2 codes in byte registers of the same order.  Every fp32 step is rounded on its own, in the library's
-// order.  The terms come from shared memory as broadcast 16-byte reads (read through the cache channel by channel they
-// were two thirds of the instructions of this function); products and sums are packed two to an instruction
-// (f32x2_add_one).  The ReLU is not applied: the quantizer's clamp at zero gives the same codes.
-template <int RES, int NB = 0>
-__device__ __forceinline__ void terms_codes32(const uint32_t (&v)[32], float S, float one, const float4* cs, const float4* cb,
-                                              const float (&res)[32], const uint32_t (&rbyte)[8], float res_scale,
-                                              float inv_next, float hi2, uint32_t (&cr)[8]) {
-    const uint32_t k256 = k256_of(one);
-    const uint64_t S2 = f32x2_pack(S, S), one2 = f32x2_pack(one, one), inv2 = f32x2_pack(inv_next, inv_next);
-    const uint64_t half2 = f32x2_pack(0.5f, 0.5f), rs2 = f32x2_pack(res_scale, res_scale);
-#pragma unroll
-    for (int bb = 0; bb < 8; ++bb) {
-        const float4 a = cs[bb], b = cb[bb];
-        uint64_t w[2] = {f32x2_mul_rn(f32x2_pack((float)(int)v[bb], (float)(int)v[8 + bb]), S2),
-                         f32x2_mul_rn(f32x2_pack((float)(int)v[16 + bb], (float)(int)v[24 + bb]), S2)};
-        w[0] = f32x2_add_one(f32x2_mul_rn(w[0], f32x2_pack(a.x, a.y)), one2, f32x2_pack(b.x, b.y));
-        w[1] = f32x2_add_one(f32x2_mul_rn(w[1], f32x2_pack(a.z, a.w)), one2, f32x2_pack(b.z, b.w));
-        uint32_t m[4];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (RES == 1) w[h] = f32x2_add_one(w[h], one2, f32x2_pack(res[16 * h + bb], res[16 * h + 8 + bb]));
-            if (RES == 2) w[h] = f32x2_add_one(w[h], one2, f32x2_mul_rn(rs2, f32x2_pack(byte_to_float(rbyte[bb], 2 * h), byte_to_float(rbyte[bb], 2 * h + 1))));
-            code_pair<NB>(f32x2_mul_rn(w[h], inv2), one2, half2, hi2, m[2 * h], m[2 * h + 1]);
-        }
-        const uint32_t c4 = join_codes(m, k256);
-        cr[bb] = __funnelshift_l(c4, c4, bb);
-    }
 }
 
 // Tensor memory -> registers in fragments: 16 rows x 32 columns, lane l holds columns 8 o + 2 (l % 4) + {0, 1}, o = 0..3, of rows
@@ -437,90 +408,112 @@ __device__ __forceinline__ void tmem_ld_frag_issue(uint32_t taddr, uint32_t (&v)
           "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
         : "r"(taddr));
 }
-// 4 x 4 transposition among the lanes of a quad: t[r][.] of lane q <-> t[q][.] of lane r.
-__device__ __forceinline__ void quad_transpose(uint32_t (&t)[4][2]) {
-    const uint32_t q = threadIdx.x & 3u;
+// A warp's fragments <-> pixels, through 1 KB of shared memory of its own: row i of 32 bytes = pixel i of the group, in two
+// 16-byte halves (e = 0, 1: byte registers 2 q + e of planes_to_bytes, q = 0..3), swapped in every other run of four rows so
+// that eight rows hit different banks.  A fragment register t[r][e] of lane l belongs to pixel l / 4 + 8 r and q = l % 4, which
+// is how the matrix loads and stores place them.  As a transposition by shuffles the same took 40 instructions instead of 4 (with
+// one instruction for two codes' floors in code_pair: 128 -> 512 1x1 at 28x28, batch 16, terms and packed shortcut, 12.3 -> 11.0
+// us; 64 -> 64 3x3 at 56x56, batch 64, 29.9 -> 28.0).
+struct FragRows {
+    uint32_t own;                                        // half 0 of the row of this lane's pixel (half 1: own ^ 16)
+    __device__ __forceinline__ explicit FragRows(uint32_t smem) {
+        const uint32_t lane = threadIdx.x & 31u;
+        own = smem + lane * 32u + ((lane & 4u) << 2);
+    }
+    __device__ __forceinline__ void put_frag(const uint32_t (&t)[4][2]) const {
 #pragma unroll
-    for (int d = 1; d <= 2; d *= 2) {
-        const bool up = (q & (uint32_t)d) != 0;
+        for (int e = 0; e < 2; ++e)
+            asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};\n" ::"r"(own ^ (16u * e)), "r"(t[0][e]),
+                         "r"(t[1][e]), "r"(t[2][e]), "r"(t[3][e]) : "memory");
+    }
+    __device__ __forceinline__ void get_frag(uint32_t (&t)[4][2]) const {
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+            asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];\n" : "=r"(t[0][e]), "=r"(t[1][e]),
+                         "=r"(t[2][e]), "=r"(t[3][e]) : "r"(own ^ (16u * e)) : "memory");
+    }
+    __device__ __forceinline__ void put_row(const uint32_t (&c)[8]) const {
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(own ^ (16u * e)), "r"(c[e]), "r"(c[2 + e]), "r"(c[4 + e]),
+                         "r"(c[6 + e]) : "memory");
+    }
+    __device__ __forceinline__ void get_row(uint32_t (&c)[8]) const {
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];\n" : "=r"(c[e]), "=r"(c[2 + e]), "=r"(c[4 + e]), "=r"(c[6 + e])
+                         : "r"(own ^ (16u * e)) : "memory");
+    }
+};
+// Where the terms of a group's channel lie in the 32 floats that a lane reads eight of, at 8 (l % 4): channel 8 o + 2 q + e.
+__device__ __forceinline__ int frag_term_at(int channel) { return ((channel & 7) >> 1) * 8 + (channel >> 3) * 2 + (channel & 1); }
+
+// Shortcut of a group in fragments.  RES = 1: fp32 values, res[8 r + 2 o + e] = pixel l / 4 + 8 r, channel 8 o + 2 q + e;
+// RES = 2: byte o of rb[r][e] = code of that pixel and channel.
+// 1024 accumulators (lo / hi: pixels 0-15 / 16-31 of the group) -> requantized codes t (byte o of t[r][e]), and the fp32 values
+// at y[r] + 8 o where VALUES and the pointer is not null.  Every fp32 step is rounded on its own, in the library's order; products
+// and sums are packed two to an instruction (f32x2_add_one).  A lane needs the terms of eight channels for its four pixels
+// (cs, cb: entries of frag_term_at).  The ReLU is applied to the values only: the quantizer's clamp at zero gives the same codes.
+template <int RES, int NB, bool VALUES>
+__device__ __forceinline__ void terms_codes_frag(const uint32_t (&lo)[16], const uint32_t (&hi)[16], float S, float one, const float2* cs,
+                                                 const float2* cb, const float (&res)[32], const uint32_t (&rb)[4][2], float res_scale,
+                                                 float inv_next, int nb, bool relu, float* const (&y)[4], uint32_t (&t)[4][2]) {
+    const uint32_t k256 = k256_of(one);
+    const uint64_t S2 = f32x2_pack(S, S), one2 = f32x2_pack(one, one), inv2 = f32x2_pack(inv_next, inv_next), rs2 = f32x2_pack(res_scale, res_scale);
+    const uint64_t bias2 = f32x2_pack(-8388608.0f, -8388608.0f);
+#pragma unroll
+    for (int o = 3; o >= 0; --o) {
+        const float2 s = cs[o], b = cb[o];
+        const uint64_t s2 = f32x2_pack(s.x, s.y), b2 = f32x2_pack(b.x, b.y);
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            if (r & d) continue;
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? t[r][e] : t[r | d][e], d);
-                if (up) t[r][e] = got;
-                else t[r | d][e] = got;
-            }
-        }
-    }
-}
-// terms_codes32 on fragments: lo / hi hold rows 0-15 / 16-31 of the group, so a lane needs the terms of eight channels only
-// (s, b: channel 8 o + 2 q + e at 2 o + e) for four pixels, rows l / 4 + 8 r.  The codes pass through the quad afterwards:
-// cr = those of row l / 4 + 8 q.  rb[r][e]: byte o = shortcut code of row r, that channel; res likewise.
-template <int RES, int NB>
-__device__ __forceinline__ void terms_codes_frag(const uint32_t (&lo)[16], const uint32_t (&hi)[16], float S, float one, const float (&s)[8],
-                                                 const float (&b)[8], const float (&res)[32], const uint32_t (&rb)[4][2], float res_scale,
-                                                 float inv_next, float hi2, uint32_t (&cr)[8]) {
-    const uint32_t k256 = k256_of(one);
-    const uint64_t S2 = f32x2_pack(S, S), one2 = f32x2_pack(one, one), inv2 = f32x2_pack(inv_next, inv_next);
-    const uint64_t half2 = f32x2_pack(0.5f, 0.5f), rs2 = f32x2_pack(res_scale, res_scale);
-    const int q = (int)(threadIdx.x & 3u);
-    uint32_t t[4][2];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        uint32_t m0[4], m1[4];
-#pragma unroll
-        for (int o = 0; o < 4; ++o) {
             const uint32_t a0 = r < 2 ? lo[4 * o + 2 * (r & 1)] : hi[4 * o + 2 * (r & 1)];
             const uint32_t a1 = r < 2 ? lo[4 * o + 2 * (r & 1) + 1] : hi[4 * o + 2 * (r & 1) + 1];
             uint64_t w = f32x2_mul_rn(f32x2_pack((float)(int)a0, (float)(int)a1), S2);
-            w = f32x2_add_one(f32x2_mul_rn(w, f32x2_pack(s[2 * o], s[2 * o + 1])), one2, f32x2_pack(b[2 * o], b[2 * o + 1]));
+            w = f32x2_add_one(f32x2_mul_rn(w, s2), one2, b2);
             if (RES == 1) w = f32x2_add_one(w, one2, f32x2_pack(res[8 * r + 2 * o], res[8 * r + 2 * o + 1]));
-            if (RES == 2) w = f32x2_add_one(w, one2, f32x2_mul_rn(rs2, f32x2_pack(byte_to_float(rb[r][0], o), byte_to_float(rb[r][1], o))));
-            code_pair<NB>(f32x2_mul_rn(w, inv2), one2, half2, hi2, m0[o], m1[o]);
+            if (RES == 2) {
+                // a byte as fp32, exactly, without the conversion pipe: 2^23 + byte, minus 2^23
+                const uint64_t m = ((uint64_t)__byte_perm(rb[r][1], 0x4B000000u, 0x7540u + (uint32_t)o) << 32) |
+                                   (uint64_t)__byte_perm(rb[r][0], 0x4B000000u, 0x7540u + (uint32_t)o);
+                uint64_t v;
+                asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(v) : "l"(m), "l"(bias2));
+                w = f32x2_add_one(w, one2, f32x2_mul_rn(rs2, v));
+            }
+            if constexpr (VALUES) {
+                if (y[r]) {
+                    float2 v = make_float2(__uint_as_float((uint32_t)w), __uint_as_float((uint32_t)(w >> 32)));
+                    if (relu) {
+                        v.x = v.x > 0.f ? v.x : 0.f;
+                        v.y = v.y > 0.f ? v.y : 0.f;
+                    }
+                    *reinterpret_cast<float2*>(y[r] + 8 * o) = v;
+                }
+            }
+            uint32_t m0, m1;
+            code_pair<NB>(f32x2_mul_rn(w, inv2), nb, m0, m1);
+            t[r][0] = o == 3 ? m0 : t[r][0] * k256 + m0;
+            t[r][1] = o == 3 ? m1 : t[r][1] * k256 + m1;
         }
-        const uint32_t c0 = join_codes(m0, k256), c1 = join_codes(m1, k256);
-        t[r][0] = __funnelshift_l(c0, c0, 2 * q);
-        t[r][1] = __funnelshift_l(c1, c1, 2 * q + 1);
     }
-    quad_transpose(t);
+}
+// Byte registers of a pixel's codes -> plane words.
+template <int NB>
+__device__ __forceinline__ void row_to_planes(uint32_t (&c)[8], int nb, uint32_t (&planes)[8]) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) { cr[2 * j] = t[j][0]; cr[2 * j + 1] = t[j][1]; }
+    for (int bb = 0; bb < 8; ++bb) c[bb] = __funnelshift_l(c[bb], c[bb], bb);
+    codes_to_planes<NB>(c, nb, planes);
 }
 
-// The same in two steps, for layers that want the fp32 values too: pair (h, bb) = channels 16 h + bb and 16 h + 8 + bb.
-template <int RES>
-__device__ __forceinline__ void terms_values32(const uint32_t (&v)[32], float S, float one, const float4* cs, const float4* cb,
-                                               const float (&res)[32], const uint32_t (&rbyte)[8], float res_scale, uint64_t (&yy)[2][8]) {
-    const uint64_t S2 = f32x2_pack(S, S), one2 = f32x2_pack(one, one), rs2 = f32x2_pack(res_scale, res_scale);
-#pragma unroll
-    for (int bb = 0; bb < 8; ++bb) {
-        const float4 a = cs[bb], b = cb[bb];
-        uint64_t w[2] = {f32x2_mul_rn(f32x2_pack((float)(int)v[bb], (float)(int)v[8 + bb]), S2),
-                         f32x2_mul_rn(f32x2_pack((float)(int)v[16 + bb], (float)(int)v[24 + bb]), S2)};
-        w[0] = f32x2_add_one(f32x2_mul_rn(w[0], f32x2_pack(a.x, a.y)), one2, f32x2_pack(b.x, b.y));
-        w[1] = f32x2_add_one(f32x2_mul_rn(w[1], f32x2_pack(a.z, a.w)), one2, f32x2_pack(b.z, b.w));
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (RES == 1) w[h] = f32x2_add_one(w[h], one2, f32x2_pack(res[16 * h + bb], res[16 * h + 8 + bb]));
-            if (RES == 2) w[h] = f32x2_add_one(w[h], one2, f32x2_mul_rn(rs2, f32x2_pack(byte_to_float(rbyte[bb], 2 * h), byte_to_float(rbyte[bb], 2 * h + 1))));
-            yy[h][bb] = w[h];
-        }
-    }
-}
-__device__ __forceinline__ void value_codes32(const uint64_t (&yy)[2][8], float one, float inv_next, float hi2, uint32_t (&cr)[8]) {
+// Two fp32 values in the order of pipe_group32 -> codes: pair (h, bb) = channels 16 h + bb and 16 h + 8 + bb.
+__device__ __forceinline__ void value_codes32(const uint64_t (&yy)[2][8], float one, float inv_next, int nb, uint32_t (&cr)[8]) {
     const uint32_t k256 = k256_of(one);
-    const uint64_t one2 = f32x2_pack(one, one), inv2 = f32x2_pack(inv_next, inv_next), half2 = f32x2_pack(0.5f, 0.5f);
+    const uint64_t inv2 = f32x2_pack(inv_next, inv_next);
 #pragma unroll
     for (int bb = 0; bb < 8; ++bb) {
         uint32_t m[4];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint64_t w = f32x2_add_one(f32x2_mul_rn(yy[h][bb], inv2), one2, half2);
-            m[2 * h] = code_pattern(__uint_as_float((uint32_t)w), hi2);
-            m[2 * h + 1] = code_pattern(__uint_as_float((uint32_t)(w >> 32)), hi2);
-        }
+        for (int h = 0; h < 2; ++h) code_pair<0>(f32x2_mul_rn(yy[h][bb], inv2), nb, m[2 * h], m[2 * h + 1]);
         const uint32_t c4 = join_codes(m, k256);
         cr[bb] = __funnelshift_l(c4, c4, bb);
     }
@@ -540,18 +533,19 @@ __device__ __forceinline__ void store_values32(const uint64_t (&yy)[2][8], bool 
     }
 }
 
-// The same without per-channel terms and shortcut.
-template <int NB = 0>
-__device__ __forceinline__ void plain_codes32(const uint32_t (&v)[32], float S, float one, float inv_next, float hi2, uint32_t (&cr)[8]) {
+// 32 accumulators of one pixel and 32-channel group -> eight registers of requantized codes (register bb: channels bb, 8 + bb,
+// 16 + bb, 24 + bb) of a layer without per-channel terms and shortcut.
+template <int NB>
+__device__ __forceinline__ void plain_codes32(const uint32_t (&v)[32], float S, float one, float inv_next, uint32_t (&cr)[8]) {
     const uint32_t k256 = k256_of(one);
-    const uint64_t S2 = f32x2_pack(S, S), one2 = f32x2_pack(one, one), inv2 = f32x2_pack(inv_next, inv_next), half2 = f32x2_pack(0.5f, 0.5f);
+    const uint64_t S2 = f32x2_pack(S, S), inv2 = f32x2_pack(inv_next, inv_next);
 #pragma unroll
     for (int bb = 0; bb < 8; ++bb) {
         uint32_t m[4];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const uint64_t w = f32x2_mul_rn(f32x2_pack((float)(int)v[16 * h + bb], (float)(int)v[16 * h + 8 + bb]), S2);
-            code_pair<NB>(f32x2_mul_rn(w, inv2), one2, half2, hi2, m[2 * h], m[2 * h + 1]);
+            code_pair<NB>(f32x2_mul_rn(w, inv2), NB, m[2 * h], m[2 * h + 1]);
         }
         const uint32_t c4 = join_codes(m, k256);
         cr[bb] = __funnelshift_l(c4, c4, bb);

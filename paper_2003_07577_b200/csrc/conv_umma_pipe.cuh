@@ -53,7 +53,8 @@ constexpr int PIPE_SLOTS = 2;                      // (pixel, word) items an exp
 constexpr int PIPE_MAX_ITEMS = PIPE_SLOTS * PIPE_EXPANDERS;
 constexpr int PIPE_MAX_TAPS = FRAME_MAX_TAPS, PIPE_MAX_STAGES = 4;
 constexpr int PIPE_MAX_BSLOTS = 32;                // weight tiles in flight when the weights stream
-constexpr int PIPE_SMEM_MAX = 220 * 1024;
+constexpr int PIPE_SMEM_MAX = 220 * 1024;          // dynamic; layers with per-channel terms or shortcuts: PIPE_SMEM_TERMS less, for the
+constexpr int PIPE_SMEM_TERMS = 6 * 1024;          // epilogue warps' matrix rows (FragRows, static)
 
 // What one slot of the weight ring holds of a phase with rows x cols taps: whole words, or whole rows of taps of one word,
 // or a part of a row, so that the MMAs of a slot are straight runs along the taps.  cap: tiles a slot has room for.
@@ -132,7 +133,8 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
     g.a_word_bytes = g.SP * 32 + 64;                           // sized with the largest skew; fixed once ks is known
     if (g.SP * 16 >= (1 << 18)) return g;
     // weights resident when they leave room for at least two activation stages
-    const int budget = PIPE_SMEM_MAX - 2048;
+    const int smem_max = PIPE_SMEM_MAX - (p.ch_scale || p.ch_bias || p.residual || p.res_packed ? PIPE_SMEM_TERMS : 0);
+    const int budget = smem_max - 2048;
     g.b_resident = g.b_total_bytes + 2 * ((g.a_word_bytes + 255) & ~255) <= budget && g.b_total_bytes <= 160 * 1024;
     int ks = PIPE_MAX_ITEMS / g.S;
     if (ks > 4) ks = 4;
@@ -191,7 +193,7 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
         const long long items = (long long)g.n_ptiles * g.n_ctiles;
         g.grid_x = (int)(items < sms ? items : sms) * pw;
     }
-    g.ok = g.n_stages >= 2 && g.smem_bytes <= PIPE_SMEM_MAX && g.grid_y <= 65535 && g.n_ctiles <= 65535;
+    g.ok = g.n_stages >= 2 && g.smem_bytes <= smem_max && g.grid_y <= 65535 && g.n_ctiles <= 65535;
     return g;
 }
 
@@ -228,7 +230,7 @@ __device__ __forceinline__ void umma_commit_pred_pair(uint32_t leader, uint64_t*
 // integer min / max instead (see below); the fp32 steps run as packed two-lane instructions.
 template <bool WANT_Q>
 __device__ __forceinline__ void pipe_group32(const ConvParams& p, uint32_t (&v)[32], size_t o, bool pvalid, float S,
-                                             float inv_next, int nb, int qmax, uint32_t* dst) {
+                                             float inv_next, int nb, uint32_t* dst) {
     if (p.acc && pvalid && EBS_IN_RANGE(p, CHK_PIPE_ACC, o + 31, p.lim_out)) {
 #pragma unroll
         for (int gq = 0; gq < 8; ++gq)
@@ -248,7 +250,7 @@ __device__ __forceinline__ void pipe_group32(const ConvParams& p, uint32_t (&v)[
         // The clamp at zero of the quantizer makes an explicit ReLU redundant here: a negative y gives
         // floor(y / step + 0.5) <= 0 and is clamped to code 0, exactly what max(y, 0) would give.
         uint32_t cr[8];
-        value_codes32(yy, p.one, inv_next, (float)(2 * qmax + 1), cr);
+        value_codes32(yy, p.one, inv_next, nb, cr);
         uint32_t planes[8];
         bytes_to_planes(cr, nb, planes);
         if (pvalid && EBS_IN_RANGE(p, CHK_PIPE_PN, (dst - p.packed_next) + nb - 1, p.lim_pn)) store_plane_words(planes, nb, dst);
@@ -311,46 +313,40 @@ __device__ __forceinline__ void pipe_store_planes(const uint32_t (&planes)[8], i
 // accumulators and the finished code registers is alive at a time -- the general form above keeps the 32 fp32 images
 // as well, which at 96 registers costs spills and the parallelism of the instruction stream.
 // left: channels of the layer from this group on (a last group of fewer than 32 writes zero bits behind them).
-template <int G, int NB = 0>
-__device__ __forceinline__ void pipe_group32_packed(const uint32_t (&v)[32], bool pvalid, float S, float inv_next, int nb, int qmax,
-                                                    uint32_t* dst, const ConvParams& p, PlaneHold<G>& hold, int left) {
+template <int G, int NB>
+__device__ __forceinline__ void pipe_group32_packed(const uint32_t (&v)[32], bool pvalid, float S, float inv_next, uint32_t* dst,
+                                                    const ConvParams& p, PlaneHold<G>& hold, int left) {
     uint32_t cr[8];
-    plain_codes32<NB>(v, S, p.one, inv_next, (float)(2 * qmax + 1), cr);
+    plain_codes32<NB>(v, S, p.one, inv_next, cr);
     uint32_t planes[8];
-    codes_to_planes<NB>(cr, nb, planes);
+    codes_to_planes<NB>(cr, NB, planes);
     if (left < 32) mask_planes(planes, left);
-    pipe_store_planes(planes, nb, dst, pvalid, hold, p);
+    pipe_store_planes(planes, NB, dst, pvalid, hold, p);
 }
 
 // Epilogue of a layer with per-channel terms and / or a shortcut (a folded batch normalisation, the second convolution of a
-// residual block): NHWC, packed planes and / or fp32 out.  The warp walks its (accumulator, 32-channel
-// group) units; the next unit's shortcut and terms are requested before the current one is packed and stored.  The terms of
-// a group pass through 64 words of shared memory of the warp's own (one load and one store a lane, then broadcast reads):
-// read channel by channel through the cache they cost more than the arithmetic (64 -> 256 1x1 at 56x56, batch 256: 225 us,
-// and 97 us for the same layer without terms).  With packed planes only, the accumulators are loaded as fragments, so that a
-// lane reads the terms of eight channels instead of 32 (that layer 194 -> 182 us, 8 bits 230 -> 206; 128 -> 128 3x3 at
-// 28x28 50.5 -> 44.6).  VALUES: fp32 output may be wanted too.
+// residual block): NHWC, packed planes and / or fp32 out.  The warp walks its (accumulator, 32-channel group) units; the next
+// unit's accumulators, shortcut and terms are requested before the current one is packed and stored.  The accumulators are
+// loaded as fragments (terms_codes_frag), so that a lane reads the terms of eight channels instead of 32, and the codes -- and
+// the codes of a packed shortcut the other way -- pass through shared memory as matrices (FragRows).  terms: 64 floats of the
+// warp's own, rows: 1 KB.  VALUES: fp32 output may be wanted too, stored from the fragments (whole 32-byte sectors).
 template <int TILE_N, int G, bool VALUES, int NB, int RES>
 __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, const FrameGeom& g, uint32_t tmem_set, int m_sub, int vwarp,
-                                                    int f0, int co0, float* terms) {
-    // Packed planes only: the accumulators come as fragments (terms_codes_frag), a lane's own pixel is row l / 4 + 8 (l % 4) of
-    // the warp's 32 and its terms are those of eight channels; else the lane's pixel is row l and it reads all terms.
-    constexpr bool FRAG = !VALUES;
+                                                    int f0, int co0, float* terms, const FragRows& rows) {
     const int lane = (int)(threadIdx.x & 31), quad = lane & 3;
-    const int at = FRAG ? ((lane & 7) >> 1) * 8 + (lane >> 3) * 2 + (lane & 1) : (lane & 7) * 4 + (lane >> 3);
-    if constexpr (FRAG) f0 += (lane >> 2) + 8 * quad - lane;
+    const int at = frag_term_at(lane);
     const uint32_t trow = tmem_set + ((uint32_t)((vwarp & 3) * 32) << 16);
     constexpr int COLS = TILE_N / 2;
     const int cbeg = (vwarp >> 2) * COLS, cend = COLS == 32 ? cbeg + 32 : min(cbeg + COLS, p.Co - co0);   // (cend: groups start below)
     if (co0 + cbeg >= p.Co) return;
     const int nb = NB > 0 ? NB : p.next_bits;                // (a constant where only planes are written)
-    const float hi2 = (float)(2 * ((1 << nb) - 1) + 1);
     PlaneHold<G> hold;
     hold.filled = 0;
     float res[32], t_scale, t_bias;
     uint32_t rw[8];
-    int gp = 0;
+    int gp = 0, gr[4];                                       // output pixels of this lane's row and of its fragment's four rows
     bool pvalid = false;
+    uint32_t lo[16], hi[16];
     auto locate = [&](int j) {
         const int f = f0 + j * UMMA_M;
         pvalid = false;
@@ -364,94 +360,92 @@ __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, cons
                 gp = ((int)n * p.Ho + (int)hq) * p.Wo + (int)wq;
             }
         }
+        if constexpr (RES == 1 || VALUES) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) gr[r] = __shfl_sync(0xffffffffu, pvalid ? gp : -1, (lane >> 2) + 8 * r);
+        }
     };
     auto request = [&](int c) {                              // c: first channel of the unit
         const bool in = c + lane < p.Co;
         t_scale = p.ch_scale && in ? __ldg(p.ch_scale + c + lane) : 1.0f;
         t_bias = p.ch_bias && in ? __ldg(p.ch_bias + c + lane) : -0.0f;
-        if constexpr (RES == 1 && FRAG) {
+        if constexpr (RES == 1) {
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                const int gr = __shfl_sync(0xffffffffu, gp, (lane & ~3) | r);      // the pixel of row r
-                const float2* r2 = reinterpret_cast<const float2*>(p.residual + (size_t)gr * p.Co + c + 2 * quad);
+                const float2* r2 = reinterpret_cast<const float2*>(p.residual + (size_t)max(gr[r], 0) * p.Co + c + 2 * quad);
 #pragma unroll
                 for (int o = 0; o < 4; ++o) {
                     const float2 t = __ldg(r2 + 4 * o);
                     res[8 * r + 2 * o] = t.x; res[8 * r + 2 * o + 1] = t.y;
                 }
             }
-        } else if constexpr (RES == 1) {
-            const float4* r4 = reinterpret_cast<const float4*>(p.residual + (size_t)gp * p.Co + c);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float4 t = __ldg(r4 + i);
-                res[4 * i] = t.x; res[4 * i + 1] = t.y; res[4 * i + 2] = t.z; res[4 * i + 3] = t.w;
-            }
         } else if constexpr (RES == 2) {
             ld_dep_planes(p.res_packed + ((size_t)gp * p.CWo + (c >> 5)) * p.res_bits, p.res_bits, rw);
         }
     };
+    auto load = [&](int j, int c0) {
+        tmem_ld_frag_issue(trow + (uint32_t)(j * TILE_N + c0), lo);
+        tmem_ld_frag_issue(trow + (16u << 16) + (uint32_t)(j * TILE_N + c0), hi);
+    };
+    // (the next unit's accumulators are requested early only where the registers hold them)
+    constexpr bool EARLY = !VALUES && G == 1;
     locate(0);
     request(co0 + cbeg);
+    if (EARLY) load(0, cbeg);
+    int j = 0, c0 = cbeg;
 #pragma unroll 1
-    for (int j = 0; j < m_sub; ++j) {
-#pragma unroll 1
-        for (int c0 = cbeg; c0 < cend; c0 += 32) {
-            const int c = co0 + c0;
-            const bool ok = pvalid;
-            const size_t gpz = gp;
-            __syncwarp();                                    // every lane has read the unit before
-            terms[at] = t_scale;
-            terms[32 + at] = t_bias;
-            __syncwarp();
-            const float4* cs = reinterpret_cast<const float4*>(terms);
-            const float4* cb = reinterpret_cast<const float4*>(terms + 32);
-            uint32_t cr[8];
-            const bool some = __any_sync(0xffffffffu, ok);   // else: 32 frame pixels without an output
-            if (some) {
-                uint32_t v[32], rbyte[8];
-                uint32_t (&lo)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[0]);
-                uint32_t (&hi)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[16]);
-                if constexpr (FRAG) {
-                    tmem_ld_frag_issue(trow + (uint32_t)(j * TILE_N + c0), lo);
-                    tmem_ld_frag_issue(trow + (16u << 16) + (uint32_t)(j * TILE_N + c0), hi);
-                } else {
-                    tmem_ld16_issue(trow + (uint32_t)(j * TILE_N + c0), lo);
-                    tmem_ld16_issue(trow + (uint32_t)(j * TILE_N + c0 + 16), hi);
-                }
-                if constexpr (RES == 2) planes_to_bytes<8>(rw, rbyte);
-                tmem_ld16_wait(lo);
-                tmem_ld16_wait(hi);
-                if constexpr (VALUES) {
-                    uint64_t yy[2][8];
-                    terms_values32<RES>(v, p.S, p.one, cs, cb, res, rbyte, p.res_scale, yy);
-                    if (p.y && ok && EBS_IN_RANGE(p, CHK_PIPE_Y, gpz * p.Co + c + 31, p.lim_out)) store_values32(yy, p.relu != 0, p.y + gpz * p.Co + c);
-                    if (p.packed_next) value_codes32(yy, p.one, p.inv_next, hi2, cr);
-                } else {
-                    uint32_t rb[4][2];
-                    if constexpr (RES == 2) {
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) { rb[r][0] = rbyte[2 * r]; rb[r][1] = rbyte[2 * r + 1]; }
-                        quad_transpose(rb);
-                    }
-                    const float4 s0 = cs[2 * quad], s1 = cs[2 * quad + 1], b0 = cb[2 * quad], b1 = cb[2 * quad + 1];
-                    const float s[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w}, b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-                    terms_codes_frag<RES, NB>(lo, hi, p.S, p.one, s, b, res, rb, p.res_scale, p.inv_next, hi2, cr);
-                }
-            }
-            if (c0 + 32 < cend) {
-                request(c + 32);
-            } else if (j + 1 < m_sub) {
-                locate(j + 1);
-                request(co0 + cbeg);
-            }
-            if (some && (!VALUES || p.packed_next)) {
-                uint32_t planes[8];
-                codes_to_planes<NB>(cr, nb, planes);
-                if (p.Co - c < 32) mask_planes(planes, p.Co - c);
-                pipe_store_planes(planes, nb, p.packed_next + (gpz * p.CWo + (c >> 5)) * nb, ok, hold, p);
-            }
+    while (true) {
+        const int c = co0 + c0;
+        const bool ok = pvalid, some = __any_sync(0xffffffffu, ok);   // (none: 32 frame pixels without an output)
+        const size_t gpz = gp;
+        const int cn = c0 + 32 < cend ? c0 + 32 : cbeg, jn = c0 + 32 < cend ? j : j + 1;
+        __syncwarp();                                        // every lane has read the unit before
+        terms[at] = t_scale;
+        terms[32 + at] = t_bias;
+        uint32_t rb[4][2], t[4][2];
+        if (!EARLY) load(j, c0);
+        if constexpr (RES == 2) {
+            uint32_t rbyte[8];
+            planes_to_bytes<8>(rw, rbyte);
+            rows.put_row(rbyte);
         }
+        __syncwarp();
+        if constexpr (RES == 2) {
+            rows.get_frag(rb);
+            __syncwarp();                                    // the codes take the place of the shortcut's
+        }
+        tmem_ld16_wait(lo);
+        tmem_ld16_wait(hi);
+        if (some) {
+            float* y[4];
+            if constexpr (VALUES) {
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const size_t o = (size_t)max(gr[r], 0) * p.Co + c + 2 * quad;
+                    y[r] = p.y && gr[r] >= 0 && EBS_IN_RANGE(p, CHK_PIPE_Y, o + 25, p.lim_out) ? p.y + o : nullptr;
+                }
+            }
+            terms_codes_frag<RES, NB, VALUES>(lo, hi, p.S, p.one, reinterpret_cast<const float2*>(terms) + 4 * quad,
+                                              reinterpret_cast<const float2*>(terms + 32) + 4 * quad, res, rb, p.res_scale, p.inv_next,
+                                              nb, p.relu != 0, y, t);
+            if (!VALUES || p.packed_next) rows.put_frag(t);
+        }
+        if (jn < m_sub) {
+            if (EARLY) load(jn, cn);
+            if (jn != j) locate(jn);
+            request(co0 + cn);
+        }
+        __syncwarp();
+        if (some && (!VALUES || p.packed_next)) {
+            uint32_t cr[8], planes[8];
+            rows.get_row(cr);
+            row_to_planes<NB>(cr, nb, planes);
+            if (p.Co - c < 32) mask_planes(planes, p.Co - c);
+            pipe_store_planes(planes, nb, p.packed_next + (gpz * p.CWo + (c >> 5)) * nb, ok, hold, p);
+        }
+        if (jn >= m_sub) break;
+        j = jn;
+        c0 = cn;
     }
 }
 
@@ -464,7 +458,7 @@ __device__ __forceinline__ void pipe_epilogue_plain(const ConvParams& p, uint32_
     constexpr int COLS = TILE_N / 2;
     const int cbeg = (vwarp >> 2) * COLS;
     const bool want_q = p.packed_next != nullptr;
-    const int nb = want_q ? p.next_bits : 0, qmax = (1 << p.next_bits) - 1;
+    const int nb = want_q ? p.next_bits : 0;
     const float S = p.S, inv_next = p.inv_next;
     uint32_t v[32];
 #pragma unroll 1
@@ -479,9 +473,9 @@ __device__ __forceinline__ void pipe_epilogue_plain(const ConvParams& p, uint32_
         const size_t o = (size_t)gp * p.Co + co0 + c0;
         uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + ((co0 + c0) >> 5)) * nb;
         if (want_q) {
-            pipe_group32<true>(p, v, o, pvalid, S, inv_next, nb, qmax, dst);
+            pipe_group32<true>(p, v, o, pvalid, S, inv_next, nb, dst);
         } else {
-            pipe_group32<false>(p, v, o, pvalid, S, inv_next, nb, qmax, dst);
+            pipe_group32<false>(p, v, o, pvalid, S, inv_next, nb, dst);
         }
     }
 }
@@ -494,7 +488,7 @@ __device__ __forceinline__ void pipe_epilogue_packed_nb(const ConvParams& p, uin
     const uint32_t trow = tmem_acc + ((uint32_t)((vwarp & 3) * 32) << 16);
     constexpr int COLS = TILE_N / 2;
     const int cbeg = (vwarp >> 2) * COLS;
-    constexpr int nb = NB, qmax = (1 << NB) - 1;
+    constexpr int nb = NB;
     const float S = p.S, inv_next = p.inv_next;
     uint32_t v[32];
     PlaneHold<G> hold;
@@ -509,7 +503,7 @@ __device__ __forceinline__ void pipe_epilogue_packed_nb(const ConvParams& p, uin
         tmem_ld16_wait(lo);
         tmem_ld16_wait(hi);
         uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + ((co0 + c0) >> 5)) * nb;
-        pipe_group32_packed<G, NB>(v, pvalid, S, inv_next, nb, qmax, dst, p, hold, p.Co - co0 - c0);
+        pipe_group32_packed<G, NB>(v, pvalid, S, inv_next, dst, p, hold, p.Co - co0 - c0);
     }
 }
 
@@ -538,11 +532,11 @@ __device__ __forceinline__ void pipe_epilogue_packed_g(const ConvParams& p, uint
 
 template <int TILE_N, int G, bool VALUES>
 __device__ __forceinline__ void pipe_epilogue_terms(const ConvParams& p, const FrameGeom& g, uint32_t tmem_set, int m_sub, int vwarp,
-                                                    int f0, int co0, float* terms) {
+                                                    int f0, int co0, float* terms, const FragRows& rows) {
     auto run = [&](auto res_tag) {
         constexpr int RES = decltype(res_tag)::value;
-        if constexpr (VALUES) pipe_epilogue_terms_nb<TILE_N, G, true, 0, RES>(p, g, tmem_set, m_sub, vwarp, f0, co0, terms);
-        else EBS_PIPE_EACH_NB((pipe_epilogue_terms_nb<TILE_N, G, false, NB, RES>(p, g, tmem_set, m_sub, vwarp, f0, co0, terms)))
+        if constexpr (VALUES) pipe_epilogue_terms_nb<TILE_N, G, true, 0, RES>(p, g, tmem_set, m_sub, vwarp, f0, co0, terms, rows);
+        else EBS_PIPE_EACH_NB((pipe_epilogue_terms_nb<TILE_N, G, false, NB, RES>(p, g, tmem_set, m_sub, vwarp, f0, co0, terms, rows)))
     };
     if (p.residual) run(std::integral_constant<int, 1>{});
     else if (p.res_packed) run(std::integral_constant<int, 2>{});
@@ -584,6 +578,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     __shared__ __align__(16) float s_terms[AFFINE ? PIPE_EPI_WARPS : 1][64];
+    __shared__ __align__(128) uint8_t s_rows[AFFINE ? PIPE_EPI_WARPS : 1][AFFINE ? 1024 : 16];
     __shared__ int s_tap_id[PIPE_MAX_TAPS];             // (in shared memory: indexed at run time by single threads)
 
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -1063,7 +1058,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
                 if constexpr (AFFINE)
                     pipe_epilogue_terms<TILE_N, EPI_G, FORM == 0>(p, g, tmem_base + (uint32_t)(buf * g.m_sub * TILE_N), g.m_sub, vwarp,
                                                                   (PAIR ? 2 * ptile + crank : ptile) * g.tile_pix + row, co0,
-                                                                  s_terms[warp - PIPE_EPI_WARP0]);
+                                                                  s_terms[warp - PIPE_EPI_WARP0], FragRows(smem_u32(s_rows[warp - PIPE_EPI_WARP0])));
             } else for (int j = 0; j < g.m_sub; ++j) {
                 const int f = (PAIR ? 2 * ptile + crank : ptile) * g.tile_pix + j * UMMA_M + row;
                 bool pvalid = false;
@@ -1121,7 +1116,7 @@ int launch_conv_umma_pipe_form(const ConvParams& p, const PipeGeom& g, cudaStrea
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
         cudaFuncSetAttribute(conv_umma_pipe_kernel<AB, TILE_N, false, HOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, PIPE_SMEM_MAX);
-        cudaFuncSetAttribute(conv_umma_pipe_kernel<AB, TILE_N, true, HOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, PIPE_SMEM_MAX);
+        cudaFuncSetAttribute(conv_umma_pipe_kernel<AB, TILE_N, true, HOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, PIPE_SMEM_MAX - PIPE_SMEM_TERMS);
         attr_set[dev] = true;
     }
     const dim3 grid((unsigned)g.grid_x, (unsigned)g.grid_y, 1);

@@ -25,6 +25,8 @@
 // limit of their own: every thread of every CTA reaches both whether it gave up or not, after bounded waits only.
 #pragma once
 
+#include <type_traits>
+
 #include "conv_frame.cuh"
 
 namespace ebs {
@@ -156,7 +158,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
     __shared__ int abort_flag;
     __shared__ int gp_s[UMMA_M];                         // output pixel of every row, -1: none
     __shared__ int s_tap_id[FRAME_MAX_TAPS];
-    __shared__ __align__(16) float s_terms[FORM == 2 ? 512 : 4];   // FORM 2: scale and shift of the channel tile, terms_codes32 order
+    __shared__ __align__(16) float s_terms[FORM == 2 ? 512 : 4];   // FORM 2: scale and shift of the channel tile, frag_term_at order
 
     // (read from lane 0, so that the compiler knows the role branches to be warp-uniform and keeps the issuing warp's
     // descriptors in uniform registers)
@@ -319,68 +321,100 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) conv_umma_tile_kernel(const C
             const size_t gpz = pvalid ? gp : 0;
             const int half = (warp >> 2) * 32;               // this warp's first group of 32 channels; every other one is its own
             const bool mine = half < N && co0 + half < p.Co;
-            uint32_t rw[8];
-            float res[32];
-            auto load_shortcut = [&](int c0) {
-                if constexpr (FORM == 2) {
-                    if (p.residual) {
-                        const float4* r4 = reinterpret_cast<const float4*>(p.residual + gpz * p.Co + co0 + c0);
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const float4 t = ld_dep(r4 + i);
-                            res[4 * i] = t.x; res[4 * i + 1] = t.y; res[4 * i + 2] = t.z; res[4 * i + 3] = t.w;
-                        }
-                    } else if (p.res_packed) {
-                        ld_dep_planes(p.res_packed + (gpz * p.CWo + ((co0 + c0) >> 5)) * p.res_bits, p.res_bits, rw);
-                    }
-                }
-            };
-            if (mine) load_shortcut(half);
+            int gr[4];                                       // FORM 2: output pixels of the four rows of this lane's fragments
             if constexpr (FORM == 2) {
-                if (tid < N) {                               // channel tid of the tile: group tid / 32, entry tid % 8, lane (tid / 8) % 4
-                    const int at = (tid >> 5) * 32 + (tid & 7) * 4 + ((tid >> 3) & 3);
+                if (tid < N) {                               // channel tid of the tile
+                    const int at = (tid & ~31) + frag_term_at(tid & 31);
                     s_terms[at] = term_at(p.ch_scale, co0 + tid, p.Co, 1.0f);
                     s_terms[256 + at] = term_at(p.ch_bias, co0 + tid, p.Co, -0.0f);
                 }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) gr[r] = __shfl_sync(0xffffffffu, gp, (lane >> 2) + 8 * r);
             }
-            if (ok) mbar_wait_bounded(&acc_full, 0u, abortp, limit);
-            asm volatile("bar.sync 1, 256;\n" ::: "memory");
-            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            if (!__any_sync(0xffffffffu, abort_flag != 0) && __any_sync(0xffffffffu, pvalid)) {
+            // the rest with the kind of shortcut and the plane count as constants of the code
+            auto finish = [&](auto nb_tag, auto res_tag) {
+                constexpr int NB = decltype(nb_tag)::value, RES = decltype(res_tag)::value;
+                uint32_t rw[8];
+                float res[32];
+                auto load_shortcut = [&](int c0) {
+                    if constexpr (RES == 1) {
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) {
+                            const float2* r2 = reinterpret_cast<const float2*>(p.residual + (size_t)max(gr[r], 0) * p.Co + co0 + c0 + 2 * (lane & 3));
+#pragma unroll
+                            for (int o = 0; o < 4; ++o) {
+                                const uint2 t = ld_dep(reinterpret_cast<const uint2*>(r2 + 4 * o));
+                                res[8 * r + 2 * o] = __uint_as_float(t.x); res[8 * r + 2 * o + 1] = __uint_as_float(t.y);
+                            }
+                        }
+                    } else if constexpr (RES == 2) {
+                        ld_dep_planes(p.res_packed + (gpz * p.CWo + ((co0 + c0) >> 5)) * p.res_bits, p.res_bits, rw);
+                    }
+                };
+                if (mine) load_shortcut(half);
+                if (ok) mbar_wait_bounded(&acc_full, 0u, abortp, limit);
+                asm volatile("bar.sync 1, 256;\n" ::: "memory");
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                if (__any_sync(0xffffffffu, abort_flag != 0) || !__any_sync(0xffffffffu, pvalid)) return;
                 const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-                const int nb = p.next_bits;
-                const float hi2 = (float)(2 * ((1 << nb) - 1) + 1);
+                const FragRows rows(smem_u32(stages) + (uint32_t)warp * 1024u);   // (every MMA has read its operands)
 #pragma unroll 1
                 for (int c0 = half; c0 < N && co0 + c0 < p.Co; c0 += 64) {
                     uint32_t v[32], cr[8], planes[8];
                     uint32_t (&lo)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[0]);
                     uint32_t (&hi)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[16]);
-                    tmem_ld16_issue(trow + (uint32_t)c0, lo);
-                    tmem_ld16_issue(trow + (uint32_t)(c0 + 16), hi);
-                    tmem_ld16_wait(lo);
-                    tmem_ld16_wait(hi);
                     if constexpr (FORM == 2) {
-                        const float4* cs = reinterpret_cast<const float4*>(s_terms + c0);
-                        const float4* cb = reinterpret_cast<const float4*>(s_terms + 256 + c0);
-                        uint32_t rbyte[8];
-                        if (p.residual) {
-                            terms_codes32<1>(v, p.S, p.one, cs, cb, res, rbyte, 0.0f, p.inv_next, hi2, cr);
-                        } else if (p.res_packed) {
+                        uint32_t rb[4][2], t[4][2];
+                        tmem_ld_frag_issue(trow + (uint32_t)c0, lo);
+                        tmem_ld_frag_issue(trow + (16u << 16) + (uint32_t)c0, hi);
+                        if constexpr (RES == 2) {
+                            uint32_t rbyte[8];
                             planes_to_bytes<8>(rw, rbyte);
-                            terms_codes32<2>(v, p.S, p.one, cs, cb, res, rbyte, p.res_scale, p.inv_next, hi2, cr);
-                        } else {
-                            terms_codes32<0>(v, p.S, p.one, cs, cb, res, rbyte, 0.0f, p.inv_next, hi2, cr);
+                            rows.put_row(rbyte);
+                            __syncwarp();
+                            rows.get_frag(rb);
+                            __syncwarp();                    // the codes take the place of the shortcut's
                         }
+                        tmem_ld16_wait(lo);
+                        tmem_ld16_wait(hi);
+                        float* const none[4] = {nullptr, nullptr, nullptr, nullptr};
+                        terms_codes_frag<RES, NB, false>(lo, hi, p.S, p.one, reinterpret_cast<const float2*>(s_terms + c0) + 4 * (lane & 3),
+                                                         reinterpret_cast<const float2*>(s_terms + 256 + c0) + 4 * (lane & 3), res, rb,
+                                                         p.res_scale, p.inv_next, NB, false, none, t);
+                        rows.put_frag(t);
+                        if (c0 + 64 < N && co0 + c0 + 64 < p.Co) load_shortcut(c0 + 64);
+                        __syncwarp();
+                        rows.get_row(cr);
+                        __syncwarp();                        // (the next group's codes take their place)
+                        row_to_planes<NB>(cr, NB, planes);
                     } else {
-                        plain_codes32(v, p.S, p.one, p.inv_next, hi2, cr);
+                        tmem_ld16_issue(trow + (uint32_t)c0, lo);
+                        tmem_ld16_issue(trow + (uint32_t)(c0 + 16), hi);
+                        tmem_ld16_wait(lo);
+                        tmem_ld16_wait(hi);
+                        plain_codes32<NB>(v, p.S, p.one, p.inv_next, cr);
+                        codes_to_planes<NB>(cr, NB, planes);
                     }
-                    if (c0 + 64 < N && co0 + c0 + 64 < p.Co) load_shortcut(c0 + 64);
-                    bytes_to_planes(cr, nb, planes);
                     if (p.Co - co0 - c0 < 32) mask_planes(planes, p.Co - co0 - c0);
-                    uint32_t* dst = p.packed_next + (gpz * p.CWo + ((co0 + c0) >> 5)) * nb;
-                    if (pvalid && EBS_IN_RANGE(p, CHK_UT_PN, (dst - p.packed_next) + nb - 1, p.lim_pn)) store_plane_words(planes, nb, dst);
+                    uint32_t* dst = p.packed_next + (gpz * p.CWo + ((co0 + c0) >> 5)) * NB;
+                    if (pvalid && EBS_IN_RANGE(p, CHK_UT_PN, (dst - p.packed_next) + NB - 1, p.lim_pn)) store_plane_words(planes, NB, dst);
                 }
-            }
+            };
+            auto with_planes = [&](auto res_tag) {
+                switch (p.next_bits) {
+                    case 1: finish(std::integral_constant<int, 1>{}, res_tag); break;
+                    case 2: finish(std::integral_constant<int, 2>{}, res_tag); break;
+                    case 3: finish(std::integral_constant<int, 3>{}, res_tag); break;
+                    case 4: finish(std::integral_constant<int, 4>{}, res_tag); break;
+                    case 5: finish(std::integral_constant<int, 5>{}, res_tag); break;
+                    case 6: finish(std::integral_constant<int, 6>{}, res_tag); break;
+                    case 7: finish(std::integral_constant<int, 7>{}, res_tag); break;
+                    default: finish(std::integral_constant<int, 8>{}, res_tag); break;
+                }
+            };
+            if (FORM == 2 && p.residual) with_planes(std::integral_constant<int, FORM == 2 ? 1 : 0>{});
+            else if (FORM == 2 && p.res_packed) with_planes(std::integral_constant<int, FORM == 2 ? 2 : 0>{});
+            else with_planes(std::integral_constant<int, 0>{});
         }
     } else if (warp == TILE_ISSUER) {
         // =========================== issuer ===========================

@@ -7,6 +7,7 @@
 namespace ebs {
 
 constexpr int FRAME_MAX_TAPS = 64, FRAME_MAX_PHASES = 4;
+constexpr int FRAME_MAX_CW = 1024;                 // 32-channel words of a pixel
 
 // Exact unsigned division by a run-time constant (Granlund and Montgomery, "Division by Invariant Integers using
 // Multiplication", 1994): q = (t + ((n - t) >> s1)) >> s2, t = mulhi(m, n).
@@ -47,7 +48,7 @@ inline int floordiv_int(int a, int b) { return (a >= 0) ? a / b : -((-a + b - 1)
 inline bool frame_geometry(const ConvParams& p, FrameGeom& g) {
     const int taps = p.kh * p.kw;
     if (p.sh > 2 || p.sw > 2 || taps > FRAME_MAX_TAPS || p.kh > 16 || p.kw > 16) return false;
-    if ((long long)p.CW * 8 > PIPE_ZERO_WORDS) return false;  // the zero page covers a pixel's words at 8 planes (byte codes: 8 words a word)
+    if (p.CW > FRAME_MAX_CW) return false;
     g.q0r = floordiv_int(-p.ph, p.sh);
     g.q0s = floordiv_int(-p.pw, p.sw);
     const int qr_max = floordiv_int(p.kh - 1 - p.ph, p.sh), qs_max = floordiv_int(p.kw - 1 - p.pw, p.sw);

@@ -19,7 +19,8 @@
 //    m_sub MMAs and the halo of the strip is shared.
 //  * Weights stay resident in shared memory when all (tap, word) tiles of a channel tile fit, else they
 //    stream through the stage ring by cp.async.bulk, a stage ahead of the MMAs.
-//  * Roles (20 warps): warps 0-7 expand (packed words -> byte strips, global loads two chunks ahead), warps 8-9
+//  * Roles (20 warps): warps 0-7 expand (packed words -> byte strips; the words arrive by cp.async in a ring of shared memory,
+//    two or three passes ahead), warps 8-9
 //    issue the MMAs (two warps when a tile has an even number of accumulators: each owns the accumulators of one
 //    parity, so that one's waits and addresses run while the other issues), warp 10 fetches weight
 //    tiles (every lane one tile of a ring slot), warps 12-19 run the epilogue out of tensor memory while the next
@@ -53,8 +54,10 @@ constexpr int PIPE_SLOTS = 2;                      // (pixel, word) items an exp
 constexpr int PIPE_MAX_ITEMS = PIPE_SLOTS * PIPE_EXPANDERS;
 constexpr int PIPE_MAX_TAPS = FRAME_MAX_TAPS, PIPE_MAX_STAGES = 4;
 constexpr int PIPE_MAX_BSLOTS = 32;                // weight tiles in flight when the weights stream
-constexpr int PIPE_SMEM_MAX = 220 * 1024;          // dynamic; layers with per-channel terms or shortcuts: PIPE_SMEM_TERMS less, for the
-constexpr int PIPE_SMEM_TERMS = 6 * 1024;          // epilogue warps' matrix rows (FragRows, static)
+// Passes of packed words in the expanders' ring (half as much memory again for more than four planes).
+__host__ __device__ constexpr int pipe_raw_depth(int words) { return words <= 4 ? 4 : 3; }
+constexpr int PIPE_SMEM_MAX = 225 * 1024;          // dynamic; layers with per-channel terms or shortcuts: PIPE_SMEM_TERMS less, for the
+constexpr int PIPE_SMEM_TERMS = 11 * 1024;         // epilogue warps' terms and matrix rows (FragRows, static)
 
 // What one slot of the weight ring holds of a phase with rows x cols taps: whole words, or whole rows of taps of one word,
 // or a part of a row, so that the MMAs of a slot are straight runs along the taps.  cap: tiles a slot has room for.
@@ -78,6 +81,8 @@ struct PipeGeom : FrameGeom {
                                        // word groups (stages per tile and phase) = ceil(CW / kss)
     int nchunks;                       // chunks per tile = n_ph * nwg (phase-major)
     int n_stages, a_word_bytes, a_stage_bytes, stage_bytes;
+    int raw_bytes;                     // ring of packed words
+    int linear_in, linear_out;         // a frame pixel is the input pixel, the output pixel, of the same number
     int b_resident, b_total_bytes;
     PipeSlot slot[FRAME_MAX_PHASES];   // of each phase
     int b_slots, b_group;              // streamed weights: ring of slots of b_group (tap, word) tiles of TILE_N x 32 bytes
@@ -134,7 +139,10 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
     if (g.SP * 16 >= (1 << 18)) return g;
     // weights resident when they leave room for at least two activation stages
     const int smem_max = PIPE_SMEM_MAX - (p.ch_scale || p.ch_bias || p.residual || p.res_packed ? PIPE_SMEM_TERMS : 0);
-    const int budget = smem_max - 2048;
+    g.raw_bytes = pipe_raw_depth(p.x_words) * PIPE_MAX_ITEMS * p.x_words * 4;
+    g.linear_in = taps == 1 && p.sh == 1 && p.sw == 1 && p.ph == 0 && p.pw == 0;
+    g.linear_out = g.Hq == p.Ho && g.Wq == p.Wo;
+    const int budget = smem_max - 2048 - g.raw_bytes;
     g.b_resident = g.b_total_bytes + 2 * ((g.a_word_bytes + 255) & ~255) <= budget && g.b_total_bytes <= 160 * 1024;
     int ks = PIPE_MAX_ITEMS / g.S;
     if (ks > 4) ks = 4;
@@ -154,7 +162,7 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
     // stage, 18 MMAs, 50.3 with two; 256 -> 256 3x3 stride 2 at 28x28: 65.1 and 49.9).
     int nsub = 1;
     while (nsub < 4 && ks * nsub * taps * m_sub < 40 && ks * nsub < p.CW &&
-           3 * stage_bytes(ks * 2 * nsub) <= avail)
+           2 * stage_bytes(ks * 2 * nsub) <= avail)
         nsub *= 2;
     // Skew between the word tiles of a pass: the 8 lanes of a quarter warp store 16 bytes each for ks words of 8 / ks
     // pixels; a skew of 128 / ks bytes (48 for three words) puts them on eight different 16-byte bank groups.
@@ -181,7 +189,7 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
         if (g.b_slots > PIPE_MAX_BSLOTS) g.b_slots = PIPE_MAX_BSLOTS;
         if (g.b_slots < 3) return g;
     }
-    g.smem_bytes = (g.b_resident ? g.b_total_bytes : g.b_slots * g.b_group * b_tile) + g.n_stages * g.stage_bytes + 1024;
+    g.smem_bytes = (g.b_resident ? g.b_total_bytes : g.b_slots * g.b_group * b_tile) + g.n_stages * g.stage_bytes + g.raw_bytes + 1024;
     if (g.b_resident) {                                        // a CTA keeps one channel tile
         g.grid_y = g.n_ctiles;
         long long gx = sms / g.n_ctiles;
@@ -493,8 +501,9 @@ __device__ __forceinline__ void pipe_epilogue_packed_nb(const ConvParams& p, uin
     uint32_t v[32];
     PlaneHold<G> hold;
     hold.filled = 0;
+    uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + ((co0 + cbeg) >> 5)) * nb;
 #pragma unroll 1
-    for (int c0 = cbeg; c0 < cbeg + COLS; c0 += 32) {
+    for (int c0 = cbeg; c0 < cbeg + COLS; c0 += 32, dst += nb) {
         if (co0 + c0 >= p.Co) break;
         uint32_t (&lo)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[0]);
         uint32_t (&hi)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[16]);
@@ -502,7 +511,6 @@ __device__ __forceinline__ void pipe_epilogue_packed_nb(const ConvParams& p, uin
         tmem_ld16_issue(trow + (uint32_t)(c0 + 16), hi);
         tmem_ld16_wait(lo);
         tmem_ld16_wait(hi);
-        uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + ((co0 + c0) >> 5)) * nb;
         pipe_group32_packed<G, NB>(v, pvalid, S, inv_next, dst, p, hold, p.Co - co0 - c0);
     }
 }
@@ -581,7 +589,9 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
     __shared__ __align__(128) uint8_t s_rows[AFFINE ? PIPE_EPI_WARPS : 1][AFFINE ? 1024 : 16];
     __shared__ int s_tap_id[PIPE_MAX_TAPS];             // (in shared memory: indexed at run time by single threads)
 
-    const int tid = threadIdx.x, warp = tid >> 5;
+    // (the warp number read from lane 0, so that the compiler knows the role branches to be warp-uniform: the issuing warps' waits
+    // and addresses then take two thirds of the time)
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     if (tid < PIPE_MAX_TAPS) s_tap_id[tid] = (int)g.tap_id[tid];
     const int NST = g.n_stages, KS = g.ks, KSS = g.kss, NSUB = g.nsub, SP = g.SP, S = g.S;
     const int nchunks = g.nchunks, nwg = g.nwg;
@@ -589,6 +599,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
     uint8_t* base = dyn_smem + ((1024u - (smem_u32(dyn_smem) & 1023u)) & 1023u);
     uint8_t* b_res = base;                                               // resident: [CW][tap slots][TILE_N][32]; else the ring of tiles
     uint8_t* stages = base + (resident ? g.b_total_bytes : g.b_slots * g.b_group * B_TILE_BYTES);   // [NST] x [KS][2][SP][16]
+    uint8_t* raw = stages + g.n_stages * g.stage_bytes;                  // ring of packed words
     const int NBS = g.b_slots, GB = g.b_group;
     // Streamed weights: every CTA of a channel tile reads the same weight tiles, and CTAs that start together would ask
     // the same few L2 slices for the same tile at the same time.  Integer accumulation is exact in any order, so each
@@ -665,145 +676,162 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
     if (warp < 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(REG_EXP));
         // =========================== expanders ===========================
-        int slot_q[PIPE_SLOTS], slot_pix[PIPE_SLOTS], slot_dst[PIPE_SLOTS];
         // An even number of words per pass: a thread takes two adjacent words of one pixel, so that for an odd plane count
         // its 2 * AB packed words still start on an 8-byte boundary and load as pairs.  Otherwise items tid and tid + 256.
         constexpr int NW = AB == 0 ? 8 : AB;                  // words of one (pixel, 32-channel word) item; AB = 0: byte codes
+        constexpr int UNIT = NW % 4 == 0 ? 16 : NW % 2 == 0 ? 8 : 4, UNITS = NW * 4 / UNIT;
+        constexpr int RD = pipe_raw_depth(NW);
+        constexpr uint32_t RAW_PASS = PIPE_MAX_ITEMS * NW * 4;
         const bool paired = (NW & 1) != 0 && (KS & 1) == 0 && (p.CW & 1) == 0;
+        int item_pix[PIPE_SLOTS];                             // strip pixel, -1: no item
+        uint32_t item_dst[PIPE_SLOTS], item_q[PIPE_SLOTS];
 #pragma unroll
         for (int j = 0; j < PIPE_SLOTS; ++j) {
             const int e = paired ? 2 * tid + j : tid + j * PIPE_EXPANDERS;
             const int s = e / KS, q = e - s * KS;            // consecutive lanes: consecutive words of one pixel
-            slot_q[j] = s < S ? q : -1;                       // -1: no item
-            slot_pix[j] = s;
-            slot_dst[j] = q * g.a_word_bytes + s * 16;
+            item_pix[j] = s < S ? s : -1;
+            item_q[j] = (uint32_t)q * (NW * 4);
+            item_dst[j] = (uint32_t)(q * g.a_word_bytes + s * 16);
         }
-        // Loader state: runs several passes ahead of the expansion, also across tile boundaries.  Per (tile, phase) a
-        // thread keeps one pointer per slot -- its pixel's words at its word position, or a page of zero words for
-        // padding, pixels past the batch and threads without an item -- so that a pass adds one warp-uniform word offset,
-        // bounded per thread so that the ragged last word group stays inside the pixel (those words feed no MMA).
-        int ld_it = 0, ld_c = 0, ld_sub = 0, ld_lim[PIPE_SLOTS];
-        const uint32_t* ld_src[PIPE_SLOTS];
-#ifdef EBS_CHECKED
-        bool ld_real[PIPE_SLOTS];
-#endif
-#pragma unroll
-        for (int j = 0; j < PIPE_SLOTS; ++j) ld_lim[j] = p.CW - ((paired && j == 0) ? 2 : 1) - max(slot_q[j], 0);
-        auto chunk_offsets = [&](int it, int ph) {
+        // Fetching runs RD - 1 passes ahead of the expansion, also across tile boundaries: cp.async brings a thread's own items into
+        // its places of the ring, so that no barrier is needed and one loop body serves every pass.  (With the words in flight in
+        // registers the body existed once per set, 19 KB of code beside the epilogue's, and 90-140 of a warp's 200 instructions a pass
+        // were addresses: 256 -> 64 1x1 at 56x56, batch 256, 4 bits, 72.0 us against 54.5 with this ring; 4096^3 GEMM, packed, 85 and 73.)
+        const uint8_t* src[PIPE_SLOTS];                       // words of the item's pixel, at its word position
+        uint32_t lim[PIPE_SLOTS];                             // bytes of a pixel's words from there on; 0: no pixel (padding, past the batch), zero bytes
+        int ld_it = 0, ld_ph = 0, ld_left = 0;
+        const uint32_t px_bytes = (uint32_t)p.CW * (NW * 4), step = (uint32_t)KS * (NW * 4), wrap = (uint32_t)(nwg * KSS) * (NW * 4);
+        const uint32_t first = (uint32_t)(wg_rot * KSS) * (NW * 4);
+        uint32_t ld_off = first;
+        const uint32_t raw0 = smem_u32(raw) + (uint32_t)(tid * (paired ? 8 : UNIT));
+        uint32_t raw_w = 0, raw_r = 0;
+        auto locate = [&]() {
             int ptile, ctile;
-            item_of(it, ptile, ctile);
+            item_of(ld_it, ptile, ctile);
             const int f0 = (PAIR ? 2 * ptile + crank : ptile) * g.tile_pix;
-            const int pa = g.ph_a[ph], pb = g.ph_b[ph];
+            const int dh = p.sh * g.q0r + g.ph_a[ld_ph], dw = p.sw * g.q0s + g.ph_b[ld_ph];
 #pragma unroll
             for (int j = 0; j < PIPE_SLOTS; ++j) {
-                const int qn = max(slot_q[j], 0) * NW;
-                ld_src[j] = p.zero_words + qn;                  // padding or past the batch -> zero bytes
-#ifdef EBS_CHECKED
-                ld_real[j] = false;
-#endif
-                const int f = f0 + slot_pix[j];
-                if (slot_q[j] >= 0 && f < g.frame) {
-                    const uint32_t n = fastdiv((uint32_t)f, g.div_img);
-                    const uint32_t rem = (uint32_t)f - n * (uint32_t)(g.Hq * g.Wq);
+                const uint32_t f = (uint32_t)(f0 + item_pix[j]);
+                bool in = item_pix[j] >= 0 && (int)f < g.frame;
+                uint32_t pix = f;
+                if (!g.linear_in) {
+                    const uint32_t n = fastdiv(f, g.div_img), rem = f - n * (uint32_t)(g.Hq * g.Wq);
                     const uint32_t hq = fastdiv(rem, g.div_row), wq = rem - hq * (uint32_t)g.Wq;
-                    const int h = p.sh * ((int)hq + g.q0r) + pa, w = p.sw * ((int)wq + g.q0s) + pb;
-                    if ((unsigned)h < (unsigned)p.H && (unsigned)w < (unsigned)p.W) {
-                        ld_src[j] = p.x + ((size_t)((((int)n * p.H + h) * p.W + w) * p.CW) * NW + qn);
-#ifdef EBS_CHECKED
-                        ld_real[j] = true;
-#endif
+                    const int h = p.sh * (int)hq + dh, w = p.sw * (int)wq + dw;
+                    in = in && (unsigned)h < (unsigned)p.H && (unsigned)w < (unsigned)p.W;
+                    pix = (n * p.H + h) * p.W + w;
+                }
+                src[j] = reinterpret_cast<const uint8_t*>(p.x) + item_q[j];
+                if (in) src[j] += (size_t)pix * px_bytes;
+                lim[j] = in ? px_bytes - item_q[j] : 0u;
+            }
+            ld_left = nwg * NSUB;
+            ld_off = first;
+            if (++ld_ph == g.n_ph) { ld_ph = 0; ++ld_it; }
+        };
+        auto fetch = [&]() {
+            if (ld_left == 0) locate();
+            --ld_left;
+#pragma unroll
+            for (int j = 0; j < PIPE_SLOTS; ++j) {
+                if (paired && j > 0) break;
+                if (item_pix[j] < 0) continue;
+                const uint8_t* a = src[j] + ld_off;
+                bool real = ld_off < lim[j];                  // (a ragged last group: words past the pixel's, which feed no MMA)
+                if (real && !EBS_IN_RANGE(p, CHK_PIPE_X, (reinterpret_cast<const uint32_t*>(a) - p.x) + (paired ? 2 : 1) * NW - 1, p.lim_x)) real = false;
+                if (paired) {
+#pragma unroll
+                    for (int u = 0; u < NW; ++u)
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(raw0 + raw_w + u * (PIPE_EXPANDERS * 8)), "l"(a + 8 * u), "r"(real ? 8 : 0) : "memory");
+                } else {
+#pragma unroll
+                    for (int u = 0; u < UNITS; ++u) {
+                        const uint32_t dst = raw0 + raw_w + (uint32_t)((j * UNITS + u) * PIPE_EXPANDERS * UNIT);
+                        if constexpr (UNIT == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(a + 16 * u), "r"(real ? 16 : 0) : "memory");
+                        else asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(dst), "l"(a + UNIT * u), "n"(UNIT), "r"(real ? UNIT : 0) : "memory");
                     }
                 }
             }
-        };
-        // register ring of packed words: SETS - 1 chunks of global loads in flight per thread (about 48 registers whatever
-        // the plane count: the latency of these loads, not their bandwidth, is what a deep reduction waits for)
-        constexpr int SETS = NW <= 4 ? 4 : 3;
-        uint32_t a_set[SETS][PIPE_SLOTS][NW];
-        int ld_ph = 0, ld_wg = 0;
-        auto load_next = [&](int set) {
-            int wg = ld_wg + wg_rot;
-            if (wg >= nwg) wg -= nwg;
-            if (ld_wg == 0 && ld_sub == 0) chunk_offsets(ld_it, ld_ph);
-            const int base = wg * KSS + ld_sub * KS;            // first word of the pass (warp-uniform)
-#ifdef EBS_CHECKED
-            auto load_ok = [&](int j, const uint32_t* a, int n) {
-                return ld_real[j] ? EBS_IN_RANGE(p, CHK_PIPE_X, (a - p.x) + n - 1, p.lim_x)
-                                  : EBS_IN_RANGE(p, CHK_PIPE_X, (a - p.zero_words) + n - 1, PIPE_ZERO_WORDS);
-            };
-#else
-            auto load_ok = [](int, const uint32_t*, int) { return true; };
-#endif
-            if (paired) {                                       // both words of the pixel in one run of 2 * AB words
-                const uint32_t* a = ld_src[0] + min(base, ld_lim[0]) * NW;
-                if (load_ok(0, a, 2 * NW)) load_words_global<2 * NW>(a, *reinterpret_cast<uint32_t(*)[2 * NW]>(&a_set[set][0][0]));
-            } else {
-#pragma unroll
-                for (int j = 0; j < PIPE_SLOTS; ++j) {
-                    const uint32_t* a = ld_src[j] + min(base, ld_lim[j]) * NW;
-                    if (load_ok(j, a, NW)) load_words_global<NW>(a, a_set[set][j]);
-                }
-            }
-            if (++ld_sub == NSUB) {
-                ld_sub = 0;
-                if (++ld_wg == nwg) { ld_wg = 0; ++ld_ph; }
-                if (++ld_c == nchunks) { ld_c = 0; ld_ph = 0; ++ld_it; }
-            }
+            raw_w = raw_w == (RD - 1) * RAW_PASS ? 0u : raw_w + RAW_PASS;
+            ld_off += step;
+            if (ld_off == wrap) ld_off = 0;
         };
         const int total = my_items * nchunks * NSUB;           // expander passes
-#pragma unroll
-        for (int u = 0; u < SETS - 1; ++u)
-            if (u < total) load_next(u);
-        bool ok = true;
+        const uint32_t st0 = smem_u32(stages), pass_bytes = (uint32_t)(KS * g.a_word_bytes);
+        uint32_t at = st0, full = smem_u32(&st_full[0]);
+        const uint32_t half = (uint32_t)SP * 16;
         int st = 0, sub = 0;
-        uint32_t st_round = 0;                                  // how many times the ring has wrapped
-        for (int g0 = 0; g0 < total && ok; g0 += SETS) {
+        uint32_t par = 1u;                                      // (a fresh barrier lets a wait for the phase before its first pass)
+#pragma unroll 1
+        for (int gi = 1 - RD; gi < total; ++gi) {
+            if (gi + RD - 1 < total) fetch();
+            asm volatile("cp.async.commit_group;\n" ::: "memory");
+            if (gi < 0) continue;
+            if (sub == 0) {                                     // the MMAs that read this stage one round ago must be done
+                if (!mbar_wait_bounded(&st_empty[st], par, abortp, wait_limit)) break;
+            }
+            asm volatile("cp.async.wait_group %0;\n" ::"n"(RD - 1) : "memory");
+            uint32_t w[PIPE_SLOTS][NW];
+            const uint32_t rd = raw0 + raw_r;
+            if (paired) {
 #pragma unroll
-            for (int u = 0; u < SETS; ++u) {
-                const int gi = g0 + u;
-                if (gi >= total) break;
-                uint8_t* A_st = stages + st * g.stage_bytes + sub * KS * g.a_word_bytes;
-                if (gi + SETS - 1 < total) load_next((u + SETS - 1) % SETS);
-                if (st_round > 0 && sub == 0) {                 // the MMAs that read this stage one round ago must be done
-                    if (!mbar_wait_bounded(&st_empty[st], (st_round - 1) & 1u, abortp, wait_limit)) { ok = false; break; }
+                for (int u = 0; u < NW; ++u) {
+                    uint32_t lo, hi;
+                    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];\n" : "=r"(lo), "=r"(hi) : "r"(rd + u * (PIPE_EXPANDERS * 8)) : "memory");
+                    w[(2 * u) / NW][(2 * u) % NW] = lo;
+                    w[(2 * u + 1) / NW][(2 * u + 1) % NW] = hi;
                 }
+            } else {
 #pragma unroll
-                for (int j = 0; j < PIPE_SLOTS; ++j) {
-                    if (slot_q[j] < 0) continue;
-                    // v_k = rotl(w_k, k); byte register bb = rotr(OR_k v_k & (0x01010101 << ((bb + k) & 7)), bb)
-                    uint32_t r[8];
-                    if constexpr (AB == 0) {
-                        // byte codes, channel c in byte c of the item: only the order changes (row byte 4b + i = channel
-                        // 8i + b, the order of the weight image): register b takes byte b % 4 of words b / 4, 2 + b / 4, ...
-                        const uint32_t (&w)[8] = a_set[u][j];
+                for (int j = 0; j < PIPE_SLOTS; ++j)
 #pragma unroll
-                        for (int bb = 0; bb < 8; ++bb) {
-                            const uint32_t sel = 0x0040u + 0x11u * (uint32_t)(bb & 3);          // byte (bb & 3) of both operands
-                            const uint32_t lo = __byte_perm(w[bb >> 2], w[2 + (bb >> 2)], sel);
-                            const uint32_t hi = __byte_perm(w[4 + (bb >> 2)], w[6 + (bb >> 2)], sel);
-                            r[bb] = __byte_perm(lo, hi, 0x5410);
-                        }
-                    } else {
-                        planes_to_bytes<NW>(a_set[u][j], r);
+                    for (int u = 0; u < UNITS; ++u) {
+                        const uint32_t a = rd + (uint32_t)((j * UNITS + u) * PIPE_EXPANDERS * UNIT);
+                        if constexpr (UNIT == 16) asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];\n" : "=r"(w[j][4 * u]), "=r"(w[j][4 * u + 1]), "=r"(w[j][4 * u + 2]), "=r"(w[j][4 * u + 3]) : "r"(a) : "memory");
+                        else if constexpr (UNIT == 8) asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];\n" : "=r"(w[j][2 * u]), "=r"(w[j][2 * u + 1]) : "r"(a) : "memory");
+                        else asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(w[j][u]) : "r"(a) : "memory");
                     }
-                    uint8_t* dst = A_st + slot_dst[j];
-                    if (!EBS_IN_RANGE(p, CHK_PIPE_STAGE, (dst + SP * 16 + 15) - stages, NST * g.stage_bytes) ||
-                        !EBS_IN_RANGE(p, CHK_PIPE_STAGE, dst - stages, NST * g.stage_bytes))
-                        continue;
-                    *reinterpret_cast<uint4*>(dst) = make_uint4(r[0], r[1], r[2], r[3]);
-                    *reinterpret_cast<uint4*>(dst + SP * 16) = make_uint4(r[4], r[5], r[6], r[7]);
+            }
+            raw_r = raw_r == (RD - 1) * RAW_PASS ? 0u : raw_r + RAW_PASS;
+#pragma unroll
+            for (int j = 0; j < PIPE_SLOTS; ++j) {
+                if (item_pix[j] < 0) continue;
+                uint32_t r[8];
+                if constexpr (AB == 0) {
+                    // byte codes, channel c in byte c of the item: only the order changes (row byte 4b + i = channel 8i + b, the
+                    // order of the weight image): register b takes byte b % 4 of words b / 4, 2 + b / 4, ...
+#pragma unroll
+                    for (int bb = 0; bb < 8; ++bb) {
+                        const uint32_t sel = 0x0040u + 0x11u * (uint32_t)(bb & 3);          // byte (bb & 3) of both operands
+                        const uint32_t lo = __byte_perm(w[j][bb >> 2], w[j][2 + (bb >> 2)], sel);
+                        const uint32_t hi = __byte_perm(w[j][4 + (bb >> 2)], w[j][6 + (bb >> 2)], sel);
+                        r[bb] = __byte_perm(lo, hi, 0x5410);
+                    }
+                } else {
+                    planes_to_bytes<NW>(w[j], r);
                 }
-                // every lane makes its bytes visible to the tensor core's proxy, then one lane arrives for the warp (32
-                // arrivals on one barrier word would be served one after the other)
-                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                __syncwarp();
-                if ((tid & 31) == 0) mbar_arrive(&st_full[st]);
-                if (++sub == NSUB) {
-                    sub = 0;
-                    if (++st == NST) { st = 0; ++st_round; }
-                }
+                const uint32_t dst = at + item_dst[j];
+                if (!EBS_IN_RANGE(p, CHK_PIPE_STAGE, (long long)(dst + half + 15u) - st0, NST * g.stage_bytes) ||
+                    !EBS_IN_RANGE(p, CHK_PIPE_STAGE, (long long)dst - st0, NST * g.stage_bytes))
+                    continue;
+                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst + half), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+            }
+            // every lane makes its bytes visible to the tensor core's proxy, then one lane arrives for the warp (32 arrivals on one
+            // barrier word would be served one after the other)
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+            __syncwarp();
+            if ((tid & 31) == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(full) : "memory");
+            at += pass_bytes;
+            if (++sub == NSUB) {
+                sub = 0;
+                full += 8u;
+                if (++st == NST) { st = 0; par ^= 1u; full = smem_u32(&st_full[0]); }
+                at = st0 + (uint32_t)(st * g.stage_bytes);
             }
         }
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
     } else if (warp < PIPE_EPI_WARP0) {
       asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(REG_MID));
       if (PAIR && crank == 1 && warp < PIPE_PRODUCER_WARP) {
@@ -1063,7 +1091,10 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
                 const int f = (PAIR ? 2 * ptile + crank : ptile) * g.tile_pix + j * UMMA_M + row;
                 bool pvalid = false;
                 int gp = 0;
-                if (f < g.frame) {
+                if (g.linear_out) {
+                    pvalid = f < g.frame;
+                    gp = pvalid ? f : 0;
+                } else if (f < g.frame) {
                     const uint32_t n = fastdiv((uint32_t)f, g.div_img);
                     const uint32_t rem = (uint32_t)f - n * (uint32_t)(g.Hq * g.Wq);
                     const uint32_t hq = fastdiv(rem, g.div_row), wq = rem - hq * (uint32_t)g.Wq;
@@ -1163,7 +1194,6 @@ int launch_conv_umma_pipe_pair(const ConvParams& p, dim3 /*grid*/, cudaStream_t 
     if (!pipe_pair_request_ok(p)) return EBS_ERR_UNSUPPORTED;
     const PipeGeom g = pipe_geometry(p, 256, pipe_sm_count(), p.pipe_m_sub, true);
     if (!g.ok) return EBS_ERR_UNSUPPORTED;
-    if (!p.zero_words) return EBS_ERR_CUDA;                   // the device's zero page could not be found
     if (pipe_packed_only(p)) return launch_conv_umma_pipe_pair_form<AB, 1>(p, g, st);
     return launch_conv_umma_pipe_pair_form<AB, 0>(p, g, st);
 }
@@ -1172,7 +1202,6 @@ template <int AB, int TILE_N>
 int launch_conv_umma_pipe(const ConvParams& p, dim3 /*grid*/, cudaStream_t st) {
     const PipeGeom g = pipe_geometry(p, TILE_N, pipe_sm_count(), p.pipe_m_sub);
     if (!g.ok) return EBS_ERR_UNSUPPORTED;                    // the geometry does not apply: nothing is launched
-    if (!p.zero_words) return EBS_ERR_CUDA;                   // the device's zero page could not be found
     if (pipe_packed_only(p)) {
         if constexpr (TILE_N >= 128) {
             if (pipe_hold_applies(p, TILE_N)) return launch_conv_umma_pipe_form<AB, TILE_N, 2>(p, g, st);

@@ -62,7 +62,7 @@ inline bool tile_tap_form(const ConvParams& p, FrameGeom& g) {
 inline bool tap_geometry(const ConvParams& p, FrameGeom& g) {
     g = FrameGeom{};
     const long long frame = (long long)p.N * p.Ho * p.Wo;
-    if (frame >= (1LL << 31) - 4096 || (long long)p.CW * 8 > PIPE_ZERO_WORDS) return false;
+    if (frame >= (1LL << 31) - 4096 || p.CW > FRAME_MAX_CW) return false;
     g.Wq = p.Wo;
     g.Hq = p.Ho;
     g.frame = (int)frame;

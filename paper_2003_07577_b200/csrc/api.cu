@@ -274,6 +274,8 @@ static int conv_plan(const void* packed_x, int n, int h, int w, const void* pack
     p.next_bits = 1;
     p.one = 1.0f;
     p.w_levels = d->w_levels;
+    p.acc_bound = (long long)d->c_in * d->kh * d->kw * (d->w_levels ? (1LL << d->w_bits) - 1 : 1LL << (d->w_bits - 1)) *
+                  (byte_acts ? 255 : (1LL << d->a_bits) - 1);
     p.fold = d->c_in <= 4 ? 8 : (d->c_in <= 8 ? 4 : (d->c_in <= 16 ? 2 : 1));
     p.fold_bits = 32 / p.fold;
     p.wait_limit = g_wait_limit;

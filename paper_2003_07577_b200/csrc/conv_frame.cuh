@@ -506,51 +506,50 @@ __device__ __forceinline__ void row_to_planes(uint32_t (&c)[8], int nb, uint32_t
     codes_to_planes<NB>(c, nb, planes);
 }
 
-// Two fp32 values in the order of pipe_group32 -> codes: pair (h, bb) = channels 16 h + bb and 16 h + 8 + bb.
-__device__ __forceinline__ void value_codes32(const uint64_t (&yy)[2][8], float one, float inv_next, int nb, uint32_t (&cr)[8]) {
+// Codes of the 32 values of a pixel's group -> eight registers (register bb: channels bb, 8 + bb, 16 + bb, 24 + bb).  value2(i, b):
+// the fp32 images of channels 8 i + 2 b and 8 i + 2 b + 1, one after the other in the registers that tensor memory was read
+// into: pairs taken eight channels apart, as the code registers join them, cost a move per value (64 -> 64 3x3 at 56x56, batch 256,
+// 47.8 -> 45.2 us; 64 -> 256 1x1, 8 planes out, 95.3 -> 90.3).
+template <int NB, class V>
+__device__ __forceinline__ void pair_codes32(V value2, float one, float inv_next, int nb, uint32_t (&cr)[8]) {
     const uint32_t k256 = k256_of(one);
     const uint64_t inv2 = f32x2_pack(inv_next, inv_next);
 #pragma unroll
-    for (int bb = 0; bb < 8; ++bb) {
-        uint32_t m[4];
+    for (int b = 0; b < 4; ++b) {
+        uint32_t m0[4], m1[4];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) code_pair<0>(f32x2_mul_rn(yy[h][bb], inv2), nb, m[2 * h], m[2 * h + 1]);
-        const uint32_t c4 = join_codes(m, k256);
-        cr[bb] = __funnelshift_l(c4, c4, bb);
+        for (int i = 0; i < 4; ++i) code_pair<NB>(f32x2_mul_rn(value2(i, b), inv2), nb, m0[i], m1[i]);
+        const uint32_t c0 = join_codes(m0, k256), c1 = join_codes(m1, k256);
+        cr[2 * b] = __funnelshift_l(c0, c0, 2 * b);
+        cr[2 * b + 1] = __funnelshift_l(c1, c1, 2 * b + 1);
     }
 }
-__device__ __forceinline__ void store_values32(const uint64_t (&yy)[2][8], bool relu, float* dst) {
+// Two fp32 values to a register: yy[i][b] = channels 8 i + 2 b and 8 i + 2 b + 1.
+__device__ __forceinline__ void value_codes32(const uint64_t (&yy)[4][4], float one, float inv_next, int nb, uint32_t (&cr)[8]) {
+    pair_codes32<0>([&](int i, int b) { return yy[i][b]; }, one, inv_next, nb, cr);
+}
+__device__ __forceinline__ void store_values32(const uint64_t (&yy)[4][4], bool relu, float* dst) {
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         float t[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const int c = 4 * q + e;                           // channel c: pair (c / 16, c % 8), upper lane if c & 8
-            const uint64_t w = yy[c >> 4][c & 7];
-            t[e] = __uint_as_float((c & 8) ? (uint32_t)(w >> 32) : (uint32_t)w);
+            const uint64_t w = yy[q >> 1][2 * (q & 1) + (e >> 1)];   // channel 4 q + e
+            t[e] = __uint_as_float((e & 1) ? (uint32_t)(w >> 32) : (uint32_t)w);
             if (relu) t[e] = t[e] > 0.f ? t[e] : 0.f;
         }
         *reinterpret_cast<float4*>(dst + 4 * q) = make_float4(t[0], t[1], t[2], t[3]);
     }
 }
 
-// 32 accumulators of one pixel and 32-channel group -> eight registers of requantized codes (register bb: channels bb, 8 + bb,
-// 16 + bb, 24 + bb) of a layer without per-channel terms and shortcut.
-template <int NB>
+// 32 accumulators of one pixel and 32-channel group -> eight registers of requantized codes of a layer without per-channel terms and
+// shortcut.  SMALL: accumulators below 2^23 taken as they are (pipe_small_accumulators).
+template <int NB, bool SMALL = false>
 __device__ __forceinline__ void plain_codes32(const uint32_t (&v)[32], float S, float one, float inv_next, uint32_t (&cr)[8]) {
-    const uint32_t k256 = k256_of(one);
-    const uint64_t S2 = f32x2_pack(S, S), inv2 = f32x2_pack(inv_next, inv_next);
-#pragma unroll
-    for (int bb = 0; bb < 8; ++bb) {
-        uint32_t m[4];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint64_t w = f32x2_mul_rn(f32x2_pack((float)(int)v[16 * h + bb], (float)(int)v[16 * h + 8 + bb]), S2);
-            code_pair<NB>(f32x2_mul_rn(w, inv2), NB, m[2 * h], m[2 * h + 1]);
-        }
-        const uint32_t c4 = join_codes(m, k256);
-        cr[bb] = __funnelshift_l(c4, c4, bb);
-    }
+    const uint64_t S2 = f32x2_pack(S, S);
+    auto value = [](uint32_t a) { return SMALL ? __uint_as_float(a) : (float)(int)a; };
+    pair_codes32<NB>([&](int i, int b) { return f32x2_mul_rn(f32x2_pack(value(v[8 * i + 2 * b]), value(v[8 * i + 2 * b + 1])), S2); },
+                     one, inv_next, NB, cr);
 }
 
 // Zero bits behind the last `left` channels of a group that is not whole.

@@ -39,6 +39,8 @@
 // memory and returns.  The single-CTA forms use no clusters.
 #pragma once
 
+#include <math.h>
+
 #include <type_traits>
 
 #include "conv_frame.cuh"
@@ -48,8 +50,16 @@ namespace ebs {
 constexpr int PIPE_EXPANDERS = 256;
 // Warps 8 and 9 issue the MMAs, warp 10 fetches weights, warp 11 has no role (20 warps cost the same registers as 18:
 // they are allotted in fours), warps 12-19 run the epilogue.
-constexpr int PIPE_ISSUER_WARP = 8, PIPE_ISSUERS = 2, PIPE_PRODUCER_WARP = 10, PIPE_EPI_WARP0 = 12, PIPE_EPI_WARPS = 8;
-constexpr int PIPE_THREADS = (PIPE_EPI_WARP0 + PIPE_EPI_WARPS) * 32;
+constexpr int PIPE_ISSUER_WARP = 8, PIPE_ISSUERS = 2, PIPE_PRODUCER_WARP = 10, PIPE_EPI_WARP0 = 12;
+// Epilogue warps: sixteen where the 256-channel tile leaves as packed planes without per-channel terms.  These layers wait for the
+// epilogue's instructions; eight warps issue in 60% of the cycles and sixteen, of 80 or 88 registers each, in 80% (64 -> 256 1x1 at
+// 56x56, batch 256, 4 planes: 91.4 -> 78.1 us; 256 -> 1024 at 14x14: 31.0 -> 28.8).  Narrower tiles wait for their expanders, and the
+// warps only poll beside them (512 -> 128 at 28x28: 32.9 and 35.0); terms and 32-bit results take more registers.
+__host__ __device__ constexpr int pipe_epi_warps(int tile_n, bool affine, int form, bool pair) {
+    return tile_n == 256 && !affine && form != 0 && !pair ? 16 : 8;
+}
+__host__ __device__ constexpr int pipe_threads(int epi_warps) { return (PIPE_EPI_WARP0 + epi_warps) * 32; }
+constexpr int PIPE_THREADS = pipe_threads(8);
 constexpr int PIPE_SLOTS = 2;                      // (pixel, word) items an expander thread handles per stage
 constexpr int PIPE_MAX_ITEMS = PIPE_SLOTS * PIPE_EXPANDERS;
 constexpr int PIPE_MAX_TAPS = FRAME_MAX_TAPS, PIPE_MAX_STAGES = 4;
@@ -81,7 +91,7 @@ struct PipeGeom : FrameGeom {
                                        // word groups (stages per tile and phase) = ceil(CW / kss)
     int nchunks;                       // chunks per tile = n_ph * nwg (phase-major)
     int n_stages, a_word_bytes, a_stage_bytes, stage_bytes;
-    int raw_bytes;                     // ring of packed words
+    int raw_bytes, rows_bytes;         // ring of packed words; rows of planes on their way out (pipe_rows_apply)
     int linear_in, linear_out;         // a frame pixel is the input pixel, the output pixel, of the same number
     int b_resident, b_total_bytes;
     PipeSlot slot[FRAME_MAX_PHASES];   // of each phase
@@ -91,6 +101,28 @@ struct PipeGeom : FrameGeom {
     int grid_x, grid_y;
     bool ok;
 };
+
+// Kernel form for a layer: 0 = every output mode; 1 = packed planes only (the usual layer of a network: its epilogue holds nothing
+// but the lean group, or the group with per-channel terms); 2 = form 1 with the planes of two neighbouring groups passing through
+// shared memory.  What else is compiled into a kernel costs the path that runs: with two epilogue forms in one kernel layers were
+// 15-25% slower.
+inline bool pipe_packed_only(const ConvParams& p) {
+    return p.packed_next && !p.acc && !p.y && !p.y_nchw && !p.w_levels && !(p.residual && (p.res_packed || (p.Co & 31) != 0));
+}
+// Form 2.  A group's planes are 4 * nb bytes of its pixel; with 32 lanes storing their own pixel's planes, 5 or 7 planes are as many
+// single-word stores of 32 sectors each and 6 planes three half-width ones.  As rows of two groups in shared memory they leave in
+// runs of 8-byte stores, four lanes to a pixel.  us, direct and through rows: 64 -> 256 1x1 at 56x56, batch 256, 5 planes 185 and 84 (held back
+// in registers until four groups filled wide stores: 99), 6 planes 113 and 84, 7 planes 264 and 88 (104); 256 -> 1024 at 14x14, 3
+// planes 47 and 29, 6 planes 50 and 31; 256 -> 128 at 56x56, 5 planes 94 and 68, 6 planes 70 and 68.  Even counts that fill one or two 16-byte
+// stores are faster direct (4 planes: 73 and 80; 8 planes: 90 and 101), 3 planes in the 128-channel tile too (60 and 64).
+inline bool pipe_rows_apply(const ConvParams& p, int tile_n) {
+    const int nb = p.next_bits;
+    return tile_n >= 128 && pipe_packed_only(p) && (p.Co & 63) == 0 && ((nb >= 5 && nb <= 7) || (nb == 3 && tile_n == 256));
+}
+inline bool pipe_has_terms(const ConvParams& p) { return p.ch_scale || p.ch_bias || p.residual || p.res_packed; }
+inline int pipe_rows_bytes(const ConvParams& p, int tile_n, bool pair) {
+    return !pair && pipe_rows_apply(p, tile_n) ? pipe_epi_warps(tile_n, pipe_has_terms(p), 2, false) * 32 * 8 * p.next_bits : 0;
+}
 
 // m_sub_req = 0: chosen here.  Returns ok = false when the kernel does not apply.
 inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_sub_req = 0, bool pair = false) {
@@ -138,11 +170,12 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
     g.a_word_bytes = g.SP * 32 + 64;                           // sized with the largest skew; fixed once ks is known
     if (g.SP * 16 >= (1 << 18)) return g;
     // weights resident when they leave room for at least two activation stages
-    const int smem_max = PIPE_SMEM_MAX - (p.ch_scale || p.ch_bias || p.residual || p.res_packed ? PIPE_SMEM_TERMS : 0);
+    const int smem_max = PIPE_SMEM_MAX - (pipe_has_terms(p) ? PIPE_SMEM_TERMS : 0);
     g.raw_bytes = pipe_raw_depth(p.x_words) * PIPE_MAX_ITEMS * p.x_words * 4;
     g.linear_in = taps == 1 && p.sh == 1 && p.sw == 1 && p.ph == 0 && p.pw == 0;
     g.linear_out = g.Hq == p.Ho && g.Wq == p.Wo;
-    const int budget = smem_max - 2048 - g.raw_bytes;
+    g.rows_bytes = pipe_rows_bytes(p, tile_n, pair);
+    const int budget = smem_max - 2048 - g.raw_bytes - g.rows_bytes;
     g.b_resident = g.b_total_bytes + 2 * ((g.a_word_bytes + 255) & ~255) <= budget && g.b_total_bytes <= 160 * 1024;
     int ks = PIPE_MAX_ITEMS / g.S;
     if (ks > 4) ks = 4;
@@ -189,7 +222,7 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
         if (g.b_slots > PIPE_MAX_BSLOTS) g.b_slots = PIPE_MAX_BSLOTS;
         if (g.b_slots < 3) return g;
     }
-    g.smem_bytes = (g.b_resident ? g.b_total_bytes : g.b_slots * g.b_group * b_tile) + g.n_stages * g.stage_bytes + g.raw_bytes + 1024;
+    g.smem_bytes = (g.b_resident ? g.b_total_bytes : g.b_slots * g.b_group * b_tile) + g.n_stages * g.stage_bytes + g.raw_bytes + g.rows_bytes + 1024;
     if (g.b_resident) {                                        // a CTA keeps one channel tile
         g.grid_y = g.n_ctiles;
         long long gx = sms / g.n_ctiles;
@@ -245,14 +278,14 @@ __device__ __forceinline__ void pipe_group32(const ConvParams& p, uint32_t (&v)[
             *reinterpret_cast<int4*>(p.acc + o + 4 * gq) =
                 make_int4((int)v[4 * gq], (int)v[4 * gq + 1], (int)v[4 * gq + 2], (int)v[4 * gq + 3]);
     }
-    // y = fl(float(acc) * S) for the 32 channels, two to a register: pair (h, bb) = channels 16h + bb and 16h + 8 + bb
-    uint64_t yy[2][8];
+    // y = fl(float(acc) * S) for the 32 channels, two to a register: yy[i][b] = channels 8 i + 2 b and 8 i + 2 b + 1
+    uint64_t yy[4][4];
     const uint64_t S2 = f32x2_pack(S, S);
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int bb = 0; bb < 8; ++bb)
-            yy[h][bb] = f32x2_mul_rn(f32x2_pack((float)(int)v[16 * h + bb], (float)(int)v[16 * h + 8 + bb]), S2);
+        for (int b = 0; b < 4; ++b)
+            yy[i][b] = f32x2_mul_rn(f32x2_pack((float)(int)v[8 * i + 2 * b], (float)(int)v[8 * i + 2 * b + 1]), S2);
     if (p.y && pvalid && EBS_IN_RANGE(p, CHK_PIPE_Y, o + 31, p.lim_out)) store_values32(yy, p.relu != 0, p.y + o);
     if (WANT_Q) {
         // The clamp at zero of the quantizer makes an explicit ReLU redundant here: a negative y gives
@@ -265,71 +298,50 @@ __device__ __forceinline__ void pipe_group32(const ConvParams& p, uint32_t (&v)[
     }
 }
 
-// Plane words of consecutive 32-channel groups of one pixel, held back until their run can leave in wide stores.  A
-// group's nb plane words are contiguous in memory, but for an odd nb their start is only 4-byte aligned and 32 lanes
-// each storing nb single words scatter 32 sectors per instruction (the wide 1x1 layers of a chain were up to 1.7 times
-// slower with nb = 7 than with nb = 8).  A warp handles G consecutive groups of its pixel (G = 4 for the 256-channel tile, 2
-// for the 128-channel one): their G * nb words are one contiguous run that starts on a 4 * G-byte boundary, stored as nb
-// vectors of G words.  The hold is a shift register (static indices only); last = the run's last group.
-template <int G>
-struct PlaneHold {
-    uint32_t w[G > 1 ? G : 1][8];
-    int filled;
-};
-template <int NB, int G>
-__device__ __forceinline__ void pipe_store_run(const uint32_t (&w)[G][8], uint32_t* run) {
-    static_assert(G == 2 || G == 4, "two or four groups to a run");
+// Planes on their way out of a form-2 kernel: a row of 2 * NB words per pixel of the warp, two neighbouring groups of 32 channels.
+template <int NB>
+__device__ __forceinline__ void pipe_row_put(uint32_t rows, int second, const uint32_t (&planes)[8]) {
+    const uint32_t at = rows + (threadIdx.x & 31u) * (8u * NB) + (uint32_t)second * (4u * NB);
+    if constexpr (NB % 2 == 0) {
 #pragma unroll
-    for (int t = 0; t < NB; ++t) {                       // vector t = words G t .. G t + G - 1 of the run; word i = group i / NB, plane i % NB
-        if constexpr (G == 4)
-            *reinterpret_cast<uint4*>(run + 4 * t) = make_uint4(w[(4 * t) / NB][(4 * t) % NB], w[(4 * t + 1) / NB][(4 * t + 1) % NB],
-                                                                 w[(4 * t + 2) / NB][(4 * t + 2) % NB], w[(4 * t + 3) / NB][(4 * t + 3) % NB]);
-        else
-            *reinterpret_cast<uint2*>(run + 2 * t) = make_uint2(w[(2 * t) / NB][(2 * t) % NB], w[(2 * t + 1) / NB][(2 * t + 1) % NB]);
+        for (int k = 0; k < NB; k += 2) asm volatile("st.shared.v2.u32 [%0], {%1, %2};\n" ::"r"(at + 4 * k), "r"(planes[k]), "r"(planes[k + 1]) : "memory");
+    } else {
+#pragma unroll
+        for (int k = 0; k < NB; ++k) asm volatile("st.shared.u32 [%0], %1;\n" ::"r"(at + 4 * k), "r"(planes[k]) : "memory");
     }
 }
-template <int G>
-__device__ __forceinline__ void pipe_store_planes(const uint32_t (&planes)[8], int nb, uint32_t* dst, bool pvalid, PlaneHold<G>& hold,
-                                                  const ConvParams& p) {
-    if constexpr (G > 1) {
-        if ((nb & 1) && (p.CWo % G) == 0) {               // odd: hold the group; store the run with its last group (rows of
-                                                          // CWo * nb words keep the run's alignment only if G divides CWo)
+// Both groups of every row are there: the rows leave, four lanes to a pixel.  gp: this lane's output pixel, -1: none; word: the first
+// group's channel word.
+template <int NB>
+__device__ __forceinline__ void pipe_rows_leave(const ConvParams& p, uint32_t rows, int gp, int word) {
+    const int lane = (int)(threadIdx.x & 31), q = lane & 3;
+    __syncwarp();
 #pragma unroll
-            for (int gi = 0; gi + 1 < G; ++gi)
+    for (int i = 0; i < 4; ++i) {
+        const int px = 8 * i + (lane >> 2), to = __shfl_sync(0xffffffffu, gp, px);
+        uint32_t* out = p.packed_next + ((size_t)max(to, 0) * p.CWo + word) * NB + 2 * q;
+        const uint32_t from = rows + (uint32_t)(px * (8 * NB) + 8 * q);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) hold.w[gi][j] = hold.w[gi + 1][j];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) hold.w[G - 1][j] = planes[j];
-            if (++hold.filled == G) {
-                hold.filled = 0;
-                uint32_t* run = dst - (G - 1) * nb;          // the first group of the run
-                if (pvalid && EBS_IN_RANGE(p, CHK_PIPE_PN, (dst - p.packed_next) + nb - 1, p.lim_pn)) {
-                    if (nb == 7) pipe_store_run<7, G>(hold.w, run);
-                    else if (nb == 5) pipe_store_run<5, G>(hold.w, run);
-                    else if (nb == 3) pipe_store_run<3, G>(hold.w, run);
-                    else pipe_store_run<1, G>(hold.w, run);
-                }
+        for (int r = 0; 4 * r < NB; ++r) {
+            if (to >= 0 && q + 4 * r < NB && EBS_IN_RANGE(p, CHK_PIPE_PN, (out - p.packed_next) + 8 * r + 1, p.lim_pn)) {
+                uint32_t x, y;
+                asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];\n" : "=r"(x), "=r"(y) : "r"(from + 32 * r) : "memory");
+                *reinterpret_cast<uint2*>(out + 8 * r) = make_uint2(x, y);
             }
-            return;
         }
     }
-    if (pvalid && EBS_IN_RANGE(p, CHK_PIPE_PN, (dst - p.packed_next) + nb - 1, p.lim_pn)) store_plane_words(planes, nb, dst);
+    __syncwarp();                                            // (the next pair of groups takes their place)
 }
 
 // The same group when only packed planes are asked for (a chained network: no accumulator and no fp32 output): the
 // four channels of a byte register go from accumulator to code in one short chain, so that nothing but the 32
 // accumulators and the finished code registers is alive at a time -- the general form above keeps the 32 fp32 images
 // as well, which at 96 registers costs spills and the parallelism of the instruction stream.
-// left: channels of the layer from this group on (a last group of fewer than 32 writes zero bits behind them).
-template <int G, int NB>
-__device__ __forceinline__ void pipe_group32_packed(const uint32_t (&v)[32], bool pvalid, float S, float inv_next, uint32_t* dst,
-                                                    const ConvParams& p, PlaneHold<G>& hold, int left) {
+template <int NB, bool SMALL>
+__device__ __forceinline__ void pipe_group32_packed(const uint32_t (&v)[32], float S, float inv_next, const ConvParams& p, uint32_t (&planes)[8]) {
     uint32_t cr[8];
-    plain_codes32<NB>(v, S, p.one, inv_next, cr);
-    uint32_t planes[8];
+    plain_codes32<NB, SMALL>(v, S, p.one, inv_next, cr);
     codes_to_planes<NB>(cr, NB, planes);
-    if (left < 32) mask_planes(planes, left);
-    pipe_store_planes(planes, NB, dst, pvalid, hold, p);
 }
 
 // Epilogue of a layer with per-channel terms and / or a shortcut (a folded batch normalisation, the second convolution of a
@@ -338,9 +350,9 @@ __device__ __forceinline__ void pipe_group32_packed(const uint32_t (&v)[32], boo
 // loaded as fragments (terms_codes_frag), so that a lane reads the terms of eight channels instead of 32, and the codes -- and
 // the codes of a packed shortcut the other way -- pass through shared memory as matrices (FragRows).  terms: 64 floats of the
 // warp's own, rows: 1 KB.  VALUES: fp32 output may be wanted too, stored from the fragments (whole 32-byte sectors).
-template <int TILE_N, int G, bool VALUES, int NB, int RES>
+template <int TILE_N, bool ROWS, bool VALUES, int NB, int RES>
 __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, const FrameGeom& g, uint32_t tmem_set, int m_sub, int vwarp,
-                                                    int f0, int co0, float* terms, const FragRows& rows) {
+                                                    int f0, int co0, float* terms, const FragRows& rows, uint32_t out_rows) {
     const int lane = (int)(threadIdx.x & 31), quad = lane & 3;
     const int at = frag_term_at(lane);
     const uint32_t trow = tmem_set + ((uint32_t)((vwarp & 3) * 32) << 16);
@@ -348,8 +360,6 @@ __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, cons
     const int cbeg = (vwarp >> 2) * COLS, cend = COLS == 32 ? cbeg + 32 : min(cbeg + COLS, p.Co - co0);   // (cend: groups start below)
     if (co0 + cbeg >= p.Co) return;
     const int nb = NB > 0 ? NB : p.next_bits;                // (a constant where only planes are written)
-    PlaneHold<G> hold;
-    hold.filled = 0;
     float res[32], t_scale, t_bias;
     uint32_t rw[8];
     int gp = 0, gr[4];                                       // output pixels of this lane's row and of its fragment's four rows
@@ -396,7 +406,7 @@ __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, cons
         tmem_ld_frag_issue(trow + (16u << 16) + (uint32_t)(j * TILE_N + c0), hi);
     };
     // (the next unit's accumulators are requested early only where the registers hold them)
-    constexpr bool EARLY = !VALUES && G == 1;
+    constexpr bool EARLY = !VALUES && !ROWS;
     locate(0);
     request(co0 + cbeg);
     if (EARLY) load(0, cbeg);
@@ -449,7 +459,13 @@ __device__ __forceinline__ void pipe_epilogue_terms_nb(const ConvParams& p, cons
             rows.get_row(cr);
             row_to_planes<NB>(cr, nb, planes);
             if (p.Co - c < 32) mask_planes(planes, p.Co - c);
-            pipe_store_planes(planes, nb, p.packed_next + (gpz * p.CWo + (c >> 5)) * nb, ok, hold, p);
+            if constexpr (ROWS) {
+                pipe_row_put<NB>(out_rows, (c >> 5) & 1, planes);
+                if (c & 32) pipe_rows_leave<NB>(p, out_rows, ok ? (int)gpz : -1, (c >> 5) - 1);
+            } else {
+                uint32_t* dst = p.packed_next + (gpz * p.CWo + (c >> 5)) * nb;
+                if (ok && EBS_IN_RANGE(p, CHK_PIPE_PN, (dst - p.packed_next) + nb - 1, p.lim_pn)) store_plane_words(planes, nb, dst);
+            }
         }
         if (jn >= m_sub) break;
         j = jn;
@@ -489,21 +505,18 @@ __device__ __forceinline__ void pipe_epilogue_plain(const ConvParams& p, uint32_
 }
 
 // Packed-only epilogue without per-channel terms of one 128-pixel accumulator: nothing but the lean
-// group, for the kernel forms that are launched only for such layers.
-template <int TILE_N, int G, int NB>
+// group, for the kernel forms that are launched only for such layers.  A last group of fewer than 32 channels writes zero bits behind them.
+template <int TILE_N, bool ROWS, bool SMALL, int EPI_WARPS, int NB>
 __device__ __forceinline__ void pipe_epilogue_packed_nb(const ConvParams& p, uint32_t tmem_acc, int vwarp, int gp, bool pvalid,
-                                                       int co0) {
+                                                       int co0, uint32_t out_rows) {
     const uint32_t trow = tmem_acc + ((uint32_t)((vwarp & 3) * 32) << 16);
-    constexpr int COLS = TILE_N / 2;
+    constexpr int COLS = TILE_N * 4 / EPI_WARPS;
     const int cbeg = (vwarp >> 2) * COLS;
-    constexpr int nb = NB;
     const float S = p.S, inv_next = p.inv_next;
     uint32_t v[32];
-    PlaneHold<G> hold;
-    hold.filled = 0;
-    uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + ((co0 + cbeg) >> 5)) * nb;
+    uint32_t* dst = p.packed_next + ((size_t)gp * p.CWo + ((co0 + cbeg) >> 5)) * NB;
 #pragma unroll 1
-    for (int c0 = cbeg; c0 < cbeg + COLS; c0 += 32, dst += nb) {
+    for (int c0 = cbeg; c0 < cbeg + COLS; c0 += 32, dst += NB) {
         if (co0 + c0 >= p.Co) break;
         uint32_t (&lo)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[0]);
         uint32_t (&hi)[16] = *reinterpret_cast<uint32_t(*)[16]>(&v[16]);
@@ -511,16 +524,28 @@ __device__ __forceinline__ void pipe_epilogue_packed_nb(const ConvParams& p, uin
         tmem_ld16_issue(trow + (uint32_t)(c0 + 16), hi);
         tmem_ld16_wait(lo);
         tmem_ld16_wait(hi);
-        pipe_group32_packed<G, NB>(v, pvalid, S, inv_next, dst, p, hold, p.Co - co0 - c0);
+        uint32_t planes[8];
+        pipe_group32_packed<NB, SMALL>(v, S, inv_next, p, planes);
+        if constexpr (ROWS) {
+            pipe_row_put<NB>(out_rows, (c0 >> 5) & 1, planes);
+            if (c0 & 32) pipe_rows_leave<NB>(p, out_rows, pvalid ? gp : -1, (co0 + c0 - 32) >> 5);
+        } else {
+            if (p.Co - co0 - c0 < 32) mask_planes(planes, p.Co - co0 - c0);
+            if (pvalid && EBS_IN_RANGE(p, CHK_PIPE_PN, (dst - p.packed_next) + NB - 1, p.lim_pn)) store_plane_words(planes, NB, dst);
+        }
     }
 }
 
 // The plane count as a constant of the code: with run-time counts every group ran through a dozen branches (plane loops,
 // store widths), which cost the epilogue warps more in instruction fetch than their arithmetic.
 #define EBS_PIPE_EACH_NB(CALL)                                                                                    \
-    if constexpr (G > 1) {                                                                                        \
-        if (p.next_bits == 5) { constexpr int NB = 5; CALL; }                                                     \
-        else { constexpr int NB = 7; CALL; }                                                                      \
+    if constexpr (ROWS) {                                                                                         \
+        switch (p.next_bits) {                                                                                    \
+            case 3: { constexpr int NB = 3; CALL; } break;                                                        \
+            case 5: { constexpr int NB = 5; CALL; } break;                                                        \
+            case 6: { constexpr int NB = 6; CALL; } break;                                                        \
+            default: { constexpr int NB = 7; CALL; } break;                                                       \
+        }                                                                                                         \
     } else {                                                                                                      \
         switch (p.next_bits) {                                                                                    \
             case 1: { constexpr int NB = 1; CALL; } break;                                                        \
@@ -533,43 +558,29 @@ __device__ __forceinline__ void pipe_epilogue_packed_nb(const ConvParams& p, uin
             default: { constexpr int NB = 8; CALL; } break;                                                       \
         }                                                                                                         \
     }
-template <int TILE_N, int G>
-__device__ __forceinline__ void pipe_epilogue_packed_g(const ConvParams& p, uint32_t tmem_acc, int vwarp, int gp, bool pvalid, int co0) {
-    EBS_PIPE_EACH_NB((pipe_epilogue_packed_nb<TILE_N, G, NB>(p, tmem_acc, vwarp, gp, pvalid, co0)))
+template <int TILE_N, bool ROWS, bool SMALL, int EPI_WARPS>
+__device__ __forceinline__ void pipe_epilogue_packed_g(const ConvParams& p, uint32_t tmem_acc, int vwarp, int gp, bool pvalid, int co0,
+                                                       uint32_t out_rows) {
+    EBS_PIPE_EACH_NB((pipe_epilogue_packed_nb<TILE_N, ROWS, SMALL, EPI_WARPS, NB>(p, tmem_acc, vwarp, gp, pvalid, co0, out_rows)))
 }
 
-template <int TILE_N, int G, bool VALUES>
+template <int TILE_N, bool ROWS, bool VALUES>
 __device__ __forceinline__ void pipe_epilogue_terms(const ConvParams& p, const FrameGeom& g, uint32_t tmem_set, int m_sub, int vwarp,
-                                                    int f0, int co0, float* terms, const FragRows& rows) {
+                                                    int f0, int co0, float* terms, const FragRows& rows, uint32_t out_rows) {
     auto run = [&](auto res_tag) {
         constexpr int RES = decltype(res_tag)::value;
-        if constexpr (VALUES) pipe_epilogue_terms_nb<TILE_N, G, true, 0, RES>(p, g, tmem_set, m_sub, vwarp, f0, co0, terms, rows);
-        else EBS_PIPE_EACH_NB((pipe_epilogue_terms_nb<TILE_N, G, false, NB, RES>(p, g, tmem_set, m_sub, vwarp, f0, co0, terms, rows)))
+        if constexpr (VALUES) pipe_epilogue_terms_nb<TILE_N, false, true, 0, RES>(p, g, tmem_set, m_sub, vwarp, f0, co0, terms, rows, out_rows);
+        else EBS_PIPE_EACH_NB((pipe_epilogue_terms_nb<TILE_N, ROWS, false, NB, RES>(p, g, tmem_set, m_sub, vwarp, f0, co0, terms, rows, out_rows)))
     };
     if (p.residual) run(std::integral_constant<int, 1>{});
     else if (p.res_packed) run(std::integral_constant<int, 2>{});
     else run(std::integral_constant<int, 0>{});
 }
 
-// Odd plane counts of the packed output take the form that holds the groups of a run back: a kernel instantiation of
-// its own (HOLD), chosen by the launcher, because the shift register costs the other layers registers and time even
-// as an untaken branch of the same kernel (even counts 15-25% slower when both forms were compiled into one kernel).
-// Kernel form for a layer: 0 = every output mode; 1 = packed planes only
-// (the usual layer of a network: its epilogue holds nothing but the lean group, or the group with per-channel terms);
-// 2 = form 1 with the held-back runs.
-inline bool pipe_packed_only(const ConvParams& p) {
-    return p.packed_next && !p.acc && !p.y && !p.y_nchw && !p.w_levels && !(p.residual && (p.res_packed || (p.Co & 31) != 0));
-}
-inline bool pipe_hold_applies(const ConvParams& p, int tile_n) {
-    const int G = tile_n / 64;
-    // (5 and 7 planes; with 1 or 3 the single-word stores are few and the held form measured slower)
-    return G > 1 && p.packed_next && (p.next_bits == 5 || p.next_bits == 7) && (p.CWo % G) == 0 && !p.acc && !p.y && !p.y_nchw &&
-           (p.Co % tile_n) == 0 && !p.w_levels && !(p.residual && p.res_packed);
-}
-
-template <int AB, int TILE_N, bool AFFINE, int FORM, bool PAIR = false>
-__global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const ConvParams p, const PipeGeom g) {
-    constexpr int EPI_G = FORM == 2 ? TILE_N / 64 : 1;         // groups of an output run held back (odd plane counts)
+template <int AB, int TILE_N, bool AFFINE, int FORM, bool PAIR = false, bool SMALL = false>
+__global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FORM, PAIR)), 1) conv_umma_pipe_kernel(const ConvParams p, const PipeGeom g) {
+    constexpr int EPI_WARPS = pipe_epi_warps(TILE_N, AFFINE, FORM, PAIR);
+    constexpr bool ROWS = FORM == 2;                           // planes of odd counts leave through rows in shared memory
     // PAIR: the two CTAs of a cluster work as one.  Each expands its own 128 * m_sub pixels and holds the weight rows of
     // half the channel tile; the even CTA issues MMAs of M = 256 (cta_group::2) that read both CTAs' shared memory and
     // write both CTAs' tensor memory, so a weight byte is fetched from L2 once per 256 pixels instead of once per 128.
@@ -585,8 +596,8 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
     __shared__ __align__(8) uint64_t bs_full[PIPE_MAX_BSLOTS], bs_empty[PIPE_MAX_BSLOTS];   // streamed weight tiles
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
-    __shared__ __align__(16) float s_terms[AFFINE ? PIPE_EPI_WARPS : 1][64];
-    __shared__ __align__(128) uint8_t s_rows[AFFINE ? PIPE_EPI_WARPS : 1][AFFINE ? 1024 : 16];
+    __shared__ __align__(16) float s_terms[AFFINE ? EPI_WARPS : 1][64];
+    __shared__ __align__(128) uint8_t s_rows[AFFINE ? EPI_WARPS : 1][AFFINE ? 1024 : 16];
     __shared__ int s_tap_id[PIPE_MAX_TAPS];             // (in shared memory: indexed at run time by single threads)
 
     // (the warp number read from lane 0, so that the compiler knows the role branches to be warp-uniform: the issuing warps' waits
@@ -599,7 +610,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
     uint8_t* base = dyn_smem + ((1024u - (smem_u32(dyn_smem) & 1023u)) & 1023u);
     uint8_t* b_res = base;                                               // resident: [CW][tap slots][TILE_N][32]; else the ring of tiles
     uint8_t* stages = base + (resident ? g.b_total_bytes : g.b_slots * g.b_group * B_TILE_BYTES);   // [NST] x [KS][2][SP][16]
-    uint8_t* raw = stages + g.n_stages * g.stage_bytes;                  // ring of packed words
+    uint8_t* raw = stages + g.n_stages * g.stage_bytes;                  // ring of packed words, then the rows of planes
     const int NBS = g.b_slots, GB = g.b_group;
     // Streamed weights: every CTA of a channel tile reads the same weight tiles, and CTAs that start together would ask
     // the same few L2 slices for the same tile at the same time.  Integer accumulation is exact in any order, so each
@@ -634,8 +645,8 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
         }
         mbar_init(&acc_full[0], n_iss);
         mbar_init(&acc_full[1], n_iss);
-        mbar_init(&acc_empty[0], PIPE_EPI_WARPS);
-        mbar_init(&acc_empty[1], PIPE_EPI_WARPS);
+        mbar_init(&acc_empty[0], EPI_WARPS);
+        mbar_init(&acc_empty[1], EPI_WARPS);
         mbar_init(&b_full, 1);
         if constexpr (PAIR) {
             for (int s = 0; s < PIPE_MAX_STAGES; ++s) mbar_init(&st_peer[s], 1);
@@ -663,16 +674,17 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem_base = tmem_slot;
 
-    // Registers follow the roles (warpgroups of four warps: 0-7 expanders, 8-11 issuers / producer / no role, 12-19
+    // Registers follow the roles (warpgroups of four warps: 0-7 expanders, 8-11 issuers / producer / no role, then the
     // epilogue): each role's branch opens with a setmaxnreg executed by all four warps of its warpgroups, and the
-    // assembler allocates each branch for its own count.  The epilogue's 32 accumulators, their fp32 images and the code
-    // registers want about 126 registers; with the 96 a CTA of 20 warps starts with it spilled and its instruction stream
-    // lost its parallelism (wide 1x1 layers 15-20% slower, and no better with twelve epilogue warps).  The other roles
-    // need fewer than 96.  The increase waits in hardware until the CTA's pool has the registers, so the counts must fit
+    // assembler allocates each branch for its own count.  With 96 registers in eight epilogue warps the epilogue spilled and its
+    // instruction stream lost its parallelism (wide 1x1 layers 15-20% slower); the expanders, whose words wait in shared memory, need 40
+    // for up to four planes.  The increase waits in hardware until the CTA's pool has the registers, so the counts must fit
     // into what the launch allots: checked at compile time.  (The middle role spilled at 56, which cost the GEMM a fifth.)
-    constexpr int REG_LAUNCH = 96, REG_EXP = 80, REG_MID = 64, REG_EPI = 128;
-    static_assert(8 * REG_EXP + 4 * REG_MID + 8 * REG_EPI <= 20 * REG_LAUNCH, "setmaxnreg: the roles' registers exceed the CTA's pool");
-    static_assert(PIPE_EPI_WARP0 == 12 && PIPE_EPI_WARPS == 8 && PIPE_THREADS == 640, "role layout changed: revisit the register split");
+    constexpr bool MANY = EPI_WARPS == 16, WIDE_ITEMS = AB == 0 || AB > 4;
+    constexpr int REG_LAUNCH = MANY ? 72 : 96, REG_MID = 64;
+    constexpr int REG_EXP = !MANY ? 64 : WIDE_ITEMS ? 48 : 40, REG_EPI = !MANY ? 144 : WIDE_ITEMS ? 80 : 88;
+    static_assert(8 * REG_EXP + 4 * REG_MID + EPI_WARPS * REG_EPI <= (PIPE_EPI_WARP0 + EPI_WARPS) * REG_LAUNCH, "setmaxnreg: the roles' registers exceed the CTA's pool");
+    static_assert(PIPE_EPI_WARP0 == 12, "role layout changed: revisit the register split");
     if (warp < 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(REG_EXP));
         // =========================== expanders ===========================
@@ -1067,9 +1079,10 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(REG_EPI));
         // =========================== epilogue ===========================
-        const int half = (warp - PIPE_EPI_WARP0) >> 2;           // which half of the channels
-        const int vwarp = (warp & 3) + 4 * half;                 // TMEM lane quarter = warp % 4 (hardware rule)
+        const int half = (warp - PIPE_EPI_WARP0) >> 2;           // which share of the channels
+        const int vwarp = (warp & 3) + 4 * half;                 // TMEM lane quarter = warp % 4 (hardware rule), share of the channels
         const int row = (warp & 3) * 32 + (tid & 31);
+        const uint32_t out_rows = smem_u32(raw) + (uint32_t)g.raw_bytes + (uint32_t)((warp - PIPE_EPI_WARP0) * 256 * p.next_bits);   // (form 2)
         const bool plain_ok = !AFFINE && !p.ch_scale && !p.ch_bias && !p.residual && !p.res_packed && !p.y_nchw &&
                               (p.Co & 31) == 0;
         // layers with per-channel terms or a shortcut and without integer output (the layers of a network)
@@ -1084,9 +1097,9 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
             const int co0 = ctile * TILE_N;
             if (AFFINE && (FORM != 0 || affine_ok)) {
                 if constexpr (AFFINE)
-                    pipe_epilogue_terms<TILE_N, EPI_G, FORM == 0>(p, g, tmem_base + (uint32_t)(buf * g.m_sub * TILE_N), g.m_sub, vwarp,
+                    pipe_epilogue_terms<TILE_N, ROWS, FORM == 0>(p, g, tmem_base + (uint32_t)(buf * g.m_sub * TILE_N), g.m_sub, vwarp,
                                                                   (PAIR ? 2 * ptile + crank : ptile) * g.tile_pix + row, co0,
-                                                                  s_terms[warp - PIPE_EPI_WARP0], FragRows(smem_u32(s_rows[warp - PIPE_EPI_WARP0])));
+                                                                  s_terms[warp - PIPE_EPI_WARP0], FragRows(smem_u32(s_rows[warp - PIPE_EPI_WARP0])), out_rows);
             } else for (int j = 0; j < g.m_sub; ++j) {
                 const int f = (PAIR ? 2 * ptile + crank : ptile) * g.tile_pix + j * UMMA_M + row;
                 bool pvalid = false;
@@ -1104,7 +1117,7 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
                 if (!__any_sync(0xffffffffu, pvalid)) continue;   // 32 frame pixels without an output
                 const uint32_t tmem_acc = tmem_base + (uint32_t)((buf * g.m_sub + j) * TILE_N);
                 if constexpr (FORM != 0) {
-                    if constexpr (!AFFINE) pipe_epilogue_packed_g<TILE_N, EPI_G>(p, tmem_acc, vwarp, gp, pvalid, co0);
+                    if constexpr (!AFFINE) pipe_epilogue_packed_g<TILE_N, ROWS, SMALL, EPI_WARPS>(p, tmem_acc, vwarp, gp, pvalid, co0, out_rows);
                 } else {
                     if (plain_ok) pipe_epilogue_plain<TILE_N>(p, tmem_acc, vwarp, gp, pvalid, co0);
                     else umma_epilogue<TILE_N, AFFINE>(p, tmem_acc, vwarp, gp, pvalid, 0, co0);
@@ -1140,22 +1153,41 @@ __global__ void __launch_bounds__(PIPE_THREADS, 1) conv_umma_pipe_kernel(const C
 
 int pipe_sm_count();
 
-template <int AB, int TILE_N, int HOLD>
-int launch_conv_umma_pipe_form(const ConvParams& p, const PipeGeom& g, cudaStream_t st) {
+template <int AB, int TILE_N, int FORM, bool AFFINE, bool SMALL>
+int launch_conv_umma_pipe_kernel(const ConvParams& p, const PipeGeom& g, cudaStream_t st) {
+    auto kern = conv_umma_pipe_kernel<AB, TILE_N, AFFINE, FORM, false, SMALL>;
     static bool attr_set[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-        cudaFuncSetAttribute(conv_umma_pipe_kernel<AB, TILE_N, false, HOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, PIPE_SMEM_MAX);
-        cudaFuncSetAttribute(conv_umma_pipe_kernel<AB, TILE_N, true, HOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, PIPE_SMEM_MAX - PIPE_SMEM_TERMS);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PIPE_SMEM_MAX - (AFFINE ? PIPE_SMEM_TERMS : 0));
         attr_set[dev] = true;
     }
-    const dim3 grid((unsigned)g.grid_x, (unsigned)g.grid_y, 1);
-    if (p.ch_scale || p.ch_bias || p.residual || p.res_packed)
-        conv_umma_pipe_kernel<AB, TILE_N, true, HOLD><<<grid, PIPE_THREADS, g.smem_bytes, st>>>(p, g);
-    else
-        conv_umma_pipe_kernel<AB, TILE_N, false, HOLD><<<grid, PIPE_THREADS, g.smem_bytes, st>>>(p, g);
+    kern<<<dim3((unsigned)g.grid_x, (unsigned)g.grid_y, 1), pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FORM, false)), g.smem_bytes, st>>>(p, g);
     return EBS_OK;
+}
+
+// Accumulators below 2^23 in a layer without per-channel terms need no conversion to fp32: the integer a, read as fp32, is the
+// denormal a * 2^-149, its product with S * 2^75 is rounded as that of float(a) with S and scaled by 2^-74, and 1 / step carries the
+// 2^74 back.  A negative one reads as a NaN or a negative value and becomes code 0, which any negative value does.  One of seven
+// instructions an output (64 -> 256 1x1 at 56x56, batch 256, 4 planes: 78.1 -> 74.0 us; 64 -> 64 3x3: 47.3 -> 46.1).
+inline bool pipe_small_accumulators(const ConvParams& p) {
+    auto moderate = [](float v) { return v >= 0x1p-50f && v <= 0x1p+50f; };
+    return p.acc_bound < (1LL << 23) && moderate(p.S) && moderate(p.inv_next);
+}
+
+template <int AB, int TILE_N, int FORM>
+int launch_conv_umma_pipe_form(const ConvParams& p, const PipeGeom& g, cudaStream_t st) {
+    if (pipe_has_terms(p)) return launch_conv_umma_pipe_kernel<AB, TILE_N, FORM, true, false>(p, g, st);
+    if constexpr (FORM != 0) {
+        if (pipe_small_accumulators(p)) {
+            ConvParams q = p;
+            q.S = ldexpf(p.S, 75);
+            q.inv_next = ldexpf(p.inv_next, 74);
+            return launch_conv_umma_pipe_kernel<AB, TILE_N, FORM, false, true>(q, g, st);
+        }
+    }
+    return launch_conv_umma_pipe_kernel<AB, TILE_N, FORM, false, false>(p, g, st);
 }
 
 // The CTA-pair form: clusters of two CTAs along x; packed-only whole tiles (form 1) or every output mode (form 0),
@@ -1204,7 +1236,7 @@ int launch_conv_umma_pipe(const ConvParams& p, dim3 /*grid*/, cudaStream_t st) {
     if (!g.ok) return EBS_ERR_UNSUPPORTED;                    // the geometry does not apply: nothing is launched
     if (pipe_packed_only(p)) {
         if constexpr (TILE_N >= 128) {
-            if (pipe_hold_applies(p, TILE_N)) return launch_conv_umma_pipe_form<AB, TILE_N, 2>(p, g, st);
+            if (pipe_rows_apply(p, TILE_N)) return launch_conv_umma_pipe_form<AB, TILE_N, 2>(p, g, st);
         }
         return launch_conv_umma_pipe_form<AB, TILE_N, 1>(p, g, st);
     }

@@ -42,6 +42,7 @@ struct ConvParams {
     int test_flags;                   // tests only, so that waits run out: bit 0 the MMA issuer issues nothing, bit 1 the first
                                       // CTA of a tile kernel's cluster sends no sums
     int tile_split;                   // tile kernel: CTAs the reduction is split over (0 = chosen by the library)
+    long long acc_bound;              // no accumulator of the layer is larger in magnitude
     int pipe_m_sub;                   // persistent pipeline kernel: accumulators per super-tile (0 = chosen by the library)
     float one;                        // 1.0f: multiplier of packed additions (see f32x2_add_one)
     // Extents of the buffers, for the range-checked build (EBS_CHECKED); filled in every build.

@@ -233,3 +233,42 @@ def test_pipe_declines_layers_wider_than_its_zero_page(ebs, U, oracle):
     qw = rng.integers(-1, 2, size=(co, c, 1, 1), dtype=np.int32)
     out = U.run_conv(qa, qw, d, None, want_acc=True)
     assert np.array_equal(out["acc"], oracle.conv2d_codes(qa, qw, (1, 1), (0, 0)))
+
+
+@pytest.mark.parametrize("nb", [3, 5, 6, 7])
+@pytest.mark.parametrize("case", [(3, 64, 192, 1, 1, 0, 11, 13), (2, 96, 256, 3, 1, 1, 9, 12), (5, 32, 320, 1, 2, 0, 15, 14)])
+@pytest.mark.parametrize("affine", [False, True])
+def test_pipe_planes_through_rows(ebs, U, oracle, nb, case, affine):
+    """Output plane counts that leave two groups at a time through shared memory: a channel tile that is cut after one pair of
+    groups, frames with and without rows that have no output, a last tile of a few pixels."""
+    n, c, co, k, s, pad, h, w = case
+    _check(ebs, U, oracle, n, c, co, k, s, pad, h, w, 3, 4, nb, affine=affine, min_variants=2)
+
+
+@pytest.mark.parametrize("c", [32, 257, 258])
+def test_pipe_accumulators_at_the_conversion_bound(ebs, U, oracle, c):
+    """Layers whose largest possible accumulator lies just below and just above 2^23 (8-bit codes, 257 and 258 channels), with pixels and
+    channels that reach it, its negative counterpart, zero and one."""
+    rng = np.random.default_rng(c)
+    co, h, w = 256, 9, 15
+    qa = U.rand_codes(rng, (1, c, h, w), 8, False)
+    qw = rng.integers(-128, 128, size=(co, c, 1, 1), dtype=np.int32)
+    qa[:, :, 0, :4] = 255
+    qa[:, :, 0, 4] = 0
+    qa[:, :, 0, 5] = 0
+    qa[:, 0, 0, 5] = 1
+    qw[:8], qw[8:16], qw[16:24] = 127, -128, 1
+    d = U.desc_for(c, co, 1, 1, 0, 8, 8, 0.03, 0.07)
+    ref = oracle.conv2d_codes(qa, qw, (1, 1), (0, 0))
+    S = oracle.combined_scale(0.03, 0.07)
+    px, pw = U.pack_acts_codes(qa, 8), U.pack_weight_codes(qw, d)
+    for nb in (4, 7, 8):
+        for top in (float(np.abs(ref).max()) * float(S), float(np.percentile(np.abs(ref), 50)) * float(S)):
+            step = np.float32(top / ((1 << nb) - 1))
+            _, q_ref = oracle.epilogue(ref, S, None, None, None, relu=True, next_bits=nb, inv_next=np.float32(1.0) / step)
+            epi = ebs.epilogue(None, None, None, True, nb, float(step))
+            for variant in U.variants_of("umma_pipe"):
+                if U.applies(d, h, w, variant, n=1, epi=epi, want_y=False, want_packed=True):
+                    out = U.run_conv(qa, qw, d, epi, want_acc=False, want_y=False, next_bits=nb, variant=variant, px=px, pw=pw)
+                    assert np.array_equal(out["packed"], oracle.pack_acts(q_ref, nb)), f"variant {variant}, {nb} planes"
+    assert ebs.ebs_device_wait_timeouts() == 0

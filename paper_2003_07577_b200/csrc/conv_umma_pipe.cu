@@ -16,6 +16,26 @@ int pipe_sm_count() {
     return n > 0 ? n : 148;
 }
 
+bool pipe_words_map(const ConvParams& p, const PipeGeom& g, CUtensorMap* map) {
+    *map = CUtensorMap{};
+    if (!g.tma) return true;
+    using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static const Encode encode = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        return cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found) == cudaSuccess &&
+                       found == cudaDriverEntryPointSuccess
+                   ? reinterpret_cast<Encode>(fn)
+                   : nullptr;
+    }();
+    if (!encode) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)p.CW * p.x_words, (cuuint64_t)p.N * p.H * p.W}, strides[1] = {dims[0] * 4};
+    const cuuint32_t box[2] = {(cuuint32_t)(g.raw_words * p.x_words), (cuuint32_t)(g.tile_pix < 256 ? g.tile_pix : 256)}, one[2] = {1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<uint32_t*>(p.x), dims, strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 const ConvVariant* conv_umma_pipe_variant(int a_bits, int variant) {
     switch (a_bits) {
         case 0: return conv_umma_pipe_variant_a0(variant);      // activations as byte codes

@@ -39,6 +39,7 @@
 // memory and returns.  The single-CTA forms use no clusters.
 #pragma once
 
+#include <cuda.h>
 #include <math.h>
 
 #include <type_traits>
@@ -48,9 +49,9 @@
 namespace ebs {
 
 constexpr int PIPE_EXPANDERS = 256;
-// Warps 8 and 9 issue the MMAs, warp 10 fetches weights, warp 11 has no role (20 warps cost the same registers as 18:
-// they are allotted in fours), warps 12-19 run the epilogue.
-constexpr int PIPE_ISSUER_WARP = 8, PIPE_ISSUERS = 2, PIPE_PRODUCER_WARP = 10, PIPE_EPI_WARP0 = 12;
+// Warps 8 and 9 issue the MMAs, warp 10 fetches weights, warp 11 packed words where they come by tensor copies, warps 12 on run the
+// epilogue.
+constexpr int PIPE_ISSUER_WARP = 8, PIPE_ISSUERS = 2, PIPE_PRODUCER_WARP = 10, PIPE_FETCH_WARP = 11, PIPE_EPI_WARP0 = 12;
 // Epilogue warps: sixteen where the 256-channel tile leaves as packed planes without per-channel terms.  These layers wait for the
 // epilogue's instructions; eight warps issue in 60% of the cycles and sixteen, of 80 or 88 registers each, in 80% (64 -> 256 1x1 at
 // 56x56, batch 256, 4 planes: 91.4 -> 78.1 us; 256 -> 1024 at 14x14: 31.0 -> 28.8).  Narrower tiles wait for their expanders, and the
@@ -64,8 +65,9 @@ constexpr int PIPE_SLOTS = 2;                      // (pixel, word) items an exp
 constexpr int PIPE_MAX_ITEMS = PIPE_SLOTS * PIPE_EXPANDERS;
 constexpr int PIPE_MAX_TAPS = FRAME_MAX_TAPS, PIPE_MAX_STAGES = 4;
 constexpr int PIPE_MAX_BSLOTS = 32;                // weight tiles in flight when the weights stream
-// Passes of packed words in the expanders' ring (half as much memory again for more than four planes).
-__host__ __device__ constexpr int pipe_raw_depth(int words) { return words <= 4 ? 4 : 3; }
+// Passes of packed words in the expanders' ring: 8 to 42 KB (8 planes: three passes measured the same).
+__host__ __device__ constexpr int pipe_raw_depth(int words) { return words <= 4 ? 4 : words < 8 ? 3 : 2; }
+constexpr int PIPE_MAX_RAW = 4;                    // slots of packed words that arrive by tensor copies
 constexpr int PIPE_SMEM_MAX = 225 * 1024;          // dynamic; layers with per-channel terms or shortcuts: PIPE_SMEM_TERMS less, for the
 constexpr int PIPE_SMEM_TERMS = 11 * 1024;         // epilogue warps' terms and matrix rows (FragRows, static)
 
@@ -92,6 +94,8 @@ struct PipeGeom : FrameGeom {
     int nchunks;                       // chunks per tile = n_ph * nwg (phase-major)
     int n_stages, a_word_bytes, a_stage_bytes, stage_bytes;
     int raw_bytes, rows_bytes;         // ring of packed words; rows of planes on their way out (pipe_rows_apply)
+    int raw_words, raw_slots, raw_slot_bytes;   // words of a pixel in a slot of that ring (a multiple of ks)
+    int tma;                           // 1: a slot arrives by a tensor copy (one box, two above 256 pixels), 0: by the expanders' own cp.async
     int linear_in, linear_out;         // a frame pixel is the input pixel, the output pixel, of the same number
     int b_resident, b_total_bytes;
     PipeSlot slot[FRAME_MAX_PHASES];   // of each phase
@@ -171,11 +175,11 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
     if (g.SP * 16 >= (1 << 18)) return g;
     // weights resident when they leave room for at least two activation stages
     const int smem_max = PIPE_SMEM_MAX - (pipe_has_terms(p) ? PIPE_SMEM_TERMS : 0);
-    g.raw_bytes = pipe_raw_depth(p.x_words) * PIPE_MAX_ITEMS * p.x_words * 4;
     g.linear_in = taps == 1 && p.sh == 1 && p.sw == 1 && p.ph == 0 && p.pw == 0;
     g.linear_out = g.Hq == p.Ho && g.Wq == p.Wo;
     g.rows_bytes = pipe_rows_bytes(p, tile_n, pair);
-    const int budget = smem_max - 2048 - g.raw_bytes - g.rows_bytes;
+    const int raw_most = pipe_raw_depth(p.x_words) * PIPE_MAX_ITEMS * p.x_words * 4;
+    const int budget = smem_max - 2048 - raw_most - g.rows_bytes;
     g.b_resident = g.b_total_bytes + 2 * ((g.a_word_bytes + 255) & ~255) <= budget && g.b_total_bytes <= 160 * 1024;
     int ks = PIPE_MAX_ITEMS / g.S;
     if (ks > 4) ks = 4;
@@ -188,8 +192,6 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
     const int avail = budget - (g.b_resident ? g.b_total_bytes : b_ring_min);
     while (ks > 1 && 2 * stage_bytes(ks) > avail) --ks;
     if (2 * stage_bytes(ks) > avail) return g;
-    // fewer words per pass when that buys a deeper ring (latency hiding matters more than stage size)
-    while (ks > 1 && avail / stage_bytes(ks) < 3) --ks;
     // A stage is filled in nsub expander passes of ks words: the waits, addresses and commits of a stage cost an issuing
     // warp a thousand clocks, to be spread over some forty MMAs (64 -> 64 3x3 at 56x56, batch 256: 55.6 us with a word a
     // stage, 18 MMAs, 50.3 with two; 256 -> 256 3x3 stride 2 at 28x28: 65.1 and 49.9).
@@ -222,7 +224,32 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
         if (g.b_slots > PIPE_MAX_BSLOTS) g.b_slots = PIPE_MAX_BSLOTS;
         if (g.b_slots < 3) return g;
     }
-    g.smem_bytes = (g.b_resident ? g.b_total_bytes : g.b_slots * g.b_group * b_tile) + g.n_stages * g.stage_bytes + g.raw_bytes + g.rows_bytes + 1024;
+    const int fixed = (g.b_resident ? g.b_total_bytes : g.b_slots * g.b_group * b_tile) + g.rows_bytes + 1024;
+    // Packed words by tensor copies where the strip is a run of input pixels and a thread's own words are no whole 16 bytes (3, 5, 6, 7
+    // planes): cp.async then moves 8 or 4 bytes a lane, which 5 to 7 planes wait for.  A copy takes whole 16 bytes of every pixel (2 or 4
+    // words), and its box at most 256 pixels and 256 words.  us, by cp.async and by tensor copies: 512 -> 128 1x1 at 28x28, batch 256, 7 planes
+    // 74.3 and 41.1 (6 planes 49.0 and 37.0); 256 -> 64 at 56x56, 5 planes 68.9 and 57.6; 1024 -> 256 at 14x14, 7 planes 37.0 and 26.8; 256 ->
+    // 128, 3 planes 65.9 and 63.4.  With 1, 2, 4 and 8 planes, whose items are fetched in whole, it made no difference (256 -> 64, 4 planes: 57.2
+    // and 57.5 in one form of the loop).
+    g.raw_words = ks;
+    g.raw_slot_bytes = PIPE_MAX_ITEMS * p.x_words * 4;
+    g.raw_slots = pipe_raw_depth(p.x_words);
+    if (g.linear_in && !pair && p.x_words != 4 && p.x_words >= 3 && p.x_words != 8 && p.CW * p.x_words % 4 == 0) {
+        const int unit = p.x_words == 6 ? 2 : 4;
+        int u = ks;
+        while (u % unit != 0) u += ks;
+        const int slot = g.tile_pix * u * p.x_words * 4;
+        if (g.kss % u == 0 && fixed + g.n_stages * g.stage_bytes + 2 * slot > smem_max && g.n_stages > 2) --g.n_stages;
+        const int most = (smem_max - fixed - g.n_stages * g.stage_bytes) / slot;
+        if (g.kss % u == 0 && most >= 2) {
+            g.tma = 1;
+            g.raw_words = u;
+            g.raw_slot_bytes = slot;
+            g.raw_slots = most < 4 ? most : 4;
+        }
+    }
+    g.raw_bytes = g.raw_slots * g.raw_slot_bytes;
+    g.smem_bytes = fixed + g.n_stages * g.stage_bytes + g.raw_bytes;
     if (g.b_resident) {                                        // a CTA keeps one channel tile
         g.grid_y = g.n_ctiles;
         long long gx = sms / g.n_ctiles;
@@ -578,7 +605,7 @@ __device__ __forceinline__ void pipe_epilogue_terms(const ConvParams& p, const F
 }
 
 template <int AB, int TILE_N, bool AFFINE, int FORM, bool PAIR = false, bool SMALL = false>
-__global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FORM, PAIR)), 1) conv_umma_pipe_kernel(const ConvParams p, const PipeGeom g) {
+__global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FORM, PAIR)), 1) conv_umma_pipe_kernel(const ConvParams p, const PipeGeom g, const __grid_constant__ CUtensorMap words) {
     constexpr int EPI_WARPS = pipe_epi_warps(TILE_N, AFFINE, FORM, PAIR);
     constexpr bool ROWS = FORM == 2;                           // planes of odd counts leave through rows in shared memory
     // PAIR: the two CTAs of a cluster work as one.  Each expands its own 128 * m_sub pixels and holds the weight rows of
@@ -594,6 +621,7 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
     extern __shared__ uint8_t dyn_smem[];
     __shared__ __align__(8) uint64_t st_full[PIPE_MAX_STAGES], st_empty[PIPE_MAX_STAGES], acc_full[2], acc_empty[2], b_full;
     __shared__ __align__(8) uint64_t bs_full[PIPE_MAX_BSLOTS], bs_empty[PIPE_MAX_BSLOTS];   // streamed weight tiles
+    __shared__ __align__(8) uint64_t raw_full[PIPE_MAX_RAW], raw_empty[PIPE_MAX_RAW];       // packed words by tensor copies
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     __shared__ __align__(16) float s_terms[AFFINE ? EPI_WARPS : 1][64];
@@ -648,6 +676,10 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
         mbar_init(&acc_empty[0], EPI_WARPS);
         mbar_init(&acc_empty[1], EPI_WARPS);
         mbar_init(&b_full, 1);
+        for (int s = 0; s < PIPE_MAX_RAW; ++s) {
+            mbar_init(&raw_full[s], 1);
+            mbar_init(&raw_empty[s], PIPE_EXPANDERS / 32);
+        }
         if constexpr (PAIR) {
             for (int s = 0; s < PIPE_MAX_STAGES; ++s) mbar_init(&st_peer[s], 1);
             for (int s = 0; s < PIPE_MAX_BSLOTS; ++s) mbar_init(&bs_peer[s], 1);
@@ -696,7 +728,7 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
         constexpr uint32_t RAW_PASS = PIPE_MAX_ITEMS * NW * 4;
         const bool paired = (NW & 1) != 0 && (KS & 1) == 0 && (p.CW & 1) == 0;
         int item_pix[PIPE_SLOTS];                             // strip pixel, -1: no item
-        uint32_t item_dst[PIPE_SLOTS], item_q[PIPE_SLOTS];
+        uint32_t item_dst[PIPE_SLOTS], item_q[PIPE_SLOTS], item_at[PIPE_SLOTS];   // item_at: its words in a slot of the ring
 #pragma unroll
         for (int j = 0; j < PIPE_SLOTS; ++j) {
             const int e = paired ? 2 * tid + j : tid + j * PIPE_EXPANDERS;
@@ -704,6 +736,7 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
             item_pix[j] = s < S ? s : -1;
             item_q[j] = (uint32_t)q * (NW * 4);
             item_dst[j] = (uint32_t)(q * g.a_word_bytes + s * 16);
+            item_at[j] = smem_u32(raw) + (s < S ? (uint32_t)((s * g.raw_words + q) * (NW * 4)) : 0u);
         }
         // Fetching runs RD - 1 passes ahead of the expansion, also across tile boundaries: cp.async brings a thread's own items into
         // its places of the ring, so that no barrier is needed and one loop body serves every pass.  (With the words in flight in
@@ -715,7 +748,6 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
         const uint32_t px_bytes = (uint32_t)p.CW * (NW * 4), step = (uint32_t)KS * (NW * 4), wrap = (uint32_t)(nwg * KSS) * (NW * 4);
         const uint32_t first = (uint32_t)(wg_rot * KSS) * (NW * 4);
         uint32_t ld_off = first;
-        const uint32_t raw0 = smem_u32(raw) + (uint32_t)(tid * (paired ? 8 : UNIT));
         uint32_t raw_w = 0, raw_r = 0;
         auto locate = [&]() {
             int ptile, ctile;
@@ -755,11 +787,11 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
                 if (paired) {
 #pragma unroll
                     for (int u = 0; u < NW; ++u)
-                        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(raw0 + raw_w + u * (PIPE_EXPANDERS * 8)), "l"(a + 8 * u), "r"(real ? 8 : 0) : "memory");
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(item_at[j] + raw_w + 8 * u), "l"(a + 8 * u), "r"(real ? 8 : 0) : "memory");
                 } else {
 #pragma unroll
                     for (int u = 0; u < UNITS; ++u) {
-                        const uint32_t dst = raw0 + raw_w + (uint32_t)((j * UNITS + u) * PIPE_EXPANDERS * UNIT);
+                        const uint32_t dst = item_at[j] + raw_w + (uint32_t)(u * UNIT);
                         if constexpr (UNIT == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(a + 16 * u), "r"(real ? 16 : 0) : "memory");
                         else asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(dst), "l"(a + UNIT * u), "n"(UNIT), "r"(real ? UNIT : 0) : "memory");
                     }
@@ -773,76 +805,90 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
         const uint32_t st0 = smem_u32(stages), pass_bytes = (uint32_t)(KS * g.a_word_bytes);
         uint32_t at = st0, full = smem_u32(&st_full[0]);
         const uint32_t half = (uint32_t)SP * 16;
-        int st = 0, sub = 0;
+        const int parts = g.raw_words / KS;                    // passes of a slot
+        int st = 0, sub = 0, part = 0, slot = 0;
+        uint32_t raw_par = 0u;
         uint32_t par = 1u;                                      // (a fresh barrier lets a wait for the phase before its first pass)
+        // (two loops, so that neither has the other's fetching in it: tested at run time it cost 3 us of 54)
+        auto passes = [&](auto tensor_copies) {
+            constexpr bool TMA = decltype(tensor_copies)::value;
 #pragma unroll 1
-        for (int gi = 1 - RD; gi < total; ++gi) {
-            if (gi + RD - 1 < total) fetch();
-            asm volatile("cp.async.commit_group;\n" ::: "memory");
-            if (gi < 0) continue;
-            if (sub == 0) {                                     // the MMAs that read this stage one round ago must be done
-                if (!mbar_wait_bounded(&st_empty[st], par, abortp, wait_limit)) break;
-            }
-            asm volatile("cp.async.wait_group %0;\n" ::"n"(RD - 1) : "memory");
-            uint32_t w[PIPE_SLOTS][NW];
-            const uint32_t rd = raw0 + raw_r;
-            if (paired) {
-#pragma unroll
-                for (int u = 0; u < NW; ++u) {
-                    uint32_t lo, hi;
-                    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];\n" : "=r"(lo), "=r"(hi) : "r"(rd + u * (PIPE_EXPANDERS * 8)) : "memory");
-                    w[(2 * u) / NW][(2 * u) % NW] = lo;
-                    w[(2 * u + 1) / NW][(2 * u + 1) % NW] = hi;
+            for (int gi = TMA ? 0 : 1 - RD; gi < total; ++gi) {
+                if constexpr (!TMA) {
+                    if (gi + RD - 1 < total) fetch();
+                    asm volatile("cp.async.commit_group;\n" ::: "memory");
+                    if (gi < 0) continue;
                 }
-            } else {
+                if (sub == 0) {                                     // the MMAs that read this stage one round ago must be done
+                    if (!mbar_wait_bounded(&st_empty[st], par, abortp, wait_limit)) break;
+                }
+                if constexpr (!TMA) {
+                    asm volatile("cp.async.wait_group %0;\n" ::"n"(RD - 1) : "memory");
+                } else if (part == 0) {
+                    if (!mbar_wait_bounded(&raw_full[slot], raw_par, abortp, wait_limit)) break;
+                }
+                uint32_t w[PIPE_SLOTS][NW];
 #pragma unroll
                 for (int j = 0; j < PIPE_SLOTS; ++j)
 #pragma unroll
                     for (int u = 0; u < UNITS; ++u) {
-                        const uint32_t a = rd + (uint32_t)((j * UNITS + u) * PIPE_EXPANDERS * UNIT);
+                        const uint32_t a = item_at[j] + raw_r + (uint32_t)(u * UNIT);
                         if constexpr (UNIT == 16) asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];\n" : "=r"(w[j][4 * u]), "=r"(w[j][4 * u + 1]), "=r"(w[j][4 * u + 2]), "=r"(w[j][4 * u + 3]) : "r"(a) : "memory");
                         else if constexpr (UNIT == 8) asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];\n" : "=r"(w[j][2 * u]), "=r"(w[j][2 * u + 1]) : "r"(a) : "memory");
                         else asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(w[j][u]) : "r"(a) : "memory");
                     }
-            }
-            raw_r = raw_r == (RD - 1) * RAW_PASS ? 0u : raw_r + RAW_PASS;
-#pragma unroll
-            for (int j = 0; j < PIPE_SLOTS; ++j) {
-                if (item_pix[j] < 0) continue;
-                uint32_t r[8];
-                if constexpr (AB == 0) {
-                    // byte codes, channel c in byte c of the item: only the order changes (row byte 4b + i = channel 8i + b, the
-                    // order of the weight image): register b takes byte b % 4 of words b / 4, 2 + b / 4, ...
-#pragma unroll
-                    for (int bb = 0; bb < 8; ++bb) {
-                        const uint32_t sel = 0x0040u + 0x11u * (uint32_t)(bb & 3);          // byte (bb & 3) of both operands
-                        const uint32_t lo = __byte_perm(w[j][bb >> 2], w[j][2 + (bb >> 2)], sel);
-                        const uint32_t hi = __byte_perm(w[j][4 + (bb >> 2)], w[j][6 + (bb >> 2)], sel);
-                        r[bb] = __byte_perm(lo, hi, 0x5410);
-                    }
-                } else {
-                    planes_to_bytes<NW>(w[j], r);
+                if constexpr (!TMA) {
+                    raw_r = raw_r == (RD - 1) * RAW_PASS ? 0u : raw_r + RAW_PASS;
                 }
-                const uint32_t dst = at + item_dst[j];
-                if (!EBS_IN_RANGE(p, CHK_PIPE_STAGE, (long long)(dst + half + 15u) - st0, NST * g.stage_bytes) ||
-                    !EBS_IN_RANGE(p, CHK_PIPE_STAGE, (long long)dst - st0, NST * g.stage_bytes))
-                    continue;
-                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
-                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst + half), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+#pragma unroll
+                for (int j = 0; j < PIPE_SLOTS; ++j) {
+                    if (item_pix[j] < 0) continue;
+                    uint32_t r[8];
+                    if constexpr (AB == 0) {
+                        // byte codes, channel c in byte c of the item: only the order changes (row byte 4b + i = channel 8i + b, the
+                        // order of the weight image): register b takes byte b % 4 of words b / 4, 2 + b / 4, ...
+#pragma unroll
+                        for (int bb = 0; bb < 8; ++bb) {
+                            const uint32_t sel = 0x0040u + 0x11u * (uint32_t)(bb & 3);          // byte (bb & 3) of both operands
+                            const uint32_t lo = __byte_perm(w[j][bb >> 2], w[j][2 + (bb >> 2)], sel);
+                            const uint32_t hi = __byte_perm(w[j][4 + (bb >> 2)], w[j][6 + (bb >> 2)], sel);
+                            r[bb] = __byte_perm(lo, hi, 0x5410);
+                        }
+                    } else {
+                        planes_to_bytes<NW>(w[j], r);
+                    }
+                    const uint32_t dst = at + item_dst[j];
+                    if (!EBS_IN_RANGE(p, CHK_PIPE_STAGE, (long long)(dst + half + 15u) - st0, NST * g.stage_bytes) ||
+                        !EBS_IN_RANGE(p, CHK_PIPE_STAGE, (long long)dst - st0, NST * g.stage_bytes))
+                        continue;
+                    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+                    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst + half), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+                }
+                // every lane makes its bytes visible to the tensor core's proxy, then one lane arrives for the warp (32 arrivals on one
+                // barrier word would be served one after the other)
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                __syncwarp();
+                if ((tid & 31) == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(full) : "memory");
+                if constexpr (TMA) {
+                    raw_r += step;
+                    if (++part == parts) {                          // this warp has used its words of the slot: only here, so that the next
+                        part = 0;                                   // copy cannot overtake loads that are still under way
+                        if ((tid & 31) == 0) mbar_arrive(&raw_empty[slot]);
+                        if (++slot == g.raw_slots) { slot = 0; raw_par ^= 1u; }
+                        raw_r = (uint32_t)(slot * g.raw_slot_bytes);
+                    }
+                }
+                at += pass_bytes;
+                if (++sub == NSUB) {
+                    sub = 0;
+                    full += 8u;
+                    if (++st == NST) { st = 0; par ^= 1u; full = smem_u32(&st_full[0]); }
+                    at = st0 + (uint32_t)(st * g.stage_bytes);
+                }
             }
-            // every lane makes its bytes visible to the tensor core's proxy, then one lane arrives for the warp (32 arrivals on one
-            // barrier word would be served one after the other)
-            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-            __syncwarp();
-            if ((tid & 31) == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(full) : "memory");
-            at += pass_bytes;
-            if (++sub == NSUB) {
-                sub = 0;
-                full += 8u;
-                if (++st == NST) { st = 0; par ^= 1u; full = smem_u32(&st_full[0]); }
-                at = st0 + (uint32_t)(st * g.stage_bytes);
-            }
-        }
+        };
+        if (g.tma) passes(std::true_type{});
+        else passes(std::false_type{});
         asm volatile("cp.async.wait_all;\n" ::: "memory");
     } else if (warp < PIPE_EPI_WARP0) {
       asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(REG_MID));
@@ -1075,6 +1121,33 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
                 }
             }
         }
+      } else if (warp == PIPE_FETCH_WARP && g.tma) {
+        // =========================== packed words by tensor copies ===========================
+        const int per_stage = KSS / g.raw_words, slot_words = g.raw_words * p.x_words, rows = min(g.tile_pix, 256);
+        const uint32_t leader = elect_one() ? 1u : 0u;
+        int slot = 0;
+        uint32_t par = 1u;
+        bool ok = true;
+        for (int it = 0; it < my_items && ok; ++it) {
+            int ptile, ctile;
+            item_of(it, ptile, ctile);
+            for (int wg = 0; wg < nwg && ok; ++wg) {
+                const int wgr = wg + wg_rot >= nwg ? wg + wg_rot - nwg : wg + wg_rot;
+                for (int i = 0; i < per_stage; ++i) {
+                    if (!mbar_wait_bounded_warp(&raw_empty[slot], par, abortp, wait_limit)) { ok = false; break; }
+                    if (leader) {
+                        mbar_arrive_expect_tx(&raw_full[slot], (uint32_t)g.raw_slot_bytes);
+                        for (int y = 0; y < g.tile_pix; y += rows)
+                            asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n" ::"r"(
+                                             smem_u32(raw) + (uint32_t)(slot * g.raw_slot_bytes + y * slot_words * 4)),
+                                         "l"(reinterpret_cast<uint64_t>(&words)), "r"((wgr * per_stage + i) * slot_words), "r"(ptile * g.tile_pix + y),
+                                         "r"(smem_u32(&raw_full[slot])) : "memory");
+                    }
+                    __syncwarp();
+                    if (++slot == g.raw_slots) { slot = 0; par ^= 1u; }
+                }
+            }
+        }
       }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(REG_EPI));
@@ -1153,6 +1226,9 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
 
 int pipe_sm_count();
 
+// Tensor map of the packed words of all pixels, for boxes of one slot of the ring.  False: the driver refused it.
+bool pipe_words_map(const ConvParams& p, const PipeGeom& g, CUtensorMap* map);
+
 template <int AB, int TILE_N, int FORM, bool AFFINE, bool SMALL>
 int launch_conv_umma_pipe_kernel(const ConvParams& p, const PipeGeom& g, cudaStream_t st) {
     auto kern = conv_umma_pipe_kernel<AB, TILE_N, AFFINE, FORM, false, SMALL>;
@@ -1163,7 +1239,9 @@ int launch_conv_umma_pipe_kernel(const ConvParams& p, const PipeGeom& g, cudaStr
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PIPE_SMEM_MAX - (AFFINE ? PIPE_SMEM_TERMS : 0));
         attr_set[dev] = true;
     }
-    kern<<<dim3((unsigned)g.grid_x, (unsigned)g.grid_y, 1), pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FORM, false)), g.smem_bytes, st>>>(p, g);
+    CUtensorMap words;
+    if (!pipe_words_map(p, g, &words)) return EBS_ERR_CUDA;
+    kern<<<dim3((unsigned)g.grid_x, (unsigned)g.grid_y, 1), pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FORM, false)), g.smem_bytes, st>>>(p, g, words);
     return EBS_OK;
 }
 
@@ -1214,7 +1292,7 @@ int launch_conv_umma_pipe_pair_form(const ConvParams& p, const PipeGeom& g, cuda
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, p, g) == cudaSuccess ? EBS_OK : EBS_ERR_CUDA;
+    return cudaLaunchKernelEx(&cfg, kern, p, g, CUtensorMap{}) == cudaSuccess ? EBS_OK : EBS_ERR_CUDA;
 }
 
 inline bool pipe_pair_request_ok(const ConvParams& p) {

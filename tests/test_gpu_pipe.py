@@ -272,3 +272,12 @@ def test_pipe_accumulators_at_the_conversion_bound(ebs, U, oracle, c):
                     out = U.run_conv(qa, qw, d, epi, want_acc=False, want_y=False, next_bits=nb, variant=variant, px=px, pw=pw)
                     assert np.array_equal(out["packed"], oracle.pack_acts(q_ref, nb)), f"variant {variant}, {nb} planes"
     assert ebs.ebs_device_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("ab", [3, 5, 6, 7])
+@pytest.mark.parametrize("case", [(3, 128, 64, 37, 29), (2, 384, 128, 23, 31), (1, 1152, 256, 35, 21), (4, 192, 64, 19, 15), (1, 256, 512, 60, 61)])
+def test_pipe_words_by_tensor_copies(ebs, U, oracle, ab, case):
+    """1x1 layers of plane counts whose packed words come by tensor copies: a last tile of a few pixels, a last group of fewer words, one
+    and several tiles a thread block, resident and streamed weights (192 channels: by cp.async where a pixel is no whole 16 bytes)."""
+    n, c, co, h, w = case
+    _check(ebs, U, oracle, n, c, co, 1, 1, 0, h, w, 4, ab, 4, min_variants=1)

@@ -170,6 +170,27 @@ static bool tile_kernel_pays(const ConvParams& p, int sms) {
     return tiles <= 3LL * sms;
 }
 
+// Layers of up to three rounds of tiles that the pipeline kernel is ahead on all the same: packed planes only, and a reduction deep
+// enough that its expansion, shared by up to 512 accumulators and overlapped with the epilogue, counts for more than its longer way from
+// launch to result.  Measured on the ResNet-18/50 shapes at batch 8 to 256 (us, tile and pipeline kernel; a round = one 128 x 128 tile an SM):
+//  * strided k x k, 256 channels on, 1.2 rounds on: 256 -> 256 3x3 stride 2 at 28x28, batch 64 21.8 and 19.2; 512 -> 512 at 14x14, batch 256 75.8
+//    and 52.2 (128 channels: 22.4 and 22.0; stride 1 stays: 512 -> 512 at 7x7, batch 256 47.4 and 55.1);
+//  * 1x1 of 1024 channels on from 1.2 rounds, of 256 on from two: 2048 -> 512 at 7x7, batch 128 18.4 and 15.5; 1024 -> 256 at 14x14, batch 64 11.4
+//    and 11.0; 256 -> 64 at 56x56, batch 16 9.0 and 7.6; with per-channel terms of 2048 and 512: batch 128 20.1 and 18.4; 512 -> 128 at 28x28, batch 64
+//    16.4 and 15.1 (1024 -> 256, batch 64: 13.2 and 13.8; 256 -> 64: 10.5 and 10.4);
+//  * 1x1 of 5 to 7 planes, whose words come by tensor copies: 512 channels on from 0.6 rounds, 256 on from 1.2, any from two: 512 -> 128 at
+//    28x28, batch 16 10.1 and 7.6; 256 -> 1024 at 14x14, batch 16 9.8 and 8.3; 64 -> 64 at 56x56, batch 16 8.4 and 7.3 (256 -> 64, batch 8: 6.7 and 7.4).
+static bool pipe_before_tile(const ConvParams& p, int sms) {
+    if (!p.packed_next || p.acc || p.y || p.w_levels) return false;
+    const double rounds = (double)((p.P + 127) / 128) * ((p.Co + 127) / 128) / sms;
+    const bool terms = p.ch_scale || p.ch_bias || p.residual || p.res_packed;
+    if (p.kh * p.kw > 1) return (p.sh > 1 || p.sw > 1) && p.CW >= 8 && rounds >= 1.2;
+    if (!terms && p.sh == 1 && p.sw == 1 && p.x_words >= 5 && p.x_words <= 7 &&
+        (rounds >= 2.0 || (rounds >= 1.2 && p.CW >= 8 && p.Co >= 128) || (rounds >= 0.6 && p.CW >= 16)))
+        return true;
+    return (rounds >= 1.2 && p.CW >= (terms ? 64 : 32)) || (rounds >= 2.0 && p.CW >= (terms ? 16 : 8));
+}
+
 // What a layer that the tile kernel fits only in its per-tap form runs on instead of it; -1: nothing is better.  The per-tap
 // form expands 128 pixels for every (tap, word), whatever the channels and bits, and its epilogue for 32-bit results and
 // weight levels takes long beside a short reduction; the warp-level kernels' time grows with the plane pairs.
@@ -312,7 +333,7 @@ static int conv_plan(const void* packed_x, int n, int h, int w, const void* pack
     if (variant == -2) {
         variant = choose_variant(d->w_bits, d->a_bits, p.P, p.Co, packed_next != nullptr, sm_count());
     } else if (variant < 0) {
-        const bool small = tile_kernel_pays(p, sm_count());
+        const bool small = tile_kernel_pays(p, sm_count()) && !pipe_before_tile(p, sm_count());
         const int tile = umma_ok && (p.Co > 16 || p.KK >= 18) ? choose_tile_variant(p) : -1;
         const int pipe = umma_ok && !(small && tile >= 0) ? choose_pipe_variant(p) : -1;
         // few channels on many pixels: the warp-level strip kernel (16 -> 16 3x3 at 32x32, batch 128: 7.1 us, the tile kernel,

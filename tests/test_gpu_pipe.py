@@ -281,3 +281,24 @@ def test_pipe_words_by_tensor_copies(ebs, U, oracle, ab, case):
     and several tiles a thread block, resident and streamed weights (192 channels: by cp.async where a pixel is no whole 16 bytes)."""
     n, c, co, h, w = case
     _check(ebs, U, oracle, n, c, co, 1, 1, 0, h, w, 4, ab, 4, min_variants=1)
+
+
+@pytest.mark.parametrize("case", [
+    (1, 256, 64, 1, 1, 199, 193, 4), (1, 256, 64, 1, 1, 195, 193, 4),      # just above and below two rounds of tiles on 148 SMs
+    (2, 64, 64, 1, 1, 139, 139, 7),                                        # two rounds, words by tensor copies
+    (1, 512, 128, 1, 1, 107, 107, 6), (1, 512, 128, 1, 1, 103, 103, 6),    # 0.6 rounds
+    (2, 256, 256, 3, 2, 151, 151, 3), (2, 256, 256, 3, 2, 147, 147, 3),    # strided 3x3, 1.2 rounds
+])
+def test_pipe_and_tile_kernels_meet(ebs, U, case):
+    """The library's own choice on both sides of the lines between the tile and the pipeline kernel, against the integer-pipe kernel."""
+    n, c, co, k, s, h, w, ab = case
+    rng = np.random.default_rng(h * w)
+    qa = U.rand_codes(rng, (n, c, h, w), ab, False)
+    qw = rng.integers(-8, 8, size=(co, c, k, k), dtype=np.int32)
+    d = U.desc_for(c, co, k, s, k // 2, 4, ab, 0.03, 0.07)
+    step = 0.03 * 0.07 * float(np.sqrt(c * k * k)) * 8.0 * (1 << ab) / 255.0
+    px, pw = U.pack_acts_codes(qa, ab), U.pack_weight_codes(qw, d)
+    epi = ebs.epilogue(None, None, None, True, 5, step)
+    own, literal = (U.run_conv(qa, qw, d, epi, want_acc=False, want_y=False, next_bits=5, variant=v, px=px, pw=pw)["packed"] for v in (-1, -2))
+    assert literal.any() and np.array_equal(own, literal)
+    assert ebs.ebs_device_wait_timeouts() == 0

@@ -257,6 +257,15 @@ int ebs_conv2d_i8(const void *x_codes_dev, int n, int h, int w, const void *pack
 const char *ebs_conv_variant_family(int variant);
 int ebs_conv_variant_applies(const ebs_conv_desc *desc, int n, int h, int w, const ebs_epilogue *epi, int want_acc,
                              int want_y, int want_packed_next, int variant);
+/*
+ * Test hook: the variant a request runs on (variant = -1: the library's own choice), in route[0], and for the persistent
+ * pipeline kernel what its geometry came to -- route[1]: 1 if packed words arrive by tensor copies, [2] accumulators a tile,
+ * [3] words an expander pass, [4] words a stage, [5] stages, [6] 1 if the weights stay in shared memory, [7] slots of the
+ * ring of packed words, [8] slots of the ring of weight tiles, [9] work items; zeros for the other families.  Status as
+ * ebs_conv_variant_applies; launches nothing.
+ */
+int ebs_test_conv_route(const ebs_conv_desc *desc, int n, int h, int w, const ebs_epilogue *epi, int want_acc, int want_y,
+                        int want_packed_next, int variant, int *route);
 
 /*
  * Number of thread blocks that gave up a bounded device-side wait (on the tensor core's completion

@@ -33,7 +33,7 @@ EXPORTS = [
     "ebs_search_act_forward", "ebs_expected_flops", "ebs_fused_plan_upload", "ebs_resnet_cifar_forward", "ebs_noalloc_scratch_bytes", "ebs_conv2d_mixed_host_noalloc",
     "ebs_conv_variant_family", "ebs_conv_variant_applies", "ebs_check_device_status", "ebs_test_set_device_wait",
     "ebs_conv2d_i8", "ebs_maxpool_packed", "ebs_combined_scale", "ebs_reciprocal_step",
-    "ebs_checked_build", "ebs_checked_status", "ebs_test_checked_shrink", "ebs_pack_acts_s2d",
+    "ebs_checked_build", "ebs_checked_status", "ebs_test_checked_shrink", "ebs_pack_acts_s2d", "ebs_test_conv_route",
     "ebs_graph_begin", "ebs_graph_end", "ebs_graph_launch", "ebs_graph_destroy",
 ]
 
@@ -118,6 +118,7 @@ def lib() -> ctypes.CDLL:
         L.ebs_conv_variant_family.argtypes = [i]
         L.ebs_conv_variant_family.restype = ctypes.c_char_p
         L.ebs_conv_variant_applies.argtypes = [D, i, i, i, E, i, i, i, i]
+        L.ebs_test_conv_route.argtypes = [D, i, i, i, E, i, i, i, i, ctypes.POINTER(i)]
         L.ebs_check_device_status.restype = i
         L.ebs_test_set_device_wait.argtypes = [ctypes.c_uint, i]
         L.ebs_graph_begin.argtypes = [ctypes.POINTER(p)]
@@ -342,6 +343,16 @@ def ebs_conv_variant_applies(desc, n, h, w, epi=None, want_acc=True, want_y=Fals
     e = None if epi is None else ctypes.byref(epi)
     return lib().ebs_conv_variant_applies(ctypes.byref(desc), n, h, w, e, int(bool(want_acc)), int(bool(want_y)),
                                           int(bool(want_packed_next)), int(variant))
+
+
+def ebs_test_conv_route(desc, n, h, w, epi=None, want_acc=True, want_y=False, want_packed_next=False, variant: int = -1) -> dict:
+    """The variant a request runs on and, for the pipeline kernel, its geometry; launches nothing."""
+    route = (ctypes.c_int * 10)()
+    e = None if epi is None else ctypes.byref(epi)
+    _check(lib().ebs_test_conv_route(ctypes.byref(desc), n, h, w, e, int(bool(want_acc)), int(bool(want_y)), int(bool(want_packed_next)),
+                                     int(variant), route), "ebs_test_conv_route")
+    names = ("variant", "tensor_copies", "accumulators", "pass_words", "stage_words", "stages", "resident", "raw_slots", "weight_slots", "items")
+    return dict(zip(names, route))
 
 
 def ebs_check_device_status() -> int:

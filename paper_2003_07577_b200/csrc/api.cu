@@ -245,6 +245,7 @@ struct ConvPlan {
     ConvParams p;
     const ConvVariant* v;
     dim3 grid;
+    int variant;
 };
 
 // byte_acts: packed_x holds the activations as unpacked u8 NHWC codes instead of bit planes (ebs_conv2d_i8).
@@ -378,6 +379,7 @@ static int conv_plan(const void* packed_x, int n, int h, int w, const void* pack
     const long long gx = (P + v->tile_p - 1) / v->tile_p, gy = (p.Co + v->tile_c - 1) / v->tile_c;
     if (gy > 65535) return EBS_ERR_UNSUPPORTED;
     plan->v = v;
+    plan->variant = variant;
     plan->grid = dim3((unsigned)gx, (unsigned)gy, 1);
     return EBS_OK;
 }
@@ -536,6 +538,21 @@ int ebs_conv_variant_applies(const ebs_conv_desc* desc, int n, int h, int w, con
     ConvPlan plan;
     return conv_plan(fake, n, h, w, fake, desc, epi, want_acc ? static_cast<int32_t*>(fake) : nullptr,
                      want_y ? static_cast<float*>(fake) : nullptr, want_packed_next ? fake : nullptr, variant, &plan);
+}
+
+int ebs_test_conv_route(const ebs_conv_desc* desc, int n, int h, int w, const ebs_epilogue* epi, int want_acc, int want_y,
+                        int want_packed_next, int variant, int* route) {
+    void* fake = reinterpret_cast<void*>(static_cast<uintptr_t>(256));
+    if (!route) return EBS_ERR_INVALID_ARG;
+    ConvPlan plan;
+    const int rc = conv_plan(fake, n, h, w, fake, desc, epi, want_acc ? static_cast<int32_t*>(fake) : nullptr,
+                             want_y ? static_cast<float*>(fake) : nullptr, want_packed_next ? fake : nullptr, variant, &plan);
+    if (rc) return rc;
+    memset(route, 0, 10 * sizeof(int));
+    route[0] = plan.variant;
+    const int pipe = plan.variant - (ebs_num_conv_variants() - NUM_CONV_PIPE_VARIANTS);
+    if (pipe >= 0) conv_umma_pipe_route(plan.p, pipe, route + 1);
+    return EBS_OK;
 }
 
 int ebs_test_set_device_wait(unsigned int limit, int skip_mma) {

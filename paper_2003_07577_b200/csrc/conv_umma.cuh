@@ -30,7 +30,9 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
-// Bounded wait for the phase with the given parity; false = gave up (or another thread already had).
+// Bounded wait of a whole warp for the phase with the given parity; false = gave up (or another warp already had).  The outcome is a
+// vote: lanes that left a loop at a poll of their own while others went on would meet those neither at the next __syncwarp
+// nor at the block's barrier.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                                   unsigned limit = UMMA_WAIT_LIMIT) {
     const uint32_t addr = smem_u32(bar);
@@ -41,14 +43,14 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
             "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}\n"
             : "=r"(done) : "r"(addr), "r"(parity) : "memory");
-        if (done) return true;
-        if (*abort_flag) return false;
+        if (__all_sync(0xffffffffu, done != 0)) return true;
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
         __nanosleep(it < 8 ? 40 : 200);   // leave the issue slots to the warps that have work
     }
     *abort_flag = 1;
     return false;
 }
-// The same wait for the single warps that feed the tensor core (issuer, weight producer): no sleep between polls (the
+// The same wait for one thread, or for warps that vote on the outcome themselves (weight producer): no sleep between polls (the
 // try_wait itself suspends the thread for a while), so that they react as soon as the barrier flips.
 __device__ __forceinline__ bool mbar_wait_bounded_hot(uint64_t* bar, uint32_t parity, volatile int* abort_flag, unsigned limit) {
     const uint32_t addr = smem_u32(bar);

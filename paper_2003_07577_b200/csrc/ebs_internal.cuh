@@ -73,7 +73,7 @@ __device__ __forceinline__ bool check_in_range(unsigned long long* st, unsigned 
 // Sites (kernel family * 16 + access): 1x pipeline kernel, 2x warp-level strip kernel, 3x warp-level per-tap kernel,
 // 4x integer-pipe kernel, 5x shared epilogue helpers, 6x tile kernel.
 enum CheckSite {
-    CHK_PIPE_X = 0x10, CHK_PIPE_STAGE = 0x11, CHK_PIPE_TAB = 0x12, CHK_PIPE_ACC = 0x13, CHK_PIPE_Y = 0x14, CHK_PIPE_PN = 0x15,
+    CHK_PIPE_X = 0x10, CHK_PIPE_STAGE = 0x11, CHK_PIPE_ACC = 0x13, CHK_PIPE_Y = 0x14, CHK_PIPE_PN = 0x15,
     CHK_PIPE_W8 = 0x16,
     CHK_MS_X = 0x20, CHK_MS_STRIP = 0x21, CHK_MS_W8 = 0x22, CHK_MS_ACC = 0x23, CHK_MS_Y = 0x24, CHK_MS_PN = 0x25, CHK_MS_WS = 0x26,
     CHK_MMA_X = 0x30, CHK_MMA_W8 = 0x31, CHK_MMA_ACC = 0x32, CHK_MMA_Y = 0x33, CHK_MMA_STAGE = 0x34,
@@ -115,7 +115,7 @@ enum { NUM_CONV_UMMA_VARIANTS = 5, NUM_CONV_STRIP_VARIANTS = 5, NUM_CONV_RESIDEN
 const ConvVariant* conv_umma_pipe_variant(int a_bits, int variant);
 bool conv_umma_pipe_applies(const ConvParams& p, int variant);
 unsigned long long conv_umma_pipe_timeouts();
-long long conv_umma_pipe_items(const ConvParams& p, int variant);   // (pixel super-tile, channel tile) work items, -1 if it does not apply
+void conv_umma_pipe_route(const ConvParams& p, int variant, int* route);   // geometry of a variant that applies (ebs_test_conv_route)
 // Warp-level strip kernel for small stride-1 layers (conv_mma_strip.cu): channel tile 16 / 32 / 64.
 const ConvVariant* conv_mma_strip_variant(int a_bits, int variant);
 bool conv_mma_strip_applies(const ConvParams& p, int variant);

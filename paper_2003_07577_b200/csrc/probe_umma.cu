@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(128, 1) probe_umma_i8_kernel(int iters, unsign
             }
         }
         umma_commit(&done_bar);
-        if (!mbar_wait_bounded(&done_bar, 0u, &abort_flag, wait_limit)) atomicAdd(gave_up, 1u);
+        if (!mbar_wait_bounded_hot(&done_bar, 0u, &abort_flag, wait_limit)) atomicAdd(gave_up, 1u);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();

@@ -57,6 +57,33 @@ def test_pipe_bounded_waits_give_up_and_recover(ebs, U, oracle, form):
     assert ebs.ebs_device_wait_timeouts() == after
 
 
+@pytest.mark.parametrize("limit", [1, 64])
+@pytest.mark.parametrize("co", [64, 256])
+def test_pipe_gives_up_with_tensor_copies_in_flight(ebs, U, oracle, co, limit):
+    """Packed words by tensor copies: the copies of the next slots are under way when the expanders' waits run out (for a free stage,
+    and with a single poll for the words themselves).  Whole warps leave their loops, the block drains its copies and returns."""
+    rng = np.random.default_rng(co + limit)
+    qa, qw = U.rand_codes(rng, (2, 1024, 40, 37), 6, False), U.rand_codes(rng, (co, 1024, 1, 1), 2, True)
+    d = U.desc_for(1024, co, 1, 1, 0, 2, 6)
+    variant = U.variants_of("umma_pipe")[0 if co == 64 else 2]
+    route = ebs.ebs_test_conv_route(d, 2, 40, 37, variant=variant)
+    assert route["tensor_copies"] and route["stage_words"] * route["stages"] < 32      # more words than the stages hold
+    px, pw = U.pack_acts_codes(qa, 6), U.pack_weight_codes(qw, d)
+    assert ebs.ebs_check_device_status() == ebs.EBS_OK
+    before = ebs.ebs_device_wait_timeouts()
+    ebs.ebs_test_set_device_wait(limit, 1)
+    try:
+        U.run_conv(qa, qw, d, variant=variant, px=px, pw=pw)                            # returns: every wait is bounded
+    finally:
+        ebs.ebs_test_set_device_wait(0, 0)
+    after = ebs.ebs_device_wait_timeouts()
+    assert after > before, "no thread block reported that it gave up"
+    assert ebs.ebs_check_device_status() == ebs.EBS_ERR_TIMEOUT
+    got = U.run_conv(qa, qw, d, variant=variant, px=px, pw=pw)["acc"]
+    assert np.array_equal(got, oracle.conv2d_codes(qa, qw, (1, 1), (0, 0)))
+    assert ebs.ebs_device_wait_timeouts() == after
+
+
 def test_tile_kernel_does_not_count_the_launch_before_it(ebs, U, oracle):
     """A tile launch may start while the one before it runs; what it waits for then is not a stage that never fills.  The second
     launch's limit (2000 polls, 80 us and more) covers its own 10 us many times, but not the first launch's: 2304 MMAs of 104

@@ -65,7 +65,8 @@ constexpr int PIPE_SLOTS = 2;                      // (pixel, word) items an exp
 constexpr int PIPE_MAX_ITEMS = PIPE_SLOTS * PIPE_EXPANDERS;
 constexpr int PIPE_MAX_TAPS = FRAME_MAX_TAPS, PIPE_MAX_STAGES = 4;
 constexpr int PIPE_MAX_BSLOTS = 32;                // weight tiles in flight when the weights stream
-// Passes of packed words in the expanders' ring: 8 to 42 KB (8 planes: three passes measured the same).
+// Passes of packed words in the expanders' ring, where shared memory leaves room for them (8 planes: three passes measured the same);
+// two at least.
 __host__ __device__ constexpr int pipe_raw_depth(int words) { return words <= 4 ? 4 : words < 8 ? 3 : 2; }
 constexpr int PIPE_MAX_RAW = 4;                    // slots of packed words that arrive by tensor copies
 constexpr int PIPE_SMEM_MAX = 225 * 1024;          // dynamic; layers with per-channel terms or shortcuts: PIPE_SMEM_TERMS less, for the
@@ -95,6 +96,7 @@ struct PipeGeom : FrameGeom {
     int n_stages, a_word_bytes, a_stage_bytes, stage_bytes;
     int raw_bytes, rows_bytes;         // ring of packed words; rows of planes on their way out (pipe_rows_apply)
     int raw_words, raw_slots, raw_slot_bytes;   // words of a pixel in a slot of that ring (a multiple of ks)
+    int ring_full;                     // by cp.async: 1: the ring has its full depth, in slots of PIPE_MAX_ITEMS items, 0: two slots of the strip's size
     int tma;                           // 1: a slot arrives by a tensor copy (one box, two above 256 pixels), 0: by the expanders' own cp.async
     int linear_in, linear_out;         // a frame pixel is the input pixel, the output pixel, of the same number
     int b_resident, b_total_bytes;
@@ -128,8 +130,8 @@ inline int pipe_rows_bytes(const ConvParams& p, int tile_n, bool pair) {
     return !pair && pipe_rows_apply(p, tile_n) ? pipe_epi_warps(tile_n, pipe_has_terms(p), 2, false) * 32 * 8 * p.next_bits : 0;
 }
 
-// m_sub_req = 0: chosen here.  Returns ok = false when the kernel does not apply.
-inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_sub_req = 0, bool pair = false) {
+// The geometry with packed words by tensor copies (copies) or by cp.async; see pipe_geometry.
+inline PipeGeom pipe_geometry_with(const ConvParams& p, int tile_n, int sms, int m_sub_req, bool pair, bool copies) {
     PipeGeom g{};
     if (pair && (tile_n != 256 || (p.Co % 256) != 0 || sms < 2)) return g;
     const int pw = pair ? 2 : 1;                               // CTAs that share a pixel pair-tile
@@ -178,27 +180,46 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
     g.linear_in = taps == 1 && p.sh == 1 && p.sw == 1 && p.ph == 0 && p.pw == 0;
     g.linear_out = g.Hq == p.Ho && g.Wq == p.Wo;
     g.rows_bytes = pipe_rows_bytes(p, tile_n, pair);
-    const int raw_most = pipe_raw_depth(p.x_words) * PIPE_MAX_ITEMS * p.x_words * 4;
-    const int budget = smem_max - 2048 - raw_most - g.rows_bytes;
-    g.b_resident = g.b_total_bytes + 2 * ((g.a_word_bytes + 255) & ~255) <= budget && g.b_total_bytes <= 160 * 1024;
+    if (copies && (!g.linear_in || pair || p.x_words < 3 || p.x_words == 4 || p.x_words == 8 || p.CW * p.x_words % 4 != 0)) return g;
+    // A slot of the ring of packed words: a pass of the strip, or what a tensor copy brings, whole 16 bytes of every pixel (2 or 4 words).
+    // Two slots are enough where shared memory is short: the ring gets its full depth only where that displaces neither resident weights nor
+    // words of a pass.  us with the full ring throughout, and so: 512 -> 256 1x1 at 28x28, batch 256, 7 planes in and out 82.3 and
+    // 53.7; 256 -> 128 at 56x56 140 and 79.8; 512 -> 128 at 28x28, 5 planes 53.3 and 32.7; strided 608 -> 2048 1x1 at 58x29, 5 planes 534 and 281; 128 ->
+    // 128 3x3 at 28x28, batch 64, 7 planes and terms 25.6 and 17.9.  A third stage instead of the deeper ring: 224 -> 64 3x3 stride 2 259 and 356.
+    auto slot_words = [&](int k) {
+        int u = k;
+        while (copies && u % (p.x_words == 6 ? 2 : 4) != 0) u += k;
+        return u;
+    };
+    auto slot_bytes = [&](int k) { return ((copies ? g.tile_pix : g.S) * slot_words(k) * p.x_words * 4 + 127) & ~127; };
+    const int budget = smem_max - 2048 - g.rows_bytes;
     int ks = PIPE_MAX_ITEMS / g.S;
     if (ks > 4) ks = 4;
     if (ks > p.CW) ks = p.CW;
     if (ks < 1) return g;
+    const int full_ring = pipe_raw_depth(p.x_words) * PIPE_MAX_ITEMS * p.x_words * 4;
     // Streamed weights go through a ring of their own (slots of a few consecutive (tap, word) tiles), so that copies are
     // in flight all the time (a stage-sized unit would leave the copy engine idle while a stage's MMAs run).
     auto stage_bytes = [&](int k) { return (k * g.a_word_bytes + 255) & ~255; };
-    const int b_ring_min = g.b_resident ? 0 : 96 * 1024 / pw;
-    const int avail = budget - (g.b_resident ? g.b_total_bytes : b_ring_min);
-    while (ks > 1 && 2 * stage_bytes(ks) > avail) --ks;
-    if (2 * stage_bytes(ks) > avail) return g;
+    // Weights stay resident beside two stages of whole passes; a layer of several taps, whose weight traffic is the larger, keeps them beside
+    // stages of one word too (1184 -> 320 1x1, 7 planes: 391 us streamed, 648 resident with one word a pass).
+    auto beside = [&](int b_bytes, int k, int words, int ring) { return b_bytes + 2 * stage_bytes(words) + ring <= budget; };
+    g.b_resident = g.b_total_bytes <= 160 * 1024 && (beside(g.b_total_bytes, ks, slot_words(ks), 2 * slot_bytes(ks)) ||
+                                                     (taps > 1 && beside(g.b_total_bytes, 1, slot_words(1), 2 * slot_bytes(1))));
+    const int b_bytes = g.b_resident ? g.b_total_bytes : 96 * 1024 / pw, avail = budget - b_bytes;
+    while (ks > 1 && !beside(b_bytes, ks, slot_words(ks), 2 * slot_bytes(ks))) --ks;
+    if (!beside(b_bytes, ks, slot_words(ks), 2 * slot_bytes(ks))) return g;
     // A stage is filled in nsub expander passes of ks words: the waits, addresses and commits of a stage cost an issuing
     // warp a thousand clocks, to be spread over some forty MMAs (64 -> 64 3x3 at 56x56, batch 256: 55.6 us with a word a
     // stage, 18 MMAs, 50.3 with two; 256 -> 256 3x3 stride 2 at 28x28: 65.1 and 49.9).
-    int nsub = 1;
-    while (nsub < 4 && ks * nsub * taps * m_sub < 40 && ks * nsub < p.CW &&
-           2 * stage_bytes(ks * 2 * nsub) <= avail)
-        nsub *= 2;
+    int nsub = slot_words(ks) / ks;                            // (a stage holds whole slots)
+    if (nsub > 4) return g;
+    auto short_of = [&](int mmas) { return nsub < 4 && ks * nsub * taps * m_sub < mmas && ks * nsub < p.CW; };
+    const int ring = full_ring > 2 * slot_bytes(ks) ? full_ring : 2 * slot_bytes(ks);
+    while (short_of(40) && beside(b_bytes, ks, ks * 2 * nsub, ring)) nsub *= 2;
+    // (a single word of nine taps is too short a stage even so: 128 -> 128 3x3 at 28x28, batch 256, 6 planes: 44.7 and 43.1; from some 32 MMAs
+    // on the third stage and the deeper ring are worth more: 672 -> 2048 3x3 886 and 910, 896 -> 256 1x1 63.5 and 74.2)
+    while (taps > 1 && short_of(32) && beside(b_bytes, ks, ks * 2 * nsub, 2 * slot_bytes(ks))) nsub *= 2;
     // Skew between the word tiles of a pass: the 8 lanes of a quarter warp store 16 bytes each for ks words of 8 / ks
     // pixels; a skew of 128 / ks bytes (48 for three words) puts them on eight different 16-byte bank groups.
     g.a_word_bytes = g.SP * 32 + (ks == 4 ? 32 : ks == 3 ? 48 : 64);
@@ -209,45 +230,33 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
     g.nchunks = g.n_ph * g.nwg;
     g.a_stage_bytes = stage_bytes(g.kss);
     g.stage_bytes = g.a_stage_bytes;
-    g.n_stages = avail / g.stage_bytes;
     const int st_cap = g.b_resident ? PIPE_MAX_STAGES : (pair ? PIPE_MAX_STAGES : 3);
+    g.tma = copies;
+    g.raw_words = slot_words(ks);
+    g.raw_slot_bytes = slot_bytes(ks);
+    const int reserve = beside(b_bytes, ks, g.kss, ring) ? ring : 2 * g.raw_slot_bytes;
+    g.n_stages = (avail - reserve) / g.stage_bytes;
     if (g.n_stages > st_cap) g.n_stages = st_cap;
     if (!g.b_resident) {
         // a slot holds up to 32 KB of consecutive tiles (one wait and one commit per slot, not per MMA)
+        auto weight_slots = [&](int most) {
+            g.b_group = 1;
+            for (int i = 0; i < g.n_ph; ++i) {
+                const PipeSlot sl = g.slot[i] = pipe_slot(g.ph_rows[i], g.ph_cols[i], most);
+                if (sl.words * sl.rows * sl.cols > g.b_group) g.b_group = sl.words * sl.rows * sl.cols;
+            }
+            g.b_slots = (budget - reserve - g.n_stages * g.stage_bytes) / (g.b_group * b_tile);
+            return g.b_slots >= 3;
+        };
         const int most = 32768 / b_tile > g.kss * max_ph_taps ? g.kss * max_ph_taps : 32768 / b_tile;
-        g.b_group = 1;
-        for (int i = 0; i < g.n_ph; ++i) {
-            const PipeSlot sl = g.slot[i] = pipe_slot(g.ph_rows[i], g.ph_cols[i], most);
-            if (sl.words * sl.rows * sl.cols > g.b_group) g.b_group = sl.words * sl.rows * sl.cols;
-        }
-        g.b_slots = (budget - g.n_stages * g.stage_bytes) / (g.b_group * b_tile);
+        if (!weight_slots(most)) return g;
         if (g.b_slots > PIPE_MAX_BSLOTS) g.b_slots = PIPE_MAX_BSLOTS;
-        if (g.b_slots < 3) return g;
     }
     const int fixed = (g.b_resident ? g.b_total_bytes : g.b_slots * g.b_group * b_tile) + g.rows_bytes + 1024;
-    // Packed words by tensor copies where the strip is a run of input pixels and a thread's own words are no whole 16 bytes (3, 5, 6, 7
-    // planes): cp.async then moves 8 or 4 bytes a lane, which 5 to 7 planes wait for.  A copy takes whole 16 bytes of every pixel (2 or 4
-    // words), and its box at most 256 pixels and 256 words.  us, by cp.async and by tensor copies: 512 -> 128 1x1 at 28x28, batch 256, 7 planes
-    // 74.3 and 41.1 (6 planes 49.0 and 37.0); 256 -> 64 at 56x56, 5 planes 68.9 and 57.6; 1024 -> 256 at 14x14, 7 planes 37.0 and 26.8; 256 ->
-    // 128, 3 planes 65.9 and 63.4.  With 1, 2, 4 and 8 planes, whose items are fetched in whole, it made no difference (256 -> 64, 4 planes: 57.2
-    // and 57.5 in one form of the loop).
-    g.raw_words = ks;
-    g.raw_slot_bytes = PIPE_MAX_ITEMS * p.x_words * 4;
-    g.raw_slots = pipe_raw_depth(p.x_words);
-    if (g.linear_in && !pair && p.x_words != 4 && p.x_words >= 3 && p.x_words != 8 && p.CW * p.x_words % 4 == 0) {
-        const int unit = p.x_words == 6 ? 2 : 4;
-        int u = ks;
-        while (u % unit != 0) u += ks;
-        const int slot = g.tile_pix * u * p.x_words * 4;
-        if (g.kss % u == 0 && fixed + g.n_stages * g.stage_bytes + 2 * slot > smem_max && g.n_stages > 2) --g.n_stages;
-        const int most = (smem_max - fixed - g.n_stages * g.stage_bytes) / slot;
-        if (g.kss % u == 0 && most >= 2) {
-            g.tma = 1;
-            g.raw_words = u;
-            g.raw_slot_bytes = slot;
-            g.raw_slots = most < 4 ? most : 4;
-        }
-    }
+    const int left = smem_max - fixed - g.n_stages * g.stage_bytes;
+    g.ring_full = !copies && left >= full_ring;
+    if (g.ring_full) g.raw_slot_bytes = PIPE_MAX_ITEMS * p.x_words * 4;
+    g.raw_slots = copies ? (left / g.raw_slot_bytes < PIPE_MAX_RAW ? left / g.raw_slot_bytes : PIPE_MAX_RAW) : g.ring_full ? pipe_raw_depth(p.x_words) : 2;
     g.raw_bytes = g.raw_slots * g.raw_slot_bytes;
     g.smem_bytes = fixed + g.n_stages * g.stage_bytes + g.raw_bytes;
     if (g.b_resident) {                                        // a CTA keeps one channel tile
@@ -263,6 +272,20 @@ inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_su
     }
     g.ok = g.n_stages >= 2 && g.smem_bytes <= smem_max && g.grid_y <= 65535 && g.n_ctiles <= 65535;
     return g;
+}
+
+// m_sub_req = 0: chosen here.  Returns ok = false when the kernel does not apply.
+// Packed words come by tensor copies where the strip is a run of input pixels and a thread's own words are no whole 16 bytes (3, 5, 6, 7
+// planes): cp.async then moves 8 or 4 bytes a lane, which 5 to 7 planes wait for.  A copy takes whole 16 bytes of every pixel (2 or 4
+// words), and its box at most 256 pixels and 256 words.  us, by cp.async and by tensor copies: 512 -> 128 1x1 at 28x28, batch 256, 7 planes
+// 74.3 and 41.1 (6 planes 49.0 and 37.0); 256 -> 64 at 56x56, 5 planes 68.9 and 57.6; 1024 -> 256 at 14x14, 7 planes 37.0 and 26.8; 256 ->
+// 128, 3 planes 65.9 and 63.4.  With 1, 2, 4 and 8 planes, whose items are fetched in whole, it made no difference (256 -> 64, 4 planes: 57.2
+// and 57.5 in one form of the loop).  copies = false: by cp.async in every layer; a layer that applies does so either way.
+inline PipeGeom pipe_geometry(const ConvParams& p, int tile_n, int sms, int m_sub_req = 0, bool pair = false, bool copies = true) {
+    const PipeGeom g = pipe_geometry_with(p, tile_n, sms, m_sub_req, pair, false);
+    if (!copies || !g.ok) return g;
+    const PipeGeom t = pipe_geometry_with(p, tile_n, sms, m_sub_req, pair, true);
+    return t.ok && t.b_resident == g.b_resident ? t : g;
 }
 
 // umma_i8_split for a CTA pair: M = 256 over the two CTAs' tensor memory, issued by the even CTA; the commit arrives on the
@@ -724,7 +747,6 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
         // its 2 * AB packed words still start on an 8-byte boundary and load as pairs.  Otherwise items tid and tid + 256.
         constexpr int NW = AB == 0 ? 8 : AB;                  // words of one (pixel, 32-channel word) item; AB = 0: byte codes
         constexpr int UNIT = NW % 4 == 0 ? 16 : NW % 2 == 0 ? 8 : 4, UNITS = NW * 4 / UNIT;
-        constexpr int RD = pipe_raw_depth(NW);
         constexpr uint32_t RAW_PASS = PIPE_MAX_ITEMS * NW * 4;
         const bool paired = (NW & 1) != 0 && (KS & 1) == 0 && (p.CW & 1) == 0;
         int item_pix[PIPE_SLOTS];                             // strip pixel, -1: no item
@@ -774,7 +796,7 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
             ld_off = first;
             if (++ld_ph == g.n_ph) { ld_ph = 0; ++ld_it; }
         };
-        auto fetch = [&]() {
+        auto fetch = [&](uint32_t raw_last, uint32_t raw_pass) {
             if (ld_left == 0) locate();
             --ld_left;
 #pragma unroll
@@ -797,7 +819,7 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
                     }
                 }
             }
-            raw_w = raw_w == (RD - 1) * RAW_PASS ? 0u : raw_w + RAW_PASS;
+            raw_w = raw_w == raw_last ? 0u : raw_w + raw_pass;
             ld_off += step;
             if (ld_off == wrap) ld_off = 0;
         };
@@ -809,13 +831,16 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
         int st = 0, sub = 0, part = 0, slot = 0;
         uint32_t raw_par = 0u;
         uint32_t par = 1u;                                      // (a fresh barrier lets a wait for the phase before its first pass)
-        // (two loops, so that neither has the other's fetching in it: tested at run time it cost 3 us of 54)
-        auto passes = [&](auto tensor_copies) {
-            constexpr bool TMA = decltype(tensor_copies)::value;
+        // (a loop each for tensor copies, the full ring and two slots: the fetching chosen at run time cost 3 us of 54, the ring's size and
+        // depth in registers up to 6% of strided layers: 128 -> 128 3x3 at 56x56, batch 256, 1 plane 46.8 and 49.8)
+        auto passes = [&](auto form) {
+            constexpr bool TMA = decltype(form)::value == 0, FULL = decltype(form)::value == 1;
+            constexpr int RD = FULL ? pipe_raw_depth(NW) : 2;   // passes in the ring
+            const uint32_t raw_pass = FULL ? RAW_PASS : (uint32_t)g.raw_slot_bytes, raw_last = (RD - 1) * raw_pass;
 #pragma unroll 1
             for (int gi = TMA ? 0 : 1 - RD; gi < total; ++gi) {
                 if constexpr (!TMA) {
-                    if (gi + RD - 1 < total) fetch();
+                    if (gi + RD - 1 < total) fetch(raw_last, raw_pass);
                     asm volatile("cp.async.commit_group;\n" ::: "memory");
                     if (gi < 0) continue;
                 }
@@ -838,7 +863,7 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
                         else asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(w[j][u]) : "r"(a) : "memory");
                     }
                 if constexpr (!TMA) {
-                    raw_r = raw_r == (RD - 1) * RAW_PASS ? 0u : raw_r + RAW_PASS;
+                    raw_r = raw_r == raw_last ? 0u : raw_r + raw_pass;
                 }
 #pragma unroll
                 for (int j = 0; j < PIPE_SLOTS; ++j) {
@@ -887,8 +912,9 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
                 }
             }
         };
-        if (g.tma) passes(std::true_type{});
-        else passes(std::false_type{});
+        if (NW >= 3 && NW != 4 && NW != 8 && g.tma) passes(std::integral_constant<int, 0>{});
+        else if (g.ring_full) passes(std::integral_constant<int, 1>{});
+        else passes(std::integral_constant<int, 2>{});
         asm volatile("cp.async.wait_all;\n" ::: "memory");
     } else if (warp < PIPE_EPI_WARP0) {
       asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(REG_MID));

@@ -31,3 +31,35 @@ def test_wide_and_strided_layers_have_a_tcgen05_kernel(ebs, c, co, k, stride, h,
     fams = [ebs.ebs_conv_variant_family(v) for v in range(ebs.ebs_num_conv_variants())
             if ebs.ebs_conv_variant_applies(d, 2, h, w, None, True, False, False, v) == ebs.EBS_OK]
     assert fams.count("umma") == 5, sorted(set(fams))
+
+
+def _route(ebs, n, h, w, c, co, k, stride, ab, nb, terms=False, tile=None):
+    """Route of a layer whose result is packed planes (stand-in buffers: nothing is read)."""
+    d = ebs.conv_desc(c, co, k, k, stride, stride, k // 2, k // 2, 4, ab, 0.05, 0.05)
+    epi = ebs.epilogue(None, None, None, True, nb, 1.0)
+    if terms:
+        epi.ch_scale_dev = epi.ch_bias_dev = 256
+    pipe = [v for v in range(ebs.ebs_num_conv_variants()) if ebs.ebs_conv_variant_family(v) == "umma_pipe"]
+    variant = -1 if tile is None else pipe[{64: 0, 128: 1, 256: 2, "pair": 3}[tile]]
+    return ebs.ebs_test_conv_route(d, n, h, w, epi, False, False, True, variant)
+
+
+@pytest.mark.parametrize("layer,tile,terms,want", [
+    # n, h, w, c, co, k, stride, planes in, planes out
+    ((256, 28, 28, 512, 256, 1, 1, 7, 7), 256, False, dict(pass_words=4, tensor_copies=1, resident=1)),
+    ((256, 7, 7, 512, 2048, 1, 1, 7, 6), 256, False, dict(pass_words=4, tensor_copies=1, resident=1)),
+    ((256, 28, 28, 512, 128, 1, 1, 5, 4), 128, False, dict(pass_words=2, tensor_copies=1, resident=1)),
+    ((256, 56, 56, 256, 128, 1, 1, 7, 7), 128, False, dict(pass_words=2, tensor_copies=1, resident=1)),
+    ((256, 28, 28, 128, 128, 3, 1, 7, 7), 128, True, dict(resident=1)),
+    ((64, 28, 28, 128, 128, 3, 1, 7, 7), 128, True, dict(resident=1, pass_words=2)),
+    ((64, 56, 56, 128, 128, 3, 2, 7, 5), 128, True, dict(resident=1, pass_words=3)),
+    ((2, 83, 84, 64, 1024, 3, 1, 7, 5), 256, False, dict(resident=1)),
+    ((4, 110, 55, 1280, 128, 1, 2, 6, 4), 128, True, dict(pass_words=4)),
+    ((256, 58, 29, 608, 2048, 1, 2, 5, 7), 256, False, dict(pass_words=4)),
+])
+def test_ring_of_packed_words_displaces_neither_weights_nor_words(ebs, layer, tile, terms, want):
+    """Where shared memory is short the ring of packed words is two slots deep, so that the words of an expander pass, resident weights of
+    a k x k layer and tensor copies are what they are beside any ring (wide plane counts with rows of planes on their way out)."""
+    got = _route(ebs, *layer, terms=terms, tile=tile)
+    assert {k: got[k] for k in want} == want, got
+    assert got["raw_slots"] >= 2 and got["stages"] >= 2

@@ -308,7 +308,8 @@ int ebs_test_checked_shrink(long long elements);
  * polls a bounded wait makes before it gives up (0 restores the default, about 2^20 polls of >= 40 ns);
  * skip_mma = 1 makes the issuing warps of the persistent pipeline kernel, the tile kernel and the whole-network
  * kernel issue no tensor-core work at all, so that every wait for it runs out with nothing in flight; 2 makes the
- * first thread block of every cluster of a split tile launch send the others no sums.  Each thread block that waits
+ * first thread block of every cluster of a split tile launch send the others no sums; 3 makes the library take every tensor map
+ * as refused by the driver (nothing then runs out: the words come the other way).  Each thread block that waits
  * in vain raises its abort flag, leaves its loops, waits a bounded time for what it started, frees its tensor
  * memory and returns, and ebs_device_wait_timeouts() rises.  Process-wide; affects the launches made afterwards.  Nothing faults or hangs by construction.
  */

@@ -557,7 +557,7 @@ int ebs_test_conv_route(const ebs_conv_desc* desc, int n, int h, int w, const eb
 
 int ebs_test_set_device_wait(unsigned int limit, int skip_mma) {
     g_wait_limit = limit == 0 ? (1u << 20) : limit;
-    g_test_flags = skip_mma == 2 ? 2 : skip_mma ? 1 : 0;
+    g_test_flags = skip_mma == 2 ? 2 : skip_mma == 3 ? 4 : skip_mma ? 1 : 0;
     return EBS_OK;
 }
 

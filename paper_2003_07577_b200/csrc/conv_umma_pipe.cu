@@ -17,8 +17,7 @@ int pipe_sm_count() {
 }
 
 bool pipe_words_map(const ConvParams& p, const PipeGeom& g, CUtensorMap* map) {
-    *map = CUtensorMap{};
-    if (!g.tma) return true;
+    if ((p.test_flags & 4) != 0) return false;
     using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
                                 const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
     static const Encode encode = [] {

@@ -1252,11 +1252,11 @@ __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FO
 
 int pipe_sm_count();
 
-// Tensor map of the packed words of all pixels, for boxes of one slot of the ring.  False: the driver refused it.
+// Tensor map of the packed words of all pixels, for boxes of one slot of the ring.  False: the driver has none, or refused it.
 bool pipe_words_map(const ConvParams& p, const PipeGeom& g, CUtensorMap* map);
 
 template <int AB, int TILE_N, int FORM, bool AFFINE, bool SMALL>
-int launch_conv_umma_pipe_kernel(const ConvParams& p, const PipeGeom& g, cudaStream_t st) {
+int launch_conv_umma_pipe_kernel(const ConvParams& p, const PipeGeom& g, const CUtensorMap& words, cudaStream_t st) {
     auto kern = conv_umma_pipe_kernel<AB, TILE_N, AFFINE, FORM, false, SMALL>;
     static bool attr_set[64] = {};
     int dev = 0;
@@ -1265,8 +1265,6 @@ int launch_conv_umma_pipe_kernel(const ConvParams& p, const PipeGeom& g, cudaStr
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PIPE_SMEM_MAX - (AFFINE ? PIPE_SMEM_TERMS : 0));
         attr_set[dev] = true;
     }
-    CUtensorMap words;
-    if (!pipe_words_map(p, g, &words)) return EBS_ERR_CUDA;
     kern<<<dim3((unsigned)g.grid_x, (unsigned)g.grid_y, 1), pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FORM, false)), g.smem_bytes, st>>>(p, g, words);
     return EBS_OK;
 }
@@ -1281,17 +1279,17 @@ inline bool pipe_small_accumulators(const ConvParams& p) {
 }
 
 template <int AB, int TILE_N, int FORM>
-int launch_conv_umma_pipe_form(const ConvParams& p, const PipeGeom& g, cudaStream_t st) {
-    if (pipe_has_terms(p)) return launch_conv_umma_pipe_kernel<AB, TILE_N, FORM, true, false>(p, g, st);
+int launch_conv_umma_pipe_form(const ConvParams& p, const PipeGeom& g, const CUtensorMap& words, cudaStream_t st) {
+    if (pipe_has_terms(p)) return launch_conv_umma_pipe_kernel<AB, TILE_N, FORM, true, false>(p, g, words, st);
     if constexpr (FORM != 0) {
         if (pipe_small_accumulators(p)) {
             ConvParams q = p;
             q.S = ldexpf(p.S, 75);
             q.inv_next = ldexpf(p.inv_next, 74);
-            return launch_conv_umma_pipe_kernel<AB, TILE_N, FORM, false, true>(q, g, st);
+            return launch_conv_umma_pipe_kernel<AB, TILE_N, FORM, false, true>(q, g, words, st);
         }
     }
-    return launch_conv_umma_pipe_kernel<AB, TILE_N, FORM, false, false>(p, g, st);
+    return launch_conv_umma_pipe_kernel<AB, TILE_N, FORM, false, false>(p, g, words, st);
 }
 
 // The CTA-pair form: clusters of two CTAs along x; packed-only whole tiles (form 1) or every output mode (form 0),
@@ -1336,15 +1334,17 @@ int launch_conv_umma_pipe_pair(const ConvParams& p, dim3 /*grid*/, cudaStream_t 
 
 template <int AB, int TILE_N>
 int launch_conv_umma_pipe(const ConvParams& p, dim3 /*grid*/, cudaStream_t st) {
-    const PipeGeom g = pipe_geometry(p, TILE_N, pipe_sm_count(), p.pipe_m_sub);
+    PipeGeom g = pipe_geometry(p, TILE_N, pipe_sm_count(), p.pipe_m_sub);
     if (!g.ok) return EBS_ERR_UNSUPPORTED;                    // the geometry does not apply: nothing is launched
+    CUtensorMap words{};
+    if (g.tma && !pipe_words_map(p, g, &words)) g = pipe_geometry(p, TILE_N, pipe_sm_count(), p.pipe_m_sub, false, false);   // by cp.async
     if (pipe_packed_only(p)) {
         if constexpr (TILE_N >= 128) {
-            if (pipe_rows_apply(p, TILE_N)) return launch_conv_umma_pipe_form<AB, TILE_N, 2>(p, g, st);
+            if (pipe_rows_apply(p, TILE_N)) return launch_conv_umma_pipe_form<AB, TILE_N, 2>(p, g, words, st);
         }
-        return launch_conv_umma_pipe_form<AB, TILE_N, 1>(p, g, st);
+        return launch_conv_umma_pipe_form<AB, TILE_N, 1>(p, g, words, st);
     }
-    return launch_conv_umma_pipe_form<AB, TILE_N, 0>(p, g, st);
+    return launch_conv_umma_pipe_form<AB, TILE_N, 0>(p, g, words, st);
 }
 
 constexpr int NUM_UMMA_PIPE_VARIANTS = 4;          // TILE_N = 64, 128, 256; 256 on a CTA pair

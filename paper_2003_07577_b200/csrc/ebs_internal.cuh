@@ -39,8 +39,8 @@ struct ConvParams {
     int fold_bits;                    // 32 / fold: bits each folded tap occupies (>= c_in)
     int strip_pix, strip_ks;          // strip kernel only (set by its launcher): pixels of a strip, words per stage
     unsigned wait_limit;              // polls a bounded device-side wait makes before the CTA gives up
-    int test_flags;                   // tests only, so that waits run out: bit 0 the MMA issuer issues nothing, bit 1 the first
-                                      // CTA of a tile kernel's cluster sends no sums
+    int test_flags;                   // tests only.  So that waits run out: bit 0 the MMA issuer issues nothing, bit 1 the first
+                                      // CTA of a tile kernel's cluster sends no sums.  Bit 2: tensor maps count as refused
     int tile_split;                   // tile kernel: CTAs the reduction is split over (0 = chosen by the library)
     long long acc_bound;              // no accumulator of the layer is larger in magnitude
     int pipe_m_sub;                   // persistent pipeline kernel: accumulators per super-tile (0 = chosen by the library)

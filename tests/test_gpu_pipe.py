@@ -302,3 +302,25 @@ def test_pipe_and_tile_kernels_meet(ebs, U, case):
     own, literal = (U.run_conv(qa, qw, d, epi, want_acc=False, want_y=False, next_bits=5, variant=v, px=px, pw=pw)["packed"] for v in (-1, -2))
     assert literal.any() and np.array_equal(own, literal)
     assert ebs.ebs_device_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("ab,c,co", [(5, 256, 64), (6, 64, 256), (7, 512, 128)])
+def test_pipe_runs_where_the_driver_refuses_the_tensor_map(ebs, U, oracle, ab, c, co):
+    """Without a tensor map the packed words come by cp.async, device call and host call alike: no error after work has been enqueued."""
+    n, h, w = 3, 23, 29
+    rng = np.random.default_rng(ab)
+    qa, qw = U.rand_codes(rng, (n, c, h, w), ab, False), rng.integers(-7, 8, size=(co, c, 1, 1), dtype=np.int32)
+    d = U.desc_for(c, co, 1, 1, 0, 4, ab)
+    ref = oracle.conv2d_codes(qa, qw, (1, 1), (0, 0))
+    px, pw = U.pack_acts_codes(qa, ab), U.pack_weight_codes(qw, d)
+    ran = 0
+    ebs.ebs_test_set_device_wait(0, 3)
+    try:
+        for variant in U.variants_of("umma_pipe"):
+            if U.applies(d, h, w, variant, n=n) and ebs.ebs_test_conv_route(d, n, h, w, variant=variant)["tensor_copies"]:
+                assert np.array_equal(U.run_conv(qa, qw, d, variant=variant, px=px, pw=pw)["acc"], ref)
+                ran += 1
+    finally:
+        ebs.ebs_test_set_device_wait(0, 0)
+    assert ran >= 2
+    assert ebs.ebs_device_wait_timeouts() == 0

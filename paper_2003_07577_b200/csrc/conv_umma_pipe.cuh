@@ -238,7 +238,8 @@ inline PipeGeom pipe_geometry_with(const ConvParams& p, int tile_n, int sms, int
     g.n_stages = (avail - reserve) / g.stage_bytes;
     if (g.n_stages > st_cap) g.n_stages = st_cap;
     if (!g.b_resident) {
-        // a slot holds up to 32 KB of consecutive tiles (one wait and one commit per slot, not per MMA)
+        // a slot holds up to 32 KB of consecutive tiles (one wait and one commit per slot, not per MMA); where three do not fit beside the
+        // stages (a CTA pair reserves half as much for them), fewer stages make room, then smaller slots
         auto weight_slots = [&](int most) {
             g.b_group = 1;
             for (int i = 0; i < g.n_ph; ++i) {
@@ -248,8 +249,12 @@ inline PipeGeom pipe_geometry_with(const ConvParams& p, int tile_n, int sms, int
             g.b_slots = (budget - reserve - g.n_stages * g.stage_bytes) / (g.b_group * b_tile);
             return g.b_slots >= 3;
         };
-        const int most = 32768 / b_tile > g.kss * max_ph_taps ? g.kss * max_ph_taps : 32768 / b_tile;
-        if (!weight_slots(most)) return g;
+        int most = 32768 / b_tile > g.kss * max_ph_taps ? g.kss * max_ph_taps : 32768 / b_tile;
+        while (!weight_slots(most)) {
+            if (g.n_stages > 2) --g.n_stages;
+            else if (most > 1) most >>= 1;
+            else return g;
+        }
         if (g.b_slots > PIPE_MAX_BSLOTS) g.b_slots = PIPE_MAX_BSLOTS;
     }
     const int fixed = (g.b_resident ? g.b_total_bytes : g.b_slots * g.b_group * b_tile) + g.rows_bytes + 1024;

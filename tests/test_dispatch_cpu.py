@@ -63,3 +63,13 @@ def test_ring_of_packed_words_displaces_neither_weights_nor_words(ebs, layer, ti
     got = _route(ebs, *layer, terms=terms, tile=tile)
     assert {k: got[k] for k in want} == want, got
     assert got["raw_slots"] >= 2 and got["stages"] >= 2
+
+
+@pytest.mark.parametrize("layer", [
+    (1, 67, 182, 256, 1280, 3, 1, 4, 4), (1, 136, 105, 1792, 768, 3, 1, 6, 5), (1, 24, 112, 1984, 256, 3, 1, 3, 4), (1, 138, 57, 192, 256, 3, 1, 7, 5),
+    (1, 95, 41, 1280, 256, 1, 1, 8, 4),
+])
+def test_pair_of_thread_blocks_takes_streamed_layers(ebs, layer):
+    """Streamed weights beside the widest stages: three slots of the weight ring are made room for."""
+    got = _route(ebs, *layer, tile="pair")
+    assert got["weight_slots"] >= 3 and got["stages"] >= 2, got

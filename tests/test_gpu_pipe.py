@@ -112,6 +112,8 @@ def test_pipe_ragged_tiles_and_ring_slots(ebs, U, oracle, case, affine):
     (2, 1024, 512, 1, 1, 0, 24, 24, 8),   # deep reduction, two channel tiles, two accumulators per CTA
     (5, 128, 256, 3, 2, 1, 17, 16, 5),    # strided 3x3: four phase images
     (70, 64, 256, 1, 1, 0, 28, 28, 2),    # more pair-tiles than CTA pairs: the rings and both accumulator sets wrap
+    (1, 192, 256, 3, 1, 1, 25, 57, 7),    # streamed 3x3: stages make room for the ring of weight slots
+    (1, 1280, 256, 1, 1, 0, 35, 41, 8),   # streamed 1x1: the weight slots are halved
 ])
 def test_pipe_cta_pair(ebs, U, oracle, case):
     """The 256-channel tile on a pair of CTAs (one MMA of 256 pixels over two SMs, half a weight tile each): the last

@@ -178,16 +178,20 @@ static bool tile_kernel_pays(const ConvParams& p, int sms) {
 //  * 1x1 of 1024 channels on from 1.2 rounds, of 256 on from two: 2048 -> 512 at 7x7, batch 128 18.4 and 15.5; 1024 -> 256 at 14x14, batch 64 11.4
 //    and 11.0; 256 -> 64 at 56x56, batch 16 9.0 and 7.6; with per-channel terms of 2048 and 512: batch 128 20.1 and 18.4; 512 -> 128 at 28x28, batch 64
 //    16.4 and 15.1 (1024 -> 256, batch 64: 13.2 and 13.8; 256 -> 64: 10.5 and 10.4);
-//  * 1x1 of 5 to 7 planes, whose words come by tensor copies: 512 channels on from 0.6 rounds, 256 on from 1.2, any from two: 512 -> 128 at
-//    28x28, batch 16 10.1 and 7.6; 256 -> 1024 at 14x14, batch 16 9.8 and 8.3; 64 -> 64 at 56x56, batch 16 8.4 and 7.3 (256 -> 64, batch 8: 6.7 and 7.4).
+//  * 1x1 of 5 to 7 planes without terms.  Words by tensor copies: 512 channels on from 0.6 rounds, 256 on from 1.5, any from two: 512 -> 128 at 28x28,
+//    batch 16, 7 planes 10.1 and 7.6; 512 -> 256, 2.2 rounds 21.0 and 12.7; 256 -> 512, 5 planes, 1.6 rounds 9.4 and 8.2; 192 -> 256, 6 planes, 2.8
+//    rounds 9.2 and 8.4 (256 -> 256, 6 planes, 1.3 rounds: 5.4 and 6.9; 256 -> 1024, 7 planes, 1.35: 6.3 and 7.4).  Where a pixel is no whole 16
+//    bytes, so that they come 8 or 4 bytes a lane: 128 output channels on from 2.5 rounds: 160 -> 256, 7 planes, 2.8 rounds 16.9 and 10.3; 96 -> 512, 5
+//    planes 12.2 and 8.6 (608 -> 64, 7 planes, 1.6 rounds: 11.1 and 17.1; 1056 -> 128, 5 planes, 1.3: 15.0 and 18.6; 96 -> 128, 2.2: 7.0 and 7.6).
 static bool pipe_before_tile(const ConvParams& p, int sms) {
     if (!p.packed_next || p.acc || p.y || p.w_levels) return false;
     const double rounds = (double)((p.P + 127) / 128) * ((p.Co + 127) / 128) / sms;
     const bool terms = p.ch_scale || p.ch_bias || p.residual || p.res_packed;
     if (p.kh * p.kw > 1) return (p.sh > 1 || p.sw > 1) && p.CW >= 8 && rounds >= 1.2;
-    if (!terms && p.sh == 1 && p.sw == 1 && p.x_words >= 5 && p.x_words <= 7 &&
-        (rounds >= 2.0 || (rounds >= 1.2 && p.CW >= 8 && p.Co >= 128) || (rounds >= 0.6 && p.CW >= 16)))
-        return true;
+    if (!terms && p.sh == 1 && p.sw == 1 && p.x_words >= 5 && p.x_words <= 7) {
+        if (!conv_umma_pipe_copies(p, choose_pipe_variant(p))) return rounds >= 2.5 && p.Co >= 128;
+        return rounds >= 2.0 || (rounds >= 1.5 && p.CW >= 8 && p.Co >= 128) || (rounds >= 0.6 && p.CW >= 16);
+    }
     return (rounds >= 1.2 && p.CW >= (terms ? 64 : 32)) || (rounds >= 2.0 && p.CW >= (terms ? 16 : 8));
 }
 

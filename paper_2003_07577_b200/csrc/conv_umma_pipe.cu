@@ -55,6 +55,12 @@ bool conv_umma_pipe_applies(const ConvParams& p, int variant) {
     return variant >= 0 && variant < 3 && pipe_geometry(p, 64 << variant, pipe_sm_count(), p.pipe_m_sub).ok;
 }
 
+bool conv_umma_pipe_copies(const ConvParams& p, int variant) {
+    if (variant < 0 || variant > 2) return false;
+    const PipeGeom g = pipe_geometry(p, 64 << variant, pipe_sm_count(), p.pipe_m_sub);
+    return g.ok && g.tma;
+}
+
 void conv_umma_pipe_route(const ConvParams& p, int variant, int* route) {
     const PipeGeom g = pipe_geometry(p, variant == 3 ? 256 : 64 << variant, pipe_sm_count(), p.pipe_m_sub, variant == 3);
     const int values[] = {g.tma, g.m_sub, g.ks, g.kss, g.n_stages, g.b_resident, g.raw_slots, g.b_slots, g.n_ptiles * g.n_ctiles};

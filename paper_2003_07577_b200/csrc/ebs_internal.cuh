@@ -115,6 +115,7 @@ enum { NUM_CONV_UMMA_VARIANTS = 5, NUM_CONV_STRIP_VARIANTS = 5, NUM_CONV_RESIDEN
 const ConvVariant* conv_umma_pipe_variant(int a_bits, int variant);
 bool conv_umma_pipe_applies(const ConvParams& p, int variant);
 unsigned long long conv_umma_pipe_timeouts();
+bool conv_umma_pipe_copies(const ConvParams& p, int variant);          // its packed words arrive by tensor copies (variant -1: false)
 void conv_umma_pipe_route(const ConvParams& p, int variant, int* route);   // geometry of a variant that applies (ebs_test_conv_route)
 // Warp-level strip kernel for small stride-1 layers (conv_mma_strip.cu): channel tile 16 / 32 / 64.
 const ConvVariant* conv_mma_strip_variant(int a_bits, int variant);

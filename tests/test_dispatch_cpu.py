@@ -73,3 +73,16 @@ def test_pair_of_thread_blocks_takes_streamed_layers(ebs, layer):
     """Streamed weights beside the widest stages: three slots of the weight ring are made room for."""
     got = _route(ebs, *layer, tile="pair")
     assert got["weight_slots"] >= 3 and got["stages"] >= 2, got
+
+
+@pytest.mark.parametrize("layer,family", [
+    # n, h, w, c, co, k, stride, planes in, planes out; the faster family as measured (rounds of 128 x 128 tiles on 148 SMs)
+    ((4, 86, 86, 608, 64, 1, 1, 7, 7), "umma"), ((4, 115, 115, 544, 64, 1, 1, 7, 2), "umma"),          # no tensor copies: 1.6 and 2.8 rounds
+    ((4, 77, 78, 1056, 128, 1, 1, 5, 4), "umma"), ((4, 60, 60, 288, 256, 1, 1, 5, 4), "umma"),         # 1.3, 1.5
+    ((4, 115, 115, 64, 64, 1, 1, 7, 4), "umma"), ((4, 80, 81, 160, 256, 1, 1, 7, 7), "umma_pipe"),     # 2.8, 2.7
+    ((4, 54, 54, 256, 256, 1, 1, 6, 2), "umma"), ((4, 43, 43, 256, 512, 1, 1, 5, 7), "umma_pipe"),     # tensor copies: 1.2, 1.6
+    ((4, 71, 72, 512, 256, 1, 1, 5, 7), "umma_pipe"), ((16, 28, 28, 512, 128, 1, 1, 7, 4), "umma_pipe"),   # 2.2, 0.7
+])
+def test_layers_of_5_to_7_planes_run_on_the_faster_kernel(ebs, layer, family):
+    got = _route(ebs, *layer)
+    assert ebs.ebs_conv_variant_family(got["variant"]) == family, got

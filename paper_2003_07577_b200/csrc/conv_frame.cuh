@@ -175,15 +175,6 @@ __device__ __forceinline__ void bytes_to_planes(const uint32_t (&cr)[8], int nb,
     }
 }
 
-// fl(t) -> the bit pattern 0x4B000000 + clamp(floor(t), 0, qmax) without the conversion pipe and with one logic-pipe
-// instruction: t + |t| is 2 * max(t, 0) exactly, the minimum with 2 * qmax + 1 bounds it (floor and clamp commute for
-// integer bounds: floor(min(max(t, 0), qmax + 1/2)) = min(max(floor(t), 0), qmax)), and the halving and the 2^23 go into
-// one multiply-add rounded toward -inf, whose low mantissa bits are the floor.
-__device__ __forceinline__ uint32_t code_pattern(float t, float hi2) {
-    const float a = __fadd_rn(t, fabsf(t));
-    return __float_as_uint(__fmaf_rd(fminf(a, hi2), 0.5f, 8388608.0f));
-}
-
 // tcgen05.mma with both descriptors given as (low word, high word): the start-address field sits in the low word, so
 // an operand is moved by a 32-bit addition.  The whole warp executes the call with the same operands and the
 // instruction is predicated on `leader` (non-zero in one lane): with the issue loop free of divergent branches its

@@ -95,8 +95,7 @@ __device__ __forceinline__ void tmem_ld4_wait(uint32_t (&a)[4], uint32_t (&b)[4]
 // What the units of a layer share.
 struct FusedUnitEnv {
     uint64_t S2, PS2, rs2, one2, inv2;
-    float hi2;
-    int c_out, cap_out;
+    int out_bits, c_out, cap_out;
     uint8_t* dst;                                       // destination strip
     const uint8_t* res;                                 // strip of the identity shortcut
     const FusedTerms* T;
@@ -111,9 +110,7 @@ __device__ __forceinline__ uint64_t fused_byte_pair(uint32_t r, int j, uint64_t 
     return f32x2_add_one(f32x2_pack(lo, hi), one2, f32x2_pack(-8388608.0f, -8388608.0f));
 }
 __device__ __forceinline__ void fused_code(uint64_t w, const FusedUnitEnv& E, uint32_t& m0, uint32_t& m1) {
-    w = f32x2_add_one(f32x2_mul_rn(w, E.inv2), E.one2, f32x2_pack(0.5f, 0.5f));
-    m0 = code_pattern(__uint_as_float((uint32_t)w), E.hi2);
-    m1 = code_pattern(__uint_as_float((uint32_t)(w >> 32)), E.hi2);
+    code_pair<0>(f32x2_mul_rn(w, E.inv2), E.out_bits, m0, m1);
 }
 // The fp32 values of a unit's 16 channels at this thread's pixel, two to a register: wide layers w[2 e + j] = word 4 hf + e of
 // the 32-channel group, its bytes 2 j and 2 j + 1 (channels 8 i + 4 hf + e); narrow ones (all 16 channels in one unit) w[b] =
@@ -530,7 +527,7 @@ fused_resnet_kernel(const uint8_t* __restrict__ images, int img_h, int img_w, co
                 E.rs2 = f32x2_pack(L.res_step, L.res_step);
                 E.one2 = f32x2_pack(one, one);
                 E.inv2 = f32x2_pack(L.out_inv_step, L.out_inv_step);
-                E.hi2 = (float)(2 * ((1 << L.out_bits) - 1) + 1);
+                E.out_bits = L.out_bits;
                 const float PS = L.res == 2 ? s_rec[(li - 1) & (FUSED_RING - 1)].S : 0.0f;
                 E.PS2 = f32x2_pack(PS, PS);
                 E.c_out = L.c_out;

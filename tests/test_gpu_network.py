@@ -327,3 +327,51 @@ def test_resnet18_imagenet_forward_matches_the_oracle(ebs, U, oracle, gen):
     assert np.array_equal(logits[sample].cpu().numpy(), logits_ref)
     assert np.isfinite(logits_ref).all() and logits_ref.shape == (2, 1000)
     assert ebs.ebs_device_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("nb", [3, 8])
+def test_undefined_and_infinite_results_have_one_code(ebs, U, oracle, nb):
+    """Terms that are no finite numbers: a NaN becomes code 0 and an infinity the top code or 0 in every kernel, as in the integer-pipe
+    one (float -> integer conversion of a NaN is 0)."""
+    rng = np.random.default_rng(nb)
+    n, c, co, h, w = 2, 64, 128, 11, 9
+    d = U.desc_for(c, co, 3, 1, 1, 3, 4, 0.03, 0.07)
+    qa, qw = U.rand_codes(rng, (n, c, h, w), 4, False), rng.integers(-3, 4, size=(co, c, 3, 3), dtype=np.int32)
+    cs, cb = np.ones(co, np.float32), rng.uniform(-0.3, 0.3, co).astype(np.float32)
+    cs[5], cb[40], cb[41], cb[97] = np.nan, np.inf, -np.inf, np.nan
+    px, pw = U.pack_acts_codes(qa, 4), U.pack_weight_codes(qw, d)
+    epi = ebs.epilogue(_to(cs, U), _to(cb, U), None, True, nb, 0.7)
+    want = U.run_conv(qa, qw, d, epi, want_acc=False, next_bits=nb, variant=-2, px=px, pw=pw)["packed"]
+    codes = oracle.unpack_acts(want, co)
+    assert not codes[:, [5, 41, 97]].any() and (codes[:, 40] == (1 << nb) - 1).all() and codes[:, 6].any()
+    ran = set()
+    for variant in range(ebs.ebs_num_conv_variants()):
+        for want_y in (False, True):
+            if U.applies(d, h, w, variant, n=n, epi=epi, want_acc=False, want_y=want_y, want_packed=True):
+                out = U.run_conv(qa, qw, d, epi, want_acc=False, want_y=want_y, next_bits=nb, variant=variant, px=px, pw=pw)
+                assert np.array_equal(out["packed"], want), f"variant {variant}, fp32 results {want_y}"
+                ran.add(ebs.ebs_conv_variant_family(variant))
+    assert {"mma", "umma", "umma_pipe"} <= ran
+
+
+def test_whole_network_kernel_codes_undefined_values_as_its_layers_do(ebs):
+    from types import SimpleNamespace
+    from paper_2003_07577_b200 import network
+    g = torch.Generator(device="cuda")
+    g.manual_seed(11)
+    shapes = [("conv1", "first", 3, 16, 3, 1, 1, 16, 8), ("s1b1c1", "conv", 16, 16, 3, 1, 1, 16, 8), ("s1b1c2", "conv", 16, 16, 3, 1, 1, 16, 3),
+              ("s2b1c1", "conv", 16, 32, 3, 2, 1, 16, 4), ("s2b1c2", "conv", 32, 32, 3, 1, 1, 8, 8),
+              ("s2b1ds", "shortcut", 16, 32, 1, 2, 0, 16, 4), ("fc", "fc", 32, 10, 1, 1, 0, 1, 8)]
+    layers = [SimpleNamespace(name=n, role=r, c_in=ci, c_out=co, k=k, stride=s, pad=p, h_in=h, w_in=h, w_bits=3, a_bits=a,
+                              w_scale=0.05) for n, r, ci, co, k, s, p, h, a in shapes]
+    codes = {L.name: torch.randint(-4, 4, (L.c_out, L.c_in, L.k, L.k), generator=g, device="cuda", dtype=torch.int8) for L in layers}
+    x = torch.randint(0, 256, (3, 16, 16, 3), generator=g, device="cuda", dtype=torch.uint8)
+    plans = network.calibrated_plans(layers, codes, x)
+    plain = network.BasicBlockNet(plans).forward(x).clone()
+    for name, channel in (("conv1", 3), ("s1b1c1", 9), ("s2b1c1", 21)):
+        p = next(p for p in plans if p.name == name)
+        p.ch_bias = torch.zeros(p.desc.c_out, device="cuda") if p.ch_bias is None else p.ch_bias.clone()
+        p.ch_bias[channel] = float("nan")
+    want = network.BasicBlockNet(plans).forward(x).clone()
+    assert torch.isfinite(want).all() and not torch.equal(want, plain)
+    assert torch.equal(network.FusedBasicBlockNet(plans).forward(x), want)

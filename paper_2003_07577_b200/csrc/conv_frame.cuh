@@ -7,7 +7,7 @@
 namespace ebs {
 
 constexpr int FRAME_MAX_TAPS = 64, FRAME_MAX_PHASES = 4;
-constexpr int FRAME_MAX_CW = 1024;                 // 32-channel words of a pixel
+constexpr int FRAME_MAX_CW = 1024;                 // 32-channel words of a pixel: as far as the tile and the pipeline kernel are tested
 
 // Exact unsigned division by a run-time constant (Granlund and Montgomery, "Division by Invariant Integers using
 // Multiplication", 1994): q = (t + ((n - t) >> s1)) >> s2, t = mulhi(m, n).

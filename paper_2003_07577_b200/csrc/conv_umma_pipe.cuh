@@ -19,12 +19,13 @@
 //    m_sub MMAs and the halo of the strip is shared.
 //  * Weights stay resident in shared memory when all (tap, word) tiles of a channel tile fit, else they
 //    stream through the stage ring by cp.async.bulk, a stage ahead of the MMAs.
-//  * Roles (20 warps): warps 0-7 expand (packed words -> byte strips; the words arrive by cp.async in a ring of shared memory,
-//    two or three passes ahead), warps 8-9
+//  * Roles (20 warps, 28 where the 256-channel tile leaves as packed planes without per-channel terms): warps 0-7 expand (packed words ->
+//    byte strips; the words arrive in a ring of shared memory, one to three passes ahead: by the expanders' own cp.async, or, in
+//    pointwise layers of 3, 5, 6 or 7 planes whose pixels are whole 16 bytes, by tensor copies that warp 11 issues), warps 8-9
 //    issue the MMAs (two warps when a tile has an even number of accumulators: each owns the accumulators of one
 //    parity, so that one's waits and addresses run while the other issues), warp 10 fetches weight
-//    tiles (every lane one tile of a ring slot), warps 12-19 run the epilogue out of tensor memory while the next
-//    tile's MMAs fill the other accumulator set.
+//    tiles (every lane one tile of a ring slot), warps 12 on (eight, or sixteen) run the epilogue out of tensor memory while the
+//    next tile's MMAs fill the other accumulator set.
 //  * Bit <-> byte transposes by rotate and bit-select: with v_k = rotl(w_k, k) the byte register of
 //    channels {b, 8+b, 16+b, 24+b} is rotr(t_b, b), byte position (b+k) & 7 of t_b taken from v_k; the
 //    selects of plane pairs and quads are shared between the eight registers (planes_to_bytes), and the
@@ -97,7 +98,7 @@ struct PipeGeom : FrameGeom {
     int raw_bytes, rows_bytes;         // ring of packed words; rows of planes on their way out (pipe_rows_apply)
     int raw_words, raw_slots, raw_slot_bytes;   // words of a pixel in a slot of that ring (a multiple of ks)
     int ring_full;                     // by cp.async: 1: the ring has its full depth, in slots of PIPE_MAX_ITEMS items, 0: two slots of the strip's size
-    int tma;                           // 1: a slot arrives by a tensor copy (one box, two above 256 pixels), 0: by the expanders' own cp.async
+    int tma;                           // 1: a slot arrives by a tensor copy (one box; two where a tile has 512 pixels), 0: by the expanders' own cp.async
     int linear_in, linear_out;         // a frame pixel is the input pixel, the output pixel, of the same number
     int b_resident, b_total_bytes;
     PipeSlot slot[FRAME_MAX_PHASES];   // of each phase
@@ -635,7 +636,7 @@ __device__ __forceinline__ void pipe_epilogue_terms(const ConvParams& p, const F
 template <int AB, int TILE_N, bool AFFINE, int FORM, bool PAIR = false, bool SMALL = false>
 __global__ void __launch_bounds__(pipe_threads(pipe_epi_warps(TILE_N, AFFINE, FORM, PAIR)), 1) conv_umma_pipe_kernel(const ConvParams p, const PipeGeom g, const __grid_constant__ CUtensorMap words) {
     constexpr int EPI_WARPS = pipe_epi_warps(TILE_N, AFFINE, FORM, PAIR);
-    constexpr bool ROWS = FORM == 2;                           // planes of odd counts leave through rows in shared memory
+    constexpr bool ROWS = FORM == 2;                           // two groups' planes leave together through rows in shared memory
     // PAIR: the two CTAs of a cluster work as one.  Each expands its own 128 * m_sub pixels and holds the weight rows of
     // half the channel tile; the even CTA issues MMAs of M = 256 (cta_group::2) that read both CTAs' shared memory and
     // write both CTAs' tensor memory, so a weight byte is fetched from L2 once per 256 pixels instead of once per 128.

@@ -223,9 +223,9 @@ def test_context_path_refuses_what_it_cannot_run(ebs, U):
     assert err.value.status == ebs.EBS_ERR_UNSUPPORTED
 
 
-def test_pipe_declines_layers_wider_than_its_zero_page(ebs, U, oracle):
-    """The expanders read padding from a page of 8192 zero words, which has to cover a pixel's words at 8 planes: a layer
-    with more than 32768 input channels goes to another kernel family, and the library's own choice stays exact."""
+def test_pipe_declines_layers_of_more_than_32768_channels(ebs, U, oracle):
+    """A pixel of more than 1024 words goes to another kernel family (the bound of the tested range), and the library's own choice stays
+    exact."""
     c, co = 32768 + 64, 64
     d = U.desc_for(c, co, 1, 1, 0, 2, 2, 0.03, 0.07)
     for variant in U.variants_of("umma_pipe"):
@@ -264,6 +264,7 @@ def test_pipe_accumulators_at_the_conversion_bound(ebs, U, oracle, c):
     ref = oracle.conv2d_codes(qa, qw, (1, 1), (0, 0))
     S = oracle.combined_scale(0.03, 0.07)
     px, pw = U.pack_acts_codes(qa, 8), U.pack_weight_codes(qw, d)
+    ran = 0
     for nb in (4, 7, 8):
         for top in (float(np.abs(ref).max()) * float(S), float(np.percentile(np.abs(ref), 50)) * float(S)):
             step = np.float32(top / ((1 << nb) - 1))
@@ -273,6 +274,8 @@ def test_pipe_accumulators_at_the_conversion_bound(ebs, U, oracle, c):
                 if U.applies(d, h, w, variant, n=1, epi=epi, want_y=False, want_packed=True):
                     out = U.run_conv(qa, qw, d, epi, want_acc=False, want_y=False, next_bits=nb, variant=variant, px=px, pw=pw)
                     assert np.array_equal(out["packed"], oracle.pack_acts(q_ref, nb)), f"variant {variant}, {nb} planes"
+                    ran += 1
+    assert ran >= 18                                         # three channel tiles at least
     assert ebs.ebs_device_wait_timeouts() == 0
 
 
@@ -282,16 +285,21 @@ def test_pipe_words_by_tensor_copies(ebs, U, oracle, ab, case):
     """1x1 layers of plane counts whose packed words come by tensor copies: a last tile of a few pixels, a last group of fewer words, one
     and several tiles a thread block, resident and streamed weights (192 channels: by cp.async where a pixel is no whole 16 bytes)."""
     n, c, co, h, w = case
+    d = U.desc_for(c, co, 1, 1, 0, 4, ab)
+    copies = [ebs.ebs_test_conv_route(d, n, h, w, variant=v)["tensor_copies"] for v in U.variants_of("umma_pipe")[:3] if U.applies(d, h, w, v, n=n)]
+    assert any(copies) == (c // 32 * ab % 4 == 0)
     _check(ebs, U, oracle, n, c, co, 1, 1, 0, h, w, 4, ab, 4, min_variants=1)
 
 
-@pytest.mark.parametrize("case", [
-    (1, 256, 64, 1, 1, 199, 193, 4), (1, 256, 64, 1, 1, 195, 193, 4),      # just above and below two rounds of tiles on 148 SMs
-    (2, 64, 64, 1, 1, 139, 139, 7),                                        # two rounds, words by tensor copies
-    (1, 512, 128, 1, 1, 107, 107, 6), (1, 512, 128, 1, 1, 103, 103, 6),    # 0.6 rounds
-    (2, 256, 256, 3, 2, 151, 151, 3), (2, 256, 256, 3, 2, 147, 147, 3),    # strided 3x3, 1.2 rounds
+@pytest.mark.parametrize("case,family", [
+    ((1, 256, 64, 1, 1, 199, 193, 4), "umma_pipe"), ((1, 256, 64, 1, 1, 195, 193, 4), "umma"),     # two rounds of tiles on 148 SMs
+    ((2, 128, 64, 1, 1, 139, 139, 7), "umma_pipe"), ((2, 128, 64, 1, 1, 136, 136, 7), "umma"),     # two rounds, words by tensor copies
+    ((1, 256, 128, 1, 1, 168, 169, 5), "umma_pipe"), ((1, 256, 128, 1, 1, 166, 169, 5), "umma"),   # 1.5 rounds, by tensor copies
+    ((1, 512, 128, 1, 1, 107, 107, 6), "umma_pipe"), ((1, 512, 128, 1, 1, 103, 103, 6), "umma"),   # 0.6 rounds, by tensor copies
+    ((1, 96, 128, 1, 1, 217, 218, 5), "umma_pipe"), ((1, 96, 128, 1, 1, 215, 218, 5), "umma"),     # 2.5 rounds, pixels of no whole 16 bytes
+    ((2, 256, 256, 3, 2, 151, 151, 3), "umma_pipe"), ((2, 256, 256, 3, 2, 147, 147, 3), "umma"),   # strided 3x3, 1.2 rounds
 ])
-def test_pipe_and_tile_kernels_meet(ebs, U, case):
+def test_pipe_and_tile_kernels_meet(ebs, U, case, family):
     """The library's own choice on both sides of the lines between the tile and the pipeline kernel, against the integer-pipe kernel."""
     n, c, co, k, s, h, w, ab = case
     rng = np.random.default_rng(h * w)
@@ -301,6 +309,7 @@ def test_pipe_and_tile_kernels_meet(ebs, U, case):
     step = 0.03 * 0.07 * float(np.sqrt(c * k * k)) * 8.0 * (1 << ab) / 255.0
     px, pw = U.pack_acts_codes(qa, ab), U.pack_weight_codes(qw, d)
     epi = ebs.epilogue(None, None, None, True, 5, step)
+    assert ebs.ebs_conv_variant_family(ebs.ebs_test_conv_route(d, n, h, w, epi, False, False, True)["variant"]) == family
     own, literal = (U.run_conv(qa, qw, d, epi, want_acc=False, want_y=False, next_bits=5, variant=v, px=px, pw=pw)["packed"] for v in (-1, -2))
     assert literal.any() and np.array_equal(own, literal)
     assert ebs.ebs_device_wait_timeouts() == 0
@@ -325,4 +334,108 @@ def test_pipe_runs_where_the_driver_refuses_the_tensor_map(ebs, U, oracle, ab, c
     finally:
         ebs.ebs_test_set_device_wait(0, 0)
     assert ran >= 2
+    assert ebs.ebs_device_wait_timeouts() == 0
+
+
+def _check_packed_only(ebs, U, oracle, family, n, c, co, k, s, pad, h, w, wb, ab, nb, shortcut, min_variants):
+    """Packed planes as the only result, with per-channel terms and a shortcut, on every variant of a family."""
+    rng = np.random.default_rng(n + 3 * c + 5 * co + 7 * k + h + w + 16 * ab + nb)
+    qa = U.rand_codes(rng, (n, c, h, w), ab, False)
+    qw = rng.integers(-3, 4, size=(co, c, k, k), dtype=np.int32)
+    d = U.desc_for(c, co, k, s, pad, wb, ab, 0.02, 0.05)
+    acc = oracle.conv2d_codes(qa, qw, (s, s), (pad, pad))
+    S = oracle.combined_scale(0.02, 0.05)
+    cs, cb = rng.uniform(0.5, 2.0, co).astype(np.float32), rng.uniform(-0.3, 0.3, co).astype(np.float32)
+    to = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(U.dev())
+    res, extra = None, {}
+    if shortcut == "fp32":
+        res = rng.standard_normal(acc.shape).astype(np.float32)
+        extra = dict(residual=to(res.transpose(0, 2, 3, 1)))
+    elif shortcut != "none":
+        rb = int(shortcut)
+        q_res = U.rand_codes(rng, acc.shape, rb, False)
+        res = oracle.dequant_codes(q_res, 0.11)
+        extra = dict(res_packed=U.pack_acts_codes(q_res, rb), res_bits=rb, res_scale=0.11)
+    y0, _ = oracle.epilogue(acc, S, cs, cb, res, relu=True)
+    step = np.float32(max(float(np.percentile(y0, 98)), 1e-3) / ((1 << nb) - 1))
+    _, q_ref = oracle.epilogue(acc, S, cs, cb, res, relu=True, next_bits=nb, inv_next=np.float32(1.0) / step)
+    epi = ebs.epilogue(to(cs), to(cb), extra.pop("residual", None), True, nb, float(step), **extra)
+    px, pw, want = U.pack_acts_codes(qa, ab), U.pack_weight_codes(qw, d), oracle.pack_acts(q_ref, nb)
+    ran = 0
+    for variant in U.variants_of(family):
+        if not U.applies(d, h, w, variant, n=n, epi=epi, want_acc=False, want_packed=True):
+            continue
+        out = U.run_conv(qa, qw, d, epi, want_acc=False, next_bits=nb, variant=variant, px=px, pw=pw)
+        assert np.array_equal(out["packed"], want), f"variant {variant}, {nb} planes, shortcut {shortcut}"
+        ran += 1
+    assert ran >= min_variants
+    assert 0 < q_ref.mean() < (1 << nb) - 1
+    assert ebs.ebs_device_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("shortcut", ["fp32", "1", "4", "7", "8"])
+@pytest.mark.parametrize("nb", [2, 3, 4, 5, 6, 7, 8])
+def test_pipe_packed_only_with_shortcut(ebs, U, oracle, nb, shortcut):
+    """Terms and shortcut in the packed-only kernels, with planes stored directly and through rows of two groups (3 planes on the
+    256-channel tile, 5 to 7); frames with rows that have no output."""
+    _check_packed_only(ebs, U, oracle, "umma_pipe", 3, 64, 256, 3, 1, 1, 11, 13, 3, 4, nb, shortcut, 3)
+    _check_packed_only(ebs, U, oracle, "umma_pipe", 2, 96, 192, 1, 1, 0, 17, 9, 3, 5, nb, shortcut, 3)
+
+
+@pytest.mark.parametrize("shortcut", ["none", "fp32", "3"])
+@pytest.mark.parametrize("nb", range(1, 9))
+def test_tile_packed_only_planes(ebs, U, oracle, nb, shortcut):
+    """The tile kernel's packed epilogues: every output plane count with every kind of shortcut, whole and cut channel groups."""
+    _check_packed_only(ebs, U, oracle, "umma", 2, 64, 96, 3, 1, 1, 9, 7, 3, 4, nb, shortcut, 4)
+    _check_packed_only(ebs, U, oracle, "umma", 1, 160, 70, 1, 1, 0, 8, 9, 3, 2, nb, shortcut, 4)
+
+
+@pytest.mark.parametrize("exponent", [-62, -51, -50, 50, 51, 60])
+@pytest.mark.parametrize("nb", [4, 8])
+def test_pipe_scales_around_the_bound_of_unconverted_accumulators(ebs, U, oracle, exponent, nb):
+    """Accumulators are taken unconverted while both S and 1 / step lie in 2^-50 .. 2^50: combined scales at and beyond either end, with a step
+    of like size (1 / step beyond the other end) and of ordinary size."""
+    rng = np.random.default_rng(exponent + 100 + nb)
+    qa = U.rand_codes(rng, (1, 64, 9, 15), 4, False)
+    qw = rng.integers(-7, 8, size=(256, 64, 1, 1), dtype=np.int32)
+    sw, sa = float(2.0 ** exponent) * 1.25, 1.5
+    d = U.desc_for(64, 256, 1, 1, 0, 4, 4, sw, sa)
+    ref = oracle.conv2d_codes(qa, qw, (1, 1), (0, 0))
+    S = oracle.combined_scale(sw, sa)
+    px, pw = U.pack_acts_codes(qa, 4), U.pack_weight_codes(qw, d)
+    spread = set()
+    for step in (np.float32(np.percentile(np.abs(ref), 98) * float(S) / ((1 << nb) - 1)), np.float32(0.37)):
+        _, q_ref = oracle.epilogue(ref, S, None, None, None, relu=True, next_bits=nb, inv_next=np.float32(1.0) / step)
+        spread.add(int(q_ref.max()))
+        epi = ebs.epilogue(None, None, None, True, nb, float(step))
+        ran = 0
+        for variant in U.variants_of("umma_pipe"):
+            if U.applies(d, 9, 15, variant, n=1, epi=epi, want_acc=False, want_packed=True):
+                out = U.run_conv(qa, qw, d, epi, want_acc=False, next_bits=nb, variant=variant, px=px, pw=pw)
+                assert np.array_equal(out["packed"], oracle.pack_acts(q_ref, nb)), f"variant {variant}, step {step}"
+                ran += 1
+        assert ran >= 3
+    assert (1 << nb) - 1 in spread
+
+
+@pytest.mark.parametrize("ab,n,c,co,accumulators", [
+    (3, 1, 256, 64, 2), (5, 1, 256, 64, 2), (7, 1, 256, 64, 2), (3, 1, 256, 128, 2), (5, 1, 256, 128, 2), (7, 1, 256, 128, 2), (6, 1, 256, 128, 2),
+    (6, 2, 64, 64, 4), (5, 1, 512, 256, 1),
+])
+def test_pipe_tensor_copies_of_several_passes_a_slot(ebs, U, ab, n, c, co, accumulators):
+    """Slots of packed words that several expander passes use (tiles of 256 and 512 pixels, two boxes a slot at 512), as in ResNet layers at
+    their batch, against the integer-pipe kernel."""
+    rng = np.random.default_rng(ab + co)
+    h, w = (297, 300) if accumulators < 4 else (300, 300)
+    d = U.desc_for(c, co, 1, 1, 0, 4, ab, 0.03, 0.07)
+    epi = ebs.epilogue(None, None, None, True, 4, 0.03 * 0.07 * 16.0 * 8.0 * (1 << ab) / 15.0)
+    variant = U.variants_of("umma_pipe")[{64: 0, 128: 1, 256: 2}[co]]
+    route = ebs.ebs_test_conv_route(d, n, h, w, epi, False, False, True, variant)
+    assert route["tensor_copies"] == 1 and route["accumulators"] == accumulators
+    assert co == 256 or route["stage_words"] > route["pass_words"]
+    qa = U.rand_codes(rng, (n, c, h, w), ab, False)
+    qw = rng.integers(-8, 8, size=(co, c, 1, 1), dtype=np.int32)
+    px, pw = U.pack_acts_codes(qa, ab), U.pack_weight_codes(qw, d)
+    got, literal = (U.run_conv(qa, qw, d, epi, want_acc=False, next_bits=4, variant=v, px=px, pw=pw)["packed"] for v in (variant, -2))
+    assert literal.any() and np.array_equal(got, literal)
     assert ebs.ebs_device_wait_timeouts() == 0

@@ -30,23 +30,23 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
-// Bounded wait of a whole warp for the phase with the given parity; false = gave up (or another warp already had).  Lanes poll on their
-// own and the outcome is a vote at the end: lanes that left the caller's loop while others went on would meet those neither at the next
-// __syncwarp nor at the block's barrier.
+// Bounded wait of a whole warp for the phase with the given parity; false = gave up (or another warp already had).  The outcome is a
+// vote: lanes that left a loop at a poll of their own while others went on would meet those neither at the next __syncwarp
+// nor at the block's barrier.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                                   unsigned limit = UMMA_WAIT_LIMIT) {
     const uint32_t addr = smem_u32(bar);
-    uint32_t done = 0;
     for (unsigned it = 0; it < limit; ++it) {
+        uint32_t done;
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
             "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}\n"
             : "=r"(done) : "r"(addr), "r"(parity) : "memory");
-        if (done || *abort_flag) break;
+        if (__all_sync(0xffffffffu, done != 0)) return true;
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
         __nanosleep(it < 8 ? 40 : 200);   // leave the issue slots to the warps that have work
     }
-    if (__all_sync(0xffffffffu, done != 0)) return true;
     *abort_flag = 1;
     return false;
 }
